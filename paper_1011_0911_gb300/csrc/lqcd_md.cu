@@ -20,9 +20,18 @@
 //            Om = Lam - Lam^dag; a leaf f0 f1 f2 f3 whose factor f_j is the
 //            link contributes (c_sw / 8) U B Om A for f_j = U and
 //            -(c_sw / 8) B Om A U^dag for f_j = U^dag, A = f0..f_{j-1},
-//            B = f_{j+1}..f3;
+//            B = f_{j+1}..f3 (summed as in k_force_clover);
 //   gauge    S_g = beta sum_P (1 - Re tr U_P / 3): M = -(beta / 3) U sum
 //            (staples).
+//
+// Re tr(T_a M) = -Re tr(T_a M^dag) for the anti-Hermitian T_a, so a term that
+// ends in U^dag is traded for minus its adjoint, and every kernel collects one
+// matrix W with M = U W.
+//
+// The kernels are bound by GB300's FP64 pipe (2 multiply-adds per clock and
+// SM), not by their loads: what counts is the number of 3x3 products per link.
+// A block works on links of one direction and parity at consecutive ranks, so
+// directions never diverge within a warp and the link loads are coalesced.
 //
 // The leapfrog step (p -= dt/2 g; U <- exp(dt P) U; p -= dt/2 g, with
 // P = sum_a p^a T_a) exponentiates with a Taylor series after scaling and
@@ -57,13 +66,43 @@ __device__ __forceinline__ M3 m3_one()
     for (int i = 0; i < 3; i++) c.m[i][i] = mk(1.0, 0.0);
     return c;
 }
+// acc += a b, every product entering its sum through a fused multiply-add
+__device__ __forceinline__ void mul_add(M3 &acc, const M3 &a, const M3 &b)
+{
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            double re = acc.m[i][j].re, im = acc.m[i][j].im;
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                re = fmx(a.m[i][k].re, b.m[k][j].re, re);
+                re = fmx(-a.m[i][k].im, b.m[k][j].im, re);
+                im = fmx(a.m[i][k].re, b.m[k][j].im, im);
+                im = fmx(a.m[i][k].im, b.m[k][j].re, im);
+            }
+            acc.m[i][j] = mk(re, im);
+        }
+}
 __device__ __forceinline__ M3 mul(const M3 &a, const M3 &b)
 {
     M3 c;
 #pragma unroll
     for (int i = 0; i < 3; i++)
 #pragma unroll
-        for (int j = 0; j < 3; j++) c.m[i][j] = a.m[i][0] * b.m[0][j] + a.m[i][1] * b.m[1][j] + a.m[i][2] * b.m[2][j];
+        for (int j = 0; j < 3; j++) {
+            double re = a.m[i][0].re * b.m[0][j].re, im = a.m[i][0].re * b.m[0][j].im;
+            re = fmx(-a.m[i][0].im, b.m[0][j].im, re);
+            im = fmx(a.m[i][0].im, b.m[0][j].re, im);
+#pragma unroll
+            for (int k = 1; k < 3; k++) {
+                re = fmx(a.m[i][k].re, b.m[k][j].re, re);
+                re = fmx(-a.m[i][k].im, b.m[k][j].im, re);
+                im = fmx(a.m[i][k].re, b.m[k][j].im, im);
+                im = fmx(a.m[i][k].im, b.m[k][j].re, im);
+            }
+            c.m[i][j] = mk(re, im);
+        }
     return c;
 }
 __device__ __forceinline__ M3 dag(const M3 &a)
@@ -83,28 +122,25 @@ __device__ __forceinline__ void add_scaled(M3 &acc, double s, const M3 &a)
         for (int j = 0; j < 3; j++) acc.m[i][j] = acc.m[i][j] + s * a.m[i][j];
 }
 
-// host-built tables: gamma_mu, sigma_{rho sigma} (rho < sigma, planes 01 02 03
-// 12 13 23) and the Gell-Mann matrices, complex (re, im)
+// host-built table of the Gell-Mann matrices, complex (re, im)
 struct Tabs {
-    double2 gam[4][4][4];
-    double2 sig[6][4][4];
     double2 lam[8][3][3];
 };
 
 __device__ __forceinline__ Cd tc(const double2 &v) { return mk(v.x, v.y); }
 
-// g_a = Re tr(T_a M) = Re tr((i/2) lambda_a M)
-__device__ __forceinline__ void project_generators(const Tabs &T, const M3 &M, double g[8])
+// g_a = Re tr(T_a M) = -1/2 Im tr(lambda_a M), the entries of the Gell-Mann
+// matrices written out
+__device__ __forceinline__ void project_generators(const M3 &M, double g[8])
 {
-#pragma unroll
-    for (int a = 0; a < 8; a++) {
-        Cd t = mk(0.0, 0.0);
-#pragma unroll
-        for (int j = 0; j < 3; j++)
-#pragma unroll
-            for (int k = 0; k < 3; k++) t = t + tc(T.lam[a][j][k]) * M.m[k][j];
-        g[a] = -0.5 * t.im;   // Re(i t / 2)
-    }
+    g[0] = -0.5 * (M.m[1][0].im + M.m[0][1].im);
+    g[1] = -0.5 * (M.m[0][1].re - M.m[1][0].re);
+    g[2] = -0.5 * (M.m[0][0].im - M.m[1][1].im);
+    g[3] = -0.5 * (M.m[2][0].im + M.m[0][2].im);
+    g[4] = -0.5 * (M.m[0][2].re - M.m[2][0].re);
+    g[5] = -0.5 * (M.m[2][1].im + M.m[1][2].im);
+    g[6] = -0.5 * (M.m[1][2].re - M.m[2][1].re);
+    g[7] = -0.28867513459481288225 * (M.m[0][0].im + M.m[1][1].im - 2.0 * M.m[2][2].im);   // 1 / (2 sqrt 3)
 }
 
 __device__ __forceinline__ void site_coords(const Geom &g, long s, int x[4])
@@ -150,256 +186,306 @@ __device__ __forceinline__ void store_grad(double *gout, long l, const double gv
     for (int a = 0; a < 8; a++) gout[8 * l + a] = (accumulate ? gout[8 * l + a] : 0.0) + scale * gv[a];
 }
 
+// the link of this thread: direction and parity from the block's y index, rank
+// from x; false past the last rank
+__device__ __forceinline__ bool my_link(const Geom &g, int &mu, int &p, int &r, int x[4], long &l)
+{
+    mu = blockIdx.y >> 1;
+    p = blockIdx.y & 1;
+    r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= g.Vh) return false;
+    rank_coords(g, p, r, x);
+    l = 4 * site_index(g, x) + mu;
+    return true;
+}
+
 // ------------------------------------------------------------------ hops
+// h = psi_up + sgn e_mu psi_lo, the half spinor of (1 + sgn g_mu) psi
+__device__ __forceinline__ void half_spinor(int mu, double sgn, const Cd v[4][3], Cd h[2][3])
+{
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        const Cd l0 = v[2][c], l1 = v[3][c];
+        Cd e0, e1;
+        switch (mu) {
+            case 0: e0 = -l0; e1 = -l1; break;
+            case 1: e0 = timesmI(l1); e1 = timesmI(l0); break;
+            case 2: e0 = -l1; e1 = l0; break;
+            default: e0 = timesmI(l0); e1 = timesI(l1); break;
+        }
+        h[0][c] = mk(fmx(sgn, e0.re, v[0][c].re), fmx(sgn, e0.im, v[0][c].im));
+        h[1][c] = mk(fmx(sgn, e1.re, v[1][c].re), fmx(sgn, e1.im, v[1][c].im));
+    }
+}
+// acc[k][i] += a[k] conj(b[i])
+__device__ __forceinline__ void outer_add(M3 &acc, const Cd a[3], const Cd b[3])
+{
+#pragma unroll
+    for (int k = 0; k < 3; k++)
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            Cd &m = acc.m[k][i];
+            m.re = fmx(a[k].re, b[i].re, m.re);
+            m.re = fmx(a[k].im, b[i].im, m.re);
+            m.im = fmx(a[k].im, b[i].re, m.im);
+            m.im = fmx(-a[k].re, b[i].im, m.im);
+        }
+}
+
+// The lower half of (1 -+ g_mu) psi follows from the upper half h, so the spin
+// sums of B1 and B2 are sum_{s < 2} h_s(X) h_s(Y)^dag with the same projection
+// of both fields, and M = -1/2 s U (B1 + B2^dag).
 __global__ void __launch_bounds__(128) k_force_hop(Geom g, const double2 *__restrict__ U, const double2 *__restrict__ X,
                                                    const double2 *__restrict__ Y, double *gout, double scale,
-                                                   int accumulate, Tabs T)
+                                                   int accumulate)
 {
-    const long l = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (l >= 4L * g.V) return;
-    const long s = l >> 2;
-    const int mu = (int)(l & 3);
-    int x[4], y[4];
-    site_coords(g, s, x);
-    for (int i = 0; i < 4; i++) y[i] = x[i];
+    int mu, p, r, x[4];
+    long l;
+    if (!my_link(g, mu, p, r, x, l)) return;
+    int y[4] = {x[0], x[1], x[2], x[3]};
     shift(g, y, mu, +1);
-    const long sy = site_index(g, y);
+    const long s = site_index(g, x), sy = site_index(g, y);
     const double sgn = (mu == 0 && x[0] == g.L[0] - 1) ? double(g.bc_t) : 1.0;
-    const M3 u = link_at(g, U, x, mu);
-    Cd Xx[4][3], Xy[4][3], Yx[4][3], Yy[4][3];
-    spinor_at(X, s, Xx);
-    spinor_at(X, sy, Xy);
-    spinor_at(Y, s, Yx);
-    spinor_at(Y, sy, Yy);
-    M3 B1 = m3_zero(), B2 = m3_zero();
-#pragma unroll
-    for (int sp = 0; sp < 4; sp++) {
-        Cd a[3], b[3];   // [(1 - g_mu) X(x+mu)]_sp, [(1 + g_mu) X(x)]_sp
-#pragma unroll
-        for (int k = 0; k < 3; k++) {
-            a[k] = Xy[sp][k];
-            b[k] = Xx[sp][k];
-#pragma unroll
-            for (int t = 0; t < 4; t++) {
-                const Cd gm = tc(T.gam[mu][sp][t]);
-                a[k] = a[k] - gm * Xy[t][k];
-                b[k] = b[k] + gm * Xx[t][k];
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < 3; k++)
-#pragma unroll
-            for (int i = 0; i < 3; i++) {
-                B1.m[k][i] = B1.m[k][i] + a[k] * conjx(Yx[sp][i]);
-                B2.m[k][i] = B2.m[k][i] + b[k] * conjx(Yy[sp][i]);
-            }
-    }
-    M3 M = m3_zero();
-    add_scaled(M, -0.5 * sgn, mul(u, B1));
-    add_scaled(M, 0.5 * sgn, mul(B2, dag(u)));
+    M3 W = m3_zero();
+    Cd v[4][3], a[2][3], b[2][3];
+    // B1 = sum_s [(1 - g_mu) X(x+mu)]_s Y(x)_s^dag
+    spinor_at(X, sy, v);
+    half_spinor(mu, -1.0, v, a);
+    spinor_at(Y, s, v);
+    half_spinor(mu, -1.0, v, b);
+    outer_add(W, a[0], b[0]);
+    outer_add(W, a[1], b[1]);
+    // B2^dag = sum_s Y(x+mu)_s [(1 + g_mu) X(x)]_s^dag
+    spinor_at(Y, sy, v);
+    half_spinor(mu, +1.0, v, a);
+    spinor_at(X, s, v);
+    half_spinor(mu, +1.0, v, b);
+    outer_add(W, a[0], b[0]);
+    outer_add(W, a[1], b[1]);
     double gv[8];
-    project_generators(T, M, gv);
-    store_grad(gout, l, gv, scale, accumulate);
+    project_generators(mul(link_at(g, U, x, mu), W), gv);
+    store_grad(gout, l, gv, -0.5 * sgn * scale, accumulate);
 }
 
 // ------------------------------------------------------------------ clover
 // plane index of (rho, sigma), rho < sigma
 __device__ __forceinline__ int plane_of(int r, int s) { return r == 0 ? s - 1 : (r == 1 ? s + 1 : 5); }
 
-// Om[site][plane][9]: from X Y^dag (src = 0) or from A^-1 on the sites of
-// parity par (src = 1; other sites get zero)
+// Om[parity][plane][9][Vh].  In the chiral basis sigma is block diagonal, with
+// Pauli matrix s_k of the upper / lower block in the planes
+//   sigma_0k: +s_k / -s_k,   sigma_23, sigma_12: -s_1, -s_3 / -s_1, -s_3,
+//   sigma_13: +s_2 / +s_2,
+// so six colour matrices T_k^h = sum_ab (s_k)_ab N_ab (N_ab the colour block of
+// M between spins b and a of half h) give all planes: Lam = (i/4)(+-T^0 +-T^1),
+// Om = (i/4)(+-G^0 +-G^1) with G = T + T^dag.
+// G[k] = T_k + T_k^dag of one half from its N_ab
+__device__ __forceinline__ void pauli_sums(const M3 &n00, const M3 &n01, const M3 &n10, const M3 &n11, M3 G[3])
+{
+#pragma unroll
+    for (int k = 0; k < 3; k++)
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            // T1 = N01 + N10, T2 = -i N01 + i N10, T3 = N00 - N11
+            const Cd t1 = n01.m[k][i] + n10.m[k][i], t1t = n01.m[i][k] + n10.m[i][k];
+            const Cd t2 = timesI(n10.m[k][i] - n01.m[k][i]), t2t = timesI(n10.m[i][k] - n01.m[i][k]);
+            const Cd t3 = n00.m[k][i] - n11.m[k][i], t3t = n00.m[i][k] - n11.m[i][k];
+            G[0].m[k][i] = t1 + conjx(t1t);
+            G[1].m[k][i] = t2 + conjx(t2t);
+            G[2].m[k][i] = t3 + conjx(t3t);
+        }
+}
+
+// src = 0: M = X Y^dag on every site; src = 1: M = A^-1 on the sites of parity
+// par (blockIdx.y runs over the parities written)
 __global__ void __launch_bounds__(128) k_omega(Geom g, int src, const double2 *__restrict__ X,
                                                const double2 *__restrict__ Y, const double2 *__restrict__ Ai,
-                                               int par, double2 *Om, Tabs T)
+                                               int par, double2 *Om)
 {
-    const long s = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (s >= g.V) return;
-    int x[4];
-    site_coords(g, s, x);
-    const int p = (x[0] + x[1] + x[2] + x[3]) & 1;
-    Cd lam[6][3][3];
-#pragma unroll
-    for (int pl = 0; pl < 6; pl++)
-#pragma unroll
-        for (int k = 0; k < 3; k++)
-#pragma unroll
-            for (int i = 0; i < 3; i++) lam[pl][k][i] = mk(0.0, 0.0);
+    const int p = src == 0 ? (int)blockIdx.y : par;
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= g.Vh) return;
+    const long Vh = g.Vh;
+    M3 G[2][3];
     if (src == 0) {
+        int x[4];
+        rank_coords(g, p, r, x);
+        const long s = site_index(g, x);
         Cd Xs[4][3], Ys[4][3];
         spinor_at(X, s, Xs);
         spinor_at(Y, s, Ys);
-        for (int a = 0; a < 4; a++)
-            for (int b = 0; b < 4; b++) {
-                Cd m[3][3];   // M_{(b k),(a i)} = X[b][k] conj(Y[a][i])
 #pragma unroll
-                for (int k = 0; k < 3; k++)
+        for (int h = 0; h < 2; h++) {
+            M3 n[2][2];
 #pragma unroll
-                    for (int i = 0; i < 3; i++) m[k][i] = Xs[b][k] * conjx(Ys[a][i]);
+            for (int a = 0; a < 2; a++)
 #pragma unroll
-                for (int pl = 0; pl < 6; pl++) {
-                    const Cd sab = tc(T.sig[pl][a][b]);
-#pragma unroll
-                    for (int k = 0; k < 3; k++)
-#pragma unroll
-                        for (int i = 0; i < 3; i++) lam[pl][k][i] = lam[pl][k][i] + sab * m[k][i];
+                for (int b = 0; b < 2; b++) {
+                    n[a][b] = m3_zero();
+                    outer_add(n[a][b], Xs[2 * h + b], Ys[2 * h + a]);
                 }
-            }
-    } else if (p == par) {
-        const long Vh = g.Vh, r = s >> 1;
-        for (int h = 0; h < 2; h++) {   // chirality block: spins 2h, 2h+1
-            double d[6];
-            Cd o[15];
+            pauli_sums(n[0][0], n[0][1], n[1][0], n[1][1], G[h]);
+        }
+    } else {
+#pragma unroll
+        for (int h = 0; h < 2; h++) {   // packed Hermitian block: 6 real diagonal, 15 upper entries
             const double2 *bp = Ai + (long)(18 * h) * Vh + r;
+            double d[6];
+            Cd blk[6][6];
+#pragma unroll
             for (int q = 0; q < 3; q++) {
                 const double2 v = bp[q * Vh];
                 d[2 * q] = v.x;
                 d[2 * q + 1] = v.y;
             }
-            for (int q = 0; q < 15; q++) o[q] = tc(bp[(3 + q) * Vh]);
-            Cd blk[6][6];
             int kk = 0;
+#pragma unroll
             for (int i = 0; i < 6; i++) {
                 blk[i][i] = mk(d[i], 0.0);
+#pragma unroll
                 for (int j = i + 1; j < 6; j++) {
-                    blk[i][j] = o[kk];
-                    blk[j][i] = conjx(o[kk]);
-                    kk++;
+                    const Cd o = tc(bp[(3 + kk++) * Vh]);
+                    blk[i][j] = o;
+                    blk[j][i] = conjx(o);
                 }
             }
-            for (int al = 0; al < 2; al++)
-                for (int bl = 0; bl < 2; bl++) {
-                    const int a = 2 * h + al, b = 2 * h + bl;
-                    for (int pl = 0; pl < 6; pl++) {
-                        const Cd sab = tc(T.sig[pl][a][b]);
-                        for (int k = 0; k < 3; k++)
-                            for (int i = 0; i < 3; i++)
-                                lam[pl][k][i] = lam[pl][k][i] + sab * blk[3 * bl + k][3 * al + i];
-                    }
-                }
+            M3 n[2][2];
+#pragma unroll
+            for (int a = 0; a < 2; a++)
+#pragma unroll
+                for (int b = 0; b < 2; b++)
+#pragma unroll
+                    for (int k = 0; k < 3; k++)
+#pragma unroll
+                        for (int i = 0; i < 3; i++) n[a][b].m[k][i] = blk[3 * b + k][3 * a + i];
+            pauli_sums(n[0][0], n[0][1], n[1][0], n[1][1], G[h]);
         }
     }
-    // Lam = (i/4) sum, Om = Lam - Lam^dag
-#pragma unroll
-    for (int pl = 0; pl < 6; pl++)
-#pragma unroll
-        for (int k = 0; k < 3; k++)
-#pragma unroll
-            for (int i = 0; i < 3; i++) {
-                const Cd lk = timesI(lam[pl][k][i]), li = timesI(lam[pl][i][k]);
-                const Cd om = 0.25 * (lk - conjx(li));
-                Om[(s * 6 + pl) * 9 + 3 * k + i] = make_double2(om.re, om.im);
-            }
-}
-
-// factor q of leaf l in the ordered plane (rho, sigma) at y: offset (in rho,
-// sigma steps) of the link's site, its direction (0: rho, 1: sigma) and
-// whether it enters as U^dag.  The four leaves run the same way round.
-__device__ __forceinline__ void leaf_factor(int l, int q, int &dr, int &ds, int &dir, int &dg)
-{
-    // [leaf][factor] = (dr, ds, dir, dag)
-    const signed char tab[4][4][4] = {
-        {{0, 0, 0, 0}, {1, 0, 1, 0}, {0, 1, 0, 1}, {0, 0, 1, 1}},
-        {{0, 0, 1, 0}, {-1, 1, 0, 1}, {-1, 0, 1, 1}, {-1, 0, 0, 0}},
-        {{-1, 0, 0, 1}, {-1, -1, 1, 1}, {-1, -1, 0, 0}, {0, -1, 1, 0}},
-        {{0, -1, 1, 1}, {0, -1, 0, 0}, {1, -1, 1, 0}, {0, 0, 0, 1}},
+    double2 *op = Om + (long)p * 54 * Vh + r;
+    auto put = [&](int pl, int e, Cd t) {   // (i/4) t
+        op[(pl * 9L + e) * Vh] = make_double2(-0.25 * t.im, 0.25 * t.re);
     };
-    dr = tab[l][q][0];
-    ds = tab[l][q][1];
-    dir = tab[l][q][2];
-    dg = tab[l][q][3];
+#pragma unroll
+    for (int e = 0; e < 9; e++) {
+        const int k = e / 3, i = e % 3;
+        const Cd u0 = G[0][0].m[k][i], l0 = G[1][0].m[k][i], u1 = G[0][1].m[k][i], l1 = G[1][1].m[k][i],
+                 u2 = G[0][2].m[k][i], l2 = G[1][2].m[k][i];
+        put(0, e, u0 - l0);      // 01
+        put(1, e, u1 - l1);      // 02
+        put(2, e, u2 - l2);      // 03
+        put(3, e, -(u2 + l2));   // 12
+        put(4, e, u1 + l1);      // 13
+        put(5, e, -(u0 + l0));   // 23
+    }
 }
 
+__device__ __forceinline__ M3 om_at(const Geom &g, const double2 *__restrict__ Om, const int x[4], int pl)
+{
+    const int p = (x[0] + x[1] + x[2] + x[3]) & 1;
+    const double2 *b = Om + (long)(p * 54 + pl * 9) * g.Vh + coords_rank(g, x);
+    M3 m;
+#pragma unroll
+    for (int e = 0; e < 9; e++) m.m[e / 3][e % 3] = tc(b[e * (long)g.Vh]);
+    return m;
+}
+
+// The places where U_mu(x) sits in a clover leaf, summed.  The leaf of plane
+// (nu, mu) is the adjoint of that of (mu, nu) and Om changes sign with the
+// order, so the two orders contribute equally and one is taken, twice.  With
+// the staples a b c = U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag and
+// a' b' c' = U_nu(x+mu-nu)^dag U_mu(x-nu)^dag U_nu(x-nu), D = a b c - a' b' c'
+// and Om at the four corners of each staple, the eight leaves of a plane give
+//   W = Om(x+mu) D + D Om(x) + (a Om(x+mu+nu) b + a b Om(x+nu)) c
+//                            - (a' Om(x+mu-nu) b' + a' b' Om(x-nu)) c',
+// M = (c_sw / 4) U sum_nu (+-) W: 14 products a plane and 43 a link where the
+// sum over (order, leaf, place) took 288.  Om is nonzero on one parity only in
+// the log det force: SEL = 1 (the parity of x) and SEL = 2 (the other one) leave
+// out the products with zero.  Measured at 32 x 16^3: loading the field, the
+// clover term and the three forces 116.5 -> 14.1 ms (two of these kernels took
+// 105 ms of it).
+template <int SEL>
 __global__ void __launch_bounds__(64) k_force_clover(Geom g, const double2 *__restrict__ U,
                                                      const double2 *__restrict__ Om, double coef, double *gout,
-                                                     double scale, int accumulate, Tabs T)
+                                                     double scale, int accumulate, int par)
 {
-    const long l = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (l >= 4L * g.V) return;
-    const long s = l >> 2;
-    const int mu = (int)(l & 3);
+    constexpr bool AT_X = SEL != 2, AT_N = SEL != 1;   // Om nonzero at x, x+mu+-nu / at x+mu, x+-nu
+    const int mu = SEL == 0 ? blockIdx.y >> 1 : blockIdx.y;
+    const int p = SEL == 0 ? (int)(blockIdx.y & 1) : (SEL == 1 ? par : 1 - par);
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= g.Vh) return;
     int x[4];
-    site_coords(g, s, x);
-    const M3 u = link_at(g, U, x, mu);
-    M3 M = m3_zero();
-    for (int nu = 0; nu < 4; nu++) {
-        if (nu == mu) continue;
-        for (int ord = 0; ord < 2; ord++) {   // ordered planes (mu, nu) and (nu, mu)
-            const int rho = ord == 0 ? mu : nu, sg = ord == 0 ? nu : mu;
-            const int dirmu = ord == 0 ? 0 : 1;   // the link's role in the plane
-            const int pl = plane_of(min(rho, sg), max(rho, sg));
-            const double osign = rho < sg ? 1.0 : -1.0;   // Om_{sigma rho} = -Om_{rho sigma}
-            for (int lf = 0; lf < 4; lf++)
-                for (int j = 0; j < 4; j++) {
-                    int dr, ds, dir, dg;
-                    leaf_factor(lf, j, dr, ds, dir, dg);
-                    if (dir != dirmu) continue;
-                    // the leaf's site: x = y + dr rho + ds sigma
-                    int y[4] = {x[0], x[1], x[2], x[3]};
-                    shift(g, y, rho, -dr);
-                    shift(g, y, sg, -ds);
-                    M3 A = m3_one(), B = m3_one();
-                    for (int q = 0; q < 4; q++) {
-                        if (q == j) continue;
-                        int qr, qs, qd, qg;
-                        leaf_factor(lf, q, qr, qs, qd, qg);
-                        int z[4] = {y[0], y[1], y[2], y[3]};
-                        shift(g, z, rho, qr);
-                        shift(g, z, sg, qs);
-                        M3 f = link_at(g, U, z, qd == 0 ? rho : sg);
-                        if (qg) f = dag(f);
-                        if (q < j)
-                            A = mul(A, f);
-                        else
-                            B = mul(B, f);
-                    }
-                    M3 om;
-                    const double2 *op = Om + (site_index(g, y) * 6 + pl) * 9;
-#pragma unroll
-                    for (int e = 0; e < 9; e++) om.m[e / 3][e % 3] = osign * tc(op[e]);
-                    const M3 BOA = mul(mul(B, om), A);
-                    if (!dg)
-                        add_scaled(M, coef / 8.0, mul(u, BOA));
-                    else
-                        add_scaled(M, -coef / 8.0, mul(BOA, dag(u)));
-                }
+    rank_coords(g, p, r, x);
+    const long l = 4 * site_index(g, x) + mu;
+    M3 W = m3_zero();
+#pragma unroll 1
+    for (int k = 1; k < 4; k++) {
+        const int nu = (mu + k) & 3;
+        const int pl = plane_of(min(mu, nu), max(mu, nu));
+        int xm[4] = {x[0], x[1], x[2], x[3]};
+        shift(g, xm, mu, +1);
+        M3 Wn = m3_zero(), D;
+#pragma unroll 1
+        for (int dn = 0; dn < 2; dn++) {   // the staple at +nu, then the one at -nu
+            int ys[4] = {x[0], x[1], x[2], x[3]}, yn[4] = {x[0], x[1], x[2], x[3]}, xmn[4] = {xm[0], xm[1], xm[2], xm[3]};
+            shift(g, yn, nu, dn ? -1 : +1);    // the staple's mu link starts here
+            shift(g, xmn, nu, dn ? -1 : +1);   // and ends here
+            M3 a = link_at(g, U, dn ? xmn : xm, nu);
+            M3 c = link_at(g, U, dn ? yn : ys, nu);
+            if (dn)
+                a = dag(a);
+            else
+                c = dag(c);
+            const M3 b = dag(link_at(g, U, yn, mu));
+            const M3 ab = mul(a, b);
+            const M3 S = mul(ab, c);
+            M3 t;
+            if (AT_X) {
+                t = mul(mul(a, om_at(g, Om, xmn, pl)), b);
+                if (AT_N) mul_add(t, ab, om_at(g, Om, yn, pl));
+            } else {
+                t = mul(ab, om_at(g, Om, yn, pl));
+            }
+            if (dn == 0) {
+                D = S;
+                mul_add(Wn, t, c);
+            } else {
+                add_scaled(D, -1.0, S);
+                add_scaled(Wn, -1.0, mul(t, c));
+            }
         }
+        if (AT_X) mul_add(Wn, D, om_at(g, Om, x, pl));
+        if (AT_N) mul_add(Wn, om_at(g, Om, xm, pl), D);
+        add_scaled(W, mu < nu ? 1.0 : -1.0, Wn);   // Om_{nu mu} = -Om_{mu nu}
     }
     double gv[8];
-    project_generators(T, M, gv);
-    store_grad(gout, l, gv, scale, accumulate);
+    project_generators(mul(link_at(g, U, x, mu), W), gv);
+    store_grad(gout, l, gv, 0.25 * coef * scale, accumulate);
 }
 
 // ------------------------------------------------------------------ gauge
 __global__ void __launch_bounds__(128) k_force_gauge(Geom g, const double2 *__restrict__ U, double beta, double *gout,
-                                                     double scale, int accumulate, Tabs T)
+                                                     double scale, int accumulate)
 {
-    const long l = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (l >= 4L * g.V) return;
-    const long s = l >> 2;
-    const int mu = (int)(l & 3);
-    int x[4];
-    site_coords(g, s, x);
-    const M3 u = link_at(g, U, x, mu);
+    int mu, p, r, x[4];
+    long l;
+    if (!my_link(g, mu, p, r, x, l)) return;
     M3 st = m3_zero();
-    for (int nu = 0; nu < 4; nu++) {
-        if (nu == mu) continue;
+#pragma unroll 1
+    for (int k = 1; k < 4; k++) {
+        const int nu = (mu + k) & 3;
         int xm[4] = {x[0], x[1], x[2], x[3]}, xn[4] = {x[0], x[1], x[2], x[3]};
         shift(g, xm, mu, +1);
         shift(g, xn, nu, +1);
         // up: U_nu(x+mu) U_mu(x+nu)^dag U_nu(x)^dag
-        add_scaled(st, 1.0, mul(mul(link_at(g, U, xm, nu), dag(link_at(g, U, xn, mu))), dag(link_at(g, U, x, nu))));
+        mul_add(st, mul(link_at(g, U, xm, nu), dag(link_at(g, U, xn, mu))), dag(link_at(g, U, x, nu)));
         // down: U_nu(x+mu-nu)^dag U_mu(x-nu)^dag U_nu(x-nu)
         int xmn[4] = {xm[0], xm[1], xm[2], xm[3]}, xd[4] = {x[0], x[1], x[2], x[3]};
         shift(g, xmn, nu, -1);
         shift(g, xd, nu, -1);
-        add_scaled(st, 1.0,
-                   mul(mul(dag(link_at(g, U, xmn, nu)), dag(link_at(g, U, xd, mu))), link_at(g, U, xd, nu)));
+        mul_add(st, mul(dag(link_at(g, U, xmn, nu)), dag(link_at(g, U, xd, mu))), link_at(g, U, xd, nu));
     }
-    M3 M = m3_zero();
-    add_scaled(M, -beta / 3.0, mul(u, st));
     double gv[8];
-    project_generators(T, M, gv);
-    store_grad(gout, l, gv, scale, accumulate);
+    project_generators(mul(link_at(g, U, x, mu), st), gv);
+    store_grad(gout, l, gv, -beta / 3.0 * scale, accumulate);
 }
 
 // per-site sum over the six planes of 1 - Re tr U_P / 3
@@ -493,41 +579,6 @@ Tabs make_tabs()
 {
     Tabs T{};
     auto set = [](double2 &d, double re, double im) { d = make_double2(re, im); };
-    // chiral basis: g0 = [[0,-1],[-1,0]], gk = [[0,-i s_k],[i s_k,0]]
-    double re[4][4][4] = {}, im[4][4][4] = {};
-    re[0][0][2] = re[0][1][3] = re[0][2][0] = re[0][3][1] = -1;
-    // s1 = [[0,1],[1,0]]: -i s1 upper right, i s1 lower left
-    im[1][0][3] = im[1][1][2] = -1;
-    im[1][2][1] = im[1][3][0] = 1;
-    // s2 = [[0,-i],[i,0]]: -i s2 = [[0,-1],[1,0]], i s2 = [[0,1],[-1,0]]
-    re[2][0][3] = -1;
-    re[2][1][2] = 1;
-    re[2][2][1] = 1;
-    re[2][3][0] = -1;
-    // s3 = diag(1,-1): -i s3 = diag(-i, i), i s3 = diag(i, -i)
-    im[3][0][2] = -1;
-    im[3][1][3] = 1;
-    im[3][2][0] = 1;
-    im[3][3][1] = -1;
-    for (int m = 0; m < 4; m++)
-        for (int a = 0; a < 4; a++)
-            for (int b = 0; b < 4; b++) set(T.gam[m][a][b], re[m][a][b], im[m][a][b]);
-    // sigma_{rs} = (i/2) [g_r, g_s]
-    const int pr[6][2] = {{0, 1}, {0, 2}, {0, 3}, {1, 2}, {1, 3}, {2, 3}};
-    for (int pl = 0; pl < 6; pl++) {
-        const int r = pr[pl][0], s = pr[pl][1];
-        for (int a = 0; a < 4; a++)
-            for (int b = 0; b < 4; b++) {
-                double cr = 0, ci = 0;   // [g_r, g_s]_{ab}
-                for (int c = 0; c < 4; c++) {
-                    cr += re[r][a][c] * re[s][c][b] - im[r][a][c] * im[s][c][b];
-                    ci += re[r][a][c] * im[s][c][b] + im[r][a][c] * re[s][c][b];
-                    cr -= re[s][a][c] * re[r][c][b] - im[s][a][c] * im[r][c][b];
-                    ci -= re[s][a][c] * im[r][c][b] + im[s][a][c] * re[r][c][b];
-                }
-                set(T.sig[pl][a][b], -0.5 * ci, 0.5 * cr);   // (i/2)(cr + i ci)
-            }
-    }
     // Gell-Mann matrices
     const double r3 = 1.0 / std::sqrt(3.0);
     set(T.lam[0][0][1], 1, 0);
@@ -556,7 +607,8 @@ const Tabs &tabs()
     return T;
 }
 
-int grid_links(const lqcd_ctx *c, int tpb) { return div_up(4L * c->g.V, tpb); }
+// one block row per (direction, parity)
+dim3 grid_links(const lqcd_ctx *c, int tpb, int rows = 8) { return dim3(div_up(c->g.Vh, tpb), rows); }
 
 lqcd_status need_state(lqcd_ctx *c)
 {
@@ -569,20 +621,19 @@ lqcd_status need_state(lqcd_ctx *c)
 lqcd_status force_dD(lqcd_ctx *c, const double *X, const double *Y, double *g, double scale, int accumulate)
 {
     LQCD_TRY(need_state(c));
-    const Tabs &T = tabs();
     k_force_hop<<<grid_links(c, 128), 128, 0, c->stream>>>(c->g, c->U64, (const double2 *)X, (const double2 *)Y, g,
-                                                           scale, accumulate, T);
+                                                           scale, accumulate);
     c->n_kernel_launches++;
     LQCD_LAUNCH_CHECK(c);
     if (c->csw != 0.0) {
         void *om;
         LQCD_TRY(ws_get(c, WS_MD_OMEGA, (size_t)c->g.V * 6 * 9 * sizeof(double2), &om));
-        k_omega<<<div_up(c->g.V, 128), 128, 0, c->stream>>>(c->g, 0, (const double2 *)X, (const double2 *)Y, nullptr, 0,
-                                                            (double2 *)om, T);
+        k_omega<<<grid_links(c, 128, 2), 128, 0, c->stream>>>(c->g, 0, (const double2 *)X, (const double2 *)Y, nullptr,
+                                                              0, (double2 *)om);
         c->n_kernel_launches++;
         LQCD_LAUNCH_CHECK(c);
-        k_force_clover<<<grid_links(c, 64), 64, 0, c->stream>>>(c->g, c->U64, (const double2 *)om, c->csw, g, scale, 1,
-                                                                T);
+        k_force_clover<0><<<grid_links(c, 64), 64, 0, c->stream>>>(c->g, c->U64, (const double2 *)om, c->csw, g, scale,
+                                                                   1, 0);
         c->n_kernel_launches++;
         LQCD_LAUNCH_CHECK(c);
     }
@@ -597,16 +648,17 @@ lqcd_status force_logdet(lqcd_ctx *c, int parity, double *g, double scale, int a
         if (!accumulate) LQCD_TRY(blas_zero(c, (size_t)c->g.V * 32 * sizeof(double), g));
         return LQCD_OK;
     }
-    const Tabs &T = tabs();
     void *om;
     LQCD_TRY(ws_get(c, WS_MD_OMEGA, (size_t)c->g.V * 6 * 9 * sizeof(double2), &om));
-    k_omega<<<div_up(c->g.V, 128), 128, 0, c->stream>>>(c->g, 1, nullptr, nullptr, c->Ai64[parity], parity,
-                                                        (double2 *)om, T);
+    k_omega<<<grid_links(c, 128, 1), 128, 0, c->stream>>>(c->g, 1, nullptr, nullptr, c->Ai64[parity], parity,
+                                                          (double2 *)om);
     c->n_kernel_launches++;
     LQCD_LAUNCH_CHECK(c);
-    k_force_clover<<<grid_links(c, 64), 64, 0, c->stream>>>(c->g, c->U64, (const double2 *)om, c->csw, g, scale,
-                                                            accumulate, T);
-    c->n_kernel_launches++;
+    k_force_clover<1><<<grid_links(c, 64, 4), 64, 0, c->stream>>>(c->g, c->U64, (const double2 *)om, c->csw, g, scale,
+                                                                  accumulate, parity);
+    k_force_clover<2><<<grid_links(c, 64, 4), 64, 0, c->stream>>>(c->g, c->U64, (const double2 *)om, c->csw, g, scale,
+                                                                  accumulate, parity);
+    c->n_kernel_launches += 2;
     LQCD_LAUNCH_CHECK(c);
     return LQCD_OK;
 }
@@ -614,7 +666,7 @@ lqcd_status force_logdet(lqcd_ctx *c, int parity, double *g, double scale, int a
 lqcd_status force_gauge(lqcd_ctx *c, double beta, double *g, double scale, int accumulate)
 {
     if (!c->have_gauge) return set_err(c, LQCD_ERR_STATE, "gauge field not set");
-    k_force_gauge<<<grid_links(c, 128), 128, 0, c->stream>>>(c->g, c->U64, beta, g, scale, accumulate, tabs());
+    k_force_gauge<<<grid_links(c, 128), 128, 0, c->stream>>>(c->g, c->U64, beta, g, scale, accumulate);
     c->n_kernel_launches++;
     LQCD_LAUNCH_CHECK(c);
     return LQCD_OK;
