@@ -1,6 +1,7 @@
-// Wilson-clover stencil kernels on native (site-minor) layouts: the
-// single-field form and the dispatch of D, Dhat (Eq. 1, Eq. 2) over it and
-// the register-blocked multi-field form (lqcd_dirac_mr.cu).
+// Wilson-clover stencil kernels on native (site-minor) layouts: the float
+// single-field form and the dispatch of D, Dhat (Eq. 1, Eq. 2) over it, the
+// register-blocked multi-field form (lqcd_dirac_mr.cu), the staged form
+// (lqcd_dirac_sm.cu) and the FP64 form (lqcd_dirac_d.cu).
 //
 // One thread per (output site, right-hand side).  A CTA is blockDim.x sites
 // by blockDim.y right-hand sides, so a warp reads 32 consecutive sites of one
@@ -153,7 +154,13 @@ std::vector<TuneChoice> hop_candidates(int nrhs)
 }
 
 // LQCD_HOP_KIND = hop | mr | sm restricts the search to one kernel form
-// (test instrumentation; ignored where that form does not exist)
+// (test instrumentation; ignored where that form does not exist, as in FP64),
+// LQCD_HOP_KIND = d1 | d2 | d4 the FP64 search to one split G
+int hop_force_split()
+{
+    const char *e = getenv("LQCD_HOP_KIND");
+    return e && e[0] == 'd' && (e[1] == '1' || e[1] == '2' || e[1] == '4') && !e[2] ? e[1] - '0' : 0;
+}
 int hop_force_kind(bool has_alt, int nrhs)
 {
     const char *e = getenv("LQCD_HOP_KIND");
@@ -214,6 +221,20 @@ std::vector<TuneChoice> hop_mr_candidates(int nrhs)
     return v;
 }
 
+// FP64 splits: 2 G threads per site (nr = G)
+std::vector<TuneChoice> hop_d_candidates(int only)
+{
+    std::vector<TuneChoice> v;
+    for (int G : {1, 2, 4})
+        if (only == 0 || only == G) {
+            TuneChoice t;
+            t.kind = KIND_D;
+            t.nr = G;
+            v.push_back(t);
+        }
+    return v;
+}
+
 template <class R, class SP, class LK, class CL, int MODE>
 lqcd_status launch_choice(lqcd_ctx *c, const TuneChoice &t, const HopArgs<SP, LK, CL> &a)
 {
@@ -221,7 +242,10 @@ lqcd_status launch_choice(lqcd_ctx *c, const TuneChoice &t, const HopArgs<SP, LK
         if (t.kind == KIND_MR) return launch_hop_mr<R, SP, LK, CL, MODE>(c, t.nr, t.variant, dim3(t.tx, t.ty), a);
         if (t.kind == KIND_SM) return launch_hop_sm<R, SP, LK, CL, MODE>(c, t.variant, dim3(t.tx, t.ty), a);
     }
-    return launch_var<R, SP, LK, CL, MODE>(c, t.variant, dim3(t.tx, t.ty), a);
+    if constexpr (std::is_same<R, double>::value)
+        return launch_hop_d<MODE>(c, t.nr, a);
+    else
+        return launch_var<R, SP, LK, CL, MODE>(c, t.variant, dim3(t.tx, t.ty), a);
 }
 
 template <class R, class SP, class LK, class CL, int MODE>
@@ -240,17 +264,25 @@ lqcd_status launch_hop(lqcd_ctx *c, int p_out, const SP *in_other, long in_rs, c
     a.out_rs = out_rs;
     a.U = U;
     a.clov = clov;
-    const int prec = sizeof(R) == 8 ? 0 : (std::is_same<SP, h16s>::value ? 2 : 1);
+    constexpr bool dbl = std::is_same<R, double>::value;
+    const int prec = dbl ? 0 : (std::is_same<SP, h16s>::value ? 2 : 1);
     constexpr bool has_alt = std::is_same<R, float>::value && MODE != MODE_HOP;
     const int force = hop_force_kind(has_alt, nrhs);
     static const char *kname[3] = {"k_hop4_hop", "k_hop4_mr", "k_hop4_sm"};
-    std::string key = tune_key(c, force >= 0 ? kname[force] : "k_hop4", MODE, prec, nrhs);
+    static const char *dname[5] = {"k_hop_d", "k_hop_d1", "k_hop_d2", "", "k_hop_d4"};
+    const int split = dbl ? hop_force_split() : 0;
+    std::string key = tune_key(c, dbl ? dname[split] : (force >= 0 ? kname[force] : "k_hop4"), MODE, prec, nrhs);
     TuneChoice tc;
     if (!tune_lookup(key, &tc)) {
         tc = TuneChoice();
         tc.tx = nrhs == 1 ? 128 : 32;
         tc.ty = nrhs == 1 ? 1 : std::min(nrhs, 8);
-        if (force == KIND_MR) {
+        if (dbl) {
+            // without timings: split until each of the 608 schedulers has two warps
+            const long w = (long)c->g.Vh * nrhs / 16;
+            tc.kind = KIND_D;
+            tc.nr = split ? split : (w >= 1216 ? 1 : (w >= 608 ? 2 : 4));
+        } else if (force == KIND_MR) {
             tc.kind = KIND_MR;
             tc.nr = 2;
             tc.tx = 64;
@@ -263,7 +295,10 @@ lqcd_status launch_hop(lqcd_ctx *c, int p_out, const SP *in_other, long in_rs, c
         if (tune_enabled()) {
             float best = 1e30f;
             std::vector<TuneChoice> cands;
-            if (force < 0 || force == KIND_HOP) cands = hop_candidates(nrhs);
+            if (dbl)
+                cands = hop_d_candidates(split);
+            else if (force < 0 || force == KIND_HOP)
+                cands = hop_candidates(nrhs);
             if (has_alt && (force < 0 || force == KIND_MR))
                 for (const TuneChoice &m : hop_mr_candidates(nrhs)) cands.push_back(m);
             if (has_alt && (force < 0 || force == KIND_SM))

@@ -393,7 +393,10 @@ template <class R, class SP, class LK, class CL, int MODE>
 lqcd_status launch_hop_sm(lqcd_ctx *c, int var, dim3 b, const HopArgs<SP, LK, CL> &a);
 constexpr int NVAR_SM = 3;
 inline int var_sm_max_threads(int v) { return v == 2 ? 256 : 384; }
+// FP64 form (lqcd_dirac_d.cu): 2 G threads per site, G = 1, 2, 4; every mode
+template <int MODE>
+lqcd_status launch_hop_d(lqcd_ctx *c, int G, const HopArgs<double2, double2, double2> &a);
 // kernel forms known to the autotuner
-enum { KIND_HOP = 0, KIND_MR = 1, KIND_SM = 2 };
+enum { KIND_HOP = 0, KIND_MR = 1, KIND_SM = 2, KIND_D = 3 };
 
 }  // namespace stencil
