@@ -117,6 +117,7 @@ __device__ __forceinline__ void site_of(const Geom &g, int nsub, long i, int &p,
     }
 }
 
+// any alignment of the canonical field (k_pack_t wants 16 bytes)
 template <class CT, int PREC>
 __global__ void k_pack(Geom g, int nsub, int nrhs, const CT *__restrict__ canon, void *native, int unpack)
 {
@@ -169,6 +170,112 @@ __global__ void k_pack(Geom g, int nsub, int nrhs, const CT *__restrict__ canon,
             }
         }
     }
+}
+
+// The same through shared memory: the canonical side of a tile of 64 sites is one
+// contiguous run, read or written in 16-byte words by consecutive threads; on
+// the native side a warp takes one word of 32 consecutive ranks of one parity.
+// HBM (L2 on small lattices) bounds it; in k_pack every canonical word of a warp
+// lies in its own sector row.  The odd pitch keeps both sides free of bank
+// conflicts.  Measured, pack / unpack, against k_pack: FP64 48 x 24^3 52 -> 20 / 18 us
+// (127 MB, 6.4 - 7 TB/s), 8^4 4.9 -> 2.2 us, FP32 D fields 28 x 12 x 10 x 14, 5
+// right-hand sides 20 -> 9 / 6 us.
+template <int PREC>
+struct PackT {
+    using W = float4;                      // 16-byte word of the canonical field
+    static constexpr int U = 6;            // words per site
+};
+template <>
+struct PackT<LQCD_F64> {
+    using W = double2;
+    static constexpr int U = 12;
+};
+constexpr int PACK_SITES = 64, PACK_THREADS = 128;
+
+template <int PREC, bool UNPACK>
+__global__ void __launch_bounds__(PACK_THREADS) k_pack_t(Geom g, int nsub, typename PackT<PREC>::W *canon, void *native)
+{
+    using W = typename PackT<PREC>::W;
+    constexpr int U = PackT<PREC>::U, LD = U + 1;
+    __shared__ W tile[PACK_SITES * LD];
+    const long Vh = g.Vh, nsite = nsub * Vh, i0 = (long)blockIdx.x * PACK_SITES;
+    const int ns = (int)min((long)PACK_SITES, nsite - i0), k = blockIdx.y;
+    W *cs = canon + (k * nsite + i0) * U;
+    if (!UNPACK) {
+        for (int e = threadIdx.x; e < ns * U; e += PACK_THREADS) tile[(e / U) * LD + e % U] = cs[e];
+        __syncthreads();
+    }
+    // slot t of the tile on the native side: nsub = 1: site t; nsub = 2: parity t / 32,
+    // pair of sites t % 32 (a pair holds one site of each parity)
+    auto slot = [&](int t, int &sl, long &h, long &r) {
+        if (nsub == 1) {
+            sl = t;
+            h = k;
+            r = i0 + t;
+            return t < ns;
+        }
+        const int p = t >> 5, j = t & 31;
+        r = (i0 >> 1) + j;
+        h = 2L * k + p;
+        if (2 * j >= ns) return false;
+        int x[4];
+        rank_coords(g, p, (int)r, x);
+        sl = 2 * j + (x[3] & 1);
+        return true;
+    };
+    if constexpr (PREC == LQCD_F16S) {
+        const int t = threadIdx.x;
+        int sl;
+        long h, r;
+        if (t < PACK_SITES && slot(t, sl, h, r)) {
+            h16s *n = (h16s *)native + h * f16s_half_units(Vh);
+            cx<float> v[12];
+            if (UNPACK) {
+                f16s_load<false>(n, Vh, r, v);
+#pragma unroll
+                for (int q = 0; q < 6; q++)
+                    tile[sl * LD + q] = make_float4(v[2 * q].re, v[2 * q].im, v[2 * q + 1].re, v[2 * q + 1].im);
+            } else {
+#pragma unroll
+                for (int q = 0; q < 6; q++) {
+                    const float4 w = tile[sl * LD + q];
+                    v[2 * q] = mk(w.x, w.y);
+                    v[2 * q + 1] = mk(w.z, w.w);
+                }
+                f16s_store(n, Vh, r, v);
+            }
+        }
+    } else {
+        const int t = threadIdx.x % PACK_SITES;
+        int sl;
+        long h, r;
+        if (slot(t, sl, h, r)) {
+            W *n = (W *)native + h * U * Vh + r;
+#pragma unroll
+            for (int q = threadIdx.x / PACK_SITES; q < U; q += PACK_THREADS / PACK_SITES) {
+                if (UNPACK)
+                    tile[sl * LD + q] = n[q * Vh];
+                else
+                    n[q * Vh] = tile[sl * LD + q];
+            }
+        }
+    }
+    if (UNPACK) {
+        __syncthreads();
+        for (int e = threadIdx.x; e < ns * U; e += PACK_THREADS) cs[e] = tile[(e / U) * LD + e % U];
+    }
+}
+
+template <int PREC>
+void launch_pack_t(lqcd_ctx *c, int nsub, const void *canon, void *native, int nrhs, bool unpack)
+{
+    using W = typename PackT<PREC>::W;
+    const dim3 grid(div_up((long)nsub * c->g.Vh, PACK_SITES), nrhs);
+    W *w = (W *)canon;
+    if (unpack)
+        k_pack_t<PREC, true><<<grid, PACK_THREADS, 0, c->stream>>>(c->g, nsub, w, native);
+    else
+        k_pack_t<PREC, false><<<grid, PACK_THREADS, 0, c->stream>>>(c->g, nsub, w, native);
 }
 
 // native F64 <-> native F32 (same site/chunk structure), nhalf half fields
@@ -276,18 +383,25 @@ lqcd_status pack_field(lqcd_ctx *c, lqcd_prec p, int nsub, const void *canon, vo
 {
     if (nsub != 1 && nsub != 2) return set_err(c, LQCD_ERR_ARG, "nsub must be 1 or 2");
     if (nrhs < 1 || nrhs > 65535) return set_err(c, LQCD_ERR_ARG, "bad nrhs %d", nrhs);
+    if (p != LQCD_F64 && p != LQCD_F32 && p != LQCD_F16S)
+        return set_err(c, LQCD_ERR_ARG, "pack: precision %d has no canonical form", (int)p);
     dim3 grid(div_up((long)nsub * c->g.Vh, 256), nrhs);
-    if (p == LQCD_F64)
+    if ((uintptr_t)canon % 16 == 0) {
+        if (p == LQCD_F64)
+            launch_pack_t<LQCD_F64>(c, nsub, canon, native, nrhs, unpack);
+        else if (p == LQCD_F32)
+            launch_pack_t<LQCD_F32>(c, nsub, canon, native, nrhs, unpack);
+        else
+            launch_pack_t<LQCD_F16S>(c, nsub, canon, native, nrhs, unpack);
+    } else if (p == LQCD_F64)
         k_pack<double, LQCD_F64><<<grid, 256, 0, c->stream>>>(c->g, nsub, nrhs, (const double *)canon, native,
                                                                unpack);
     else if (p == LQCD_F32)
         k_pack<float, LQCD_F32><<<grid, 256, 0, c->stream>>>(c->g, nsub, nrhs, (const float *)canon, native,
                                                              unpack);
-    else if (p == LQCD_F16S)
+    else
         k_pack<float, LQCD_F16S><<<grid, 256, 0, c->stream>>>(c->g, nsub, nrhs, (const float *)canon, native,
                                                                unpack);
-    else
-        return set_err(c, LQCD_ERR_ARG, "pack: precision %d has no canonical form", (int)p);
     c->n_kernel_launches++;
     LQCD_LAUNCH_CHECK(c);
     return LQCD_OK;
