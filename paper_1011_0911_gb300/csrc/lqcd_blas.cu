@@ -13,10 +13,7 @@ constexpr int DOT_CHUNK = 8;
 __global__ void k_axpy(long n, double ar, double ai, const double2 *__restrict__ x, double2 *y)
 {
     for (long j = blockIdx.x * (long)blockDim.x + threadIdx.x; j < n; j += (long)gridDim.x * blockDim.x) {
-        double2 a = x[j], b = y[j];
-        b.x += ar * a.x - ai * a.y;
-        b.y += ar * a.y + ai * a.x;
-        y[j] = b;
+        y[j] = caxpy(make_double2(ar, ai), x[j], y[j]);
     }
 }
 __global__ void k_xpay(long n, const double2 *__restrict__ x, double ar, double2 *y)
@@ -40,24 +37,6 @@ __global__ void k_sub(long n, const double2 *__restrict__ x, const double2 *__re
         z[j] = make_double2(a.x - b.x, a.y - b.y);
     }
 }
-// y += sign * sum_i c_i X_i  (c complex, up to 64 terms)
-struct Coefs {
-    double c[2 * 64];
-};
-__global__ void k_multi_axpy(long n, int k, Coefs cf, const double2 *__restrict__ X, long stride, double2 *y,
-                             double sign)
-{
-    for (long j = blockIdx.x * (long)blockDim.x + threadIdx.x; j < n; j += (long)gridDim.x * blockDim.x) {
-        double2 b = y[j];
-        double sr = 0, si = 0;
-        for (int i = 0; i < k; i++) {
-            double2 a = X[i * stride + j];
-            sr += cf.c[2 * i] * a.x - cf.c[2 * i + 1] * a.y;
-            si += cf.c[2 * i] * a.y + cf.c[2 * i + 1] * a.x;
-        }
-        y[j] = make_double2(b.x + sign * sr, b.y + sign * si);
-    }
-}
 // gamma5 = diag(1,1,-1,-1): negate spins 2,3 = complex components 6..11
 __global__ void k_gamma5_64(long Vh, long nhalf, const double2 *__restrict__ in, double2 *out)
 {
@@ -75,74 +54,67 @@ __global__ void k_gamma5_64(long Vh, long nhalf, const double2 *__restrict__ in,
 inline int grid_for(long n) { return (int)std::min<long>(4 * 152, (n + 255) / 256); }
 
 // ---------------------------------------------------------------- batched
-// partial[(r*nb + b)*64 + i] = block b's share of <A_{i,r}, B_r>
+// partial[(r*nb + b)*64 + i] = block b's share of <A_{i,r}, B_r>, k0 <= i < k0 + kn,
+// kn <= KN.  NORM: KN = 1 and A = B, the real part alone.  FP64-pipe bound: 4
+// multiply-adds per element and vector; the CTA's reduction is kept short
+// (warp_multi_sum), as the 608 CTAs of a launch repeat it.
+template <int KN, bool NORM>
 __global__ void __launch_bounds__(RED_THREADS) k_bdot_partial(long n, const double2 *__restrict__ A, long sa,
                                                               long fa, const double2 *__restrict__ B, long fb,
                                                               int k0, int kn, double2 *partial)
 {
     const int r = blockIdx.y;
     const double2 *Br = B + r * fb;
-    const double2 *Ar = A + r * fa;
-    double re[DOT_CHUNK], im[DOT_CHUNK];
+    const double2 *Ar = A + r * fa + k0 * sa;
+    double v[2 * KN];   // re, im of each vector
 #pragma unroll
-    for (int i = 0; i < DOT_CHUNK; i++) re[i] = im[i] = 0;
+    for (int i = 0; i < 2 * KN; i++) v[i] = 0;
     const long st = (long)gridDim.x * blockDim.x;
     long j = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (kn <= 2) {
+    if (KN <= 2) {
         // few vectors: four grid-strided elements per pass, their loads issued
         // together (one element per pass leaves too few loads in flight to
         // cover the memory latency)
         for (; j + 3 * st < n; j += 4 * st) {
-            double2 b[4], a0[4], a1[4];
+            double2 b[4], a[KN][4];
 #pragma unroll
             for (int u = 0; u < 4; u++) {
                 b[u] = Br[j + u * st];
-                a0[u] = Ar[k0 * sa + j + u * st];
-                if (kn == 2) a1[u] = Ar[(k0 + 1) * sa + j + u * st];
+#pragma unroll
+                for (int i = 0; i < KN; i++)
+                    if (!NORM) a[i][u] = Ar[i * sa + j + u * st];
             }
 #pragma unroll
-            for (int u = 0; u < 4; u++) {
-                re[0] += a0[u].x * b[u].x + a0[u].y * b[u].y;
-                im[0] += a0[u].x * b[u].y - a0[u].y * b[u].x;
-                if (kn == 2) {
-                    re[1] += a1[u].x * b[u].x + a1[u].y * b[u].y;
-                    im[1] += a1[u].x * b[u].y - a1[u].y * b[u].x;
+            for (int u = 0; u < 4; u++)
+#pragma unroll
+                for (int i = 0; i < KN; i++) {
+                    if (NORM)
+                        v[0] = norm_add(v[0], b[u]);
+                    else
+                        cdot_add(v[2 * i], v[2 * i + 1], a[i][u], b[u]);
                 }
-            }
         }
     }
     for (; j < n; j += st) {
-        double2 b = Br[j];
+        const double2 b = Br[j];
+        if (NORM) {
+            v[0] = norm_add(v[0], b);
+        } else {
 #pragma unroll
-        for (int i = 0; i < DOT_CHUNK; i++)
-            if (i < kn) {
-                double2 a = Ar[(k0 + i) * sa + j];
-                re[i] += a.x * b.x + a.y * b.y;
-                im[i] += a.x * b.y - a.y * b.x;
-            }
-    }
-    __shared__ double sh[RED_THREADS / 32][DOT_CHUNK][2];
-    int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i < DOT_CHUNK; i++) {
-        double x = re[i], m = im[i];
-        for (int o = 16; o > 0; o >>= 1) {
-            x += __shfl_down_sync(0xffffffffu, x, o);
-            m += __shfl_down_sync(0xffffffffu, m, o);
-        }
-        if (lane == 0) {
-            sh[warp][i][0] = x;
-            sh[warp][i][1] = m;
+            for (int i = 0; i < KN; i++)
+                if (i < kn) cdot_add(v[2 * i], v[2 * i + 1], Ar[i * sa + j], b);
         }
     }
+    __shared__ double sh[RED_THREADS / 32][2 * KN];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    warp_multi_sum(v);
+    constexpr int L = 32 / (2 * KN);   // lanes holding the same value
+    if (lane % L == 0) sh[warp][lane / L] = v[0];
     __syncthreads();
-    if (threadIdx.x < kn) {
-        double x = 0, m = 0;
-        for (int w = 0; w < RED_THREADS / 32; w++) {
-            x += sh[w][threadIdx.x][0];
-            m += sh[w][threadIdx.x][1];
-        }
-        partial[((long)r * gridDim.x + blockIdx.x) * 64 + k0 + threadIdx.x] = make_double2(x, m);
+    if (threadIdx.x < 2 * kn) {
+        double x = 0;
+        for (int w = 0; w < RED_THREADS / 32; w++) x += sh[w][threadIdx.x];
+        reinterpret_cast<double *>(partial + ((long)r * gridDim.x + blockIdx.x) * 64 + k0)[threadIdx.x] = x;
     }
 }
 // one CTA per (vector i, rhs r): fixed-order tree over the nb partial sums
@@ -183,14 +155,11 @@ __global__ void k_bmulti_axpy(long n, int k, const __grid_constant__ CoefParam c
     const double2 *Xr = X + r * fa;
     double2 *yr = y + r * fy;
     for (long j = blockIdx.x * (long)blockDim.x + threadIdx.x; j < n; j += (long)gridDim.x * blockDim.x) {
-        double2 b = yr[j];
-        double sr = 0, si = 0;
-        for (int i = 0; i < k; i++) {
-            double2 a = Xr[i * sa + j], ci = c[i];
-            sr += ci.x * a.x - ci.y * a.y;
-            si += ci.x * a.y + ci.y * a.x;
-        }
-        yr[j] = make_double2(b.x + sign * sr, b.y + sign * si);
+        double2 s = make_double2(0, 0);
+#pragma unroll 4
+        for (int i = 0; i < k; i++) s = caxpy(c[i], Xr[i * sa + j], s);
+        const double2 b = yr[j];
+        yr[j] = make_double2(fmx(sign, s.x, b.x), fmx(sign, s.y, b.y));
     }
 }
 
@@ -203,14 +172,11 @@ __global__ void k_bmulti_axpy_dev(long n, int k, const double2 *__restrict__ cf,
     const double2 *Xr = X + r * fa;
     double2 *yr = y + r * fy;
     for (long j = blockIdx.x * (long)blockDim.x + threadIdx.x; j < n; j += (long)gridDim.x * blockDim.x) {
-        double2 b = yr[j];
-        double sr = 0, si = 0;
-        for (int i = 0; i < k; i++) {
-            double2 a = Xr[i * sa + j], ci = c[i];
-            sr += ci.x * a.x - ci.y * a.y;
-            si += ci.x * a.y + ci.y * a.x;
-        }
-        yr[j] = make_double2(b.x + sign * sr, b.y + sign * si);
+        double2 s = make_double2(0, 0);
+#pragma unroll 4
+        for (int i = 0; i < k; i++) s = caxpy(c[i], Xr[i * sa + j], s);
+        const double2 b = yr[j];
+        yr[j] = make_double2(fmx(sign, s.x, b.x), fmx(sign, s.y, b.y));
     }
 }
 
@@ -430,6 +396,29 @@ __global__ void k_bmulti_axpy_mixed(long Vh, int k, const __grid_constant__ Coef
 
 }  // namespace
 
+namespace {
+// the dot products <A_i, B>, i < k, in launches of up to DOT_CHUNK vectors
+void bdot_partials(lqcd_ctx *c, int nb, long n, int nrhs, const double2 *A, long sa, long fa, const double2 *B, long fb,
+                   int k, double2 *partial)
+{
+    const dim3 grid(nb, nrhs);
+    for (int k0 = 0; k0 < k; k0 += DOT_CHUNK) {
+        const int kn = std::min(DOT_CHUNK, k - k0);
+        if (kn == 1 && k == 1 && A == B && fa == fb)
+            k_bdot_partial<1, true><<<grid, RED_THREADS, 0, c->stream>>>(n, A, sa, fa, B, fb, k0, kn, partial);
+        else if (kn == 1)
+            k_bdot_partial<1, false><<<grid, RED_THREADS, 0, c->stream>>>(n, A, sa, fa, B, fb, k0, kn, partial);
+        else if (kn == 2)
+            k_bdot_partial<2, false><<<grid, RED_THREADS, 0, c->stream>>>(n, A, sa, fa, B, fb, k0, kn, partial);
+        else if (kn <= 4)
+            k_bdot_partial<4, false><<<grid, RED_THREADS, 0, c->stream>>>(n, A, sa, fa, B, fb, k0, kn, partial);
+        else
+            k_bdot_partial<DOT_CHUNK, false><<<grid, RED_THREADS, 0, c->stream>>>(n, A, sa, fa, B, fb, k0, kn, partial);
+        c->n_kernel_launches++;
+    }
+}
+}  // namespace
+
 // as bblas_dot, results left in device memory: out_dev[r*k + i] (complex)
 lqcd_status bblas_dot_dev(lqcd_ctx *c, long n2, int nrhs, const double *A, long sa, long fa, const double *B, long fb,
                           int k, double2 *out_dev)
@@ -440,12 +429,7 @@ lqcd_status bblas_dot_dev(lqcd_ctx *c, long n2, int nrhs, const double *A, long 
     int nb = std::max(1, (int)std::min<long>(std::max(8, 4 * 152 / nrhs), (n + 255) / 256));
     nb = std::min(nb, 4096 / nrhs);
     double2 *partial = (double2 *)c->red;
-    for (int k0 = 0; k0 < k; k0 += DOT_CHUNK) {
-        int kn = std::min(DOT_CHUNK, k - k0);
-        k_bdot_partial<<<dim3(nb, nrhs), RED_THREADS, 0, c->stream>>>(n, (const double2 *)A, sa / 2, fa / 2,
-                                                                      (const double2 *)B, fb / 2, k0, kn, partial);
-        c->n_kernel_launches++;
-    }
+    bdot_partials(c, nb, n, nrhs, (const double2 *)A, sa / 2, fa / 2, (const double2 *)B, fb / 2, k, partial);
     k_bdot_final<<<dim3(k, nrhs), 256, 0, c->stream>>>(nb, k, partial, out_dev);
     c->n_kernel_launches++;
     LQCD_LAUNCH_CHECK(c);
@@ -475,12 +459,7 @@ lqcd_status bblas_dot(lqcd_ctx *c, long n2, int nrhs, const double *A, long sa, 
     int nb = std::max(1, (int)std::min<long>(std::max(8, 4 * 152 / nrhs), (n + 255) / 256));
     nb = std::min(nb, 4096 / nrhs);
     double2 *partial = (double2 *)c->red;   // nrhs * nb * 64 double2 <= 4096 * 64 (sized at create)
-    for (int k0 = 0; k0 < k; k0 += DOT_CHUNK) {
-        int kn = std::min(DOT_CHUNK, k - k0);
-        k_bdot_partial<<<dim3(nb, nrhs), RED_THREADS, 0, c->stream>>>(n, (const double2 *)A, sa / 2, fa / 2,
-                                                                      (const double2 *)B, fb / 2, k0, kn, partial);
-        c->n_kernel_launches++;
-    }
+    bdot_partials(c, nb, n, nrhs, (const double2 *)A, sa / 2, fa / 2, (const double2 *)B, fb / 2, k, partial);
     k_bdot_final<<<dim3(k, nrhs), 256, 0, c->stream>>>(nb, k, partial, (double2 *)c->red_out);
     c->n_kernel_launches++;
     LQCD_LAUNCH_CHECK(c);
@@ -570,16 +549,7 @@ lqcd_status blas_zero(lqcd_ctx *c, size_t bytes, void *p)
 lqcd_status blas_multi_axpy(lqcd_ctx *c, long n2, int k, const double *coef_host, const double *X, long stride,
                             double *y, double sign)
 {
-    if (k < 1) return LQCD_OK;
-    if (k > 64) return set_err(c, LQCD_ERR_ARG, "multi_axpy: k=%d", k);
-    Coefs cf;
-    for (int i = 0; i < 2 * k; i++) cf.c[i] = coef_host[i];
-    long n = n2 / 2;
-    k_multi_axpy<<<grid_for(n), 256, 0, c->stream>>>(n, k, cf, (const double2 *)X, stride / 2, (double2 *)y,
-                                                     sign);
-    c->n_kernel_launches++;
-    LQCD_LAUNCH_CHECK(c);
-    return LQCD_OK;
+    return bblas_multi_axpy(c, n2, 1, k, coef_host, X, stride, 0, y, 0, sign);
 }
 lqcd_status blas_gamma5_native64(lqcd_ctx *c, long nhalf, const double2 *in, double2 *out)
 {

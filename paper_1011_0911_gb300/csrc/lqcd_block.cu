@@ -153,8 +153,7 @@ __global__ void __launch_bounds__(256) k_bdot(long Vh, int hb, int nch, const in
 #pragma unroll
             for (int q = 0; q < 12; q++) {
                 const double2 u = d.a[j][q * Vh + r], v = d.b[j][q * Vh + r];
-                re[j] += u.x * v.x + u.y * v.y;
-                im[j] += u.x * v.y - u.y * v.x;
+                cdot_add(re[j], im[j], u, v);
             }
     }
     __shared__ double sh[8][ND][2];
@@ -305,10 +304,6 @@ __global__ void k_bs_end(int nblk, BState *S)
 }
 
 // ---- elementwise updates on the even sites of active blocks
-__device__ __forceinline__ double2 cfma(double2 a, double2 x, double2 y)   // y + a x
-{
-    return make_double2(y.x + a.x * x.x - a.y * x.y, y.y + a.x * x.y + a.y * x.x);
-}
 // p = r + beta (p - omega v)
 __global__ void k_bu_p(long Vh, const int *blk, const BState *S, const double2 *r, const double2 *v, double2 *p)
 {
@@ -316,8 +311,8 @@ __global__ void k_bu_p(long Vh, const int *blk, const BState *S, const double2 *
     if (i >= 12 * Vh) return;
     const BState &s = S[blk[i % Vh]];
     if (!s.active) return;
-    const double2 w = cfma(make_double2(-s.omega.x, -s.omega.y), v[i], p[i]);
-    p[i] = cfma(s.beta, w, r[i]);
+    const double2 w = caxpy(make_double2(-s.omega.x, -s.omega.y), v[i], p[i]);
+    p[i] = caxpy(s.beta, w, r[i]);
 }
 // s = r - alpha v
 __global__ void k_bu_s(long Vh, const int *blk, const BState *S, const double2 *r, const double2 *v, double2 *sv)
@@ -326,7 +321,7 @@ __global__ void k_bu_s(long Vh, const int *blk, const BState *S, const double2 *
     if (i >= 12 * Vh) return;
     const BState &s = S[blk[i % Vh]];
     if (!s.active) return;
-    sv[i] = cfma(make_double2(-s.alpha.x, -s.alpha.y), v[i], r[i]);
+    sv[i] = caxpy(make_double2(-s.alpha.x, -s.alpha.y), v[i], r[i]);
 }
 // x += alpha p (+ omega s); r = s - omega t
 __global__ void k_bu_xr(long Vh, const int *blk, const BState *S, const double2 *p, const double2 *sv,
@@ -337,11 +332,11 @@ __global__ void k_bu_xr(long Vh, const int *blk, const BState *S, const double2 
     const BState &s = S[blk[i % Vh]];
     if (!s.active) return;
     if (s.half) {
-        x[i] = cfma(s.alpha, p[i], x[i]);
+        x[i] = caxpy(s.alpha, p[i], x[i]);
         return;
     }
-    x[i] = cfma(s.omega, sv[i], cfma(s.alpha, p[i], x[i]));
-    r[i] = cfma(make_double2(-s.omega.x, -s.omega.y), t[i], sv[i]);
+    x[i] = caxpy(s.omega, sv[i], caxpy(s.alpha, p[i], x[i]));
+    r[i] = caxpy(make_double2(-s.omega.x, -s.omega.y), t[i], sv[i]);
 }
 __global__ void k_bsub(long n, const double2 *a, const double2 *b, double2 *out)
 {

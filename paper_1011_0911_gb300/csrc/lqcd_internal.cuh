@@ -51,6 +51,48 @@ __device__ __forceinline__ cx<R> cmulc(cx<R> a, cx<R> b)
 __device__ __forceinline__ float fmx(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fmx(double a, double b, double c) { return __fma_rn(a, b, c); }
 
+// (re, im) += conj(a) b and += c x with one fused multiply-add per real product
+// (a sum of products written out compiles to a product, a fused multiply-add
+// and an addition: half as much again on the FP64 pipe that bounds FP64 BLAS)
+__device__ __forceinline__ void cdot_add(double &re, double &im, double2 a, double2 b)
+{
+    re = fmx(a.x, b.x, re);
+    re = fmx(a.y, b.y, re);
+    im = fmx(a.x, b.y, im);
+    im = fmx(-a.y, b.x, im);
+}
+__device__ __forceinline__ double2 caxpy(double2 c, double2 x, double2 y)   // y + c x
+{
+    y.x = fmx(c.x, x.x, y.x);
+    y.x = fmx(-c.y, x.y, y.x);
+    y.y = fmx(c.x, x.y, y.y);
+    y.y = fmx(c.y, x.x, y.y);
+    return y;
+}
+__device__ __forceinline__ double norm_add(double n, double2 a) { return fmx(a.y, a.y, fmx(a.x, a.x, n)); }
+
+// Warp sums of V = 1, 2, 4, 8 or 16 values in V - 1 + 5 - log2 V additions (a
+// butterfly over each takes 5 V): in each step a lane hands half of its values
+// to its partner and adds the partner's other half to what it keeps.  On
+// return v[0] is the sum of value lane * V / 32.
+template <int V>
+__device__ __forceinline__ void warp_multi_sum(double (&v)[V])
+{
+    const int lane = threadIdx.x & 31;
+    int off = 16;
+#pragma unroll
+    for (int h = V / 2; h >= 1; h /= 2, off /= 2) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int j = 0; j < h; j++) {
+            const double send = up ? v[j] : v[j + h];
+            v[j] = (up ? v[j + h] : v[j]) + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+    }
+#pragma unroll
+    for (; off > 0; off /= 2) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+}
+
 // third row of an SU(3) matrix from the first two, u2 = (u0 x u1)^*, each real
 // part one product and three fused multiply-adds
 template <class R>
