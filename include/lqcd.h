@@ -299,9 +299,10 @@ typedef struct {
 } lqcd_solve_info;
 
 /* Solve Dhat psi_e = eta_e (Eq. 2) for nrhs even fields to a true relative
- * residual <= tol.  CGNR works on Dhat directly; the GCR solvers solve the
- * full system D chi = (eta_e, 0) and return psi_e = chi_e (Eq. 5), then
- * check the Dhat residual in FP64 and tighten the tolerance when needed.
+ * residual <= tol.  CGNR and the GCR solvers work on even fields: the GCR
+ * preconditions (rho_e, 0) on the full lattice, keeps the even half of the
+ * result (the even half of the solution of D chi = (eta_e, 0) is psi_e, Eq. 5)
+ * and stops on the FP64 residual eta_e - Dhat psi_e.
  * eta_e, psi_e: nrhs canonical FP64 even fields.  info: host array of nrhs
  * entries (may be NULL).  Returns the worst per-RHS status. */
 LQCD_API lqcd_status lqcd_solve_dhat(lqcd_ctx *ctx, const lqcd_solver_params *p, const double *eta_dev,

@@ -180,6 +180,93 @@ __global__ void k_bmulti_axpy_dev(long n, int k, const double2 *__restrict__ cf,
     }
 }
 
+// CTA sums of V values per thread, then slot o[0..V-1]
+template <int V>
+__device__ __forceinline__ void cta_sums(double (&v)[V], double *o)
+{
+    __shared__ double sh[RED_THREADS / 32][V];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    warp_multi_sum(v);
+    if (lane % (32 / V) == 0) sh[warp][lane / (32 / V)] = v[0];
+    __syncthreads();
+    if (threadIdx.x < V) {
+        double x = 0;
+        for (int w = 0; w < RED_THREADS / 32; w++) x += sh[w][threadIdx.x];
+        o[threadIdx.x] = x;
+    }
+}
+
+// |x_r|^2 and <rho_r, x_r> as partial[(r*nb + b)*64 + {0, 1}]: 6 multiply-adds per
+// element, where two dot products against x take 8
+__global__ void __launch_bounds__(RED_THREADS) k_norm_rdot64_partial(long n, const double2 *__restrict__ X, long fx,
+                                                                     const double2 *__restrict__ R, long fr,
+                                                                     double2 *partial)
+{
+    const int r = blockIdx.y;
+    const double2 *Xr = X + r * fx, *Rr = R + r * fr;
+    double v[4] = {0, 0, 0, 0};
+    const long st = (long)gridDim.x * blockDim.x;
+    long j = blockIdx.x * (long)blockDim.x + threadIdx.x;
+    for (; j + 3 * st < n; j += 4 * st) {
+        double2 x[4], u[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            x[q] = Xr[j + q * st];
+            u[q] = Rr[j + q * st];
+        }
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            v[0] = norm_add(v[0], x[q]);
+            cdot_add(v[2], v[3], u[q], x[q]);
+        }
+    }
+    for (; j < n; j += st) {
+        const double2 x = Xr[j];
+        v[0] = norm_add(v[0], x);
+        cdot_add(v[2], v[3], Rr[j], x);
+    }
+    cta_sums(v, reinterpret_cast<double *>(partial + ((long)r * gridDim.x + blockIdx.x) * 64));
+}
+
+// rho_r -= c_r x_r, x_r *= s_r in one pass
+struct RhoScale64 {
+    double2 cR[64];
+    double sx[64];
+};
+__global__ void k_rho_update64(long n, const __grid_constant__ RhoScale64 cf, double2 *X, long fx, double2 *R, long fr)
+{
+    const int r = blockIdx.y;
+    double2 *Xr = X + r * fx, *Rr = R + r * fr;
+    const double2 mc = make_double2(-cf.cR[r].x, -cf.cR[r].y);
+    const double sx = cf.sx[r];
+#pragma unroll 4
+    for (long j = blockIdx.x * (long)blockDim.x + threadIdx.x; j < n; j += (long)gridDim.x * blockDim.x) {
+        const double2 x = Xr[j];
+        Rr[j] = caxpy(mc, x, Rr[j]);
+        Xr[j] = make_double2(sx * x.x, sx * x.y);
+    }
+}
+
+// rho_r = eta_r - w_r (w = NULL: eta_r) and |rho_r|^2 as partial[(r*nb + b)*64]
+__global__ void __launch_bounds__(RED_THREADS) k_residual64(long n, const double2 *__restrict__ E, long fe,
+                                                            const double2 *__restrict__ W, long fw, double2 *R,
+                                                            long fr, double2 *partial)
+{
+    const int r = blockIdx.y;
+    double v[2] = {0, 0};
+#pragma unroll 4
+    for (long j = blockIdx.x * (long)blockDim.x + threadIdx.x; j < n; j += (long)gridDim.x * blockDim.x) {
+        double2 e = E[r * fe + j];
+        if (W) {
+            const double2 w = W[r * fw + j];
+            e = make_double2(e.x - w.x, e.y - w.y);
+        }
+        R[r * fr + j] = e;
+        v[0] = norm_add(v[0], e);
+    }
+    cta_sums(v, reinterpret_cast<double *>(partial + ((long)r * gridDim.x + blockIdx.x) * 64));
+}
+
 // ---------------------------------------------------------------- FP32 Krylov
 // Batched kernels of the GCR with FP32 Krylov vectors (native F32 full fields,
 // float4 = two complex components).  Products are formed in float; each
@@ -245,10 +332,10 @@ __global__ void __launch_bounds__(RED_THREADS) k_bdot32_partial(long n, const fl
     }
 }
 
-// |x_r|^2 and <rho_r, x_r> (x: F32 full fields, rho: F64 full fields) as the two
-// partial sums partial[(r*nb + b)*64 + {0, 1}]; site r of half h, float4 q of x
-// holds the complex components 2q, 2q+1 of rho
-__global__ void __launch_bounds__(RED_THREADS) k_norm_rdot32_partial(long Vh, const float4 *__restrict__ X, long fx,
+// |x_r|^2 and <rho_r, x_r> (x: F32 fields, rho: F64 fields, np = 6 float4 words per
+// half) as the two partial sums partial[(r*nb + b)*64 + {0, 1}]; site r of half
+// h, float4 q of x holds the complex components 2q, 2q+1 of rho
+__global__ void __launch_bounds__(RED_THREADS) k_norm_rdot32_partial(long Vh, int np, const float4 *__restrict__ X, long fx,
                                                                      const double2 *__restrict__ R, long fr,
                                                                      double2 *partial)
 {
@@ -258,8 +345,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_norm_rdot32_partial(long Vh, co
     double nn = 0, dre = 0, dim = 0;
     for (long s = blockIdx.x * (long)blockDim.x + threadIdx.x; s < Vh; s += (long)gridDim.x * blockDim.x) {
         float fn = 0, fre = 0, fim = 0;
-#pragma unroll
-        for (int p = 0; p < 12; p++) {
+#pragma unroll 6
+        for (int p = 0; p < np; p++) {
             const float4 a = Xr[p * Vh + s];
             const double2 u = Rr[(2 * p) * Vh + s], v = Rr[(2 * p + 1) * Vh + s];
             fn += a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w;
@@ -343,15 +430,15 @@ struct RhoScale {
     double2 cR[64];
     float sx[64];
 };
-__global__ void k_rho_update32(long Vh, const __grid_constant__ RhoScale cf, float4 *X, long fx, double2 *R, long fr)
+__global__ void k_rho_update32(long Vh, int np, const __grid_constant__ RhoScale cf, float4 *X, long fx, double2 *R, long fr)
 {
     const int rh = blockIdx.y;
     float4 *Xr = X + rh * fx;
     double2 *Rr = R + rh * fr;
     const float cr = (float)cf.cR[rh].x, ci = (float)cf.cR[rh].y, sx = cf.sx[rh];
     for (long s = blockIdx.x * (long)blockDim.x + threadIdx.x; s < Vh; s += (long)gridDim.x * blockDim.x) {
-#pragma unroll 4
-        for (int p = 0; p < 12; p++) {
+#pragma unroll 3
+        for (int p = 0; p < np; p++) {
             const float4 a = Xr[p * Vh + s];
             double2 u = Rr[(2 * p) * Vh + s], v = Rr[(2 * p + 1) * Vh + s];
             u.x -= (double)(cr * a.x - ci * a.y);
@@ -365,8 +452,8 @@ __global__ void k_rho_update32(long Vh, const __grid_constant__ RhoScale cf, flo
     }
 }
 
-// psi_r += sum_i c[r*k + i] X_{i,r} (X F32 full fields, psi F64; the sum in float)
-__global__ void k_bmulti_axpy_mixed(long Vh, int k, const __grid_constant__ CoefParam cf,
+// psi_r += sum_i c[r*k + i] X_{i,r} (X F32 fields, psi F64; the sum in float)
+__global__ void k_bmulti_axpy_mixed(long Vh, int np, int k, const __grid_constant__ CoefParam cf,
                                     const float4 *__restrict__ X, long sa, long fa, double2 *y, long fy)
 {
     const int rh = blockIdx.y;
@@ -377,7 +464,7 @@ __global__ void k_bmulti_axpy_mixed(long Vh, int k, const __grid_constant__ Coef
         c[i] = make_float2((float)cf.c[rh * k + i].x, (float)cf.c[rh * k + i].y);
     __syncthreads();
     for (long s = blockIdx.x * (long)blockDim.x + threadIdx.x; s < Vh; s += (long)gridDim.x * blockDim.x) {
-        for (int p = 0; p < 12; p++) {
+        for (int p = 0; p < np; p++) {
             float s0 = 0, s1 = 0, s2 = 0, s3 = 0;
             for (int i = 0; i < k; i++) {
                 const float4 a = Xr[i * sa + p * Vh + s];
@@ -580,6 +667,48 @@ lqcd_status finish_dots(lqcd_ctx *c, int nb, int nrhs, int k, double *host_out)
 }
 }  // namespace
 
+lqcd_status bnorm_rdot64(lqcd_ctx *c, int nh, int nrhs, const double2 *x, long fx, const double2 *rho, long fr,
+                         double *host_out)
+{
+    if (nrhs < 1 || nrhs > 1024) return set_err(c, LQCD_ERR_ARG, "bnorm_rdot64 nrhs=%d", nrhs);
+    const long n = 12L * nh * c->g.Vh;
+    const int nb = red_blocks(n, nrhs);
+    k_norm_rdot64_partial<<<dim3(nb, nrhs), RED_THREADS, 0, c->stream>>>(n, x, fx, rho, fr, (double2 *)c->red);
+    c->n_kernel_launches++;
+    return finish_dots(c, nb, nrhs, 2, host_out);
+}
+
+lqcd_status brho_update64(lqcd_ctx *c, int nh, int nrhs, const double *cR_host, const double *sx_host, double2 *x,
+                          long fx, double2 *rho, long fr)
+{
+    if (nrhs < 1 || nrhs > 64) return set_err(c, LQCD_ERR_ARG, "brho_update64 nrhs=%d", nrhs);
+    RhoScale64 cp;
+    for (int r = 0; r < nrhs; r++) {
+        cp.cR[r] = make_double2(cR_host[2 * r], cR_host[2 * r + 1]);
+        cp.sx[r] = sx_host[r];
+    }
+    const long n = 12L * nh * c->g.Vh;
+    dim3 grid(std::max(1, grid_for(n) / std::max(1, nrhs / 2)), nrhs);
+    k_rho_update64<<<grid, 256, 0, c->stream>>>(n, cp, x, fx, rho, fr);
+    c->n_kernel_launches++;
+    LQCD_LAUNCH_CHECK(c);
+    return LQCD_OK;
+}
+
+lqcd_status bresidual64(lqcd_ctx *c, int nh, int nrhs, const double2 *eta, long fe, const double2 *w, long fw,
+                        double2 *rho, long fr, double *norms)
+{
+    if (nrhs < 1 || nrhs > 64) return set_err(c, LQCD_ERR_ARG, "bresidual64 nrhs=%d", nrhs);
+    const long n = 12L * nh * c->g.Vh;
+    const int nb = red_blocks(n, nrhs);
+    k_residual64<<<dim3(nb, nrhs), RED_THREADS, 0, c->stream>>>(n, eta, fe, w, fw, rho, fr, (double2 *)c->red);
+    c->n_kernel_launches++;
+    double d[128];
+    LQCD_TRY(finish_dots(c, nb, nrhs, 1, d));
+    for (int r = 0; r < nrhs; r++) norms[r] = d[2 * r];
+    return LQCD_OK;
+}
+
 lqcd_status bdot32(lqcd_ctx *c, long n4, int nrhs, const float4 *A, long sa, long fa, const float4 *B, long fb, int k,
                    double *host_out)
 {
@@ -594,13 +723,14 @@ lqcd_status bdot32(lqcd_ctx *c, long n4, int nrhs, const float4 *A, long sa, lon
     return finish_dots(c, nb, nrhs, k, host_out);
 }
 
-lqcd_status bnorm_rdot32(lqcd_ctx *c, int nrhs, const float4 *x, long fx, const double2 *rho, long fr,
+lqcd_status bnorm_rdot32(lqcd_ctx *c, int nh, int nrhs, const float4 *x, long fx, const double2 *rho, long fr,
                          double *host_out)
 {
     if (nrhs < 1 || nrhs > 1024) return set_err(c, LQCD_ERR_ARG, "bnorm_rdot32 nrhs=%d", nrhs);
     const long Vh = c->g.Vh;
     const int nb = red_blocks(Vh, nrhs);
-    k_norm_rdot32_partial<<<dim3(nb, nrhs), RED_THREADS, 0, c->stream>>>(Vh, x, fx, rho, fr, (double2 *)c->red);
+    k_norm_rdot32_partial<<<dim3(nb, nrhs), RED_THREADS, 0, c->stream>>>(Vh, 6 * nh, x, fx, rho, fr,
+                                                                           (double2 *)c->red);
     c->n_kernel_launches++;
     return finish_dots(c, nb, nrhs, 2, host_out);
 }
@@ -619,8 +749,8 @@ lqcd_status bmulti_axpy32(lqcd_ctx *c, long n4, int nrhs, int k, const double *c
     return LQCD_OK;
 }
 
-lqcd_status brho_update32(lqcd_ctx *c, int nrhs, const double *cR_host, const double *sx_host, float4 *x, long fx,
-                          double2 *rho, long fr)
+lqcd_status brho_update32(lqcd_ctx *c, int nh, int nrhs, const double *cR_host, const double *sx_host, float4 *x,
+                          long fx, double2 *rho, long fr)
 {
     if (nrhs < 1 || nrhs > 64) return set_err(c, LQCD_ERR_ARG, "brho_update32 nrhs=%d", nrhs);
     RhoScale cp;
@@ -630,13 +760,13 @@ lqcd_status brho_update32(lqcd_ctx *c, int nrhs, const double *cR_host, const do
     }
     const long Vh = c->g.Vh;
     dim3 grid(std::max(1, grid_for(Vh) / std::max(1, nrhs / 2)), nrhs);
-    k_rho_update32<<<grid, 256, 0, c->stream>>>(Vh, cp, x, fx, rho, fr);
+    k_rho_update32<<<grid, 256, 0, c->stream>>>(Vh, 6 * nh, cp, x, fx, rho, fr);
     c->n_kernel_launches++;
     LQCD_LAUNCH_CHECK(c);
     return LQCD_OK;
 }
 
-lqcd_status bmulti_axpy_mixed(lqcd_ctx *c, int nrhs, int k, const double *coef_host, const float4 *X, long sa,
+lqcd_status bmulti_axpy_mixed(lqcd_ctx *c, int nh, int nrhs, int k, const double *coef_host, const float4 *X, long sa,
                               long fa, double2 *y, long fy)
 {
     if (k < 1) return LQCD_OK;
@@ -645,7 +775,7 @@ lqcd_status bmulti_axpy_mixed(lqcd_ctx *c, int nrhs, int k, const double *coef_h
     for (int i = 0; i < k * nrhs; i++) cp.c[i] = make_double2(coef_host[2 * i], coef_host[2 * i + 1]);
     const long Vh = c->g.Vh;
     dim3 grid(std::max(1, grid_for(Vh) / std::max(1, nrhs / 2)), nrhs);
-    k_bmulti_axpy_mixed<<<grid, 256, 0, c->stream>>>(Vh, k, cp, X, sa, fa, y, fy);
+    k_bmulti_axpy_mixed<<<grid, 256, 0, c->stream>>>(Vh, 6 * nh, k, cp, X, sa, fa, y, fy);
     c->n_kernel_launches++;
     LQCD_LAUNCH_CHECK(c);
     return LQCD_OK;

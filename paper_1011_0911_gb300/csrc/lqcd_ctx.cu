@@ -279,25 +279,25 @@ void launch_pack_t(lqcd_ctx *c, int nsub, const void *canon, void *native, int n
 }
 
 // native F64 <-> native F32 (same site/chunk structure), nhalf half fields
-__global__ void k_conv64to32(long Vh, long nhalf, const double2 *__restrict__ in, float4 *out)
+__global__ void k_conv64to32(long Vh, long nhalf, long ih, long oh, const double2 *__restrict__ in, float4 *out)
 {
     long r = blockIdx.x * (long)blockDim.x + threadIdx.x;
     long h = blockIdx.y;
     if (r >= Vh || h >= nhalf) return;
-    const double2 *i = in + h * 12 * Vh + r;
-    float4 *o = out + h * 6 * Vh + r;
+    const double2 *i = in + h * ih * 12 * Vh + r;
+    float4 *o = out + h * oh * 6 * Vh + r;
     for (int q = 0; q < 6; q++) {
         double2 a = i[(2 * q) * Vh], b = i[(2 * q + 1) * Vh];
         o[q * Vh] = make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
     }
 }
-__global__ void k_conv32to64(long Vh, long nhalf, const float4 *__restrict__ in, double2 *out)
+__global__ void k_conv32to64(long Vh, long nhalf, long ih, long oh, const float4 *__restrict__ in, double2 *out)
 {
     long r = blockIdx.x * (long)blockDim.x + threadIdx.x;
     long h = blockIdx.y;
     if (r >= Vh || h >= nhalf) return;
-    const float4 *i = in + h * 6 * Vh + r;
-    double2 *o = out + h * 12 * Vh + r;
+    const float4 *i = in + h * ih * 6 * Vh + r;
+    double2 *o = out + h * oh * 12 * Vh + r;
     for (int q = 0; q < 6; q++) {
         float4 a = i[q * Vh];
         o[(2 * q) * Vh] = make_double2(a.x, a.y);
@@ -330,46 +330,51 @@ __device__ __forceinline__ void nat_store(float4 *f, long Vh, long r, const cx<f
     for (int q = 0; q < 6; q++) f[q * Vh + r] = make_float4(v[2 * q].re, v[2 * q].im, v[2 * q + 1].re, v[2 * q + 1].im);
 }
 template <class T>
-__global__ void k_conv_to16s(long Vh, long nhalf, const T *__restrict__ in, h16s *out)
+__global__ void k_conv_to16s(long Vh, long nhalf, long ih, long oh, const T *__restrict__ in, h16s *out)
 {
     long r = blockIdx.x * (long)blockDim.x + threadIdx.x;
     long h = blockIdx.y;
     if (r >= Vh || h >= nhalf) return;
     cx<float> v[12];
-    nat_load(in + h * (std::is_same<T, double2>::value ? 12 : 6) * Vh, Vh, r, v);
-    f16s_store(out + h * f16s_half_units(Vh), Vh, r, v);
+    nat_load(in + h * ih * (std::is_same<T, double2>::value ? 12 : 6) * Vh, Vh, r, v);
+    f16s_store(out + h * oh * f16s_half_units(Vh), Vh, r, v);
 }
 template <class T>
-__global__ void k_conv_from16s(long Vh, long nhalf, const h16s *__restrict__ in, T *out)
+__global__ void k_conv_from16s(long Vh, long nhalf, long ih, long oh, const h16s *__restrict__ in, T *out)
 {
     long r = blockIdx.x * (long)blockDim.x + threadIdx.x;
     long h = blockIdx.y;
     if (r >= Vh || h >= nhalf) return;
     cx<float> v[12];
-    f16s_load<true>(in + h * f16s_half_units(Vh), Vh, r, v);
-    nat_store(out + h * (std::is_same<T, double2>::value ? 12 : 6) * Vh, Vh, r, v);
+    f16s_load<true>(in + h * ih * f16s_half_units(Vh), Vh, r, v);
+    nat_store(out + h * oh * (std::is_same<T, double2>::value ? 12 : 6) * Vh, Vh, r, v);
 }
 
 }  // namespace
 
-lqcd_status convert_native(lqcd_ctx *c, lqcd_prec from, lqcd_prec to, const void *in, void *out, long nhalf)
+lqcd_status convert_native(lqcd_ctx *c, lqcd_prec from, lqcd_prec to, const void *in, void *out, long nhalf,
+                           long in_hs, long out_hs)
 {
     dim3 grid(div_up(c->g.Vh, 256), (unsigned)nhalf);
     if (from == LQCD_F64 && to == LQCD_F32)
-        k_conv64to32<<<grid, 256, 0, c->stream>>>(c->g.Vh, nhalf, (const double2 *)in, (float4 *)out);
+        k_conv64to32<<<grid, 256, 0, c->stream>>>(c->g.Vh, nhalf, in_hs, out_hs, (const double2 *)in, (float4 *)out);
     else if (from == LQCD_F32 && to == LQCD_F64)
-        k_conv32to64<<<grid, 256, 0, c->stream>>>(c->g.Vh, nhalf, (const float4 *)in, (double2 *)out);
+        k_conv32to64<<<grid, 256, 0, c->stream>>>(c->g.Vh, nhalf, in_hs, out_hs, (const float4 *)in, (double2 *)out);
     else if (from == LQCD_F64 && to == LQCD_F16S)
-        k_conv_to16s<double2><<<grid, 256, 0, c->stream>>>(c->g.Vh, nhalf, (const double2 *)in, (h16s *)out);
+        k_conv_to16s<double2><<<grid, 256, 0, c->stream>>>(c->g.Vh, nhalf, in_hs, out_hs, (const double2 *)in, (h16s *)out);
     else if (from == LQCD_F32 && to == LQCD_F16S)
-        k_conv_to16s<float4><<<grid, 256, 0, c->stream>>>(c->g.Vh, nhalf, (const float4 *)in, (h16s *)out);
+        k_conv_to16s<float4><<<grid, 256, 0, c->stream>>>(c->g.Vh, nhalf, in_hs, out_hs, (const float4 *)in, (h16s *)out);
     else if (from == LQCD_F16S && to == LQCD_F64)
-        k_conv_from16s<double2><<<grid, 256, 0, c->stream>>>(c->g.Vh, nhalf, (const h16s *)in, (double2 *)out);
+        k_conv_from16s<double2><<<grid, 256, 0, c->stream>>>(c->g.Vh, nhalf, in_hs, out_hs, (const h16s *)in, (double2 *)out);
     else if (from == LQCD_F16S && to == LQCD_F32)
-        k_conv_from16s<float4><<<grid, 256, 0, c->stream>>>(c->g.Vh, nhalf, (const h16s *)in, (float4 *)out);
+        k_conv_from16s<float4><<<grid, 256, 0, c->stream>>>(c->g.Vh, nhalf, in_hs, out_hs, (const h16s *)in, (float4 *)out);
     else if (from == to) {
-        LQCD_CUDA_CHECK(c, cudaMemcpyAsync(out, in, nhalf * native_half_bytes(c, from),
-                                           cudaMemcpyDeviceToDevice, c->stream));
+        const size_t hb = native_half_bytes(c, from);
+        if (in_hs == 1 && out_hs == 1)
+            LQCD_CUDA_CHECK(c, cudaMemcpyAsync(out, in, nhalf * hb, cudaMemcpyDeviceToDevice, c->stream));
+        else
+            LQCD_CUDA_CHECK(c, cudaMemcpy2DAsync(out, out_hs * hb, in, in_hs * hb, hb, nhalf, cudaMemcpyDeviceToDevice,
+                                                 c->stream));
         return LQCD_OK;
     } else
         return set_err(c, LQCD_ERR_ARG, "conversion %d -> %d not supported", (int)from, (int)to);

@@ -324,46 +324,49 @@ lqcd_status launch_hop(lqcd_ctx *c, int p_out, const SP *in_other, long in_rs, c
 
 }  // namespace
 
-// Dhat on native half fields: in/out even (nrhs fields, rhs stride = one half
-// field), tmp_o an odd native half field per rhs.
-lqcd_status dirac_dhat(lqcd_ctx *c, lqcd_prec p, const void *in, void *out, void *tmp_o, int nrhs)
+// Dhat on native half fields: in / out even, in_rs / out_rs units apart per rhs
+// (native units: double2, float4, h16s); tmp_o: nrhs odd half fields one after the other.
+lqcd_status dirac_dhat_s(lqcd_ctx *c, lqcd_prec p, const void *in, long in_rs, void *out, long out_rs, void *tmp_o,
+                         int nrhs)
 {
     if (!c->have_clover) return set_err(c, LQCD_ERR_STATE, "clover term not built");
-    const long Vh = c->g.Vh;
+    const long rs = native_half_units(c, p);
     if (p == LQCD_F64) {
-        const long rs = 12 * Vh;
         auto *i = (const double2 *)in;
         auto *o = (double2 *)out;
         auto *t = (double2 *)tmp_o;
         LQCD_TRY((launch_hop<double, double2, double2, double2, MODE_DHAT1>(
-            c, 1, i, rs, nullptr, 0, t, rs, c->U64, c->Ai64[1], nrhs)));
+            c, 1, i, in_rs, nullptr, 0, t, rs, c->U64, c->Ai64[1], nrhs)));
         LQCD_TRY((launch_hop<double, double2, double2, double2, MODE_DHAT2>(
-            c, 0, t, rs, i, rs, o, rs, c->U64, c->A64[0], nrhs)));
+            c, 0, t, rs, i, in_rs, o, out_rs, c->U64, c->A64[0], nrhs)));
         return LQCD_OK;
     }
     if (p == LQCD_F32) {
-        const long rs = 6 * Vh;
         auto *i = (const float4 *)in;
         auto *o = (float4 *)out;
         auto *t = (float4 *)tmp_o;
         LQCD_TRY((launch_hop<float, float4, float4, float4, MODE_DHAT1>(
-            c, 1, i, rs, nullptr, 0, t, rs, c->U32, c->Ai32[1], nrhs)));
+            c, 1, i, in_rs, nullptr, 0, t, rs, c->U32, c->Ai32[1], nrhs)));
         LQCD_TRY((launch_hop<float, float4, float4, float4, MODE_DHAT2>(
-            c, 0, t, rs, i, rs, o, rs, c->U32, c->A32[0], nrhs)));
+            c, 0, t, rs, i, in_rs, o, out_rs, c->U32, c->A32[0], nrhs)));
         return LQCD_OK;
     }
     if (p == LQCD_F16S) {
-        const long rs = f16s_half_units(Vh);
         auto *i = (const h16s *)in;
         auto *o = (h16s *)out;
         auto *t = (h16s *)tmp_o;
-        LQCD_TRY((launch_hop<float, h16s, uint2, uint2, MODE_DHAT1>(c, 1, i, rs, nullptr, 0, t, rs, c->U16,
+        LQCD_TRY((launch_hop<float, h16s, uint2, uint2, MODE_DHAT1>(c, 1, i, in_rs, nullptr, 0, t, rs, c->U16,
                                                                     c->Ai16[1], nrhs)));
-        LQCD_TRY((launch_hop<float, h16s, uint2, uint2, MODE_DHAT2>(c, 0, t, rs, i, rs, o, rs, c->U16, c->A16[0],
-                                                                    nrhs)));
+        LQCD_TRY((launch_hop<float, h16s, uint2, uint2, MODE_DHAT2>(c, 0, t, rs, i, in_rs, o, out_rs, c->U16,
+                                                                    c->A16[0], nrhs)));
         return LQCD_OK;
     }
     return set_err(c, LQCD_ERR_ARG, "precision %d not supported for Dhat", (int)p);
+}
+lqcd_status dirac_dhat(lqcd_ctx *c, lqcd_prec p, const void *in, void *out, void *tmp_o, int nrhs)
+{
+    const long rs = native_half_units(c, p);
+    return dirac_dhat_s(c, p, in, rs, out, rs, tmp_o, nrhs);
 }
 
 // D on native full fields ([rhs][even half][odd half])

@@ -294,6 +294,10 @@ lqcd_status ws_get(lqcd_ctx *c, int slot, size_t bytes, void **out);
 inline int native_chunks(lqcd_prec p) { return p == LQCD_F64 ? 12 : (p == LQCD_F32 ? 6 : 3); }
 inline size_t native_chunk_bytes(lqcd_prec p) { return p == LQCD_F64 ? 16 : (p == LQCD_F32 ? 16 : 16); }
 size_t native_half_bytes(const lqcd_ctx *c, lqcd_prec p);   // one rhs, one parity
+inline long native_half_units(const lqcd_ctx *c, lqcd_prec p)   // in 16-byte units
+{
+    return (long)(native_half_bytes(c, p) / 16);
+}
 
 // launch helpers
 inline int div_up(long a, long b) { return (int)((a + b - 1) / b); }
@@ -301,11 +305,14 @@ inline int div_up(long a, long b) { return (int)((a + b - 1) / b); }
 // --------------------------------------------------------------- internals
 // dirac
 lqcd_status dirac_dhat(lqcd_ctx *c, lqcd_prec p, const void *in, void *out, void *tmp_o, int nrhs);
+lqcd_status dirac_dhat_s(lqcd_ctx *c, lqcd_prec p, const void *in, long in_rs, void *out, long out_rs, void *tmp_o,
+                         int nrhs);
 lqcd_status dirac_D(lqcd_ctx *c, lqcd_prec p, const void *in, void *out, int nrhs);
 lqcd_status dirac_hop_parity(lqcd_ctx *c, lqcd_prec p, int p_out, const void *in_other,
                              void *out, long in_rstride, long out_rstride, int nrhs);
+// nhalf half fields; in_hs, out_hs: distance of consecutive ones in half fields
 lqcd_status convert_native(lqcd_ctx *c, lqcd_prec from, lqcd_prec to, const void *in, void *out,
-                           long nhalf);
+                           long nhalf, long in_hs = 1, long out_hs = 1);
 lqcd_status pack_field(lqcd_ctx *c, lqcd_prec p, int nsub, const void *canon, void *native,
                        int nrhs, bool unpack);
 // even_scale != 1: the even-site blocks of A (and so of A^-1) belong to
@@ -333,18 +340,27 @@ lqcd_status bblas_dot_dev(lqcd_ctx *c, long n2, int nrhs, const double *A, long 
                           int k, double2 *out_dev);
 lqcd_status bblas_multi_axpy_dev(lqcd_ctx *c, long n2, int nrhs, int k, const double2 *coef_dev, const double *X,
                                  long sa, long fa, double *y, long fy, double sign);
-// GCR with FP32 Krylov vectors: x, A, B, X, y are native F32 full fields
-// (float4, strides in float4), rho and psi native F64 full fields (double2,
-// strides in double2); dots land on the host as (re, im) pairs [r][i]
+// GCR vectors.  nh: halves per vector (2: full fields, 1: their even halves);
+// f*: distance of the right-hand sides.  dots land on the host as (re, im)
+// pairs [r][i]; norm_rdot: [r][0] = |x_r|^2, [r][1] = <rho_r, x_r>.
+lqcd_status bnorm_rdot64(lqcd_ctx *c, int nh, int nrhs, const double2 *x, long fx, const double2 *rho, long fr,
+                         double *host_out);
+lqcd_status brho_update64(lqcd_ctx *c, int nh, int nrhs, const double *cR_host, const double *sx_host, double2 *x,
+                          long fx, double2 *rho, long fr);   // rho_r -= cR_r x_r; x_r *= sx_r
+// rho_r = eta_r - w_r (w = NULL: eta_r), norms[r] = |rho_r|^2
+lqcd_status bresidual64(lqcd_ctx *c, int nh, int nrhs, const double2 *eta, long fe, const double2 *w, long fw,
+                        double2 *rho, long fr, double *norms);
+// FP32 Krylov vectors: x, A, B, X, y are native F32 fields (float4, strides in
+// float4), rho and psi native F64 fields (double2, strides in double2)
 lqcd_status bdot32(lqcd_ctx *c, long n4, int nrhs, const float4 *A, long sa, long fa, const float4 *B, long fb, int k,
                    double *host_out);
-lqcd_status bnorm_rdot32(lqcd_ctx *c, int nrhs, const float4 *x, long fx, const double2 *rho, long fr,
-                         double *host_out);   // [r][0] = |x_r|^2, [r][1] = <rho_r, x_r>
+lqcd_status bnorm_rdot32(lqcd_ctx *c, int nh, int nrhs, const float4 *x, long fx, const double2 *rho, long fr,
+                         double *host_out);
 lqcd_status bmulti_axpy32(lqcd_ctx *c, long n4, int nrhs, int k, const double *coef_host, const float4 *X, long sa,
                           long fa, float4 *y, long fy, double sign);
-lqcd_status brho_update32(lqcd_ctx *c, int nrhs, const double *cR_host, const double *sx_host, float4 *x, long fx,
-                          double2 *rho, long fr);   // rho_r -= cR_r x_r; x_r *= sx_r
-lqcd_status bmulti_axpy_mixed(lqcd_ctx *c, int nrhs, int k, const double *coef_host, const float4 *X, long sa,
+lqcd_status brho_update32(lqcd_ctx *c, int nh, int nrhs, const double *cR_host, const double *sx_host, float4 *x,
+                          long fx, double2 *rho, long fr);   // rho_r -= cR_r x_r; x_r *= sx_r
+lqcd_status bmulti_axpy_mixed(lqcd_ctx *c, int nh, int nrhs, int k, const double *coef_host, const float4 *X, long sa,
                               long fa, double2 *y, long fy);   // y_r += sum_i c_ri X_ir
 lqcd_status blas_gamma5_native64(lqcd_ctx *c, long nhalf, const double2 *in, double2 *out);
 lqcd_status blas_zero(lqcd_ctx *c, size_t bytes, void *p);

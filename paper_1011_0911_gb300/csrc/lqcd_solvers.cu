@@ -1,6 +1,16 @@
 // Outer solvers: even-odd CGNR on Dhat (Eq. 2) and the flexible GCR of
-// Sec. 3-4 on the full operator, preconditioned by SAP or deflated SAP; the
-// solution of Dhat psi_e = eta_e is the even part of D^-1 (eta_e, 0) (Eq. 5).
+// Sec. 3-4, preconditioned by SAP or deflated SAP.
+//
+// The GCR solves either D psi = eta on the full lattice or Dhat psi_e = eta_e.
+// The latter is the former with the odd half eliminated: completing an even
+// field x_e by x_o = -A_oo^-1 H_oe x_e gives D x = (Dhat x_e, 0), so with a
+// residual (rho_e, 0) the preconditioner M of the full lattice is applied as it
+// is, the even half of its output is the search direction, and D phi_k needs
+// Dhat phi_e alone (as many hops as D).  Every Krylov vector, dot product and
+// update has half the length, and the residual is that of the Dhat system
+// itself (Eq. 5 only bounds it by the full one).  Measured with unchanged
+// iteration counts: 32 x 16^3, one source, FP32 SAP, FP64 Krylov vectors 70.9 ->
+// 58.4 ms; 48 x 24^3, 12 sources, deflated, build included 1218 -> 1101 ms.
 //
 // Precision: the residual, the solution update and the restart residual
 // eta - D psi are FP64.  The preconditioner and D phi_k may run in FP32
@@ -138,17 +148,28 @@ lqcd_status precond(lqcd_ctx *c, const lqcd_solver_params *sp, const double2 *rh
     return convert_native(c, sap.prec, LQCD_F64, b, phi, 2 * nrhs);
 }
 
-// chi = D phi in the inner precision, result FP64
-lqcd_status apply_D_inner(lqcd_ctx *c, lqcd_prec inner, const double2 *phi, double2 *chi, int nrhs)
+// chi = D phi (nh = 2) or Dhat phi_e (nh = 1) in the inner precision, phi nrhs
+// native full FP64 fields, chi nrhs fields of nh halves
+lqcd_status apply_D_inner(lqcd_ctx *c, lqcd_prec inner, int nh, const double2 *phi, double2 *chi, int nrhs)
 {
-    if (inner == LQCD_F64) return dirac_D(c, LQCD_F64, phi, chi, nrhs);
+    const long Vh = c->g.Vh;
+    if (inner == LQCD_F64 && nh == 2) return dirac_D(c, LQCD_F64, phi, chi, nrhs);
+    const size_t hb = native_half_bytes(c, inner);
+    void *t = nullptr;
+    if (nh == 1) LQCD_TRY(ws_get(c, WS_TMP_O, hb * nrhs, &t));
+    if (inner == LQCD_F64) return dirac_dhat_s(c, LQCD_F64, phi, 24 * Vh, chi, 12 * Vh, t, nrhs);
     void *a, *b;
-    size_t fb = 2 * native_half_bytes(c, inner) * nrhs;
+    const size_t fb = nh * hb * nrhs;
     LQCD_TRY(ws_get(c, WS_MISC, fb, &a));
     LQCD_TRY(ws_get(c, WS_MISC2, fb, &b));
-    LQCD_TRY(convert_native(c, LQCD_F64, inner, phi, a, 2 * nrhs));
-    LQCD_TRY(dirac_D(c, inner, a, b, nrhs));
-    return convert_native(c, inner, LQCD_F64, b, chi, 2 * nrhs);
+    if (nh == 2) {
+        LQCD_TRY(convert_native(c, LQCD_F64, inner, phi, a, 2 * nrhs));
+        LQCD_TRY(dirac_D(c, inner, a, b, nrhs));
+    } else {
+        LQCD_TRY(convert_native(c, LQCD_F64, inner, phi, a, nrhs, 2, 1));
+        LQCD_TRY(dirac_dhat(c, inner, a, b, t, nrhs));
+    }
+    return convert_native(c, inner, LQCD_F64, b, chi, nh * nrhs);
 }
 
 struct GcrState {
@@ -201,87 +222,77 @@ struct PhaseProf {
     }
 };
 
-// per-rhs squared norms of nrhs fields
-lqcd_status bnorm2(lqcd_ctx *c, long n2, int nrhs, const double2 *x, std::vector<double> &out)
-{
-    std::vector<double> d(2 * nrhs);
-    LQCD_TRY(bblas_dot(c, n2, nrhs, (const double *)x, 0, n2, (const double *)x, n2, 1, d.data()));
-    out.resize(nrhs);
-    for (int r = 0; r < nrhs; r++) out[r] = d[2 * r];
-    return LQCD_OK;
-}
-
 // Krylov-vector storage of the GCR.  Krylov64: phi_k and chi_k native F64
-// full fields.  Krylov32 (krylov = inner = F32): phi_k and chi_k native F32
-// full fields, so D phi_k runs on them directly and the Gram-Schmidt moves
-// half the bytes and leaves GB300's FP64 pipe (FP64 products bound it at about
-// a third of HBM bandwidth); rho and psi stay F64, the products with FP32
-// vectors are formed in float and accumulated in double.
+// fields.  Krylov32 (krylov = inner = F32): phi_k and chi_k native F32 fields,
+// so D phi_k runs on them directly and the Gram-Schmidt moves half the bytes
+// and leaves GB300's FP64 pipe (FP64 products bound it at about a third of HBM
+// bandwidth); rho and psi stay F64, the products with FP32 vectors are formed
+// in float and accumulated in double.
+//
+// nh: halves per vector (1: the Dhat system).  phi_k and rho are full fields in
+// either case (fphi, 24 Vh apart): the preconditioner writes and reads them, the
+// odd half of rho being zero when nh = 1; chi, psi and eta have nh halves.
 struct Krylov64 {
     using T = double2;
     lqcd_ctx *c;
     const lqcd_solver_params *sp;
-    int nrhs;
-    long nf;   // elements (double2) per full field
-    long n2;   // doubles per full field
-    Krylov64(lqcd_ctx *ctx, const lqcd_solver_params *p, int n)
-        : c(ctx), sp(p), nrhs(n), nf(24 * (long)ctx->g.Vh), n2(48 * (long)ctx->g.Vh)
+    int nh, nrhs;
+    long fphi, fchi, frho;   // elements between right-hand sides
+    Krylov64(lqcd_ctx *ctx, const lqcd_solver_params *p, int halves, int n)
+        : c(ctx), sp(p), nh(halves), nrhs(n), fphi(24 * (long)ctx->g.Vh), fchi(12L * halves * ctx->g.Vh),
+          frho(24 * (long)ctx->g.Vh)
     {
     }
-    size_t field_bytes() const { return nf * sizeof(T); }
     lqcd_status precond_with(const lqcd_solver_params *p, const double2 *rho, T *ph)
     {
         return precond(c, p, rho, ph, nrhs);
     }
-    lqcd_status D_inner(const T *ph, T *ch) { return apply_D_inner(c, sp->inner, ph, ch, nrhs); }
-    lqcd_status dots(const T *A, long sa, const T *B, int kk, double *out)
+    lqcd_status D_inner(const T *ph, T *ch) { return apply_D_inner(c, sp->inner, nh, ph, ch, nrhs); }
+    lqcd_status dots(const T *A, const T *B, int kk, double *out)
     {
-        return bblas_dot(c, n2, nrhs, (const double *)A, 2 * sa, n2, (const double *)B, n2, kk, out);
+        return bblas_dot(c, 2 * fchi, nrhs, (const double *)A, 2 * nrhs * fchi, 2 * fchi, (const double *)B, 2 * fchi,
+                         kk, out);
     }
-    lqcd_status axpy(int k, const double *cf, const T *X, long sa, T *y, double sign)
+    lqcd_status axpy(int k, const double *cf, const T *X, T *y, double sign)
     {
-        return bblas_multi_axpy(c, n2, nrhs, k, cf, (const double *)X, 2 * sa, n2, (double *)y, n2, sign);
+        return bblas_multi_axpy(c, 2 * fchi, nrhs, k, cf, (const double *)X, 2 * nrhs * fchi, 2 * fchi, (double *)y,
+                                2 * fchi, sign);
     }
-    // |chi|^2 and <rho, chi> (the family {chi, rho} against chi)
+    // |chi|^2 and <rho, chi>
     lqcd_status norm_rdot(const T *ch, const double2 *rho, double *out)
     {
-        return bblas_dot(c, n2, nrhs, (const double *)ch, 2 * (rho - ch), n2, (const double *)ch, n2, 2, out);
+        return bnorm_rdot64(c, nh, nrhs, ch, fchi, rho, frho, out);
     }
     // rho -= cR chi; chi *= s
     lqcd_status rho_update(const double *cR, const double *s, T *ch, double2 *rho)
     {
-        std::vector<double> cs(2 * nrhs);
-        for (int r = 0; r < nrhs; r++) {
-            cs[2 * r] = s[r] - 1.0;
-            cs[2 * r + 1] = 0.0;
-        }
-        LQCD_TRY(bblas_multi_axpy(c, n2, nrhs, 1, cR, (const double *)ch, 0, n2, (double *)rho, n2, -1.0));
-        return bblas_multi_axpy(c, n2, nrhs, 1, cs.data(), (const double *)ch, 0, n2, (double *)ch, n2, 1.0);
+        return brho_update64(c, nh, nrhs, cR, s, ch, fchi, rho, frho);
     }
-    lqcd_status psi_update(int nk, const double *cf, const T *phi, long sa, double2 *psi)
+    lqcd_status psi_update(int nk, const double *cf, const T *phi, double2 *psi)
     {
-        return bblas_multi_axpy(c, n2, nrhs, nk, cf, (const double *)phi, 2 * sa, n2, (double *)psi, n2, 1.0);
+        return bblas_multi_axpy(c, 2 * fchi, nrhs, nk, cf, (const double *)phi, 2 * nrhs * fphi, 2 * fphi,
+                                (double *)psi, 2 * fchi, 1.0);
     }
-    double final_fields() const { return 7.0; }   // F64-field transfers of norm_rdot + rho_update
+    double final_fields() const { return 5.0; }   // F64-field transfers of norm_rdot + rho_update
 };
 
 struct Krylov32 {
     using T = float4;
     lqcd_ctx *c;
     const lqcd_solver_params *sp;
-    int nrhs;
-    long nf;    // elements (float4) per full F32 field
-    long nf64;  // double2 per full F64 field
-    Krylov32(lqcd_ctx *ctx, const lqcd_solver_params *p, int n)
-        : c(ctx), sp(p), nrhs(n), nf(12 * (long)ctx->g.Vh), nf64(24 * (long)ctx->g.Vh)
+    int nh, nrhs;
+    long fphi, fchi, frho;   // elements between right-hand sides
+    Krylov32(lqcd_ctx *ctx, const lqcd_solver_params *p, int halves, int n)
+        : c(ctx), sp(p), nh(halves), nrhs(n), fphi(12 * (long)ctx->g.Vh), fchi(6L * halves * ctx->g.Vh),
+          frho(24 * (long)ctx->g.Vh)
     {
     }
-    size_t field_bytes() const { return nf * sizeof(T); }
     // the preconditioner's output in F32: SAP in F32 writes it directly, other
-    // forms are converted from their own output precision
+    // forms are converted from their own output precision (the halves in use)
     lqcd_status precond_with(const lqcd_solver_params *p, const double2 *rho, T *ph)
     {
         const lqcd_sap_params &sap = p->sap;
+        const int hs = nh == 1 ? 2 : 1;   // distance of the converted halves
         if (p->solver == LQCD_SOLVER_SAP_GCR && sap.prec != LQCD_F64) {
             void *a;
             const size_t fb = 2 * native_half_bytes(c, sap.prec) * nrhs;
@@ -291,70 +302,87 @@ struct Krylov32 {
             void *b;
             LQCD_TRY(ws_get(c, WS_SAP_PSI, fb, &b));
             LQCD_TRY(sap_apply(c, &sap, a, b, nrhs));
-            return convert_native(c, sap.prec, LQCD_F32, b, ph, 2 * nrhs);
+            return convert_native(c, sap.prec, LQCD_F32, b, ph, nh * nrhs, hs, hs);
         }
         void *t;
-        LQCD_TRY(ws_get(c, WS_PHI64, (size_t)nf64 * nrhs * sizeof(double2), &t));
+        LQCD_TRY(ws_get(c, WS_PHI64, (size_t)frho * nrhs * sizeof(double2), &t));
         LQCD_TRY(precond(c, p, rho, (double2 *)t, nrhs));
-        return convert_native(c, LQCD_F64, LQCD_F32, t, ph, 2 * nrhs);
+        return convert_native(c, LQCD_F64, LQCD_F32, t, ph, nh * nrhs, hs, hs);
     }
-    lqcd_status D_inner(const T *ph, T *ch) { return dirac_D(c, LQCD_F32, ph, ch, nrhs); }
-    lqcd_status dots(const T *A, long sa, const T *B, int kk, double *out)
+    lqcd_status D_inner(const T *ph, T *ch)
     {
-        return bdot32(c, nf, nrhs, A, sa, nf, B, nf, kk, out);
+        if (nh == 2) return dirac_D(c, LQCD_F32, ph, ch, nrhs);
+        void *t;
+        LQCD_TRY(ws_get(c, WS_TMP_O, native_half_bytes(c, LQCD_F32) * nrhs, &t));
+        return dirac_dhat_s(c, LQCD_F32, ph, fphi, ch, fchi, t, nrhs);
     }
-    lqcd_status axpy(int k, const double *cf, const T *X, long sa, T *y, double sign)
+    lqcd_status dots(const T *A, const T *B, int kk, double *out)
     {
-        return bmulti_axpy32(c, nf, nrhs, k, cf, X, sa, nf, y, nf, sign);
+        return bdot32(c, fchi, nrhs, A, nrhs * fchi, fchi, B, fchi, kk, out);
+    }
+    lqcd_status axpy(int k, const double *cf, const T *X, T *y, double sign)
+    {
+        return bmulti_axpy32(c, fchi, nrhs, k, cf, X, nrhs * fchi, fchi, y, fchi, sign);
     }
     lqcd_status norm_rdot(const T *ch, const double2 *rho, double *out)
     {
-        return bnorm_rdot32(c, nrhs, ch, nf, rho, nf64, out);
+        return bnorm_rdot32(c, nh, nrhs, ch, fchi, rho, frho, out);
     }
     lqcd_status rho_update(const double *cR, const double *s, T *ch, double2 *rho)
     {
-        return brho_update32(c, nrhs, cR, s, ch, nf, rho, nf64);
+        return brho_update32(c, nh, nrhs, cR, s, ch, fchi, rho, frho);
     }
-    lqcd_status psi_update(int nk, const double *cf, const T *phi, long sa, double2 *psi)
+    lqcd_status psi_update(int nk, const double *cf, const T *phi, double2 *psi)
     {
-        return bmulti_axpy_mixed(c, nrhs, nk, cf, phi, sa, nf, psi, nf64);
+        return bmulti_axpy_mixed(c, nh, nrhs, nk, cf, phi, nrhs * fphi, fphi, psi, 12L * nh * c->g.Vh);
     }
     double final_fields() const { return 4.5; }
 };
 
-// flexible GCR on D psi_r = eta_r, warm start from psi; tol per rhs
+// flexible GCR on D psi_r = eta_r (nh = 2) or Dhat psi_r = eta_r (nh = 1) to
+// |residual| <= tol |eta|; psi, eta: nrhs native FP64 fields of nh halves.
+// warm: start from the given psi, which is zero otherwise.
 template <class KV>
-lqcd_status gcr_impl(lqcd_ctx *c, const lqcd_solver_params *sp, const std::vector<double> &tol, const double2 *eta,
-                     double2 *psi, int nrhs, int nmx, GcrState &S)
+lqcd_status gcr_impl(lqcd_ctx *c, const lqcd_solver_params *sp, double tol, int nh, const double2 *eta,
+                     double2 *psi, bool warm, int nrhs, int nmx, GcrState &S)
 {
     using T = typename KV::T;
-    KV kv(c, sp, nrhs);
+    KV kv(c, sp, nh, nrhs);
     const long Vh = c->g.Vh;
-    const long n2 = 48 * Vh;   // doubles in one full F64 field
-    const long nf = kv.nf;     // Krylov elements per field
+    const long ne = 12L * nh * Vh;   // double2 per FP64 field of nh halves
     const int nkv = sp->nkv;
     if (nkv < 1 || nkv > 64) return set_err(c, LQCD_ERR_ARG, "nkv=%d", nkv);
     if (nrhs * nkv > 1024 || nrhs > 64) return set_err(c, LQCD_ERR_ARG, "nrhs=%d with nkv=%d too large", nrhs, nkv);
-    const long bf = nrhs * nf;   // Krylov elements per batch of fields
-    const size_t bf64 = (size_t)nrhs * 24 * Vh;   // double2 per batch of F64 fields
+    const long bphi = nrhs * kv.fphi, bchi = nrhs * kv.fchi;   // Krylov elements per batch of fields
+    const size_t brho = (size_t)nrhs * kv.frho;
     void *buf;
-    LQCD_TRY(ws_get(c, WS_SOLVER, 2 * nkv * bf * sizeof(T) + 2 * bf64 * sizeof(double2), &buf));
-    T *phi = (T *)buf, *chi = phi + nkv * bf;
-    double2 *rho = (double2 *)(chi + nkv * bf), *w = rho + bf64;
+    LQCD_TRY(ws_get(c, WS_SOLVER, nkv * (bphi + bchi) * sizeof(T) + (brho + nrhs * ne) * sizeof(double2), &buf));
+    T *phi = (T *)buf, *chi = phi + nkv * bphi;
+    double2 *rho = (double2 *)(chi + nkv * bchi), *w = rho + brho;
     const double inner_gain = sp->inner == LQCD_F64 ? 0.0 : 1e-5;
-    const double gs_field = (double)bf * sizeof(T);
+    const double gs_field = (double)bchi * sizeof(T);
     PhaseProf prof(c);
-    std::vector<double> eta2, rn2, eta_n(nrhs), res(nrhs), cycle_start(nrhs);
-    LQCD_TRY(bnorm2(c, n2, nrhs, eta, eta2));
-    LQCD_TRY(dirac_D(c, LQCD_F64, psi, w, nrhs));
-    LQCD_TRY(blas_sub(c, n2 * nrhs, (const double *)eta, (const double *)w, (double *)rho));
-    LQCD_TRY(bnorm2(c, n2, nrhs, rho, rn2));
+    std::vector<double> eta2(nrhs), rn2(nrhs), eta_n(nrhs), res(nrhs), cycle_start(nrhs);
+    if (nh == 1) LQCD_TRY(blas_zero(c, brho * sizeof(double2), rho));
+    // rho = eta - D psi (with_psi) or eta, and its norms
+    auto residual = [&](bool with_psi, std::vector<double> &norms) -> lqcd_status {
+        if (with_psi && nh == 2) LQCD_TRY(dirac_D(c, LQCD_F64, psi, w, nrhs));
+        if (with_psi && nh == 1) {
+            void *t;
+            LQCD_TRY(ws_get(c, WS_TMP_O, native_half_bytes(c, LQCD_F64) * nrhs, &t));
+            LQCD_TRY(dirac_dhat(c, LQCD_F64, psi, w, t, nrhs));
+        }
+        return bresidual64(c, nh, nrhs, eta, ne, with_psi ? w : nullptr, ne, rho, kv.frho, norms.data());
+    };
+    LQCD_TRY(residual(false, eta2));
+    rn2 = eta2;
+    if (warm) LQCD_TRY(residual(true, rn2));
     std::vector<char> active(nrhs);
     for (int r = 0; r < nrhs; r++) {
         eta_n[r] = std::sqrt(eta2[r]);
         res[r] = std::sqrt(rn2[r]);
         if (!std::isfinite(res[r])) S.status[r] = LQCD_ERR_NAN;
-        else if (eta_n[r] == 0 || res[r] <= tol[r] * eta_n[r]) S.status[r] = LQCD_OK;
+        else if (eta_n[r] == 0 || res[r] <= tol * eta_n[r]) S.status[r] = LQCD_OK;
         else S.status[r] = LQCD_ERR_NOT_CONVERGED;
         active[r] = S.status[r] == LQCD_ERR_NOT_CONVERGED;
     }
@@ -372,7 +400,7 @@ lqcd_status gcr_impl(lqcd_ctx *c, const lqcd_solver_params *sp, const std::vecto
         std::vector<char> done(nrhs, 0);
         for (int r = 0; r < nrhs; r++) cycle_start[r] = res[r];
         for (int k = 0; k < nkv && it < nmx; k++) {
-            T *ph = phi + k * bf, *ch = chi + k * bf;
+            T *ph = phi + k * bphi, *ch = chi + k * bchi;
             prof.start();
             LQCD_TRY(kv.precond_with(sp, rho, ph));
             prof.stop(0);
@@ -390,7 +418,7 @@ lqcd_status gcr_impl(lqcd_ctx *c, const lqcd_solver_params *sp, const std::vecto
                 // first pass reduces chi_0..chi_k against chi_k, which also gives |chi_k|^2.
                 for (int pass = 0; pass < 2 && k > 0; pass++) {
                     const int kk = pass == 0 ? k + 1 : k;
-                    LQCD_TRY(kv.dots(chi, bf, ch, kk, dots.data()));
+                    LQCD_TRY(kv.dots(chi, ch, kk, dots.data()));
                     bool again = false;
                     std::vector<double> cf(2 * (size_t)nrhs * k);
                     for (int r = 0; r < nrhs; r++) {
@@ -405,7 +433,7 @@ lqcd_status gcr_impl(lqcd_ctx *c, const lqcd_solver_params *sp, const std::vecto
                         }
                         if (pass == 0 && active[r] && removed > 0.5 * dots[2 * (r * kk + k)]) again = true;
                     }
-                    LQCD_TRY(kv.axpy(k, cf.data(), chi, bf, ch, -1.0));
+                    LQCD_TRY(kv.axpy(k, cf.data(), chi, ch, -1.0));
                     // bytes: the dot reads kk + 1 fields, the update k + 1 and writes one
                     c->prof_gs_bytes += (kk + 1 + k + 2) * gs_field;
                     if (!again) break;
@@ -428,14 +456,15 @@ lqcd_status gcr_impl(lqcd_ctx *c, const lqcd_solver_params *sp, const std::vecto
                 }
                 if (!reject.empty()) {
                     void *fb;
-                    LQCD_TRY(ws_get(c, WS_NET_FALLBACK, (size_t)bf * sizeof(T), &fb));
+                    LQCD_TRY(ws_get(c, WS_NET_FALLBACK, (size_t)bphi * sizeof(T), &fb));
                     lqcd_solver_params sap_only = *sp;
                     sap_only.solver = sp->solver == LQCD_SOLVER_DFL_NET_GCR ? LQCD_SOLVER_DFL_SAP_GCR
                                                                             : LQCD_SOLVER_SAP_GCR;
                     LQCD_TRY(kv.precond_with(&sap_only, rho, (T *)fb));
                     for (int r : reject) {
-                        LQCD_CUDA_CHECK(c, cudaMemcpyAsync(ph + r * nf, (T *)fb + r * nf, kv.field_bytes(),
-                                                           cudaMemcpyDeviceToDevice, c->stream));
+                        LQCD_CUDA_CHECK(c, cudaMemcpyAsync(ph + r * kv.fphi, (T *)fb + r * kv.fphi,
+                                                           kv.fphi * sizeof(T), cudaMemcpyDeviceToDevice,
+                                                           c->stream));
                         S.net_fallbacks[r]++;
                     }
                     LQCD_TRY(orth());
@@ -460,7 +489,7 @@ lqcd_status gcr_impl(lqcd_ctx *c, const lqcd_solver_params *sp, const std::vecto
                 if (active[r]) rn2[r] = std::max(0.0, rn2[r] - (cr * cr + ci * ci));
             }
             LQCD_TRY(kv.rho_update(coef.data(), sx.data(), ch, rho));
-            c->prof_gs_bytes += kv.final_fields() * (double)bf64 * sizeof(double2);
+            c->prof_gs_bytes += kv.final_fields() * (double)(nrhs * ne) * sizeof(double2);
             it++;
             nk = k + 1;
             bool recompute = false;
@@ -469,12 +498,17 @@ lqcd_status gcr_impl(lqcd_ctx *c, const lqcd_solver_params *sp, const std::vecto
                 // |rho|^2 - |c|^2 loses digits once |rho| has dropped ~1e7 within the cycle
                 if (active[r] && rn2[r] < 1e-14 * cycle_start[r] * cycle_start[r]) recompute = true;
             }
-            if (recompute) LQCD_TRY(bnorm2(c, n2, nrhs, rho, rn2));
+            if (recompute) {
+                std::vector<double> d(2 * nrhs);
+                LQCD_TRY(bblas_dot(c, 2 * ne, nrhs, (const double *)rho, 0, 2 * kv.frho, (const double *)rho,
+                                   2 * kv.frho, 1, d.data()));
+                for (int r = 0; r < nrhs; r++) rn2[r] = d[2 * r];
+            }
             prof.stop(2);
             bool all_done = true;
             for (int r = 0; r < nrhs; r++) {
                 double rr = std::sqrt(rn2[r]);
-                if (!active[r] || rr <= tol[r] * eta_n[r] || rr <= inner_gain * cycle_start[r]) done[r] = 1;
+                if (!active[r] || rr <= tol * eta_n[r] || rr <= inner_gain * cycle_start[r]) done[r] = 1;
                 all_done = all_done && done[r];
             }
             if (all_done) break;
@@ -497,11 +531,9 @@ lqcd_status gcr_impl(lqcd_ctx *c, const lqcd_solver_params *sp, const std::vecto
             }
         }
         prof.start();
-        if (nk > 0) LQCD_TRY(kv.psi_update(nk, coef.data(), phi, bf, psi));
+        if (nk > 0) LQCD_TRY(kv.psi_update(nk, coef.data(), phi, psi));
         // restart from the FP64 true residual
-        LQCD_TRY(dirac_D(c, LQCD_F64, psi, w, nrhs));
-        LQCD_TRY(blas_sub(c, n2 * nrhs, (const double *)eta, (const double *)w, (double *)rho));
-        LQCD_TRY(bnorm2(c, n2, nrhs, rho, rn2));
+        LQCD_TRY(residual(true, rn2));
         prof.stop(3);
         for (int r = 0; r < nrhs; r++) {
             if (!active[r]) continue;
@@ -510,7 +542,7 @@ lqcd_status gcr_impl(lqcd_ctx *c, const lqcd_solver_params *sp, const std::vecto
             if (!std::isfinite(res[r])) {
                 S.status[r] = LQCD_ERR_NAN;
                 active[r] = 0;
-            } else if (res[r] <= tol[r] * eta_n[r]) {
+            } else if (res[r] <= tol * eta_n[r]) {
                 S.status[r] = LQCD_OK;
                 active[r] = 0;
             }
@@ -521,33 +553,11 @@ lqcd_status gcr_impl(lqcd_ctx *c, const lqcd_solver_params *sp, const std::vecto
 }
 
 // Krylov vectors in F64 or (krylov == F32, inner == F32) in F32
-lqcd_status gcr_native(lqcd_ctx *c, const lqcd_solver_params *sp, const std::vector<double> &tol,
-                       const double2 *eta, double2 *psi, int nrhs, int nmx, GcrState &S)
+lqcd_status gcr_native(lqcd_ctx *c, const lqcd_solver_params *sp, int nh, const double2 *eta, double2 *psi, bool warm,
+                       int nrhs, GcrState &S)
 {
-    if (sp->krylov == LQCD_F32) return gcr_impl<Krylov32>(c, sp, tol, eta, psi, nrhs, nmx, S);
-    return gcr_impl<Krylov64>(c, sp, tol, eta, psi, nrhs, nmx, S);
-}
-
-// |eta_e - Dhat psi_e| / |eta_e| per rhs; eta, psi: nrhs native full fields (even halves used)
-lqcd_status dhat_relres(lqcd_ctx *c, const double2 *eta, const double2 *psi, int nrhs, std::vector<double> &out)
-{
-    const long Vh = c->g.Vh;
-    const long n2 = 24 * Vh;   // doubles in one even field
-    const long nf = 24 * Vh;   // double2 per full field
-    void *b, *tmp_o;
-    LQCD_TRY(ws_get(c, WS_MISC, 2 * native_half_bytes(c, LQCD_F64), &b));
-    LQCD_TRY(ws_get(c, WS_TMP_O, native_half_bytes(c, LQCD_F64), &tmp_o));
-    double2 *w = (double2 *)b, *rr = w + 12 * Vh;
-    out.resize(nrhs);
-    for (int r = 0; r < nrhs; r++) {
-        LQCD_TRY(dirac_dhat(c, LQCD_F64, psi + r * nf, w, tmp_o, 1));
-        LQCD_TRY(blas_sub(c, n2, (const double *)(eta + r * nf), (const double *)w, (double *)rr));
-        double x, e;
-        LQCD_TRY(blas_norm2(c, n2, (const double *)rr, &x));
-        LQCD_TRY(blas_norm2(c, n2, (const double *)(eta + r * nf), &e));
-        out[r] = e > 0 ? std::sqrt(x / e) : 0;
-    }
-    return LQCD_OK;
+    if (sp->krylov == LQCD_F32) return gcr_impl<Krylov32>(c, sp, sp->tol, nh, eta, psi, warm, nrhs, sp->nmx, S);
+    return gcr_impl<Krylov64>(c, sp, sp->tol, nh, eta, psi, warm, nrhs, sp->nmx, S);
 }
 
 lqcd_status check_params(lqcd_ctx *c, const lqcd_solver_params *p, int nrhs)
@@ -571,9 +581,7 @@ lqcd_status check_params(lqcd_ctx *c, const lqcd_solver_params *p, int nrhs)
 
 lqcd_status worst(lqcd_status a, lqcd_status b) { return a != LQCD_OK ? a : b; }
 
-// guess: psi holds the initial even-site guess x0 on entry (GCR solvers); the
-// odd part of the full-lattice start is -A_oo^-1 H_oe x0, so that the full
-// residual starts as (eta_e - Dhat x0, 0)
+// guess: psi holds the initial even-site guess x0 on entry (GCR solvers)
 lqcd_status solve_dhat_impl(lqcd_ctx *c, const lqcd_solver_params *p, const double *eta, double *psi, int nrhs,
                             lqcd_solve_info *info, bool guess)
 {
@@ -599,49 +607,25 @@ lqcd_status solve_dhat_impl(lqcd_ctx *c, const lqcd_solver_params *p, const doub
             all = worst(all, st);
         }
     } else {
-        // full fields (eta_e, 0) for every rhs, solved together
+        // the even halves of every rhs, solved together
         void *io;
-        LQCD_TRY(ws_get(c, WS_SOLVE_IO, 4 * hb * nrhs, &io));
-        double2 *eta_f = (double2 *)io, *psi_f = eta_f + nrhs * nf;
-        LQCD_TRY(blas_zero(c, 4 * hb * nrhs, io));
-        for (int k = 0; k < nrhs; k++)
-            LQCD_TRY(pack_field(c, LQCD_F64, 1, eta + (size_t)k * 24 * Vh, eta_f + k * nf, 1, false));
-        if (guess) {
-            const long hh = 12 * Vh;   // double2 in one half field
-            for (int k = 0; k < nrhs; k++)
-                LQCD_TRY(pack_field(c, LQCD_F64, 1, psi + (size_t)k * 24 * Vh, psi_f + k * nf, 1, false));
-            LQCD_TRY(dirac_hop_parity(c, LQCD_F64, 1, psi_f, psi_f + hh, nf, nf, nrhs));
-            for (int k = 0; k < nrhs; k++) {
-                double2 *po = psi_f + k * nf + hh;
-                LQCD_TRY(clover_apply_native64(c, 1, 1, po, po));
-                LQCD_TRY(blas_scal(c, 2 * hh, -1.0, 0.0, (double *)po));
-            }
-        }
+        LQCD_TRY(ws_get(c, WS_SOLVE_IO, 2 * hb * nrhs, &io));
+        double2 *eta_e = (double2 *)io, *psi_e = eta_e + nrhs * 12 * Vh;
+        LQCD_TRY(pack_field(c, LQCD_F64, 1, eta, eta_e, nrhs, false));
+        if (guess)
+            LQCD_TRY(pack_field(c, LQCD_F64, 1, psi, psi_e, nrhs, false));
+        else
+            LQCD_TRY(blas_zero(c, hb * nrhs, psi_e));
         GcrState S(nrhs);
-        std::vector<double> tol(nrhs, p->tol), rh(nrhs, 0);
-        for (int attempt = 0; attempt < 4; attempt++) {
-            int used = 0;
-            for (int k = 0; k < nrhs; k++) used = std::max(used, S.iters[k]);
-            LQCD_TRY(gcr_native(c, p, tol, eta_f, psi_f, nrhs, p->nmx - used, S));
-            LQCD_TRY(dhat_relres(c, eta_f, psi_f, nrhs, rh));
-            bool again = false;
-            for (int k = 0; k < nrhs; k++)
-                if (S.status[k] == LQCD_OK && rh[k] > p->tol) {
-                    // the Dhat residual r_e - H_eo A_oo^-1 r_o is not bounded by |r|: tighten
-                    tol[k] = tol[k] * std::max(0.05, 0.5 * p->tol / rh[k]);
-                    S.status[k] = LQCD_ERR_NOT_CONVERGED;
-                    again = true;
-                }
-            if (!again) break;
-        }
+        LQCD_TRY(gcr_native(c, p, 1, eta_e, psi_e, guess, nrhs, S));
+        LQCD_TRY(pack_field(c, LQCD_F64, 1, psi, psi_e, nrhs, true));
         for (int k = 0; k < nrhs; k++) {
-            if (S.status[k] == LQCD_OK && rh[k] > p->tol) S.status[k] = LQCD_ERR_NOT_CONVERGED;
-            LQCD_TRY(pack_field(c, LQCD_F64, 1, psi + (size_t)k * 24 * Vh, psi_f + k * nf, 1, true));
             if (info) {
                 info[k].iters = S.iters[k];
                 info[k].restarts = S.restarts[k];
+                // with psi_o = -A_oo^-1 H_oe psi_e the residual of D is that of Dhat
                 info[k].true_relres = S.relres[k];
-                info[k].relres_dhat = rh[k];
+                info[k].relres_dhat = S.relres[k];
                 info[k].status = S.status[k];
                 info[k].seconds = now_s() - t0;
                 info[k].net_fallbacks = S.net_fallbacks[k];
@@ -685,8 +669,7 @@ lqcd_status lqcd_solve_D(lqcd_ctx *c, const lqcd_solver_params *p, const double 
     LQCD_TRY(pack_field(c, LQCD_F64, 2, eta, eta_f, nrhs, false));
     LQCD_TRY(blas_zero(c, 2 * hb * nrhs, psi_f));
     GcrState S(nrhs);
-    std::vector<double> tol(nrhs, p->tol);
-    LQCD_TRY(gcr_native(c, p, tol, eta_f, psi_f, nrhs, p->nmx, S));
+    LQCD_TRY(gcr_native(c, p, 2, eta_f, psi_f, false, nrhs, S));
     LQCD_TRY(pack_field(c, LQCD_F64, 2, psi, psi_f, nrhs, true));
     lqcd_status all = LQCD_OK;
     for (int k = 0; k < nrhs; k++) {
