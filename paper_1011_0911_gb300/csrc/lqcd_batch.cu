@@ -776,9 +776,12 @@ lqcd_status lqcd_batch_solve_dhat(lqcd_batch *b, const double *const *eta_dev, d
     std::vector<BScal> S(n);
     std::vector<cudaStream_t> saved(n);
     for (int l = 0; l < n; l++) {
+        saved[l] = b->ctx[l]->stream;
+        b->ctx[l]->stream = b->st;
+    }
+    LQCD_TRY(sap_batch_refresh(b->sap, b->ctx.data(), n, b->p.sap.bs));
+    for (int l = 0; l < n; l++) {
         lqcd_ctx *c = b->ctx[l];
-        saved[l] = c->stream;
-        c->stream = b->st;
         LQCD_TRY(pack_field(c, LQCD_F64, 1, eta_dev[l], b->eta + b->lat_h[l].off64, 1, false));
         double e2 = 0;
         LQCD_TRY(blas_norm2(c, 24 * b->lat_h[l].Vh, (const double *)(b->eta + b->lat_h[l].off64), &e2));

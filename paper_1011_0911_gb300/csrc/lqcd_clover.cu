@@ -321,6 +321,7 @@ lqcd_status clover_build(lqcd_ctx *c, double kappa, double csw, double *ld_e, do
     a.logdet = logdet;
     a.singular = sing;
     a.even_scale = even_scale;
+    c->op_version++;
     k_clover<<<dim3(div_up(Vh, 128), 2), 128, 0, c->stream>>>(a);
     c->n_kernel_launches++;
     LQCD_LAUNCH_CHECK(c);

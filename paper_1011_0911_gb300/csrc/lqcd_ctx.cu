@@ -495,6 +495,7 @@ lqcd_status lqcd_set_gauge(lqcd_ctx *c, const double *U_dev)
     LQCD_LAUNCH_CHECK(c);
     c->have_gauge = true;
     c->have_clover = false;
+    c->op_version++;
     dfl_free(c);
     return LQCD_OK;
 }

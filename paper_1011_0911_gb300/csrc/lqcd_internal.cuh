@@ -198,6 +198,7 @@ struct lqcd_ctx {
     float4 *A32[2] = {nullptr, nullptr}, *Ai32[2] = {nullptr, nullptr};   // [18][Vh]
     uint2 *A16[2] = {nullptr, nullptr}, *Ai16[2] = {nullptr, nullptr};    // [18][Vh], FP16
     bool have_clover = false;
+    long op_version = 0;   // changes with the links and with the clover term
     double kappa = 0, csw = 0;
     double logdet_e = 0, logdet_o = 0;   // log|det A| of each parity, from the last clover build
     // device scratch for reductions
@@ -382,6 +383,7 @@ struct SapBatch;
 lqcd_status sap_batch_create(lqcd_ctx *hc, lqcd_ctx *const *ctx, int n, const lqcd_sap_params *sp, void *r,
                              void *psi, void *delta, const long *off, SapBatch **out_b);
 lqcd_status sap_batch_apply(lqcd_ctx *hc, SapBatch *b, const void *eta, size_t bytes, const int *active_dev);
+lqcd_status sap_batch_refresh(SapBatch *b, lqcd_ctx *const *ctx, int n, const int bs[4]);
 void sap_batch_free(SapBatch *b);
 void chrono_free(lqcd_ctx *c);
 // learned preconditioner

@@ -365,6 +365,12 @@ struct SapArgs {
     long fstride;                    // spinor units between the fields of consecutive right-hand sides
     const typename SapT<P>::LK *U;
     const typename SapT<P>::CL *Ae, *Aio;   // A on even sites, A^-1 on odd sites
+    // the operator as the resident block kernel reads it: in block order (perm = 1,
+    // site t of the block in place slot of the plan's list at slot * nh + t) or,
+    // where the copy could not be allocated, the arrays above (perm = 0)
+    const typename SapT<P>::LK *Ub;
+    const typename SapT<P>::CL *Aeb, *Aiob;
+    int perm, slot0;     // slot of block list entry 0
     int nmr;
 };
 
@@ -683,29 +689,32 @@ __device__ __forceinline__ void proj_apply_rt(float sgn, const cx<float> psi[12]
     }
 }
 
-// half of the in-block hop sum at site (l, x) from the smem field src of the
-// other parity: h = 0 forward hops, h = 1 backward hops; then the pair's halves
-// are added so both threads hold the full sum S (before the -1/2).  own: the
-// site's index par * SAPS_NH + t in the link arrays; the neighbours' links sit
-// at (1 - par) * SAPS_NH + their half index.  Both halves run the same
-// instructions (the sense, the link slot and U versus U^dag are selected per
-// lane), and a hop that leaves the block is computed with weight 0 from an
-// in-block slot instead of being skipped, so the warp never diverges here.
+// Chirality half h of the in-block hop sum S (before the -1/2) at site (l, x)
+// from the smem field src of the other parity: thread h = 0 takes the forward
+// hops, h = 1 the backward ones, each hands the other's half over and adds what
+// it gets to its own.  own: the site's index par * SAPS_NH + t in the link
+// arrays; the neighbours' links sit at (1 - par) * SAPS_NH + their half index.
+// Both threads run the same instructions (the sense, the link slot and U versus
+// U^dag are selected per lane), and a hop that leaves the block is computed
+// with weight 0 instead of being skipped, so the warp never diverges here; its
+// dummy neighbour is t itself, the neighbour of a lane nearby, so that the
+// loads stay free of bank conflicts.
 template <class SM>
 __device__ __forceinline__ void s_hopsum(const Geom &g, const BlkGeom &B, const SM &S, int h, const int l[4],
-                                         const int x[4], int own, const float4 (*src)[SAPS_NH], cx<float> acc[12])
+                                         const int x[4], int own, const float4 (*src)[SAPS_NH], cx<float> out[6])
 {
+    cx<float> acc[12];
 #pragma unroll
     for (int i = 0; i < 12; i++) acc[i] = mk(0.f, 0.f);
     const float sgn = h ? 1.f : -1.f;
     const int d = h ? -1 : 1;
-    const int oth = own < SAPS_NH ? SAPS_NH : 0;
+    const int oth = own < SAPS_NH ? SAPS_NH : 0, t = own < SAPS_NH ? own : own - SAPS_NH;
     const int xt = h ? 0 : g.L[0] - 1;
     cx<float> u[3][3], v[12];
 #pragma unroll
     for (int mu = 0; mu < 4; mu++) {
         const int ln = blk_nbr_lex(B, l, mu, d);
-        const int n = ln >= 0 ? ln >> 1 : 0;
+        const int n = ln >= 0 ? ln >> 1 : t;
         float sg = (mu == 0 && x[0] == xt) ? float(g.bc_t) : 1.f;
         sg = ln >= 0 ? sg : 0.f;
         s_link(S, mu, h ? oth + n : own, u);
@@ -723,17 +732,11 @@ __device__ __forceinline__ void s_hopsum(const Geom &g, const BlkGeom &B, const 
         }
     }
 #pragma unroll
-    for (int i = 0; i < 12; i++) {
-        acc[i].re += __shfl_xor_sync(0xffffffffu, acc[i].re, 16);
-        acc[i].im += __shfl_xor_sync(0xffffffffu, acc[i].im, 16);
+    for (int i = 0; i < 6; i++) {
+        const cx<float> give = h ? acc[i] : acc[6 + i], keep = h ? acc[6 + i] : acc[i];
+        out[i].re = keep.re + __shfl_xor_sync(0xffffffffu, give.re, 16);
+        out[i].im = keep.im + __shfl_xor_sync(0xffffffffu, give.im, 16);
     }
-}
-
-// the chirality half h of a 12-component spinor (predicated select, no local memory)
-__device__ __forceinline__ void s_half(const cx<float> acc[12], int h, cx<float> out[6])
-{
-#pragma unroll
-    for (int i = 0; i < 6; i++) out[i] = h ? acc[6 + i] : acc[i];
 }
 
 __device__ __forceinline__ void stage_site(const float4 *f, long Vh, long r, float4 o[6])
@@ -836,20 +839,24 @@ __device__ __forceinline__ void sap_block_s_body(const SapArgs<P> &a, int bi, in
         org[3] = c3 * B.bs[3];
     }
     const int tid = threadIdx.x;
+    const typename SapT<P>::LK *U = a.perm ? a.Ub : a.U;
+    const typename SapT<P>::CL *Ae = a.perm ? a.Aeb : a.Ae, *Aio = a.perm ? a.Aiob : a.Aio;
+    const long op0 = (long)(a.slot0 + bi) * nh;   // the block's first site in the block-ordered operator
     // ---- stage links, clover and r_o (one thread per block site, both parities)
     for (int i = tid; i < 2 * nh; i += blockDim.x) {
         const int par = i >= nh, t = par ? i - nh : i;
         SiteInfo s;
         block_site(a.g, B, org, par, t, s);
         const int ls = par * SAPS_NH + t;
+        const long op = a.perm ? op0 + t : s.grank;
 #pragma unroll
         for (int mu = 0; mu < 4; mu++)
 #pragma unroll
-            for (int q = 0; q < 3; q++) stage_link(S.U[mu][q][ls], a.U + ((long)(par * 4 + mu) * 3 + q) * Vh + s.grank);
+            for (int q = 0; q < 3; q++) stage_link(S.U[mu][q][ls], U + ((long)(par * 4 + mu) * 3 + q) * Vh + op);
         if constexpr (SA) {
-            const typename SapT<P>::CL *A = par ? a.Aio : a.Ae;
+            const typename SapT<P>::CL *A = par ? Aio : Ae;
 #pragma unroll
-            for (int q = 0; q < 18; q++) S.A[q][ls] = stage4(A + q * Vh + s.grank);
+            for (int q = 0; q < 18; q++) S.A[q][ls] = stage4(A + q * Vh + op);
         }
         float4 site[6];
         stage_site(par ? r_o : r_e, Vh, s.grank, site);
@@ -868,13 +875,14 @@ __device__ __forceinline__ void sap_block_s_body(const SapArgs<P> &a, int bi, in
     // array (no bank conflicts between a site's two halves)
     const int h = (tid >> 4) & 1, t = ((tid >> 5) << 4) | (tid & 15);
     const bool act = t < nh;
-    SiteInfo so, se;
+    SiteInfo so = {}, se = {};
     const int lso = SAPS_NH + t, lse = t;   // the sites' slots in the link / clover arrays
     if (act) {
         block_site(a.g, B, org, 1, t, so);
         block_site(a.g, B, org, 0, t, se);
     }
-    cx<float> acc[12], v[6], w[6];
+    const long opo = a.perm ? op0 + t : so.grank, ope = a.perm ? op0 + t : se.grank;
+    cx<float> ah[6], v[6], w[6];
     float4 chi4[3];   // this thread's half of chi_e
 #pragma unroll
     for (int q = 0; q < 3; q++) chi4[q] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -886,16 +894,14 @@ __device__ __forceinline__ void sap_block_s_body(const SapArgs<P> &a, int bi, in
             v[2 * q] = mk(x.x, x.y);
             v[2 * q + 1] = mk(x.z, x.w);
         }
-        s_clover_half<SA>(S, lso, a.Aio, Vh, so.grank, h, v, w);
+        s_clover_half<SA>(S, lso, Aio, Vh, opo, h, v, w);
 #pragma unroll
         for (int q = 0; q < 3; q++) S.to[3 * h + q][t] = make_float4(w[2 * q].re, w[2 * q].im, w[2 * q + 1].re, w[2 * q + 1].im);
     }
     __syncthreads();
     // rho = r_e - H_eo to = r_e + 1/2 S
     if (act) {
-        s_hopsum(a.g, B, S, h, se.l, se.x, lse, S.to, acc);
-        cx<float> ah[6];
-        s_half(acc, h, ah);
+        s_hopsum(a.g, B, S, h, se.l, se.x, lse, S.to, ah);
 #pragma unroll
         for (int q = 0; q < 3; q++) {
             float4 x = S.rho[3 * h + q][t];
@@ -907,11 +913,10 @@ __device__ __forceinline__ void sap_block_s_body(const SapArgs<P> &a, int bi, in
     for (int it = 0; it < a.nmr; it++) {
         // to = A_oo^-1 (-1/2 S(rho))
         if (act) {
-            s_hopsum(a.g, B, S, h, so.l, so.x, lso, S.rho, acc);
-            s_half(acc, h, v);
+            s_hopsum(a.g, B, S, h, so.l, so.x, lso, S.rho, ah);
 #pragma unroll
-            for (int i = 0; i < 6; i++) v[i] = -0.5f * v[i];
-            s_clover_half<SA>(S, lso, a.Aio, Vh, so.grank, h, v, w);
+            for (int i = 0; i < 6; i++) v[i] = -0.5f * ah[i];
+            s_clover_half<SA>(S, lso, Aio, Vh, opo, h, v, w);
 #pragma unroll
             for (int q = 0; q < 3; q++) S.to[3 * h + q][t] = make_float4(w[2 * q].re, w[2 * q].im, w[2 * q + 1].re, w[2 * q + 1].im);
         }
@@ -919,7 +924,7 @@ __device__ __forceinline__ void sap_block_s_body(const SapArgs<P> &a, int bi, in
         // p = A_ee rho + 1/2 S(to); partial <p,p>, <p,rho>
         float pp = 0.f, pr = 0.f, pi = 0.f;
         if (act) {
-            s_hopsum(a.g, B, S, h, se.l, se.x, lse, S.to, acc);
+            s_hopsum(a.g, B, S, h, se.l, se.x, lse, S.to, ah);
             cx<float> x[6];
 #pragma unroll
             for (int q = 0; q < 3; q++) {
@@ -927,9 +932,7 @@ __device__ __forceinline__ void sap_block_s_body(const SapArgs<P> &a, int bi, in
                 x[2 * q] = mk(y.x, y.y);
                 x[2 * q + 1] = mk(y.z, y.w);
             }
-            s_clover_half<SA>(S, lse, a.Ae, Vh, se.grank, h, x, w);
-            cx<float> ah[6];
-            s_half(acc, h, ah);
+            s_clover_half<SA>(S, lse, Ae, Vh, ope, h, x, w);
 #pragma unroll
             for (int i = 0; i < 6; i++) {
                 w[i] = w[i] + 0.5f * ah[i];
@@ -986,16 +989,14 @@ __device__ __forceinline__ void sap_block_s_body(const SapArgs<P> &a, int bi, in
         for (int q = 0; q < 3; q++) S.p[3 * h + q][t] = chi4[q];
     __syncthreads();
     if (act) {
-        s_hopsum(a.g, B, S, h, so.l, so.x, lso, S.p, acc);
-        cx<float> ah[6];
-        s_half(acc, h, ah);
+        s_hopsum(a.g, B, S, h, so.l, so.x, lso, S.p, ah);
 #pragma unroll
         for (int q = 0; q < 3; q++) {
             float4 x = S.ro[3 * h + q][t];
             v[2 * q] = mk(x.x + 0.5f * ah[2 * q].re, x.y + 0.5f * ah[2 * q].im);
             v[2 * q + 1] = mk(x.z + 0.5f * ah[2 * q + 1].re, x.w + 0.5f * ah[2 * q + 1].im);
         }
-        s_clover_half<SA>(S, lso, a.Aio, Vh, so.grank, h, v, w);
+        s_clover_half<SA>(S, lso, Aio, Vh, opo, h, v, w);
         cx<float> ce[6], re[6], zero[6];
 #pragma unroll
         for (int q = 0; q < 3; q++) {
@@ -1183,6 +1184,13 @@ struct SapPlan {
     BlkGeom B;
     int2 *face_dev[2] = {nullptr, nullptr};   // sites updated after colour col (k_sap_face_l)
     int nface[2] = {0, 0};
+    // the operator in block order, [F32, F16S]: links, A_ee, A_oo^-1 in one buffer
+    // (the plan's own; made again when the context's operator has changed)
+    struct Perm {
+        void *p = nullptr;
+        long version = -1;
+        bool failed = false;
+    } perm[2];
 };
 
 // one cached plan per context (keyed by block shape)
@@ -1274,14 +1282,80 @@ lqcd_status get_plan(lqcd_ctx *c, const int bs[4], SapPlan **out)
     return LQCD_OK;
 }
 
+// row-wise copy out[row Vh + slot nh + t] = in[row Vh + rank], rows of parity par0 +
+// row / rows_per_parity
+template <class T>
+__global__ void k_sap_permute(Geom g, BlkGeom B, const int *blocks, int rows_per_parity, int par0,
+                              const T *__restrict__ in, T *out)
+{
+    const long pos = blockIdx.x * (long)blockDim.x + threadIdx.x;
+    if (pos >= g.Vh) return;
+    const int row = blockIdx.y, par = par0 + row / rows_per_parity;
+    const int slot = (int)(pos / B.nh), t = (int)(pos - (long)slot * B.nh);
+    int id = blocks[slot], org[4];
+#pragma unroll
+    for (int i = 3; i >= 0; i--) {
+        org[i] = id % B.nb[i] * B.bs[i];
+        id /= B.nb[i];
+    }
+    SiteInfo s;
+    block_site(g, B, org, par, t, s);
+    out[row * (long)g.Vh + pos] = in[row * (long)g.Vh + s.grank];
+}
+
+// The block-ordered operator of the plan, in args.  A block's 128 sites per
+// parity lie in runs of bs3 / 2 ranks, so that a warp's load of one link or
+// clover word touched 16 lines: at nmr = 4 the clover loads alone were 40 % of
+// the L1 wavefronts that bounded the kernel (67 % of their peak).  In block
+// order they are one run.  With the halved lane exchange of s_hopsum, per colour
+// launch at 32 x 16^3: F16S, 12 right-hand sides, nmr 4: 444 -> 380 us; FP32, one,
+// nmr 5: 64.5 -> 49.4 us.
 template <int P>
-lqcd_status sap_run(lqcd_ctx *c, const SapPlan &P_, int ncy, int nmr, const void *eta, void *psi, void *r,
+lqcd_status sap_operator(lqcd_ctx *c, SapPlan &pl, SapArgs<P> &a)
+{
+    using LK = typename SapT<P>::LK;
+    using CL = typename SapT<P>::CL;
+    static_assert(sizeof(LK) == sizeof(CL), "one buffer");
+    const long Vh = c->g.Vh;
+    SapPlan::Perm &pm = pl.perm[P == LQCD_F32 ? 0 : 1];
+    a.perm = 0;
+    a.Ub = a.U;
+    a.Aeb = a.Ae;
+    a.Aiob = a.Aio;
+    if (!pm.p && !pm.failed) {
+        if (cudaMalloc(&pm.p, (24 + 2 * 18) * Vh * sizeof(LK)) != cudaSuccess) {
+            cudaGetLastError();
+            pm.p = nullptr;
+            pm.failed = true;   // the lattice-ordered arrays serve
+        }
+    }
+    if (!pm.p) return LQCD_OK;
+    LK *ub = (LK *)pm.p;
+    CL *ae = (CL *)(ub + 24 * Vh), *ai = ae + 18 * Vh;
+    if (pm.version != c->op_version) {
+        const int gx = div_up(Vh, 256);
+        k_sap_permute<LK><<<dim3(gx, 24), 256, 0, c->stream>>>(c->g, pl.B, pl.blocks_dev, 12, 0, a.U, ub);
+        k_sap_permute<CL><<<dim3(gx, 18), 256, 0, c->stream>>>(c->g, pl.B, pl.blocks_dev, 18, 0, a.Ae, ae);
+        k_sap_permute<CL><<<dim3(gx, 18), 256, 0, c->stream>>>(c->g, pl.B, pl.blocks_dev, 18, 1, a.Aio, ai);
+        c->n_kernel_launches += 3;
+        LQCD_LAUNCH_CHECK(c);
+        pm.version = c->op_version;
+    }
+    a.perm = 1;
+    a.Ub = ub;
+    a.Aeb = ae;
+    a.Aiob = ai;
+    return LQCD_OK;
+}
+
+template <int P>
+lqcd_status sap_run(lqcd_ctx *c, SapPlan &P_, int ncy, int nmr, const void *eta, void *psi, void *r,
                     void *delta, int nrhs)
 {
     using T = SapT<P>;
     using R = typename T::R;
     using SP = typename T::SP;
-    const SapPlan &Pl = P_;
+    SapPlan &Pl = P_;
     const size_t fb = 2 * native_half_bytes(c, (lqcd_prec)P);
     size_t smem = 5 * 12 * Pl.B.nh * sizeof(cx<R>) + 3 * 32 * sizeof(R);
     static bool attr_set = false;
@@ -1328,6 +1402,7 @@ lqcd_status sap_run(lqcd_ctx *c, const SapPlan &P_, int ncy, int nmr, const void
             attr_s = true;
         }
         resident = Pl.B.nh <= SAPS_NH && (2 * Pl.B.nh) % 32 == 0 && !sap_force_generic();
+        if (resident) LQCD_TRY(sap_operator<P>(c, Pl, a));
     }
     // clover term staged in shared memory (stage = 1, one CTA per SM) or read
     // through L1 (stage = 0): identical arithmetic, chosen by timing.  Without
@@ -1364,7 +1439,8 @@ lqcd_status sap_run(lqcd_ctx *c, const SapPlan &P_, int ncy, int nmr, const void
     for (int cyc = 0; cyc < ncy; cyc++)
         for (int col = 0; col < 2; col++) {
             if (Pl.count[col] == 0) continue;
-            a.blocks = Pl.blocks_dev + (col == 0 ? 0 : Pl.count[0]);
+            a.slot0 = col == 0 ? 0 : Pl.count[0];
+            a.blocks = Pl.blocks_dev + a.slot0;
             if (tuning) {
                 stage = (sweep + 1) & 1;   // sweep 0 (cold caches) uses stage 1, then alternate
                 cudaEventRecord(ev[0], c->stream);
@@ -1508,7 +1584,8 @@ lqcd_status sap_batch_args(lqcd_ctx *hc, lqcd_ctx *const *ctx, int n, const lqcd
             SapArgs<P> a;
             a.g = ctx[l]->g;
             a.B = pl->B;
-            a.blocks = pl->blocks_dev + (col == 0 ? 0 : pl->count[0]);
+            a.slot0 = col == 0 ? 0 : pl->count[0];
+            a.blocks = pl->blocks_dev + a.slot0;
             a.r = (SP *)b->r + off[l];
             a.psi = (SP *)b->psi + off[l];
             a.delta = (SP *)b->delta + off[l];
@@ -1523,6 +1600,8 @@ lqcd_status sap_batch_args(lqcd_ctx *hc, lqcd_ctx *const *ctx, int n, const lqcd
                 a.Aio = ctx[l]->Ai16[1];
             }
             a.nmr = sp->nmr;
+            LQCD_TRY(sap_operator<P>(ctx[l], *pl, a));
+            LQCD_CUDA_CHECK(hc, cudaStreamSynchronize(ctx[l]->stream));   // the batch runs on its own stream
             v.push_back(a);
             for (int i = 0; i < pl->count[col]; i++) it[col].push_back(make_int2(l, i));
         }
@@ -1610,6 +1689,35 @@ lqcd_status sap_batch_create(lqcd_ctx *hc, lqcd_ctx *const *ctx, int n, const lq
     return LQCD_OK;
 }
 
+// the block-ordered operators of lattices whose operator changed since the batch
+// was made, on the contexts' streams (the kernel arguments keep their pointers)
+lqcd_status sap_batch_refresh(SapBatch *b, lqcd_ctx *const *ctx, int n, const int bs[4])
+{
+    for (int l = 0; l < n; l++) {
+        SapPlan *pl;
+        LQCD_TRY(get_plan(ctx[l], bs, &pl));
+        auto again = [&](auto tag) -> lqcd_status {
+            constexpr int P = decltype(tag)::value;
+            SapArgs<P> a;
+            if constexpr (P == LQCD_F32) {
+                a.U = ctx[l]->U32;
+                a.Ae = ctx[l]->A32[0];
+                a.Aio = ctx[l]->Ai32[1];
+            } else {
+                a.U = ctx[l]->U16;
+                a.Ae = ctx[l]->A16[0];
+                a.Aio = ctx[l]->Ai16[1];
+            }
+            return sap_operator<P>(ctx[l], *pl, a);
+        };
+        if (b->p == LQCD_F32)
+            LQCD_TRY(again(std::integral_constant<int, LQCD_F32>()));
+        else
+            LQCD_TRY(again(std::integral_constant<int, LQCD_F16S>()));
+    }
+    return LQCD_OK;
+}
+
 // psi = M_sap eta on every lattice whose active flag is set (the arenas given
 // at creation; eta: an arena of the same layout, bytes long)
 lqcd_status sap_batch_apply(lqcd_ctx *hc, SapBatch *b, const void *eta, size_t bytes, const int *active)
@@ -1627,6 +1735,7 @@ void sap_free_plans(lqcd_ctx *c)
             cudaFree(it->plan.blocks_dev);
             cudaFree(it->plan.face_dev[0]);
             cudaFree(it->plan.face_dev[1]);
+            for (auto &pm : it->plan.perm) cudaFree(pm.p);
             it = g_plans.erase(it);
         } else
             ++it;
