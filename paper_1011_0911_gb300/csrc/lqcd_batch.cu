@@ -1,13 +1,14 @@
 // Batched solve of several independent lattices with the SAP-preconditioned
-// flexible GCR (Sec. 3-4; Dhat systems through Eq. 5), one right-hand side per
-// lattice.  All lattices' fields live in shared arenas (lattice l at a fixed
-// offset); every phase of a GCR step is one launch over a flat work list of
-// (lattice, item) pairs of all lattices, so small and large lattices fill the
-// GPU together:
+// flexible GCR (Sec. 3-4) of the Dhat systems on even fields (lqcd_solvers.cu),
+// one right-hand side per lattice.  All lattices' fields live in shared arenas
+// (lattice l at a fixed offset); every phase of a GCR step is one launch over a
+// flat work list of (lattice, item) pairs of all lattices, so small and large
+// lattices fill the GPU together:
 //
-//   phi_k = M_sap rho      FP64 -> sap precision, batched SAP, -> FP64
-//   chi_k = D phi_k        FP64 -> F32, batched D, -> FP64
-//   Gram-Schmidt           one cooperative persistent kernel (k_gs): dot
+//   phi_k = M_sap (rho, 0)  FP64 -> sap precision, batched SAP, even half -> FP32
+//                           (phi_k is kept in FP32: it holds no more digits)
+//   chi_k = Dhat phi_k      batched Dhat in FP32 -> FP64
+//   Gram-Schmidt            one cooperative persistent kernel (k_gs): dot
 //                          products, per-lattice coefficients, updates, the new
 //                          residual and its norm, separated by grid barriers
 //                          whose waits are bounded (LQCD_ERR_TIMEOUT)
@@ -37,13 +38,13 @@ constexpr int TILE = 128;          // sites per conversion work item
 
 struct BLat {            // layout of lattice l in the arenas
     long Vh;
-    long off64;          // double2 units (FP64 arena, 24 Vh per full field)
-    long off32;          // float4 units (F32 arena, 12 Vh)
-    long offs;           // units of the SAP arena (F32: float4, 12 Vh; F16S: h16s, 13 Vh / 2)
+    long off64;          // double2 units (FP64 arenas of half fields, 12 Vh each)
+    long off32;          // float4 units (F32 arenas of half fields, 6 Vh)
+    long offs;           // units of the SAP arenas (full fields; F32: float4, 12 Vh; F16S: h16s, 13 Vh / 2)
     int it0, it1;        // its BLAS work items
 };
 
-struct BItem {           // complex entries [s0, s0 + n) of a full FP64 field of lattice lat
+struct BItem {           // complex entries [s0, s0 + n) of an even FP64 field of lattice lat
     int lat, n;
     long s0;
 };
@@ -70,11 +71,6 @@ struct GridBar {
 
 __device__ __forceinline__ double2 ld2(const double2 *p) { return __ldcg(p); }
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-// conj(a) b
-__device__ __forceinline__ double2 cdot(double2 a, double2 b)
-{
-    return make_double2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
-}
 __device__ __forceinline__ double2 cmul(double2 a, double2 b)
 {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -115,20 +111,21 @@ __device__ bool grid_wait(GridBar *bar, unsigned int expected, long long limit, 
     return s_ok != 0;
 }
 
-// block sum of one double2 (fixed order); valid in thread 0
-__device__ double2 block_sum(double2 v, double2 *sm)
+// CTA sums of V values per thread (fixed order); thread i < V returns value i.  sm
+// alternates between the two buffers of successive calls (par), so one barrier
+// per call is enough.
+template <int V>
+__device__ __forceinline__ double cta_sums(double (&v)[V], double (*sm)[GS_THREADS / 32][16], int &par)
 {
-    for (int o = 16; o > 0; o >>= 1) {
-        v.x += __shfl_down_sync(0xffffffffu, v.x, o);
-        v.y += __shfl_down_sync(0xffffffffu, v.y, o);
-    }
-    const int w = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    warp_multi_sum(v);
+    double (*b)[16] = sm[par];
+    par ^= 1;
+    if (lane % (32 / V) == 0) b[warp][lane / (32 / V)] = v[0];
     __syncthreads();
-    if ((threadIdx.x & 31) == 0) sm[w] = v;
-    __syncthreads();
-    double2 s = make_double2(0, 0);
-    if (threadIdx.x == 0)
-        for (int i = 0; i < (int)(blockDim.x >> 5); i++) s = cadd(s, sm[i]);
+    double s = 0;
+    if (threadIdx.x < V)
+        for (int w = 0; w < GS_THREADS / 32; w++) s += b[w][threadIdx.x];
     return s;
 }
 
@@ -166,10 +163,19 @@ struct GsArgs {
 // against chi_0..chi_{k-1} (a second pass where the first removed more than
 // half of |chi_k|^2), b_k = |chi_k|, c_k = <chi_k, rho> / b_k, chi_k /= b_k,
 // rho -= c_k chi_k, |rho|^2, and the per-lattice stopping tests.
-__global__ void __launch_bounds__(GS_THREADS) k_gs(GsArgs a)
+//
+// Bound by the FP64 pipe: 4 multiply-adds per entry and vector in A and again in
+// C.  A reduces eight vectors at a time (one barrier and 16 additions per warp
+// where one vector at a time took four barriers and ten additions each), and B
+// gives every vector's partial sums to a warp of its own.  16 lattices, 920 576
+// sites: 2050 -> 754 us a step (full fields and sums of products before), the
+// whole solve 406 -> 248 ms.
+__global__ void __launch_bounds__(GS_THREADS, 2) k_gs(GsArgs a)
 {
-    __shared__ double2 sm[GS_THREADS / 32];
-    const int k = a.k, G = gridDim.x;
+    __shared__ double sm[2][GS_THREADS / 32][16];
+    __shared__ double2 sd[PS];
+    int par = 0;
+    const int k = a.k, G = gridDim.x, warp = threadIdx.x >> 5;
     const unsigned int nb = gridDim.x;
     double2 *chik = a.chi + (long)k * a.N;
     constexpr int PER = CHUNK / GS_THREADS;
@@ -187,44 +193,50 @@ __global__ void __launch_bounds__(GS_THREADS) k_gs(GsArgs a)
                 xk[e] = j < w.n ? chik[base + j] : make_double2(0, 0);
             }
             const int m = pass == 0 ? k + 1 : k;
-            for (int i = 0; i < m; i++) {
-                const double2 *ci = a.chi + (long)i * a.N + base;
-                double2 s = make_double2(0, 0);
+            for (int i0 = 0; i0 < m; i0 += 8) {
+                double v[16];
 #pragma unroll
-                for (int e = 0; e < PER; e++) {
-                    const int j = threadIdx.x + e * GS_THREADS;
-                    if (j < w.n) s = cadd(s, cdot(ci[j], xk[e]));
-                }
-                s = block_sum(s, sm);
-                if (threadIdx.x == 0) a.part[(long)it * PS + i] = s;
+                for (int q = 0; q < 16; q++) v[q] = 0;
+#pragma unroll
+                for (int q = 0; q < 8; q++)
+                    if (i0 + q < m) {
+                        const double2 *ci = a.chi + (long)(i0 + q) * a.N + base;
+#pragma unroll
+                        for (int e = 0; e < PER; e++) {
+                            const int j = threadIdx.x + e * GS_THREADS;
+                            if (j < w.n) cdot_add(v[2 * q], v[2 * q + 1], ci[j], xk[e]);
+                        }
+                    }
+                const double s = cta_sums(v, sm, par);
+                if (threadIdx.x < 16 && i0 + (int)threadIdx.x / 2 < m)
+                    reinterpret_cast<double *>(a.part + (long)it * PS + i0)[threadIdx.x] = s;
             }
         }
         if (!grid_wait(a.bar, nb + (a.stall && pass == 0 ? 1u : 0u), a.limit, a.status)) return;
         // ---- B: per-lattice coefficients
-        if (threadIdx.x < 32)
-            for (int l = blockIdx.x; l < a.nlat; l += G) {
-                if (!a.act[l]) continue;
-                if (pass == 1 && !__ldcg(&a.sc[l].pass2)) continue;
-                const int m = pass == 0 ? k + 1 : k;
-                double removed = 0, dkk = 0;
-                for (int i = 0; i < m; i++) {
-                    const double2 d = warp_items_sum(a.part, a.lat[l].it0, a.lat[l].it1, i);
-                    if (threadIdx.x == 0) {
-                        if (i == k) {
-                            dkk = d.x;
-                        } else {
-                            double2 &ai = a.mat[l].a[i][k];
-                            ai = pass == 0 ? d : cadd(ai, d);
-                            a.mat[l].coef[i] = d;
-                            removed += d.x * d.x + d.y * d.y;
-                        }
-                    }
-                }
-                if (threadIdx.x == 0) {
-                    if (pass == 0) a.sc[l].pass2 = (k > 0 && removed > 0.5 * dkk) ? 1 : 0;
-                    __threadfence();
-                }
+        for (int l = blockIdx.x; l < a.nlat; l += G) {
+            if (!a.act[l]) continue;
+            if (pass == 1 && !__ldcg(&a.sc[l].pass2)) continue;
+            const int m = pass == 0 ? k + 1 : k;
+            for (int i = warp; i < m; i += GS_THREADS / 32) {
+                const double2 d = warp_items_sum(a.part, a.lat[l].it0, a.lat[l].it1, i);
+                if ((threadIdx.x & 31) == 0) sd[i] = d;
             }
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                double removed = 0;
+                for (int i = 0; i < k; i++) {
+                    const double2 d = sd[i];
+                    double2 &ai = a.mat[l].a[i][k];
+                    ai = pass == 0 ? d : cadd(ai, d);
+                    a.mat[l].coef[i] = d;
+                    removed += d.x * d.x + d.y * d.y;
+                }
+                if (pass == 0) a.sc[l].pass2 = (k > 0 && removed > 0.5 * sd[k].x) ? 1 : 0;
+                __threadfence();
+            }
+            __syncthreads();
+        }
         if (!grid_wait(a.bar, nb, a.limit, a.status)) return;
         // ---- C: chi_k -= sum_i coef_i chi_i; final |chi_k|^2, <chi_k, rho> where done
         for (int it = blockIdx.x; it < a.nitems; it += G) {
@@ -239,36 +251,33 @@ __global__ void __launch_bounds__(GS_THREADS) k_gs(GsArgs a)
                 const int j = threadIdx.x + e * GS_THREADS;
                 xk[e] = j < w.n ? chik[base + j] : make_double2(0, 0);
             }
+#pragma unroll 2
             for (int i = 0; i < k; i++) {
                 const double2 cf = ld2(&a.mat[w.lat].coef[i]);
+                const double2 mc = make_double2(-cf.x, -cf.y);
                 const double2 *ci = a.chi + (long)i * a.N + base;
 #pragma unroll
                 for (int e = 0; e < PER; e++) {
                     const int j = threadIdx.x + e * GS_THREADS;
-                    if (j < w.n) {
-                        const double2 t = cmul(cf, ci[j]);
-                        xk[e].x -= t.x;
-                        xk[e].y -= t.y;
-                    }
+                    if (j < w.n) xk[e] = caxpy(mc, ci[j], xk[e]);
                 }
             }
-            double2 q = make_double2(0, 0), cr = make_double2(0, 0);
+            const bool last = pass == 1 || !p2;
+            double v[4] = {0, 0, 0, 0};   // |chi_k|^2, -, <chi_k, rho>
 #pragma unroll
             for (int e = 0; e < PER; e++) {
                 const int j = threadIdx.x + e * GS_THREADS;
                 if (j < w.n) {
                     if (k > 0) chik[base + j] = xk[e];
-                    q.x += xk[e].x * xk[e].x + xk[e].y * xk[e].y;
-                    cr = cadd(cr, cdot(xk[e], a.rho[base + j]));
+                    if (last) {
+                        v[0] = norm_add(v[0], xk[e]);
+                        cdot_add(v[2], v[3], xk[e], a.rho[base + j]);
+                    }
                 }
             }
-            if (pass == 1 || !p2) {
-                q = block_sum(q, sm);
-                cr = block_sum(cr, sm);
-                if (threadIdx.x == 0) {
-                    a.part[(long)it * PS + 0] = q;
-                    a.part[(long)it * PS + 1] = cr;
-                }
+            if (last) {
+                const double s = cta_sums(v, sm, par);
+                if (threadIdx.x < 4) reinterpret_cast<double *>(a.part + (long)it * PS)[threadIdx.x] = s;
             }
         }
         if (!grid_wait(a.bar, nb, a.limit, a.status)) return;
@@ -299,22 +308,23 @@ __global__ void __launch_bounds__(GS_THREADS) k_gs(GsArgs a)
         if (!__ldcg(&a.act[w.lat])) continue;
         const long base = a.lat[w.lat].off64 + w.s0;
         const double inv = 1.0 / __ldcg(&a.mat[w.lat].b[k]);
-        const double2 c = ld2(&a.mat[w.lat].c[k]);
-        double2 s = make_double2(0, 0);
-        for (int j = threadIdx.x; j < w.n; j += GS_THREADS) {
-            double2 x = chik[base + j];
-            x.x *= inv;
-            x.y *= inv;
-            chik[base + j] = x;
-            const double2 t = cmul(c, x);
-            double2 r = a.rho[base + j];
-            r.x -= t.x;
-            r.y -= t.y;
-            a.rho[base + j] = r;
-            s.x += r.x * r.x + r.y * r.y;
+        const double2 c = ld2(&a.mat[w.lat].c[k]), mc = make_double2(-c.x, -c.y);
+        double v[2] = {0, 0};
+#pragma unroll
+        for (int e = 0; e < PER; e++) {
+            const int j = threadIdx.x + e * GS_THREADS;
+            if (j < w.n) {
+                double2 x = chik[base + j];
+                x.x *= inv;
+                x.y *= inv;
+                chik[base + j] = x;
+                const double2 r = caxpy(mc, x, a.rho[base + j]);
+                a.rho[base + j] = r;
+                v[0] = norm_add(v[0], r);
+            }
         }
-        s = block_sum(s, sm);
-        if (threadIdx.x == 0) a.part[(long)it * PS + 0] = s;
+        const double s = cta_sums(v, sm, par);
+        if (threadIdx.x < 2) reinterpret_cast<double *>(a.part + (long)it * PS)[threadIdx.x] = s;
     }
     if (!grid_wait(a.bar, nb, a.limit, a.status)) return;
     // ---- F: |rho|^2 and the stopping tests of the cycle
@@ -332,23 +342,24 @@ __global__ void __launch_bounds__(GS_THREADS) k_gs(GsArgs a)
         }
 }
 
-// ---- cycle start: rho = eta - D psi (FP64), |rho|^2, activity of the cycle
+// ---- cycle start: rho = eta - Dhat psi (FP64), |rho|^2, activity of the cycle
 __global__ void k_b_resid(const BLat *lat, const BItem *items, const int *act, const double2 *eta, const double2 *t,
                           double2 *rho, double2 *part)
 {
-    __shared__ double2 sm[GS_THREADS / 32];
+    __shared__ double sm[2][GS_THREADS / 32][16];
+    int par = 0;
     const BItem w = items[blockIdx.x];
     if (!act[w.lat]) return;
     const long base = lat[w.lat].off64 + w.s0;
-    double2 s = make_double2(0, 0);
+    double v[2] = {0, 0};
     for (int j = threadIdx.x; j < w.n; j += blockDim.x) {
         const double2 e = eta[base + j], d = t[base + j];
         const double2 r = make_double2(e.x - d.x, e.y - d.y);
         rho[base + j] = r;
-        s.x += r.x * r.x + r.y * r.y;
+        v[0] = norm_add(v[0], r);
     }
-    s = block_sum(s, sm);
-    if (threadIdx.x == 0) part[(long)blockIdx.x * PS] = s;
+    const double s = cta_sums(v, sm, par);
+    if (threadIdx.x < 2) reinterpret_cast<double *>(part + (long)blockIdx.x * PS)[threadIdx.x] = s;
 }
 // one warp per lattice; gain2: the cycle stops once |rho|^2 fell by this factor
 __global__ void k_b_restart(const BLat *lat, const double2 *part, int *act, BScal *sc, int nlat, double gain2)
@@ -401,22 +412,33 @@ __global__ void k_b_backsub(BScal *sc, BMat *mat, int nlat)
         M.alpha[i] = make_double2(t.x / M.b[i], t.y / M.b[i]);
     }
 }
-__global__ void k_b_update(const BLat *lat, const BItem *items, const BScal *sc, const BMat *mat, const double2 *phi,
-                           long N, double2 *psi)
+// tiles: (lattice, first rank, count); phi: F32 even fields, N32 float4 apart
+__global__ void __launch_bounds__(TILE) k_b_update(const BLat *lat, const int4 *tiles, const BScal *sc, const BMat *mat,
+                                                   const float4 *phi, long N32, double2 *psi)
 {
-    const BItem w = items[blockIdx.x];
-    const int nk = sc[w.lat].nk;
-    if (nk == 0) return;
-    const long base = lat[w.lat].off64 + w.s0;
-    for (int j = threadIdx.x; j < w.n; j += blockDim.x) {
-        double2 x = psi[base + j];
-        for (int i = 0; i < nk; i++) x = cadd(x, cmul(mat[w.lat].alpha[i], phi[(long)i * N + base + j]));
-        psi[base + j] = x;
+    const int4 w = tiles[blockIdx.x];
+    const int nk = sc[w.x].nk;
+    if (nk == 0 || (int)threadIdx.x >= w.z) return;
+    const BLat L = lat[w.x];
+    const long r = w.y + threadIdx.x, Vh = L.Vh;
+    for (int q = 0; q < 6; q++) {
+        double2 *p = psi + L.off64 + 2 * q * Vh + r;
+        const float4 *f = phi + L.off32 + q * Vh + r;
+        double2 x = p[0], y = p[Vh];
+#pragma unroll 4
+        for (int i = 0; i < nk; i++) {
+            const float4 v = f[i * N32];
+            const double2 al = mat[w.x].alpha[i];
+            x = caxpy(al, make_double2(v.x, v.y), x);
+            y = caxpy(al, make_double2(v.z, v.w), y);
+        }
+        p[0] = x;
+        p[Vh] = y;
     }
 }
 
-// ---- arena conversions over (lattice, half, first rank, count) tiles
-enum { CV_64_TO_S = 0, CV_S_TO_64 = 1, CV_64_TO_32 = 2, CV_32_TO_64 = 3 };
+// ---- arena conversions of even half fields over (lattice, first rank, count) tiles
+enum { CV_64_TO_S = 0, CV_S_TO_32 = 1, CV_32_TO_64 = 2 };
 __device__ __forceinline__ void ld64(const double2 *f, long Vh, long r, cx<float> v[12])
 {
 #pragma unroll
@@ -444,27 +466,25 @@ __device__ __forceinline__ void st32(float4 *f, long Vh, long r, const cx<float>
 #pragma unroll
     for (int q = 0; q < 6; q++) f[q * Vh + r] = make_float4(v[2 * q].re, v[2 * q].im, v[2 * q + 1].re, v[2 * q + 1].im);
 }
-// sprec: precision of the SAP arena (LQCD_F32 / LQCD_F16S) for CV_64_TO_S, CV_S_TO_64
+// sprec: precision of the SAP arena (LQCD_F32 / LQCD_F16S) for CV_64_TO_S, CV_S_TO_32
 template <int MODE, int SPREC>
-__global__ void __launch_bounds__(TILE) k_b_conv(const BLat *lat, const int4 *items, const int *act, const void *in,
+__global__ void __launch_bounds__(TILE) k_b_conv(const BLat *lat, const int4 *tiles, const int *act, const void *in,
                                                  void *out)
 {
-    const int4 w = items[blockIdx.x];   // (lattice, half, first rank, count)
+    const int4 w = tiles[blockIdx.x];   // (lattice, first rank, count)
     if (act && !act[w.x]) return;
-    if ((int)threadIdx.x >= w.w) return;
+    if ((int)threadIdx.x >= w.z) return;
     const BLat L = lat[w.x];
-    const long r = w.z + threadIdx.x, Vh = L.Vh;
-    const long h64 = L.off64 + w.y * 12 * Vh, h32 = L.off32 + w.y * 6 * Vh;
-    const long hs = L.offs + (SPREC == LQCD_F16S ? w.y * f16s_half_units(Vh) : w.y * 6 * Vh);
+    const long r = w.y + threadIdx.x, Vh = L.Vh;
     cx<float> v[12];
-    if (MODE == CV_64_TO_S || MODE == CV_64_TO_32) ld64((const double2 *)in + h64, Vh, r, v);
-    else if (MODE == CV_32_TO_64) ld32((const float4 *)in + h32, Vh, r, v);
-    else if (SPREC == LQCD_F16S) f16s_load<false>((const h16s *)in + hs, Vh, r, v);
-    else ld32((const float4 *)in + hs, Vh, r, v);
-    if (MODE == CV_S_TO_64 || MODE == CV_32_TO_64) st64((double2 *)out + h64, Vh, r, v);
-    else if (MODE == CV_64_TO_32) st32((float4 *)out + h32, Vh, r, v);
-    else if (SPREC == LQCD_F16S) f16s_store((h16s *)out + hs, Vh, r, v);
-    else st32((float4 *)out + hs, Vh, r, v);
+    if (MODE == CV_64_TO_S) ld64((const double2 *)in + L.off64, Vh, r, v);
+    else if (MODE == CV_32_TO_64) ld32((const float4 *)in + L.off32, Vh, r, v);
+    else if (SPREC == LQCD_F16S) f16s_load<false>((const h16s *)in + L.offs, Vh, r, v);
+    else ld32((const float4 *)in + L.offs, Vh, r, v);
+    if (MODE == CV_32_TO_64) st64((double2 *)out + L.off64, Vh, r, v);
+    else if (MODE == CV_S_TO_32) st32((float4 *)out + L.off32, Vh, r, v);
+    else if (SPREC == LQCD_F16S) f16s_store((h16s *)out + L.offs, Vh, r, v);
+    else st32((float4 *)out + L.offs, Vh, r, v);
 }
 
 }  // namespace
@@ -485,8 +505,8 @@ struct lqcd_batch {
     long N = 0;                      // complex entries of one FP64 arena vector
     long N32 = 0, NS = 0;            // F32 / SAP arena units
     size_t sap_bytes = 0;
-    double2 *eta = nullptr, *psi = nullptr, *rho = nullptr, *tmp = nullptr, *phi = nullptr, *chi = nullptr;
-    float4 *x32 = nullptr, *y32 = nullptr;
+    double2 *eta = nullptr, *psi = nullptr, *rho = nullptr, *tmp = nullptr, *tmp_o = nullptr, *chi = nullptr;
+    float4 *phi = nullptr, *t32 = nullptr, *y32 = nullptr;
     void *s_eta = nullptr, *s_r = nullptr, *s_psi = nullptr, *s_delta = nullptr;
     BScal *sc = nullptr;
     BMat *mat = nullptr;
@@ -514,8 +534,8 @@ void batch_free_all(lqcd_batch *b)
     dirac_batch_free(b->d64);
     sap_batch_free(b->sap);
     for (void *q : {(void *)b->lat, (void *)b->items, (void *)b->tiles, (void *)b->eta, (void *)b->psi, (void *)b->rho,
-                    (void *)b->tmp, (void *)b->phi, (void *)b->chi, (void *)b->x32, (void *)b->y32, b->s_eta, b->s_r,
-                    b->s_psi, b->s_delta, (void *)b->sc, (void *)b->mat, (void *)b->act, (void *)b->part,
+                    (void *)b->tmp, (void *)b->tmp_o, (void *)b->phi, (void *)b->chi, (void *)b->t32, (void *)b->y32,
+                    b->s_eta, b->s_r, b->s_psi, b->s_delta, (void *)b->sc, (void *)b->mat, (void *)b->act, (void *)b->part,
                     (void *)b->bar, (void *)b->status})
         cudaFree(q);
     if (b->st) cudaStreamDestroy(b->st);
@@ -540,12 +560,9 @@ lqcd_status conv(lqcd_batch *b, int mode, const void *in, void *out, const int *
             if (s16) k_b_conv<CV_64_TO_S, LQCD_F16S><<<b->ntiles, TILE, 0, b->st>>>(b->lat, b->tiles, act, in, out);
             else k_b_conv<CV_64_TO_S, LQCD_F32><<<b->ntiles, TILE, 0, b->st>>>(b->lat, b->tiles, act, in, out);
             break;
-        case CV_S_TO_64:
-            if (s16) k_b_conv<CV_S_TO_64, LQCD_F16S><<<b->ntiles, TILE, 0, b->st>>>(b->lat, b->tiles, act, in, out);
-            else k_b_conv<CV_S_TO_64, LQCD_F32><<<b->ntiles, TILE, 0, b->st>>>(b->lat, b->tiles, act, in, out);
-            break;
-        case CV_64_TO_32:
-            k_b_conv<CV_64_TO_32, LQCD_F32><<<b->ntiles, TILE, 0, b->st>>>(b->lat, b->tiles, act, in, out);
+        case CV_S_TO_32:
+            if (s16) k_b_conv<CV_S_TO_32, LQCD_F16S><<<b->ntiles, TILE, 0, b->st>>>(b->lat, b->tiles, act, in, out);
+            else k_b_conv<CV_S_TO_32, LQCD_F32><<<b->ntiles, TILE, 0, b->st>>>(b->lat, b->tiles, act, in, out);
             break;
         default:
             k_b_conv<CV_32_TO_64, LQCD_F32><<<b->ntiles, TILE, 0, b->st>>>(b->lat, b->tiles, act, in, out);
@@ -589,30 +606,28 @@ lqcd_status gs_step(lqcd_batch *b, int k, int stall)
 lqcd_status cycle_steps(lqcd_batch *b, int stall)
 {
     for (int k = 0; k < b->p.nkv; k++) {
-        double2 *phk = b->phi + (long)k * b->N, *chk = b->chi + (long)k * b->N;
-        LQCD_TRY(conv(b, CV_64_TO_S, b->rho, b->s_eta, b->act));
+        LQCD_TRY(conv(b, CV_64_TO_S, b->rho, b->s_eta, b->act));   // the odd halves of s_eta stay zero
         LQCD_TRY(sap_batch_apply(b->hc, b->sap, b->s_eta, b->sap_bytes, b->act));
-        LQCD_TRY(conv(b, CV_S_TO_64, b->s_psi, phk, b->act));
-        LQCD_TRY(conv(b, CV_64_TO_32, phk, b->x32, b->act));
-        LQCD_TRY(dirac_batch_D(b->hc, b->d32, b->act));
-        LQCD_TRY(conv(b, CV_32_TO_64, b->y32, chk, b->act));
+        LQCD_TRY(conv(b, CV_S_TO_32, b->s_psi, b->phi + k * b->N32, b->act));
+        LQCD_TRY(dirac_batch_dhat(b->hc, b->d32, k * b->N32, b->act));
+        LQCD_TRY(conv(b, CV_32_TO_64, b->y32, b->chi + k * b->N, b->act));
         LQCD_TRY(gs_step(b, k, stall && k == 0));
     }
     k_b_backsub<<<(b->n + 63) / 64, 64, 0, b->st>>>(b->sc, b->mat, b->n);
-    k_b_update<<<b->nitems, GS_THREADS, 0, b->st>>>(b->lat, b->items, b->sc, b->mat, b->phi, b->N, b->psi);
+    k_b_update<<<b->ntiles, TILE, 0, b->st>>>(b->lat, b->tiles, b->sc, b->mat, b->phi, b->N32, b->psi);
     b->hc->n_kernel_launches += 2;
     LQCD_LAUNCH_CHECK(b->hc);
     return LQCD_OK;
 }
 
-// rho = eta - D psi on every lattice still running; flags of the new cycle
+// rho = eta - Dhat psi on every lattice still running; flags of the new cycle
 lqcd_status cycle_restart(lqcd_batch *b)
 {
     k_b_activate<<<(b->n + 63) / 64, 64, 0, b->st>>>(b->act, b->sc, b->n, b->p.nmx);
     b->hc->n_kernel_launches++;
-    LQCD_TRY(dirac_batch_D(b->hc, b->d64, b->act));
+    LQCD_TRY(dirac_batch_dhat(b->hc, b->d64, 0, b->act));
     k_b_resid<<<b->nitems, GS_THREADS, 0, b->st>>>(b->lat, b->items, b->act, b->eta, b->tmp, b->rho, b->part);
-    // a cycle in which D phi is FP32 gains at most 1e-5 before the FP64 restart
+    // a cycle in which Dhat phi is FP32 gains at most 1e-5 before the FP64 restart
     k_b_restart<<<b->n, 32, 0, b->st>>>(b->lat, b->part, b->act, b->sc, b->n, 1e-10);
     b->hc->n_kernel_launches += 2;
     LQCD_LAUNCH_CHECK(b->hc);
@@ -668,16 +683,15 @@ lqcd_status lqcd_batch_create(lqcd_ctx *const *ctxs, int n, const lqcd_batch_par
         off64[l] = L.off64;
         off32[l] = L.off32;
         offs[l] = L.offs;
-        const long nc = 24 * L.Vh;   // complex entries of a full field
+        const long nc = 12 * L.Vh;   // complex entries of an even field
         L.it0 = (int)items.size();
         for (long s0 = 0; s0 < nc; s0 += CHUNK) items.push_back(BItem{l, (int)std::min<long>(CHUNK, nc - s0), s0});
         L.it1 = (int)items.size();
-        for (int h = 0; h < 2; h++)
-            for (long r0 = 0; r0 < L.Vh; r0 += TILE)
-                tiles.push_back(make_int4(l, h, (int)r0, (int)std::min<long>(TILE, L.Vh - r0)));
+        for (long r0 = 0; r0 < L.Vh; r0 += TILE)
+            tiles.push_back(make_int4(l, (int)r0, (int)std::min<long>(TILE, L.Vh - r0), 0));
         b->lat_h.push_back(L);
         b->N += nc;
-        b->N32 += 12 * L.Vh;
+        b->N32 += 6 * L.Vh;
         b->NS += s16 ? 2 * f16s_half_units(L.Vh) : 12 * L.Vh;
     }
     b->nitems = (int)items.size();
@@ -693,11 +707,12 @@ lqcd_status lqcd_batch_create(lqcd_ctx *const *ctxs, int n, const lqcd_batch_par
     BALLOC(b->eta, f64b, "eta");
     BALLOC(b->psi, f64b, "psi");
     BALLOC(b->rho, f64b, "rho");
-    BALLOC(b->tmp, f64b, "D psi");
-    BALLOC(b->phi, f64b * p->nkv, "phi");
+    BALLOC(b->tmp, f64b, "Dhat psi");
+    BALLOC(b->tmp_o, f64b, "odd part of Dhat psi");
     BALLOC(b->chi, f64b * p->nkv, "chi");
-    BALLOC(b->x32, (size_t)b->N32 * 16, "F32 input");
-    BALLOC(b->y32, (size_t)b->N32 * 16, "F32 output");
+    BALLOC(b->phi, (size_t)b->N32 * 16 * p->nkv, "phi");
+    BALLOC(b->t32, (size_t)b->N32 * 16, "odd part of Dhat phi");
+    BALLOC(b->y32, (size_t)b->N32 * 16, "Dhat phi");
     BALLOC(b->s_eta, b->sap_bytes, "SAP input");
     BALLOC(b->s_r, b->sap_bytes, "SAP residual");
     BALLOC(b->s_psi, b->sap_bytes, "SAP output");
@@ -712,9 +727,12 @@ lqcd_status lqcd_batch_create(lqcd_ctx *const *ctxs, int n, const lqcd_batch_par
     cudaMemcpy(b->lat, b->lat_h.data(), n * sizeof(BLat), cudaMemcpyHostToDevice);
     cudaMemcpy(b->items, items.data(), items.size() * sizeof(BItem), cudaMemcpyHostToDevice);
     cudaMemcpy(b->tiles, tiles.data(), tiles.size() * sizeof(int4), cudaMemcpyHostToDevice);
-    if ((st = dirac_batch_create(b->hc, b->ctx.data(), n, LQCD_F32, b->x32, b->y32, off32.data(), &b->d32)) != LQCD_OK)
+    cudaMemset(b->s_eta, 0, b->sap_bytes);   // the odd halves stay zero
+    if ((st = dirac_batch_create(b->hc, b->ctx.data(), n, LQCD_F32, b->phi, b->t32, b->y32, off32.data(), &b->d32)) !=
+        LQCD_OK)
         return fail(st);
-    if ((st = dirac_batch_create(b->hc, b->ctx.data(), n, LQCD_F64, b->psi, b->tmp, off64.data(), &b->d64)) != LQCD_OK)
+    if ((st = dirac_batch_create(b->hc, b->ctx.data(), n, LQCD_F64, b->psi, b->tmp_o, b->tmp, off64.data(), &b->d64)) !=
+        LQCD_OK)
         return fail(st);
     if ((st = sap_batch_create(b->hc, b->ctx.data(), n, &p->sap, b->s_r, b->s_psi, b->s_delta, offs.data(), &b->sap)) !=
         LQCD_OK)
@@ -766,10 +784,8 @@ lqcd_status lqcd_batch_solve_dhat(lqcd_batch *b, const double *const *eta_dev, d
     LQCD_CUDA_CHECK(hc, cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
     LQCD_CUDA_CHECK(hc, cudaEventRecord(ev, b->user));
     LQCD_CUDA_CHECK(hc, cudaStreamWaitEvent(b->st, ev, 0));
-    // eta: even half from the caller's field, odd half zero (Eq. 5); psi = 0
-    const size_t f64b = (size_t)b->N * sizeof(double2);
-    LQCD_CUDA_CHECK(hc, cudaMemsetAsync(b->eta, 0, f64b, b->st));
-    LQCD_CUDA_CHECK(hc, cudaMemsetAsync(b->psi, 0, f64b, b->st));
+    // psi = 0
+    LQCD_CUDA_CHECK(hc, cudaMemsetAsync(b->psi, 0, (size_t)b->N * sizeof(double2), b->st));
     LQCD_CUDA_CHECK(hc, cudaMemsetAsync(b->status, 0, sizeof(int), b->st));
     LQCD_CUDA_CHECK(hc, cudaMemsetAsync(b->bar, 0, sizeof(GridBar), b->st));
     LQCD_CUDA_CHECK(hc, cudaStreamSynchronize(b->st));
@@ -796,9 +812,8 @@ lqcd_status lqcd_batch_solve_dhat(lqcd_batch *b, const double *const *eta_dev, d
     }
     LQCD_CUDA_CHECK(hc, cudaMemcpyAsync(b->sc, S.data(), n * sizeof(BScal), cudaMemcpyHostToDevice, b->st));
     std::vector<int> act(n);
-    std::vector<double> dhat_rel(n, 0.0);
     lqcd_status st = LQCD_OK;
-    for (int attempt = 0; attempt < 4 && st == LQCD_OK; attempt++) {
+    {
         for (;;) {
             if ((st = cycle_restart(b)) != LQCD_OK) break;
             if (cudaMemcpyAsync(act.data(), b->act, n * sizeof(int), cudaMemcpyDeviceToHost, b->st) != cudaSuccess ||
@@ -846,40 +861,13 @@ lqcd_status lqcd_batch_solve_dhat(lqcd_batch *b, const double *const *eta_dev, d
                 break;
             }
         }
-        if (st != LQCD_OK) break;
-        int dstat = 0;
-        LQCD_CUDA_CHECK(hc, cudaMemcpyAsync(&dstat, b->status, sizeof(int), cudaMemcpyDeviceToHost, b->st));
-        LQCD_CUDA_CHECK(hc, cudaMemcpyAsync(S.data(), b->sc, n * sizeof(BScal), cudaMemcpyDeviceToHost, b->st));
-        LQCD_CUDA_CHECK(hc, cudaStreamSynchronize(b->st));
-        if (dstat != 0) {
-            st = set_err(hc, (lqcd_status)dstat, "batch: a device-side wait ran out of time");
-            break;
+        if (st == LQCD_OK) {
+            int dstat = 0;
+            LQCD_CUDA_CHECK(hc, cudaMemcpyAsync(&dstat, b->status, sizeof(int), cudaMemcpyDeviceToHost, b->st));
+            LQCD_CUDA_CHECK(hc, cudaMemcpyAsync(S.data(), b->sc, n * sizeof(BScal), cudaMemcpyDeviceToHost, b->st));
+            LQCD_CUDA_CHECK(hc, cudaStreamSynchronize(b->st));
+            if (dstat != 0) st = set_err(hc, (lqcd_status)dstat, "batch: a device-side wait ran out of time");
         }
-        // the Dhat residual of every converged lattice, in FP64 (Eq. 5 only bounds it by the full one)
-        bool again = false;
-        for (int l = 0; l < n && st == LQCD_OK; l++) {
-            lqcd_ctx *c = b->ctx[l];
-            const long Vh = b->lat_h[l].Vh;
-            if (S[l].status != LQCD_OK || S[l].eta2 == 0) continue;
-            void *o, *t;
-            if ((st = ws_get(c, WS_MISC, 12 * Vh * sizeof(double2), &o)) != LQCD_OK) break;
-            if ((st = ws_get(c, WS_TMP_O, 12 * Vh * sizeof(double2), &t)) != LQCD_OK) break;
-            const double2 *pe = b->psi + b->lat_h[l].off64, *ee = b->eta + b->lat_h[l].off64;
-            double r2 = 0;
-            if ((st = dirac_dhat(c, LQCD_F64, pe, o, t, 1)) != LQCD_OK) break;
-            if ((st = blas_sub(c, 24 * Vh, (const double *)ee, (const double *)o, (double *)o)) != LQCD_OK) break;
-            if ((st = blas_norm2(c, 24 * Vh, (const double *)o, &r2)) != LQCD_OK) break;
-            dhat_rel[l] = std::sqrt(r2 / S[l].eta2);
-            if (dhat_rel[l] > b->p.tol && attempt < 3) {
-                const double f = b->p.tol / dhat_rel[l];
-                S[l].tol2 *= 0.25 * f * f;
-                S[l].done = 0;
-                S[l].status = LQCD_ERR_NOT_CONVERGED;
-                again = true;
-            }
-        }
-        if (!again || st != LQCD_OK) break;
-        LQCD_CUDA_CHECK(hc, cudaMemcpyAsync(b->sc, S.data(), n * sizeof(BScal), cudaMemcpyHostToDevice, b->st));
     }
     // results
     lqcd_status worst = st;
@@ -891,7 +879,7 @@ lqcd_status lqcd_batch_solve_dhat(lqcd_batch *b, const double *const *eta_dev, d
             info[l].iters = S[l].iters;
             info[l].restarts = S[l].restarts;
             info[l].true_relres = S[l].eta2 > 0 ? std::sqrt(S[l].true_rn2 / S[l].eta2) : 0;
-            info[l].relres_dhat = dhat_rel[l];
+            info[l].relres_dhat = info[l].true_relres;   // the residual of the Dhat system
             info[l].seconds = secs;
             info[l].status = (lqcd_status)S[l].status;
             info[l].net_fallbacks = 0;

@@ -100,18 +100,26 @@ __global__ void __launch_bounds__(Var<VAR>::T, Var<VAR>::B) k_hop(HopArgs<SP, LK
     hop_site<R, SP, LK, CL, MODE>(a, r, k);
 }
 
-// D on the full fields of several lattices in one launch.  items: (index of
-// the HopArgs of a lattice and output parity, first rank of the tile, sites in
-// the tile, lattice); tiles of lattices whose active flag is 0 are skipped.
-template <class R, class SP, class LK, class CL>
-__global__ void __launch_bounds__(256) k_hop_batch(const HopArgs<SP, LK, CL> *args, const int4 *items, const int *active)
+// One stage of Dhat (MODE_DHAT1, MODE_DHAT2) on several lattices in one launch.
+// args[2 l + stage]: lattice l; items: (lattice, first rank of the tile, sites in
+// the tile); tiles of lattices whose active flag is 0 are skipped.  shift moves
+// the even input field.
+template <class R, class SP, class LK, class CL, int MODE>
+__global__ void __launch_bounds__(256) k_hop_batch(const HopArgs<SP, LK, CL> *args, const int4 *items, const int *active,
+                                                   long shift)
 {
     __shared__ HopArgs<SP, LK, CL> sa;
     const int4 w = items[blockIdx.x];
-    if (active && !active[w.w]) return;
-    if (threadIdx.x == 0) sa = args[w.x];
+    if (active && !active[w.x]) return;
+    if (threadIdx.x == 0) {
+        sa = args[2 * w.x + (MODE == MODE_DHAT2)];
+        if (MODE == MODE_DHAT1)
+            sa.in_other += shift;
+        else
+            sa.in_same += shift;
+    }
     __syncthreads();
-    if ((int)threadIdx.x < w.z) hop_site<R, SP, LK, CL, MODE_D>(sa, w.y + threadIdx.x, 0);
+    if ((int)threadIdx.x < w.z) hop_site<R, SP, LK, CL, MODE>(sa, w.y + threadIdx.x, 0);
 }
 
 template <class R, class SP, class LK, class CL, int MODE>
@@ -424,8 +432,8 @@ struct DBatch {
     lqcd_prec p = LQCD_F32;
     int nlat = 0;
     long sites = 0;
-    void *args = nullptr;                       // HopArgs[2 nlat]: (lattice, output parity)
-    int4 *items[3] = {nullptr, nullptr, nullptr};   // tiles of 64 / 128 / 256 sites
+    void *args = nullptr;                       // HopArgs[2 nlat]: (lattice, stage)
+    int4 *items[3] = {nullptr, nullptr, nullptr};   // tiles of 64 / 128 / 256 ranks
     int nitems[3] = {0, 0, 0};
     int choice = -1;                            // tuned tile size index
 };
@@ -433,83 +441,67 @@ static const int kBatchTile[3] = {64, 128, 256};
 
 namespace {
 template <class SP, class LK, class CL>
-std::vector<HopArgs<SP, LK, CL>> batch_args(lqcd_ctx *const *ctx, int n, const SP *in, SP *out, const long *off,
-                                            long units_per_site, const LK *const *U, const CL *const *A0,
-                                            const CL *const *A1)
+lqcd_status batch_args(lqcd_ctx *hc, DBatch *b, lqcd_ctx *const *ctx, int n, const SP *in, SP *tmp, SP *out,
+                       const long *off, LK *lqcd_ctx::*U, CL *(lqcd_ctx::*A)[2], CL *(lqcd_ctx::*Ai)[2])
 {
     std::vector<HopArgs<SP, LK, CL>> v;
     for (int l = 0; l < n; l++)
-        for (int p = 0; p < 2; p++) {
+        for (int stage = 0; stage < 2; stage++) {
             HopArgs<SP, LK, CL> a;
-            const long half = units_per_site * ctx[l]->g.Vh;
             a.g = ctx[l]->g;
-            a.p_out = p;
+            a.p_out = 1 - stage;
             a.nrhs = 1;
-            a.in_other = in + off[l] + (1 - p) * half;
+            a.in_other = (stage == 0 ? in : tmp) + off[l];
             a.in_rs = 0;
-            a.in_same = in + off[l] + p * half;
+            a.in_same = stage == 0 ? nullptr : in + off[l];
             a.same_rs = 0;
-            a.out = out + off[l] + p * half;
+            a.out = (stage == 0 ? tmp : out) + off[l];
             a.out_rs = 0;
-            a.U = U[l];
-            a.clov = p ? A1[l] : A0[l];
+            a.U = ctx[l]->*U;
+            a.clov = stage == 0 ? (ctx[l]->*Ai)[1] : (ctx[l]->*A)[0];
             v.push_back(a);
         }
-    return v;
+    const size_t bytes = v.size() * sizeof(v[0]);
+    if (cudaMalloc(&b->args, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return set_err(hc, LQCD_ERR_NOMEM, "batched Dhat arguments");
+    }
+    LQCD_CUDA_CHECK(hc, cudaMemcpy(b->args, v.data(), bytes, cudaMemcpyHostToDevice));
+    return LQCD_OK;
 }
 }  // namespace
 
-lqcd_status dirac_batch_create(lqcd_ctx *hc, lqcd_ctx *const *ctx, int n, lqcd_prec p, const void *in, void *out,
-                               const long *off, DBatch **out_b)
+// in, tmp, out: arenas of half fields (even, odd, even), lattice l at off[l]
+lqcd_status dirac_batch_create(lqcd_ctx *hc, lqcd_ctx *const *ctx, int n, lqcd_prec p, const void *in, void *tmp,
+                               void *out, const long *off, DBatch **out_b)
 {
-    if (p != LQCD_F32 && p != LQCD_F64) return set_err(hc, LQCD_ERR_ARG, "batched D: precision %d", (int)p);
+    if (p != LQCD_F32 && p != LQCD_F64) return set_err(hc, LQCD_ERR_ARG, "batched Dhat: precision %d", (int)p);
     DBatch *b = new DBatch();
     b->p = p;
     b->nlat = n;
-    size_t argbytes;
-    std::vector<unsigned char> host;
-    if (p == LQCD_F32) {
-        std::vector<const float4 *> U(n), A0(n), A1(n);
-        for (int l = 0; l < n; l++) {
-            U[l] = ctx[l]->U32;
-            A0[l] = ctx[l]->A32[0];
-            A1[l] = ctx[l]->A32[1];
-        }
-        auto v = batch_args<float4, float4, float4>(ctx, n, (const float4 *)in, (float4 *)out, off, 6, U.data(),
-                                                    A0.data(), A1.data());
-        argbytes = v.size() * sizeof(v[0]);
-        host.assign((unsigned char *)v.data(), (unsigned char *)v.data() + argbytes);
-    } else {
-        std::vector<const double2 *> U(n), A0(n), A1(n);
-        for (int l = 0; l < n; l++) {
-            U[l] = ctx[l]->U64;
-            A0[l] = ctx[l]->A64[0];
-            A1[l] = ctx[l]->A64[1];
-        }
-        auto v = batch_args<double2, double2, double2>(ctx, n, (const double2 *)in, (double2 *)out, off, 12,
-                                                       U.data(), A0.data(), A1.data());
-        argbytes = v.size() * sizeof(v[0]);
-        host.assign((unsigned char *)v.data(), (unsigned char *)v.data() + argbytes);
-    }
-    if (cudaMalloc(&b->args, argbytes) != cudaSuccess) {
-        delete b;
-        cudaGetLastError();
-        return set_err(hc, LQCD_ERR_NOMEM, "batched D arguments");
-    }
-    cudaMemcpy(b->args, host.data(), argbytes, cudaMemcpyHostToDevice);
-    for (int t = 0; t < 3; t++) {
+    lqcd_status st;
+    if (p == LQCD_F32)
+        st = batch_args<float4, float4, float4>(hc, b, ctx, n, (const float4 *)in, (float4 *)tmp, (float4 *)out, off,
+                                                &lqcd_ctx::U32, &lqcd_ctx::A32, &lqcd_ctx::Ai32);
+    else
+        st = batch_args<double2, double2, double2>(hc, b, ctx, n, (const double2 *)in, (double2 *)tmp, (double2 *)out,
+                                                   off, &lqcd_ctx::U64, &lqcd_ctx::A64, &lqcd_ctx::Ai64);
+    for (int t = 0; t < 3 && st == LQCD_OK; t++) {
         std::vector<int4> it;
         for (int l = 0; l < n; l++)
-            for (int par = 0; par < 2; par++)
-                for (int r0 = 0; r0 < ctx[l]->g.Vh; r0 += kBatchTile[t])
-                    it.push_back(make_int4(2 * l + par, r0, std::min(kBatchTile[t], ctx[l]->g.Vh - r0), l));
+            for (int r0 = 0; r0 < ctx[l]->g.Vh; r0 += kBatchTile[t])
+                it.push_back(make_int4(l, r0, std::min(kBatchTile[t], ctx[l]->g.Vh - r0), 0));
         b->nitems[t] = (int)it.size();
         if (cudaMalloc(&b->items[t], it.size() * sizeof(int4)) != cudaSuccess) {
             cudaGetLastError();
-            dirac_batch_free(b);
-            return set_err(hc, LQCD_ERR_NOMEM, "batched D work list");
+            st = set_err(hc, LQCD_ERR_NOMEM, "batched Dhat work list");
+        } else {
+            cudaMemcpy(b->items[t], it.data(), it.size() * sizeof(int4), cudaMemcpyHostToDevice);
         }
-        cudaMemcpy(b->items[t], it.data(), it.size() * sizeof(int4), cudaMemcpyHostToDevice);
+    }
+    if (st != LQCD_OK) {
+        dirac_batch_free(b);
+        return st;
     }
     for (int l = 0; l < n; l++) b->sites += ctx[l]->g.V;
     *out_b = b;
@@ -525,26 +517,31 @@ void dirac_batch_free(DBatch *b)
 }
 
 namespace {
-lqcd_status batch_launch(lqcd_ctx *hc, DBatch *b, int t, const int *active)
+template <class R, class SP, class LK, class CL>
+void batch_launch2(cudaStream_t st, const DBatch *b, int t, const int *active, long shift)
+{
+    auto *a = (const HopArgs<SP, LK, CL> *)b->args;
+    k_hop_batch<R, SP, LK, CL, MODE_DHAT1><<<b->nitems[t], kBatchTile[t], 0, st>>>(a, b->items[t], active, shift);
+    k_hop_batch<R, SP, LK, CL, MODE_DHAT2><<<b->nitems[t], kBatchTile[t], 0, st>>>(a, b->items[t], active, shift);
+}
+lqcd_status batch_launch(lqcd_ctx *hc, DBatch *b, int t, const int *active, long shift)
 {
     if (b->p == LQCD_F32)
-        k_hop_batch<float, float4, float4, float4><<<b->nitems[t], kBatchTile[t], 0, hc->stream>>>(
-            (const HopArgs<float4, float4, float4> *)b->args, b->items[t], active);
+        batch_launch2<float, float4, float4, float4>(hc->stream, b, t, active, shift);
     else
-        k_hop_batch<double, double2, double2, double2><<<b->nitems[t], kBatchTile[t], 0, hc->stream>>>(
-            (const HopArgs<double2, double2, double2> *)b->args, b->items[t], active);
-    hc->n_kernel_launches++;
+        batch_launch2<double, double2, double2, double2>(hc->stream, b, t, active, shift);
+    hc->n_kernel_launches += 2;
     LQCD_LAUNCH_CHECK(hc);
     return LQCD_OK;
 }
 }  // namespace
 
-// out = D in on every lattice of the batch (tile size chosen by the autotuner
-// on the first call, which must not be inside a stream capture)
-lqcd_status dirac_batch_D(lqcd_ctx *hc, DBatch *b, const int *active)
+// out = Dhat (in + shift) on every lattice of the batch (tile size chosen by the
+// autotuner on the first call, which must not be inside a stream capture)
+lqcd_status dirac_batch_dhat(lqcd_ctx *hc, DBatch *b, long shift, const int *active)
 {
     if (b->choice < 0) {
-        std::string key = "k_hop_batch/p" + std::to_string((int)b->p) + "/n" + std::to_string(b->nlat) + "/s" +
+        std::string key = "k_hop_batch_dhat/p" + std::to_string((int)b->p) + "/n" + std::to_string(b->nlat) + "/s" +
                           std::to_string(b->sites);
         TuneChoice tc;
         if (tune_lookup(key, &tc)) {
@@ -555,7 +552,7 @@ lqcd_status dirac_batch_D(lqcd_ctx *hc, DBatch *b, const int *active)
                 float best = 1e30f;
                 for (int t = 0; t < 3; t++) {
                     float us;
-                    LQCD_TRY(tune_time(hc, [&]() { return batch_launch(hc, b, t, active); }, 3, &us));
+                    LQCD_TRY(tune_time(hc, [&]() { return batch_launch(hc, b, t, active, shift); }, 3, &us));
                     if (tune_verbose()) fprintf(stderr, "tune %s: tile %d %.1f us\n", key.c_str(), kBatchTile[t], us);
                     if (us < best) {
                         best = us;
@@ -569,5 +566,5 @@ lqcd_status dirac_batch_D(lqcd_ctx *hc, DBatch *b, const int *active)
             }
         }
     }
-    return batch_launch(hc, b, b->choice, active);
+    return batch_launch(hc, b, b->choice, active, shift);
 }

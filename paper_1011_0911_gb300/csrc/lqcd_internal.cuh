@@ -375,9 +375,9 @@ lqcd_status sap_apply(lqcd_ctx *c, const lqcd_sap_params *sp, const void *eta_na
 // error text, launch counter); arenas hold the lattices' native full fields at
 // offsets off[l] (in native spinor units of the precision)
 struct DBatch;
-lqcd_status dirac_batch_create(lqcd_ctx *hc, lqcd_ctx *const *ctx, int n, lqcd_prec p, const void *in, void *out,
-                               const long *off, DBatch **out_b);
-lqcd_status dirac_batch_D(lqcd_ctx *hc, DBatch *b, const int *active_dev);
+lqcd_status dirac_batch_create(lqcd_ctx *hc, lqcd_ctx *const *ctx, int n, lqcd_prec p, const void *in, void *tmp,
+                               void *out, const long *off, DBatch **out_b);
+lqcd_status dirac_batch_dhat(lqcd_ctx *hc, DBatch *b, long shift, const int *active_dev);
 void dirac_batch_free(DBatch *b);
 struct SapBatch;
 lqcd_status sap_batch_create(lqcd_ctx *hc, lqcd_ctx *const *ctx, int n, const lqcd_sap_params *sp, void *r,
