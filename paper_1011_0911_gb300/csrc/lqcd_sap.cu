@@ -1032,75 +1032,17 @@ int sap_stage_forced()
     return e[0] == '1' ? 1 : 0;
 }
 
-// r(x) -= sum of the hops into x from neighbours y that lie in another block
-// of colour col (delta holds chi there).  One thread per (site, rhs); i is the
-// parity-major site index 0 .. V-1.
+// r(x) -= sum of the hops into x from neighbours y that lie in another block of
+// colour col (delta holds chi there), over a precomputed list of the sites that
+// receive such hops: entry (i, mask) with i the parity-major site index and bit
+// 2 mu + (d > 0) of mask set for each hop from x + d mu.  The list is sorted by
+// mask, so the threads of a warp take the same hops (a thread per lattice site
+// branches per site and took twice the time).
 template <int P>
-__device__ __forceinline__ void sap_face_body(const SapArgs<P> &a, int col, long i, int rhs)
+__device__ __forceinline__ void sap_face_site(const SapArgs<P> &a, int2 fs, int rhs)
 {
     using R = typename SapT<P>::R;
     using SP = typename SapT<P>::SP;
-    const BlkGeom &B = a.B;
-    if (i >= 2L * a.g.Vh) return;
-    const long Vh = a.g.Vh;
-    const int par = i >= Vh;
-    const long rk = par ? i - Vh : i;
-    const long half = SapT<P>::half(Vh);
-    const long foff = rhs * a.fstride;
-    int x[4];
-    rank_coords(a.g, par, (int)rk, x);
-    int bx[4];
-    for (int m = 0; m < 4; m++) bx[m] = x[m] / B.bs[m];
-    cx<R> acc[12], u[3][3], v[12];
-    bool any = false;
-#pragma unroll
-    for (int c = 0; c < 12; c++) acc[c] = mk(R(0), R(0));
-    const SP *din = a.delta + foff + (1 - par) * half;
-    for (int mu = 0; mu < 4; mu++)
-        for (int d = -1; d <= 1; d += 2) {
-            int y[4] = {x[0], x[1], x[2], x[3]};
-            int vv = y[mu] + d;
-            y[mu] = vv < 0 ? vv + a.g.L[mu] : (vv >= a.g.L[mu] ? vv - a.g.L[mu] : vv);
-            int by = y[mu] / B.bs[mu];
-            if (by == bx[mu]) continue;   // same block (also covers a block spanning the direction)
-            int csum = by - bx[mu];
-            for (int m = 0; m < 4; m++) csum += bx[m];
-            if ((csum & 1) != col) continue;
-            long ry = coords_rank(a.g, y);
-            gload(din, Vh, ry, v);
-            if (d > 0) {
-                R sg = (mu == 0 && x[0] == a.g.L[0] - 1) ? R(a.g.bc_t) : R(1);
-                glink(a.U, Vh, par, mu, rk, u);
-                proj_apply<R>(mu, -1, v, u, false, sg, acc);
-            } else {
-                R sg = (mu == 0 && x[0] == 0) ? R(a.g.bc_t) : R(1);
-                glink(a.U, Vh, 1 - par, mu, ry, u);
-                proj_apply<R>(mu, +1, v, u, true, sg, acc);
-            }
-            any = true;
-        }
-    if (!any) return;
-    // r -= H delta = r + 1/2 S
-#pragma unroll
-    for (int c = 0; c < 12; c++) acc[c] = R(0.5) * acc[c];
-    gadd(a.r + foff + par * half, Vh, rk, acc);
-}
-
-// The update of sap_face_body driven by a precomputed list of the sites that receive hops
-// from blocks of colour col: entry (i, mask) with i the parity-major site index
-// and bit 2 mu + (d > 0) of mask set for each hop from x + d mu that enters
-// from such a block.  The list is sorted by mask, so the threads of a warp
-// take the same hops (the site-ordered form branches per site); the hops are
-// those of sap_face_body in the same order, so the result is bitwise the same.
-template <int P>
-__global__ void __launch_bounds__(128) k_sap_face_l(SapArgs<P> a, const int2 *__restrict__ list, int n)
-{
-    using R = typename SapT<P>::R;
-    using SP = typename SapT<P>::SP;
-    const long e = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (e >= n) return;
-    const int rhs = blockIdx.y;
-    const int2 fs = list[e];
     const long Vh = a.g.Vh;
     const int par = fs.x >= Vh;
     const long rk = par ? fs.x - Vh : fs.x;
@@ -1127,9 +1069,16 @@ __global__ void __launch_bounds__(128) k_sap_face_l(SapArgs<P> a, const int2 *__
                 proj_apply<R>(mu, +1, v, u, true, sg, acc);
             }
         }
+    // r -= H delta = r + 1/2 S
 #pragma unroll
     for (int c = 0; c < 12; c++) acc[c] = R(0.5) * acc[c];
     gadd(a.r + foff + par * half, Vh, rk, acc);
+}
+template <int P>
+__global__ void __launch_bounds__(128) k_sap_face_l(SapArgs<P> a, const int2 *__restrict__ list, int n)
+{
+    const long e = blockIdx.x * (long)blockDim.x + threadIdx.x;
+    if (e < n) sap_face_site<P>(a, list[e], blockIdx.y);
 }
 
 // ------------------------------------------------------------------ batches
@@ -1157,17 +1106,18 @@ __global__ void __launch_bounds__(2 * SAPS_NH, sap_ctas<P, SA>())
     }
 }
 
-// face items: (lattice, first parity-major site of a 128-site tile)
+// items: (lattice, first list entry of a tile of up to 128, entries in the tile);
+// lists[2 l + col]: the face list of lattice l after colour col
 template <int P>
 __global__ void __launch_bounds__(128)
-    k_sap_face_batch(const SapArgs<P> *args, int col, const int2 *items, int nitems, const int *active)
+    k_sap_face_batch(const SapArgs<P> *args, int col, const int2 *const *lists, const int4 *items, const int *active)
 {
-    const int2 w = items[blockIdx.x];
+    const int4 w = items[blockIdx.x];
     if (active && !active[w.x]) return;
     __shared__ SapArgs<P> sa;
     if (threadIdx.x == 0) sa = args[2 * w.x + col];
     __syncthreads();
-    sap_face_body<P>(sa, col, (long)w.y + threadIdx.x, 0);
+    if ((int)threadIdx.x < w.z) sap_face_site<P>(sa, lists[2 * w.x + col][w.y + threadIdx.x], 0);
 }
 
 // LQCD_SAP_GENERIC=1 selects the generic (L1-cached) FP32 block kernel
@@ -1549,8 +1499,9 @@ struct SapBatch {
     void *args = nullptr;                  // SapArgs<p>[2 nlat]
     int2 *blk[2] = {nullptr, nullptr};     // (lattice, index in its colour list)
     int nblk[2] = {0, 0};
-    int2 *face = nullptr;                  // (lattice, first site of a 128-site tile)
-    int nface = 0;
+    const int2 **lists = nullptr;          // [2 nlat] face lists (the plans' own)
+    int4 *face[2] = {nullptr, nullptr};    // (lattice, first list entry, entries) per colour
+    int nface[2] = {0, 0};
     int *queue = nullptr;                  // one work counter per block launch of an application
     void *r = nullptr, *psi = nullptr, *delta = nullptr;
 };
@@ -1561,7 +1512,9 @@ void sap_batch_free(SapBatch *b)
     cudaFree(b->args);
     cudaFree(b->blk[0]);
     cudaFree(b->blk[1]);
-    cudaFree(b->face);
+    cudaFree(b->lists);
+    cudaFree(b->face[0]);
+    cudaFree(b->face[1]);
     cudaFree(b->queue);
     delete b;
 }
@@ -1573,7 +1526,9 @@ lqcd_status sap_batch_args(lqcd_ctx *hc, lqcd_ctx *const *ctx, int n, const lqcd
 {
     using SP = typename SapT<P>::SP;
     std::vector<SapArgs<P>> v;
-    std::vector<int2> it[2], face;
+    std::vector<int2> it[2];
+    std::vector<int4> face[2];
+    std::vector<const int2 *> lists;
     for (int l = 0; l < n; l++) {
         SapPlan *pl;
         LQCD_TRY(get_plan(ctx[l], sp->bs, &pl));
@@ -1604,8 +1559,10 @@ lqcd_status sap_batch_args(lqcd_ctx *hc, lqcd_ctx *const *ctx, int n, const lqcd
             LQCD_CUDA_CHECK(hc, cudaStreamSynchronize(ctx[l]->stream));   // the batch runs on its own stream
             v.push_back(a);
             for (int i = 0; i < pl->count[col]; i++) it[col].push_back(make_int2(l, i));
+            lists.push_back(pl->face_dev[col]);
+            for (int e = 0; e < pl->nface[col]; e += 128)
+                face[col].push_back(make_int4(l, e, std::min(128, pl->nface[col] - e), 0));
         }
-        for (int s0 = 0; s0 < 2 * ctx[l]->g.Vh; s0 += 128) face.push_back(make_int2(l, s0));
     }
     LQCD_CUDA_CHECK(hc, cudaMalloc(&b->args, v.size() * sizeof(v[0])));
     LQCD_CUDA_CHECK(hc, cudaMemcpy(b->args, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice));
@@ -1614,9 +1571,15 @@ lqcd_status sap_batch_args(lqcd_ctx *hc, lqcd_ctx *const *ctx, int n, const lqcd
         LQCD_CUDA_CHECK(hc, cudaMalloc(&b->blk[col], std::max<size_t>(1, it[col].size()) * sizeof(int2)));
         LQCD_CUDA_CHECK(hc, cudaMemcpy(b->blk[col], it[col].data(), it[col].size() * sizeof(int2), cudaMemcpyHostToDevice));
     }
-    b->nface = (int)face.size();
-    LQCD_CUDA_CHECK(hc, cudaMalloc(&b->face, face.size() * sizeof(int2)));
-    LQCD_CUDA_CHECK(hc, cudaMemcpy(b->face, face.data(), face.size() * sizeof(int2), cudaMemcpyHostToDevice));
+    LQCD_CUDA_CHECK(hc, cudaMalloc((void **)&b->lists, lists.size() * sizeof(lists[0])));
+    LQCD_CUDA_CHECK(hc, cudaMemcpy((void *)b->lists, lists.data(), lists.size() * sizeof(lists[0]),
+                                   cudaMemcpyHostToDevice));
+    for (int col = 0; col < 2; col++) {
+        b->nface[col] = (int)face[col].size();
+        LQCD_CUDA_CHECK(hc, cudaMalloc(&b->face[col], std::max<size_t>(1, face[col].size()) * sizeof(int4)));
+        LQCD_CUDA_CHECK(hc, cudaMemcpy(b->face[col], face[col].data(), face[col].size() * sizeof(int4),
+                                       cudaMemcpyHostToDevice));
+    }
     return LQCD_OK;
 }
 
@@ -1651,7 +1614,8 @@ lqcd_status sap_batch_run(lqcd_ctx *hc, SapBatch *b, const int *active)
             hc->n_kernel_launches++;
             LQCD_LAUNCH_CHECK(hc);
             if (cyc == b->ncy - 1 && col == last_col) continue;
-            k_sap_face_batch<P><<<b->nface, 128, 0, hc->stream>>>(args, col, b->face, b->nface, active);
+            if (b->nface[col] == 0) continue;
+            k_sap_face_batch<P><<<b->nface[col], 128, 0, hc->stream>>>(args, col, b->lists, b->face[col], active);
             hc->n_kernel_launches++;
             LQCD_LAUNCH_CHECK(hc);
         }
