@@ -195,6 +195,7 @@ constexpr int PACK_SITES = 64, PACK_THREADS = 128;
 template <int PREC, bool UNPACK>
 __global__ void __launch_bounds__(PACK_THREADS) k_pack_t(Geom g, int nsub, typename PackT<PREC>::W *canon, void *native)
 {
+    after_previous();
     using W = typename PackT<PREC>::W;
     constexpr int U = PackT<PREC>::U, LD = U + 1;
     __shared__ W tile[PACK_SITES * LD];
@@ -272,10 +273,11 @@ void launch_pack_t(lqcd_ctx *c, int nsub, const void *canon, void *native, int n
     using W = typename PackT<PREC>::W;
     const dim3 grid(div_up((long)nsub * c->g.Vh, PACK_SITES), nrhs);
     W *w = (W *)canon;
+    const bool pdl = !c->capturing;
     if (unpack)
-        k_pack_t<PREC, true><<<grid, PACK_THREADS, 0, c->stream>>>(c->g, nsub, w, native);
+        launch_pdl(pdl, k_pack_t<PREC, true>, grid, PACK_THREADS, c->stream, c->g, nsub, w, native);
     else
-        k_pack_t<PREC, false><<<grid, PACK_THREADS, 0, c->stream>>>(c->g, nsub, w, native);
+        launch_pdl(pdl, k_pack_t<PREC, false>, grid, PACK_THREADS, c->stream, c->g, nsub, w, native);
 }
 
 // native F64 <-> native F32 (same site/chunk structure), nhalf half fields
@@ -463,6 +465,7 @@ lqcd_status lqcd_destroy(lqcd_ctx *c)
     cudaFree(c->red);
     cudaFree(c->red_out);
     if (c->red_host) cudaFreeHost(c->red_host);
+    if (c->cg_stream) cudaStreamDestroy(c->cg_stream);
     for (auto &w : c->ws)
         if (w.p) cudaFree(w.p);
     delete c;

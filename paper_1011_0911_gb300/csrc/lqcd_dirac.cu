@@ -279,8 +279,19 @@ lqcd_status launch_hop(lqcd_ctx *c, int p_out, const SP *in_other, long in_rs, c
     static const char *kname[3] = {"k_hop4_hop", "k_hop4_mr", "k_hop4_sm"};
     static const char *dname[5] = {"k_hop_d", "k_hop_d1", "k_hop_d2", "", "k_hop_d4"};
     const int split = dbl ? hop_force_split() : 0;
-    std::string key = tune_key(c, dbl ? dname[split] : (force >= 0 ? kname[force] : "k_hop4"), MODE, prec, nrhs);
+    TuneMemo &memo = c->tune[MODE][prec][p_out];
+    const int forced = dbl ? 16 + split : force;
     TuneChoice tc;
+    if (memo.gen == tune_generation() && memo.nrhs == nrhs && memo.force == forced) {
+        tc.variant = memo.variant;
+        tc.tx = memo.tx;
+        tc.ty = memo.ty;
+        tc.nr = memo.nr;
+        tc.kind = memo.kind;
+        return launch_choice<R, SP, LK, CL, MODE>(c, tc, a);
+    }
+    std::string key = tune_key(c, dbl ? dname[split] : (force >= 0 ? kname[force] : "k_hop4"), MODE, prec, nrhs);
+    bool settled = true;   // a choice of the table, not a default taken while the search is off
     if (!tune_lookup(key, &tc)) {
         tc = TuneChoice();
         tc.tx = nrhs == 1 ? 128 : 32;
@@ -325,8 +336,11 @@ lqcd_status launch_hop(lqcd_ctx *c, int p_out, const SP *in_other, long in_rs, c
                 }
             }
             tune_store(key, tc);
+        } else {
+            settled = false;
         }
     }
+    if (settled) memo = TuneMemo{tune_generation(), nrhs, forced, tc.variant, tc.tx, tc.ty, tc.nr, tc.kind};
     return launch_choice<R, SP, LK, CL, MODE>(c, tc, a);
 }
 

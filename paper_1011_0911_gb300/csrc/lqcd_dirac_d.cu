@@ -171,6 +171,7 @@ template <int MODE, int G>
 __global__ void __launch_bounds__(HOP_D_THREADS, 3) k_hop_d(HopArgs<double2, double2, double2> a)
 {
     constexpr int P = 2 * G, SW = 32 / P;
+    after_previous();
     const long Vh = a.g.Vh;
     const int kf = blockIdx.x % a.nrhs;
     const int lane = threadIdx.x & 31, part = lane / SW, s = part & 1;
@@ -299,14 +300,16 @@ lqcd_status launch_hop_d(lqcd_ctx *c, int G, const HopArgs<double2, double2, dou
     const long nb = (long)div_up(c->g.Vh, sites) * a.nrhs;
     if (nb > 0x7fffffffL) return set_err(c, LQCD_ERR_ARG, "FP64 stencil: grid of %ld CTAs", nb);
     const int grid = (int)nb;
+    const bool pdl = !c->capturing;
+    cudaError_t e = cudaSuccess;
     switch (G) {
-        case 1: k_hop_d<MODE, 1><<<grid, HOP_D_THREADS, 0, c->stream>>>(a); break;
-        case 2: k_hop_d<MODE, 2><<<grid, HOP_D_THREADS, 0, c->stream>>>(a); break;
-        case 4: k_hop_d<MODE, 4><<<grid, HOP_D_THREADS, 0, c->stream>>>(a); break;
+        case 1: e = launch_pdl(pdl, k_hop_d<MODE, 1>, grid, HOP_D_THREADS, c->stream, a); break;
+        case 2: e = launch_pdl(pdl, k_hop_d<MODE, 2>, grid, HOP_D_THREADS, c->stream, a); break;
+        case 4: e = launch_pdl(pdl, k_hop_d<MODE, 4>, grid, HOP_D_THREADS, c->stream, a); break;
         default: return set_err(c, LQCD_ERR_ARG, "FP64 stencil: split %d", G);
     }
     c->n_kernel_launches++;
-    LQCD_LAUNCH_CHECK(c);
+    LQCD_CUDA_CHECK(c, e);
     return LQCD_OK;
 }
 

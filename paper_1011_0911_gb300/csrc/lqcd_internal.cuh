@@ -179,6 +179,15 @@ struct Workspace {
     size_t bytes = 0;
 };
 
+// the autotuner's choice for a stencil launch, kept with the context while nothing
+// it depends on changes (building and looking up its key took longer than the
+// launch)
+struct TuneMemo {
+    long gen = -1;      // generation of the tuner's table
+    int nrhs = 0, force = 0;
+    int variant = 0, tx = 0, ty = 0, nr = 0, kind = 0;
+};
+
 struct DflState;   // deflation subspace (lqcd_dfl.cu)
 struct NetState;   // learned preconditioner (lqcd_ptc.cu)
 struct ChronoState;   // stored solutions for initial guesses (lqcd_chrono.cu)
@@ -211,6 +220,9 @@ struct lqcd_ctx {
     NetState *net = nullptr;
     ChronoState *chrono = nullptr;
     long n_kernel_launches = 0;
+    TuneMemo tune[4][3][2];   // [mode][precision][output parity]
+    bool capturing = false;               // launches go into a graph being captured
+    cudaStream_t cg_stream = nullptr;     // CGNR on small lattices (lqcd_cgnr.cu)
     // LQCD_PROFILE=1: synchronised wall time of solver phases, reported on
     // stderr by the GCR (developer instrumentation; off by default)
     bool prof_on = false;
@@ -300,6 +312,37 @@ inline long native_half_units(const lqcd_ctx *c, lqcd_prec p)   // in 16-byte un
     return (long)(native_half_bytes(c, p) / 16);
 }
 
+// Launch whose CTAs may be set up while the kernel before it in the stream is
+// still running (programmatic dependent launch); the kernel begins with
+// after_previous(), which waits until that kernel has finished and its writes are
+// visible.  It hides about 2 us per kernel: Dhat FP64 on 8^4 (four kernels) 28.7
+// -> 19.3 us.  Kernels must let the next one be set up only after their own wait:
+// signalled before it, the launches of a chain pile up on the SMs (43.6 us).  In
+// captured graphs plain launches are faster (CGNR on 8^4: 6.97 against 7.97 ms).
+template <class... KP, class... A>
+inline cudaError_t launch_pdl(bool pdl, void (*kernel)(KP...), dim3 grid, dim3 block, cudaStream_t st, A... args)
+{
+    if (!pdl) {
+        kernel<<<grid, block, 0, st>>>(args...);
+        return cudaGetLastError();
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KP>(args)...);
+}
+__device__ __forceinline__ void after_previous()
+{
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();   // the next kernel may be set up now, but no later one
+}
+
 // launch helpers
 inline int div_up(long a, long b) { return (int)((a + b - 1) / b); }
 
@@ -365,6 +408,9 @@ lqcd_status bmulti_axpy_mixed(lqcd_ctx *c, int nh, int nrhs, int k, const double
                               long fa, double2 *y, long fy);   // y_r += sum_i c_ri X_ir
 lqcd_status blas_gamma5_native64(lqcd_ctx *c, long nhalf, const double2 *in, double2 *out);
 lqcd_status blas_zero(lqcd_ctx *c, size_t bytes, void *p);
+
+// even-odd CGNR (lqcd_cgnr.cu)
+lqcd_status cgnr_native(lqcd_ctx *c, const double2 *eta, double2 *x, double tol, int nmx, lqcd_solve_info *info);
 
 // sap
 lqcd_status sap_axpby_native(lqcd_ctx *c, lqcd_prec p, const void *eta, void *r);

@@ -1,5 +1,5 @@
-// Outer solvers: even-odd CGNR on Dhat (Eq. 2) and the flexible GCR of
-// Sec. 3-4, preconditioned by SAP or deflated SAP.
+// Outer solvers: the flexible GCR of Sec. 3-4, preconditioned by SAP or deflated
+// SAP, and the solver entry points (CGNR: lqcd_cgnr.cu).
 //
 // The GCR solves either D psi = eta on the full lattice or Dhat psi_e = eta_e.
 // The latter is the former with the odd half eliminated: completing an even
@@ -36,93 +36,6 @@ struct Cplx {
 };
 inline Cplx cmul(Cplx a, Cplx b) { return {a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re}; }
 inline Cplx cdiv(Cplx a, double b) { return {a.re / b, a.im / b}; }
-
-// ---------------------------------------------------------------- CGNR
-lqcd_status cgnr_native(lqcd_ctx *c, const double2 *eta, double2 *x, double tol, int nmx, lqcd_solve_info *info)
-{
-    const long Vh = c->g.Vh;
-    const long n2 = 24 * Vh;   // doubles in one even field
-    const size_t hb = native_half_bytes(c, LQCD_F64);
-    void *buf;
-    LQCD_TRY(ws_get(c, WS_CGNR, 5 * hb, &buf));
-    double2 *r = (double2 *)buf, *z = r + 12 * Vh, *p = z + 12 * Vh, *w = p + 12 * Vh, *t = w + 12 * Vh;
-    void *tmp_o;
-    LQCD_TRY(ws_get(c, WS_TMP_O, hb, &tmp_o));
-    auto dhat = [&](const double2 *in, double2 *out) { return dirac_dhat(c, LQCD_F64, in, out, tmp_o, 1); };
-    auto dhat_dag = [&](const double2 *in, double2 *out) -> lqcd_status {
-        LQCD_TRY(blas_gamma5_native64(c, 1, in, t));
-        LQCD_TRY(dirac_dhat(c, LQCD_F64, t, out, tmp_o, 1));
-        return blas_gamma5_native64(c, 1, out, out);
-    };
-    double t0 = now_s();
-    LQCD_TRY(blas_zero(c, hb, x));
-    LQCD_TRY(blas_copy(c, n2, (const double *)eta, (double *)r));
-    double eta2;
-    LQCD_TRY(blas_norm2(c, n2, (const double *)eta, &eta2));
-    int it = 0;
-    lqcd_status st = LQCD_ERR_NOT_CONVERGED;
-    double rr = eta2;
-    if (eta2 == 0) {
-        st = LQCD_OK;
-    } else if (!std::isfinite(eta2)) {
-        st = LQCD_ERR_NAN;
-    } else {
-        LQCD_TRY(dhat_dag(r, z));
-        LQCD_TRY(blas_copy(c, n2, (const double *)z, (double *)p));
-        double zz;
-        LQCD_TRY(blas_norm2(c, n2, (const double *)z, &zz));
-        while (it < nmx) {
-            LQCD_TRY(dhat(p, w));
-            double ww;
-            LQCD_TRY(blas_norm2(c, n2, (const double *)w, &ww));
-            if (!std::isfinite(ww)) {
-                st = LQCD_ERR_NAN;
-                break;
-            }
-            if (ww == 0) {
-                st = LQCD_ERR_BREAKDOWN;
-                break;
-            }
-            double alpha = zz / ww;
-            LQCD_TRY(blas_axpy(c, n2, alpha, 0, (const double *)p, (double *)x));
-            LQCD_TRY(blas_axpy(c, n2, -alpha, 0, (const double *)w, (double *)r));
-            it++;
-            LQCD_TRY(blas_norm2(c, n2, (const double *)r, &rr));
-            if (rr <= tol * tol * eta2) {
-                // recompute the residual before accepting
-                LQCD_TRY(dhat(x, w));
-                LQCD_TRY(blas_sub(c, n2, (const double *)eta, (const double *)w, (double *)r));
-                LQCD_TRY(blas_norm2(c, n2, (const double *)r, &rr));
-                if (rr <= tol * tol * eta2) {
-                    st = LQCD_OK;
-                    break;
-                }
-                LQCD_TRY(dhat_dag(r, z));
-                LQCD_TRY(blas_copy(c, n2, (const double *)z, (double *)p));
-                LQCD_TRY(blas_norm2(c, n2, (const double *)z, &zz));
-                continue;
-            }
-            LQCD_TRY(dhat_dag(r, z));
-            double zz1;
-            LQCD_TRY(blas_norm2(c, n2, (const double *)z, &zz1));
-            LQCD_TRY(blas_xpay(c, n2, (const double *)z, zz1 / zz, (double *)p));
-            zz = zz1;
-        }
-    }
-    // final true residual
-    LQCD_TRY(dhat(x, w));
-    LQCD_TRY(blas_sub(c, n2, (const double *)eta, (const double *)w, (double *)r));
-    LQCD_TRY(blas_norm2(c, n2, (const double *)r, &rr));
-    if (info) {
-        info->iters = it;
-        info->restarts = 0;
-        info->relres_dhat = eta2 > 0 ? std::sqrt(rr / eta2) : 0;
-        info->true_relres = info->relres_dhat;
-        info->seconds = now_s() - t0;
-        info->status = st;
-    }
-    return st;
-}
 
 // ---------------------------------------------------------------- GCR
 // All fields below are native full FP64 fields; nrhs of them are stored one

@@ -7,6 +7,7 @@
 // ($LQCD_TUNE_CACHE, default $HOME/.cache/lqcd_tune.json) so later processes
 // skip the search.  Kernels whose results do not depend on the launch shape
 // (no reductions) are the only ones tuned, so tuning never changes numerics.
+#include <atomic>
 #include <cstdlib>
 #include <fstream>
 #include <map>
@@ -22,6 +23,7 @@ namespace {
 std::mutex g_mu;
 std::map<std::string, TuneChoice> g_cache;
 bool g_loaded = false;
+std::atomic<long> g_generation{0};
 std::string g_gpu;
 
 std::string cache_path()
@@ -112,8 +114,11 @@ void tune_store(const std::string &key, const TuneChoice &t)
     std::lock_guard<std::mutex> lk(g_mu);
     load_locked();
     g_cache[key] = t;
+    g_generation++;
     save_locked();
 }
+
+long tune_generation() { return g_generation.load(); }
 
 bool tune_enabled()
 {
@@ -160,6 +165,7 @@ extern "C" LQCD_API lqcd_status lqcd_tune_reset(void)
 {
     std::lock_guard<std::mutex> lk(g_mu);
     g_cache.clear();
+    g_generation++;
     g_loaded = false;   // the next lookup reads the cache file again
     return LQCD_OK;
 }

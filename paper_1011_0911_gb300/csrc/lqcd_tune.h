@@ -19,6 +19,7 @@ struct TuneChoice {
 std::string tune_key(const lqcd_ctx *c, const char *kernel, int mode, int prec, int nrhs);
 bool tune_lookup(const std::string &key, TuneChoice *out);
 void tune_store(const std::string &key, const TuneChoice &t);
+long tune_generation();   // changes whenever the table of choices does
 bool tune_enabled();
 bool tune_verbose();   // LQCD_TUNE_VERBOSE=1: report every timed candidate on stderr
 lqcd_status tune_time(lqcd_ctx *c, const std::function<lqcd_status()> &launch, int reps, float *us);
