@@ -9,7 +9,8 @@
 //   p = r + beta (p - omega v), v = Dhat_blk p, alpha = rho / <rhat, v>,
 //   s = r - alpha v, (|s| <= tol |eta|: x += alpha p, done), t = Dhat_blk s,
 //   omega = <t, s> / <t, t>, x += alpha p + omega s, r = s - omega t.
-// The operator is one pair of lattice-wide launches; inner products are
+// The operator is one pair of lattice-wide launches of the FP64 stencil with the
+// hops out of a block left out (lqcd_dirac_d.cu); inner products are
 // per-block reductions over a block-major list of the even sites (fixed order:
 // per-CTA partials, then a per-block sum); the scalars and the activity flags
 // live per block in device memory, and a block that has converged (or broken
@@ -32,88 +33,6 @@ __device__ __forceinline__ int blk_id(const BlkG &B, const int x[4])
 {
     return x[3] / B.bs[3] + B.nb[3] * (x[2] / B.bs[2] + B.nb[2] * (x[1] / B.bs[1] + B.nb[1] * (x[0] / B.bs[0])));
 }
-// does the hop from x by d along mu stay in x's block (after the periodic wrap)?
-__device__ __forceinline__ bool in_blk(const Geom &g, const BlkG &B, const int x[4], int mu, int d)
-{
-    int v = x[mu] + d;
-    v = v < 0 ? v + g.L[mu] : (v >= g.L[mu] ? v - g.L[mu] : v);
-    return v / B.bs[mu] == x[mu] / B.bs[mu];
-}
-
-// the hops of direction MU into x, each kept only inside x's block (same
-// arithmetic as the lattice-wide stencil)
-template <int MU>
-__device__ __forceinline__ void bhop_dir(const Geom &g, const BlkG &B, int p_out, int r, const int x[4],
-                                         const double2 *in, long Vh, const double2 *U, Spinor<double> &acc)
-{
-    cx<double> h[2][3], w[2][3], u[3][3];
-    Spinor<double> psi;
-    if (in_blk(g, B, x, MU, +1)) {
-        const int ry = nbr_rank(g, x, MU, +1);
-        const double sg = (MU == 0 && x[0] == g.L[0] - 1) ? double(g.bc_t) : 1.0;
-        load_spinor(in, Vh, ry, psi);
-        project<double, MU, -1>(psi, h);
-        load_link(U, Vh, p_out, MU, r, u);
-        su3_vec(u, h[0], w[0]);
-        su3_vec(u, h[1], w[1]);
-        accumulate<double, MU, -1, MU == 0>(acc, w, sg);
-    }
-    if (in_blk(g, B, x, MU, -1)) {
-        const int rz = nbr_rank(g, x, MU, -1);
-        const double sg = (MU == 0 && x[0] == 0) ? double(g.bc_t) : 1.0;
-        load_spinor(in, Vh, rz, psi);
-        project<double, MU, +1>(psi, h);
-        load_link(U, Vh, 1 - p_out, MU, rz, u);
-        su3dag_vec(u, h[0], w[0]);
-        su3dag_vec(u, h[1], w[1]);
-        accumulate<double, MU, +1, MU == 0>(acc, w, sg);
-    }
-}
-
-// MODE_DHAT1: out_o = A_oo^-1 (-1/2 S_blk in_e);  MODE_DHAT2: out_e = A_ee same_e + 1/2 S_blk in_o
-template <int MODE>
-__global__ void __launch_bounds__(128) k_bhop(Geom g, BlkG B, const double2 *in, const double2 *same, double2 *out,
-                                              const double2 *U, const double2 *cl)
-{
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= g.Vh) return;
-    const long Vh = g.Vh;
-    const int p_out = MODE == MODE_DHAT1 ? 1 : 0;
-    int x[4];
-    rank_coords(g, p_out, r, x);
-    Spinor<double> acc;
-    if (MODE == MODE_DHAT1) {
-#pragma unroll
-        for (int s = 0; s < 4; s++)
-#pragma unroll
-            for (int c = 0; c < 3; c++) acc.s[s][c] = mk(0.0, 0.0);
-    } else {
-        Spinor<double> self;
-        load_spinor(same, Vh, r, self);
-        clover_apply<double, double2>(cl, Vh, r, self, acc);
-#pragma unroll
-        for (int s = 0; s < 4; s++)
-#pragma unroll
-            for (int c = 0; c < 3; c++) acc.s[s][c] = 2.0 * acc.s[s][c];
-    }
-    bhop_dir<0>(g, B, p_out, r, x, in, Vh, U, acc);
-    bhop_dir<1>(g, B, p_out, r, x, in, Vh, U, acc);
-    bhop_dir<2>(g, B, p_out, r, x, in, Vh, U, acc);
-    bhop_dir<3>(g, B, p_out, r, x, in, Vh, U, acc);
-    const double f = MODE == MODE_DHAT2 ? 0.5 : -0.5;
-#pragma unroll
-    for (int s = 0; s < 4; s++)
-#pragma unroll
-        for (int c = 0; c < 3; c++) acc.s[s][c] = f * acc.s[s][c];
-    if (MODE == MODE_DHAT1) {
-        Spinor<double> res;
-        clover_apply<double, double2>(cl, Vh, r, acc, res);
-        store_spinor(out, Vh, r, res);
-    } else {
-        store_spinor(out, Vh, r, acc);
-    }
-}
-
 // list[b*hb + k] = rank of the k-th even site of block b (local lexicographic
 // order; the block origin has even parity, so k = local lex / 2), blk[r] = b
 __global__ void k_blist(Geom g, BlkG B, int *list, int *blk)
@@ -132,7 +51,8 @@ __global__ void k_blist(Geom g, BlkG B, int *list, int *blk)
 }
 
 // per-block inner products <a_j, b_j> (j < ND) over the block's even sites:
-// partial[(b*nch + c)*ND + j] for chunk c of the block's list
+// partial[(b*nch + c)*ND + j] for chunk c of the block's list; a_j = b_j gives the
+// norm (imaginary part 0) at half the products
 template <int ND>
 struct DotSet {
     const double2 *a[ND], *b[ND];
@@ -143,41 +63,40 @@ __global__ void __launch_bounds__(256) k_bdot(long Vh, int hb, int nch, const in
 {
     const int b = blockIdx.x, c = blockIdx.y;   // blocks on x (no 65535 limit), chunks on y
     const int per = (hb + nch - 1) / nch, k0 = c * per, k1 = min(hb, k0 + per);
-    double re[ND], im[ND];
+    double v[2 * ND];
 #pragma unroll
-    for (int j = 0; j < ND; j++) re[j] = im[j] = 0;
-    for (int k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
-        const long r = list[(long)b * hb + k];
+    for (int j = 0; j < 2 * ND; j++) v[j] = 0;
+    // two threads per site, six components each
+    const int hq = 6 * (threadIdx.x & 1);
+    for (int k = k0 + (threadIdx.x >> 1); k < k1; k += blockDim.x >> 1) {
+        const long r = list[(long)b * hb + k] + hq * Vh;
 #pragma unroll
-        for (int j = 0; j < ND; j++)
+        for (int j = 0; j < ND; j++) {
+            double2 x[6], y[6];
 #pragma unroll
-            for (int q = 0; q < 12; q++) {
-                const double2 u = d.a[j][q * Vh + r], v = d.b[j][q * Vh + r];
-                cdot_add(re[j], im[j], u, v);
+            for (int q = 0; q < 6; q++) {
+                x[q] = d.a[j][q * Vh + r];
+                if (d.a[j] != d.b[j]) y[q] = d.b[j][q * Vh + r];
             }
-    }
-    __shared__ double sh[8][ND][2];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+            if (d.a[j] == d.b[j]) {
 #pragma unroll
-    for (int j = 0; j < ND; j++) {
-        double x = re[j], m = im[j];
-        for (int o = 16; o > 0; o >>= 1) {
-            x += __shfl_down_sync(0xffffffffu, x, o);
-            m += __shfl_down_sync(0xffffffffu, m, o);
-        }
-        if (lane == 0) {
-            sh[warp][j][0] = x;
-            sh[warp][j][1] = m;
+                for (int q = 0; q < 6; q++) v[2 * j] = norm_add(v[2 * j], x[q]);
+            } else {
+#pragma unroll
+                for (int q = 0; q < 6; q++) cdot_add(v[2 * j], v[2 * j + 1], x[q], y[q]);
+            }
         }
     }
+    __shared__ double sh[8][2 * ND];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int L = 32 / (2 * ND);
+    warp_multi_sum(v);
+    if (lane % L == 0) sh[warp][lane / L] = v[0];
     __syncthreads();
-    if (threadIdx.x < ND) {
-        double x = 0, m = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++) {
-            x += sh[w][threadIdx.x][0];
-            m += sh[w][threadIdx.x][1];
-        }
-        partial[((long)b * nch + c) * ND + threadIdx.x] = make_double2(x, m);
+    if (threadIdx.x < 2 * ND) {
+        double x = 0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); w++) x += sh[w][threadIdx.x];
+        reinterpret_cast<double *>(partial + ((long)b * nch + c) * ND)[threadIdx.x] = x;
     }
 }
 // dots[b*ND + j] = sum over the block's chunks, in order
@@ -383,12 +302,7 @@ struct BlockRun {
     // out_e = Dhat_blk in_e (tmp_o: one odd FP64 half field)
     lqcd_status dhat(const double2 *in, double2 *out, double2 *tmp)
     {
-        const int grid = div_up(c->g.Vh, 128);
-        k_bhop<MODE_DHAT1><<<grid, 128, 0, c->stream>>>(c->g, B, in, nullptr, tmp, c->U64, c->Ai64[1]);
-        k_bhop<MODE_DHAT2><<<grid, 128, 0, c->stream>>>(c->g, B, tmp, in, out, c->U64, c->A64[0]);
-        c->n_kernel_launches += 2;
-        LQCD_LAUNCH_CHECK(c);
-        return LQCD_OK;
+        return launch_dhat_block_d(c, B.bs, in, tmp, out);
     }
     template <int ND>
     lqcd_status bdots(DotSet<ND> d)

@@ -29,6 +29,7 @@ constexpr int HOP_D_THREADS = 128;
 
 struct HopSite {
     int x[4], lex;
+    unsigned keep;   // bit 2 mu + fwd: the hop stays in the site's block
 };
 
 __device__ __forceinline__ double shx(double v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
@@ -49,12 +50,20 @@ __device__ __forceinline__ unsigned sign_mask(bool neg) { return neg ? 0x8000000
 // w = s_bc U h or s_bc U^dag h, s_bc the time-boundary sign.  Signs, factors i
 // and (SENSE = 0: fwd at run time; +1, -1: fixed) the adjoint are selected on
 // the integer side: the FP64 pipe sees 6 + 36 operations.
-template <int SENSE>
+// BLK: a hop out of the site's block gives w = 0 (and no work where no lane of
+// the warp keeps its hop).
+template <int SENSE, bool BLK>
 __device__ __forceinline__ void hop_w(const Geom &g, int p_out, int r, const HopSite &S, int mu, bool fwd_rt, int s,
                                       const double2 *__restrict__ in, const double2 *__restrict__ U, cx<double> w[3])
 {
     const bool fwd = SENSE == 0 ? fwd_rt : SENSE > 0;
     const long Vh = g.Vh;
+    const bool keep = !BLK || (S.keep >> (2 * mu + fwd) & 1);
+    if (BLK && !__any_sync(0xffffffffu, keep)) {
+#pragma unroll
+        for (int c = 0; c < 3; c++) w[c] = mk(0.0, 0.0);
+        return;
+    }
     const bool swap = mu == 1 || mu == 2, imag = mu & 1;
     const int xm = mu == 0 ? S.x[0] : (mu == 1 ? S.x[1] : (mu == 2 ? S.x[2] : S.x[3]));
     const int Lm = mu == 0 ? g.L[0] : (mu == 1 ? g.L[1] : (mu == 2 ? g.L[2] : g.L[3]));
@@ -96,7 +105,10 @@ __device__ __forceinline__ void hop_w(const Geom &g, int p_out, int r, const Hop
         su3dag_vec(m, h, w);
     const unsigned bc = sign_mask(mu == 0 && edge && g.bc_t < 0);
 #pragma unroll
-    for (int c = 0; c < 3; c++) w[c] = mk(flip(bc, w[c].re), flip(bc, w[c].im));
+    for (int c = 0; c < 3; c++) {
+        w[c] = mk(flip(bc, w[c].re), flip(bc, w[c].im));
+        if (BLK && !keep) w[c] = mk(0.0, 0.0);
+    }
 }
 
 // what w adds to the lower spin: sgn e_mu^dag w
@@ -116,23 +128,24 @@ __device__ __forceinline__ void add3(cx<double> a[3], const cx<double> b[3])
 }
 
 // the four hops of kind k (directions ma, mb), forward first
+template <bool BLK>
 __device__ __forceinline__ void hop_kind(const Geom &g, int p_out, int r, const HopSite &S, int ma, int mb, int s,
                                          const double2 *__restrict__ in, const double2 *__restrict__ U,
                                          cx<double> up[3], cx<double> lo[3])
 {
     cx<double> w[3], l[3];
-    hop_w<1>(g, p_out, r, S, ma, true, s, in, U, up);
+    hop_w<1, BLK>(g, p_out, r, S, ma, true, s, in, U, up);
     lower_of(ma, true, s, up, lo);
     auto more = [&](int mu, bool fwd) {
         add3(up, w);
         lower_of(mu, fwd, s, w, l);
         add3(lo, l);
     };
-    hop_w<1>(g, p_out, r, S, mb, true, s, in, U, w);
+    hop_w<1, BLK>(g, p_out, r, S, mb, true, s, in, U, w);
     more(mb, true);
-    hop_w<-1>(g, p_out, r, S, ma, false, s, in, U, w);
+    hop_w<-1, BLK>(g, p_out, r, S, ma, false, s, in, U, w);
     more(ma, false);
-    hop_w<-1>(g, p_out, r, S, mb, false, s, in, U, w);
+    hop_w<-1, BLK>(g, p_out, r, S, mb, false, s, in, U, w);
     more(mb, false);
 }
 
@@ -167,8 +180,12 @@ __device__ __forceinline__ cx<double> herm_row(const double2 *__restrict__ A, lo
 // Modes as in k_hop.  Lane = part * (32 / P) + site, P = 2 G parts per site:
 // part bit 0 is s, bit 1 (G >= 2) the kind k, bit 2 (G = 4) the sense.
 // One-dimensional grid, the fields of a site tile next to each other.
-template <int MODE, int G>
-__global__ void __launch_bounds__(HOP_D_THREADS, 3) k_hop_d(HopArgs<double2, double2, double2> a)
+// BLK: the Dirichlet operator of blocks of extents bs.
+struct BlkExt {
+    int bs[4];
+};
+template <int MODE, int G, bool BLK = false>
+__global__ void __launch_bounds__(HOP_D_THREADS, 3) k_hop_d(HopArgs<double2, double2, double2> a, BlkExt bx)
 {
     constexpr int P = 2 * G, SW = 32 / P;
     after_previous();
@@ -182,6 +199,15 @@ __global__ void __launch_bounds__(HOP_D_THREADS, 3) k_hop_d(HopArgs<double2, dou
     HopSite S;
     rank_coords(a.g, a.p_out, r, S.x);
     S.lex = S.x[3] + a.g.L[3] * (S.x[2] + a.g.L[2] * (S.x[1] + a.g.L[1] * S.x[0]));
+    if (BLK) {
+        S.keep = 0;
+#pragma unroll
+        for (int m = 0; m < 4; m++) {
+            const int L = a.g.L[m], b = bx.bs[m], l = S.x[m] % b;
+            // a block that spans the direction keeps its wrapped hop
+            S.keep |= (unsigned)(l + 1 < b || b == L) << (2 * m + 1) | (unsigned)(l > 0 || b == L) << (2 * m);
+        }
+    }
     const double2 *in = a.in_other + kf * a.in_rs;
     // sums of the hops: up of spin s, lo of the lower spin reached from it; for
     // G = 4 the thread keeps one of the two (up for sense bit 0, lo for 1) in up
@@ -191,8 +217,8 @@ __global__ void __launch_bounds__(HOP_D_THREADS, 3) k_hop_d(HopArgs<double2, dou
     int sl = s;   // the lower spin that lo ends on
     if (G == 4) {
         cx<double> wa[3], wb[3], oa[3], ob[3], l[3];
-        hop_w<0>(a.g, a.p_out, r, S, ma, d0 == 0, s, in, a.U, wa);
-        hop_w<0>(a.g, a.p_out, r, S, mb, d0 == 0, s, in, a.U, wb);
+        hop_w<0, BLK>(a.g, a.p_out, r, S, ma, d0 == 0, s, in, a.U, wa);
+        hop_w<0, BLK>(a.g, a.p_out, r, S, mb, d0 == 0, s, in, a.U, wb);
         shx3(wa, 4 * SW, oa);
         shx3(wb, 4 * SW, ob);
         auto pick = [&](int mu, bool fwd, const cx<double> mine[3], const cx<double> other[3], cx<double> o[3]) {
@@ -221,11 +247,11 @@ __global__ void __launch_bounds__(HOP_D_THREADS, 3) k_hop_d(HopArgs<double2, dou
         add3(up, t);
         sl = k0 ? 1 - s : s;
     } else {
-        hop_kind(a.g, a.p_out, r, S, ma, mb, s, in, a.U, up, lo);
+        hop_kind<BLK>(a.g, a.p_out, r, S, ma, mb, s, in, a.U, up, lo);
         cx<double> t[3];
         if (G == 1) {
             cx<double> u1[3], l1[3];
-            hop_kind(a.g, a.p_out, r, S, 1, 2, s, in, a.U, u1, l1);
+            hop_kind<BLK>(a.g, a.p_out, r, S, 1, 2, s, in, a.U, u1, l1);
             add3(up, u1);
             shx3(l1, SW, t);   // kind 1 of thread 1 - s ends on lower spin s
             add3(lo, t);
@@ -293,8 +319,9 @@ __global__ void __launch_bounds__(HOP_D_THREADS, 3) k_hop_d(HopArgs<double2, dou
 
 }  // namespace
 
-template <int MODE>
-lqcd_status launch_hop_d(lqcd_ctx *c, int G, const HopArgs<double2, double2, double2> &a)
+namespace {
+template <int MODE, bool BLK>
+lqcd_status launch_d(lqcd_ctx *c, int G, const HopArgs<double2, double2, double2> &a, BlkExt bx)
 {
     const int sites = HOP_D_THREADS / (2 * G);   // per CTA
     const long nb = (long)div_up(c->g.Vh, sites) * a.nrhs;
@@ -303,14 +330,45 @@ lqcd_status launch_hop_d(lqcd_ctx *c, int G, const HopArgs<double2, double2, dou
     const bool pdl = !c->capturing;
     cudaError_t e = cudaSuccess;
     switch (G) {
-        case 1: e = launch_pdl(pdl, k_hop_d<MODE, 1>, grid, HOP_D_THREADS, c->stream, a); break;
-        case 2: e = launch_pdl(pdl, k_hop_d<MODE, 2>, grid, HOP_D_THREADS, c->stream, a); break;
-        case 4: e = launch_pdl(pdl, k_hop_d<MODE, 4>, grid, HOP_D_THREADS, c->stream, a); break;
+        case 1: e = launch_pdl(pdl, k_hop_d<MODE, 1, BLK>, grid, HOP_D_THREADS, c->stream, a, bx); break;
+        case 2: e = launch_pdl(pdl, k_hop_d<MODE, 2, BLK>, grid, HOP_D_THREADS, c->stream, a, bx); break;
+        case 4: e = launch_pdl(pdl, k_hop_d<MODE, 4, BLK>, grid, HOP_D_THREADS, c->stream, a, bx); break;
         default: return set_err(c, LQCD_ERR_ARG, "FP64 stencil: split %d", G);
     }
     c->n_kernel_launches++;
     LQCD_CUDA_CHECK(c, e);
     return LQCD_OK;
+}
+}  // namespace
+
+template <int MODE>
+lqcd_status launch_hop_d(lqcd_ctx *c, int G, const HopArgs<double2, double2, double2> &a)
+{
+    return launch_d<MODE, false>(c, G, a, BlkExt{});
+}
+
+lqcd_status launch_dhat_block_d(lqcd_ctx *c, const int bs[4], const double2 *in, double2 *tmp, double2 *out)
+{
+    HopArgs<double2, double2, double2> a;
+    a.g = c->g;
+    a.nrhs = 1;
+    a.in_rs = a.same_rs = a.out_rs = 0;
+    a.U = c->U64;
+    const BlkExt bx = {{bs[0], bs[1], bs[2], bs[3]}};
+    // as the untuned rule of the lattice-wide operator
+    const int G = c->g.Vh >= 16 * 1216 ? 1 : (c->g.Vh >= 16 * 608 ? 2 : 4);
+    a.p_out = 1;
+    a.in_other = in;
+    a.in_same = nullptr;
+    a.out = tmp;
+    a.clov = c->Ai64[1];
+    LQCD_TRY((launch_d<MODE_DHAT1, true>(c, G, a, bx)));
+    a.p_out = 0;
+    a.in_other = tmp;
+    a.in_same = in;
+    a.out = out;
+    a.clov = c->A64[0];
+    return launch_d<MODE_DHAT2, true>(c, G, a, bx);
 }
 
 template lqcd_status launch_hop_d<MODE_HOP>(lqcd_ctx *, int, const HopArgs<double2, double2, double2> &);

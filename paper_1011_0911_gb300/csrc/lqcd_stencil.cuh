@@ -396,6 +396,8 @@ inline int var_sm_max_threads(int v) { return v == 2 ? 256 : 384; }
 // FP64 form (lqcd_dirac_d.cu): 2 G threads per site, G = 1, 2, 4; every mode
 template <int MODE>
 lqcd_status launch_hop_d(lqcd_ctx *c, int G, const HopArgs<double2, double2, double2> &a);
+// out_e = Dhat_blk in_e on Dirichlet blocks of extents bs (tmp: an odd half field)
+lqcd_status launch_dhat_block_d(lqcd_ctx *c, const int bs[4], const double2 *in, double2 *tmp, double2 *out);
 // kernel forms known to the autotuner
 enum { KIND_HOP = 0, KIND_MR = 1, KIND_SM = 2, KIND_D = 3 };
 
