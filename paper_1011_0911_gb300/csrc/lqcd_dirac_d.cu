@@ -185,10 +185,12 @@ struct BlkExt {
     int bs[4];
 };
 template <int MODE, int G, bool BLK = false>
-__global__ void __launch_bounds__(HOP_D_THREADS, 3) k_hop_d(HopArgs<double2, double2, double2> a, BlkExt bx)
+__global__ void __launch_bounds__(HOP_D_THREADS, 3) k_hop_d(const HopArgs<double2, double2, double2> args,
+                                                            BlkExt bx)
 {
     constexpr int P = 2 * G, SW = 32 / P;
     after_previous();
+    const HopArgs<double2, double2, double2> a = hop_args<MODE>(args);
     const long Vh = a.g.Vh;
     const int kf = blockIdx.x % a.nrhs;
     const int lane = threadIdx.x & 31, part = lane / SW, s = part & 1;
@@ -326,7 +328,7 @@ lqcd_status launch_d(lqcd_ctx *c, int G, const HopArgs<double2, double2, double2
     const int sites = HOP_D_THREADS / (2 * G);   // per CTA
     const long nb = (long)div_up(c->g.Vh, sites) * a.nrhs;
     if (nb > 0x7fffffffL) return set_err(c, LQCD_ERR_ARG, "FP64 stencil: grid of %ld CTAs", nb);
-    const int grid = (int)nb;
+    const dim3 grid((unsigned)nb, hop_grid_y<MODE>());
     const bool pdl = !c->capturing;
     cudaError_t e = cudaSuccess;
     switch (G) {
@@ -349,7 +351,7 @@ lqcd_status launch_hop_d(lqcd_ctx *c, int G, const HopArgs<double2, double2, dou
 
 lqcd_status launch_dhat_block_d(lqcd_ctx *c, const int bs[4], const double2 *in, double2 *tmp, double2 *out)
 {
-    HopArgs<double2, double2, double2> a;
+    HopArgs<double2, double2, double2> a = {};
     a.g = c->g;
     a.nrhs = 1;
     a.in_rs = a.same_rs = a.out_rs = 0;

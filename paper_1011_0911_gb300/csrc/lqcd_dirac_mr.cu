@@ -99,8 +99,10 @@ struct VarMR<2> {
 // all field groups of a site tile run next to each other and share its links
 // and clover term through L1/L2.
 template <class R, class SP, class LK, class CL, int MODE, int NR, int VAR>
-__global__ void __launch_bounds__(VarMR<VAR>::T, VarMR<VAR>::B) k_hop_mr(HopArgs<SP, LK, CL> a, int ngy)
+__global__ void __launch_bounds__(VarMR<VAR>::T, VarMR<VAR>::B) k_hop_mr(const HopArgs<SP, LK, CL> args, int ngy)
 {
+    after_previous();
+    const HopArgs<SP, LK, CL> a = hop_args<MODE>(args);
     const int gy = blockIdx.x % ngy, tile = blockIdx.x / ngy;
     const int r = tile * blockDim.x + threadIdx.x;
     const int k0 = (gy * blockDim.y + threadIdx.y) * NR;
@@ -181,12 +183,12 @@ __global__ void __launch_bounds__(VarMR<VAR>::T, VarMR<VAR>::B) k_hop_mr(HopArgs
 }
 
 template <class R, class SP, class LK, class CL, int MODE, int NR>
-void launch_nr(int var, int grid, dim3 b, int ngy, cudaStream_t st, const HopArgs<SP, LK, CL> &a)
+cudaError_t launch_nr(bool pdl, int var, dim3 grid, dim3 b, int ngy, cudaStream_t st, const HopArgs<SP, LK, CL> &a)
 {
     switch (var) {
-        case 0: k_hop_mr<R, SP, LK, CL, MODE, NR, 0><<<grid, b, 0, st>>>(a, ngy); break;
-        case 1: k_hop_mr<R, SP, LK, CL, MODE, NR, 1><<<grid, b, 0, st>>>(a, ngy); break;
-        default: k_hop_mr<R, SP, LK, CL, MODE, NR, 2><<<grid, b, 0, st>>>(a, ngy); break;
+        case 0: return launch_pdl(pdl, k_hop_mr<R, SP, LK, CL, MODE, NR, 0>, grid, b, st, a, ngy);
+        case 1: return launch_pdl(pdl, k_hop_mr<R, SP, LK, CL, MODE, NR, 1>, grid, b, st, a, ngy);
+        default: return launch_pdl(pdl, k_hop_mr<R, SP, LK, CL, MODE, NR, 2>, grid, b, st, a, ngy);
     }
 }
 
@@ -199,14 +201,16 @@ lqcd_status launch_hop_mr(lqcd_ctx *c, int nr, int var, dim3 b, const HopArgs<SP
     const int ngy = div_up(groups, b.y);
     const long grid = (long)div_up(c->g.Vh, b.x) * ngy;
     if (grid > 0x7fffffffL) return set_err(c, LQCD_ERR_ARG, "blocked stencil: grid of %ld CTAs", grid);
+    const dim3 g((unsigned)grid, hop_grid_y<MODE>());
+    cudaError_t e;
     if (nr == 2)
-        launch_nr<R, SP, LK, CL, MODE, 2>(var, (int)grid, b, ngy, c->stream, a);
+        e = launch_nr<R, SP, LK, CL, MODE, 2>(!c->capturing, var, g, b, ngy, c->stream, a);
     else if (nr == 3)
-        launch_nr<R, SP, LK, CL, MODE, 3>(var, (int)grid, b, ngy, c->stream, a);
+        e = launch_nr<R, SP, LK, CL, MODE, 3>(!c->capturing, var, g, b, ngy, c->stream, a);
     else
         return set_err(c, LQCD_ERR_ARG, "no blocked stencil for %d fields per thread", nr);
     c->n_kernel_launches++;
-    LQCD_LAUNCH_CHECK(c);
+    LQCD_CUDA_CHECK(c, e);
     return LQCD_OK;
 }
 

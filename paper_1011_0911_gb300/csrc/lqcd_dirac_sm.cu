@@ -119,8 +119,10 @@ struct VarSM<2> {
 };
 
 template <class SP, class LK, class CL, int MODE, int TS, int VAR>
-__global__ void __launch_bounds__(VarSM<VAR>::T, VarSM<VAR>::B) k_hop_sm(HopArgs<SP, LK, CL> a, int ngy)
+__global__ void __launch_bounds__(VarSM<VAR>::T, VarSM<VAR>::B) k_hop_sm(const HopArgs<SP, LK, CL> args, int ngy)
 {
+    after_previous();
+    const HopArgs<SP, LK, CL> a = hop_args<MODE>(args);
     __shared__ SmStage<TS> S;
     const long Vh = a.g.Vh;
     // one-dimensional grid, the field blocks of a site tile next to each other
@@ -190,12 +192,12 @@ __global__ void __launch_bounds__(VarSM<VAR>::T, VarSM<VAR>::B) k_hop_sm(HopArgs
 }
 
 template <class SP, class LK, class CL, int MODE, int TS>
-void launch_ts(int var, int grid, dim3 b, int ngy, cudaStream_t st, const HopArgs<SP, LK, CL> &a)
+cudaError_t launch_ts(bool pdl, int var, dim3 grid, dim3 b, int ngy, cudaStream_t st, const HopArgs<SP, LK, CL> &a)
 {
     switch (var) {
-        case 0: k_hop_sm<SP, LK, CL, MODE, TS, 0><<<grid, b, 0, st>>>(a, ngy); break;
-        case 1: k_hop_sm<SP, LK, CL, MODE, TS, 1><<<grid, b, 0, st>>>(a, ngy); break;
-        default: k_hop_sm<SP, LK, CL, MODE, TS, 2><<<grid, b, 0, st>>>(a, ngy); break;
+        case 0: return launch_pdl(pdl, k_hop_sm<SP, LK, CL, MODE, TS, 0>, grid, b, st, a, ngy);
+        case 1: return launch_pdl(pdl, k_hop_sm<SP, LK, CL, MODE, TS, 1>, grid, b, st, a, ngy);
+        default: return launch_pdl(pdl, k_hop_sm<SP, LK, CL, MODE, TS, 2>, grid, b, st, a, ngy);
     }
 }
 
@@ -207,14 +209,16 @@ lqcd_status launch_hop_sm(lqcd_ctx *c, int var, dim3 b, const HopArgs<SP, LK, CL
     const int ngy = div_up(a.nrhs, b.y);
     const long nb = (long)div_up(c->g.Vh, b.x) * ngy;
     if (nb > 0x7fffffffL) return set_err(c, LQCD_ERR_ARG, "staged stencil: grid of %ld CTAs", nb);
+    const dim3 g((unsigned)nb, hop_grid_y<MODE>());
+    cudaError_t e;
     if (b.x == 16)
-        launch_ts<SP, LK, CL, MODE, 16>(var, (int)nb, b, ngy, c->stream, a);
+        e = launch_ts<SP, LK, CL, MODE, 16>(!c->capturing, var, g, b, ngy, c->stream, a);
     else if (b.x == 32)
-        launch_ts<SP, LK, CL, MODE, 32>(var, (int)nb, b, ngy, c->stream, a);
+        e = launch_ts<SP, LK, CL, MODE, 32>(!c->capturing, var, g, b, ngy, c->stream, a);
     else
         return set_err(c, LQCD_ERR_ARG, "staged stencil: tile of %d sites", (int)b.x);
     c->n_kernel_launches++;
-    LQCD_LAUNCH_CHECK(c);
+    LQCD_CUDA_CHECK(c, e);
     return LQCD_OK;
 }
 

@@ -379,7 +379,28 @@ struct HopArgs {
     long out_rs;
     const LK *U;
     const CL *clov;   // parity p_out: A^-1 (DHAT1) or A (DHAT2, D)
+    // MODE_D writes both parities in one launch: the members above are output
+    // parity 0 (blockIdx.y = 0), these parity 1
+    const SP *in_other1, *in_same1;
+    SP *out1;
+    const CL *clov1;
 };
+// the arguments of this CTA's output parity
+template <int MODE, class SP, class LK, class CL>
+__device__ __forceinline__ HopArgs<SP, LK, CL> hop_args(const HopArgs<SP, LK, CL> &a)
+{
+    HopArgs<SP, LK, CL> b = a;
+    if (MODE == MODE_D && blockIdx.y) {
+        b.p_out = 1;
+        b.in_other = a.in_other1;
+        b.in_same = a.in_same1;
+        b.out = a.out1;
+        b.clov = a.clov1;
+    }
+    return b;
+}
+template <int MODE>
+constexpr int hop_grid_y() { return MODE == MODE_D ? 2 : 1; }
 
 // register-blocked form (lqcd_dirac_mr.cu): nr = 2 fields per thread,
 // occupancy variant var (0..2); float arithmetic, modes DHAT1 / DHAT2 / D
