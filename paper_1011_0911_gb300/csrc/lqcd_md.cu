@@ -399,9 +399,8 @@ __device__ __forceinline__ M3 om_at(const Geom &g, const double2 *__restrict__ O
 // M = (c_sw / 4) U sum_nu (+-) W: 14 products a plane and 43 a link where the
 // sum over (order, leaf, place) took 288.  Om is nonzero on one parity only in
 // the log det force: SEL = 1 (the parity of x) and SEL = 2 (the other one) leave
-// out the products with zero.  Measured at 32 x 16^3: loading the field, the
-// clover term and the three forces 116.5 -> 14.1 ms (two of these kernels took
-// 105 ms of it).
+// out the products with zero.  Measured at 32 x 16^3: 52.7 -> 4.29 ms (SEL = 0;
+// floor of the FP64 pipe 3.9), log det 52.7 -> 1.80 + 1.51 ms.
 template <int SEL>
 __global__ void __launch_bounds__(64) k_force_clover(Geom g, const double2 *__restrict__ U,
                                                      const double2 *__restrict__ Om, double coef, double *gout,
