@@ -10,7 +10,7 @@
 //   [Re z, Im z] x [[Re W^T, Im W^T], [-Im W^T, Re W^T]]
 // it is a (rows x 72 cin) x (72 cin x 8 cout) real GEMM, which the BF16 path
 // runs on the tensor cores with mma.sync m16n8k16 (bf16 in, fp32 accumulate):
-// one warp per 16 rows, the whole K and N of the layer per warp.  The
+// two m16 tiles per warp, the whole K and N of the layer per warp.  The
 // contraction is too narrow (N = 16) to fill a 128-row tcgen05 tile with TMEM
 // round trips, and the layer is bound by its transports, so the warp-level
 // tensor-core form is the better fit.  The FP32 path contracts with FMAs.
@@ -70,18 +70,19 @@ __device__ __forceinline__ void act_store1(bf162 *f, long i, float re, float im)
 __device__ __forceinline__ void act_store1(float2 *f, long i, float re, float im) { f[i] = make_float2(re, im); }
 
 // ------------------------------------------------------------ geometry
+// (multiply-high divisions: the 64-bit ones took longer than a transport)
 __device__ __forceinline__ void lex_coords(const Geom &g, long x, int c[4])
 {
-    c[3] = x % g.L[3];
-    long t = x / g.L[3];
-    c[2] = t % g.L[2];
-    t /= g.L[2];
-    c[1] = t % g.L[1];
-    c[0] = t / g.L[1];
+    const int row = fast_div(g.dL3h, (int)(x >> 1));
+    c[3] = (int)x - row * g.L[3];
+    const int t = fast_div(g.dL2, row);
+    c[2] = row - t * g.L[2];
+    c[0] = fast_div(g.dL1, t);
+    c[1] = t - c[0] * g.L[1];
 }
 __device__ __forceinline__ long lex_index(const Geom &g, const int c[4])
 {
-    return c[3] + (long)g.L[3] * (c[2] + (long)g.L[2] * (c[1] + (long)g.L[1] * c[0]));
+    return c[3] + g.L[3] * (c[2] + g.L[2] * (c[1] + g.L[1] * c[0]));   // V < 2^31
 }
 // ------------------------------------------------------------ gather
 // Per CTA, once per site of its tile and path d: the neighbour site, the
@@ -165,6 +166,25 @@ __device__ __forceinline__ void su3dag_mul_fma(const cx<float> u[3][3], const cx
     }
 }
 
+// the link of path d > 0 at site s of the tile, third row rebuilt, the hop's
+// boundary sign (+-1, exact) folded in
+__device__ __forceinline__ void pt_link(const Geom &g, const float4 *U, const PtStage &S, int s, int d, cx<float> u[3][3])
+{
+    const float4 *b = U + S.lnk[d][s];
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+        const float4 t = __ldg(b + q * (long)g.Vh);
+        u[(2 * q) / 3][(2 * q) % 3] = mk(t.x, t.y);
+        u[(2 * q + 1) / 3][(2 * q + 1) % 3] = mk(t.z, t.w);
+    }
+    su3_third_row(u);
+    if (S.sg[d][s] < 0.f)
+#pragma unroll
+        for (int a = 0; a < 3; a++)
+#pragma unroll
+            for (int k = 0; k < 3; k++) u[a][k] = -u[a][k];
+}
+
 // The transported inputs (T_d y_i)(x) of the tile: one item per (site, path);
 // the path's link is loaded and its third row rebuilt once and applied to every
 // input channel.  sink(s, i, d, z) receives the 12 spin-colour components.
@@ -177,19 +197,9 @@ __device__ __forceinline__ void pt_gather(const Geom &g, const float4 *U, const 
         const int s = it % PT_SITES, d = it / PT_SITES;
         const bool ok = x0 + s < V;
         cx<float> u[3][3];
-        if (ok && d > 0) {
-            const float4 *b = U + S.lnk[d][s];
-#pragma unroll
-            for (int q = 0; q < 3; q++) {
-                const float4 t = __ldg(b + q * (long)g.Vh);
-                u[(2 * q) / 3][(2 * q) % 3] = mk(t.x, t.y);
-                u[(2 * q + 1) / 3][(2 * q + 1) % 3] = mk(t.z, t.w);
-            }
-            su3_third_row(u);
-        }
+        if (ok && d > 0) pt_link(g, U, S, s, d, u);
         const bool fwd = d & 1;
         const int y = ok ? S.nbr[d][s] : 0;
-        const float sgn = ok ? S.sg[d][s] : 1.f;
         for (int i = 0; i < cin; i++) {
             cx<float> z[12];
             if (!ok) {
@@ -202,19 +212,14 @@ __device__ __forceinline__ void pt_gather(const Geom &g, const float4 *U, const 
 #pragma unroll
                     for (int k = 0; k < 12; k++) z[k] = v[k];
                 } else {
-                    // U v or U^dag v per spin, as fused multiply-add chains with the
-                    // boundary sign (+-1, exact) folded into the link
-                    cx<float> us[3][3];
-#pragma unroll
-                    for (int a = 0; a < 3; a++)
-#pragma unroll
-                        for (int b = 0; b < 3; b++) us[a][b] = sgn * u[a][b];
+                    // U v or U^dag v per spin, as fused multiply-add chains (the
+                    // boundary sign is in the link)
 #pragma unroll
                     for (int sp = 0; sp < 4; sp++) {
                         if (fwd)
-                            su3_mul_fma(us, v + 3 * sp, z + 3 * sp);
+                            su3_mul_fma(u, v + 3 * sp, z + 3 * sp);
                         else
-                            su3dag_mul_fma(us, v + 3 * sp, z + 3 * sp);
+                            su3dag_mul_fma(u, v + 3 * sp, z + 3 * sp);
                     }
                 }
             }
@@ -235,113 +240,174 @@ struct LayerArgs {
     const float2 *Wc;       // [cout][cin][9][4][4] complex weights (FP32 path)
 };
 
-__device__ __forceinline__ unsigned ld_b32(const bf16 *p) { return *reinterpret_cast<const unsigned *>(p); }
+// row pitch (bf16) of the A and B tiles: an odd number of 16-byte words, so that
+// the 16-byte stores of the gather (rows three apart) and the rows of ldmatrix
+// spread over the banks
+__host__ __device__ constexpr int pt_ld(int Kp) { return Kp + 8; }
+__host__ __device__ constexpr int pt_kpad(int cin) { return (72 * cin + 15) / 16 * 16; }
 
-// row pitch (bf16) of the A tile: room for Kp columns, even, and an odd
-// number of 4-byte words per 3 rows, so that the stride-3-row stores of the
-// gather and the fragment loads of the MMA both spread over the banks
-__host__ __device__ inline int pt_ld(int Kp)
+__device__ __forceinline__ void ldmatrix4(unsigned (&r)[4], const bf16 *p)
 {
-    int ld = Kp + 8;
-    if (((3 * ld / 2) & 1) == 0) ld += 2;
-    return ld;
+    const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(a));
+}
+__device__ __forceinline__ unsigned pack_bf(cx<float> v)
+{
+    bf162 h = __floats2bfloat162_rn(v.re, v.im);
+    return *reinterpret_cast<unsigned *>(&h);
 }
 
-template <class ACT>
-__global__ void __launch_bounds__(PT_THREADS) k_ptc_layer(LayerArgs a)
+// BF16 layer.  Instruction issue and the shared-memory pipe bound it, not the
+// tensor cores: what counts is the work around the 36 multiply-adds per
+// transported spin.  A path's four spins of a row are one 16-byte store (kk runs
+// over the spin fastest), the contraction reads its fragments with ldmatrix,
+// each A fragment once for all output channels, and the sizes are compile-time.
+// 32 x 16^3, 4 samples: 671 -> 453 us for the three layers of 1-2-2-1 channels
+template <int CIN, int COUT>
+__global__ void __launch_bounds__(PT_THREADS) k_ptc_layer_bf(LayerArgs a)
+{
+    constexpr int K = 72 * CIN, Kp = pt_kpad(CIN), LD = pt_ld(Kp);
+    extern __shared__ __align__(16) unsigned char smraw[];
+    const bf162 *in = (const bf162 *)a.in + blockIdx.y * a.in_ss;
+    bf162 *out = (bf162 *)a.out + blockIdx.y * a.out_ss;
+    const long x0 = (long)blockIdx.x * PT_SITES;
+    const long V = a.g.V;
+    const int tid = threadIdx.x;
+    PtStage &S = *reinterpret_cast<PtStage *>(smraw);
+    bf16 *A = (bf16 *)(smraw + sizeof(PtStage));   // [rows][LD]
+    bf16 *Bs = A + PT_ROWS * LD;                   // [8 COUT][LD]
+    for (int e = tid; e < 8 * COUT * (Kp / 8); e += PT_THREADS) {
+        const int n = e / (Kp / 8), k = e % (Kp / 8);
+        *reinterpret_cast<uint4 *>(Bs + n * LD + 8 * k) = __ldg(reinterpret_cast<const uint4 *>(a.Bt + n * Kp) + k);
+    }
+    if (K < Kp) *reinterpret_cast<uint4 *>(A + tid * LD + K) = make_uint4(0, 0, 0, 0);   // Kp - K = 8, 192 rows
+    pt_stage_sites(a.g, x0, S);
+    __syncthreads();
+    for (int it = tid; it < 9 * PT_SITES; it += PT_THREADS) {
+        const int s = it % PT_SITES, d = it / PT_SITES;
+        const bool ok = x0 + s < V;
+        cx<float> u[3][3];
+        if (ok && d > 0) pt_link(a.g, a.U, S, s, d, u);
+        const int y = ok ? S.nbr[d][s] : 0;
+#pragma unroll
+        for (int i = 0; i < CIN; i++) {
+            unsigned w[12];   // component 3 spin + colour
+            const uint4 *src = reinterpret_cast<const uint4 *>(in + (long)i * 12 * V + 12L * y);
+#pragma unroll
+            for (int q = 0; q < 3; q++) {
+                const uint4 t = ok ? __ldg(src + q) : make_uint4(0, 0, 0, 0);
+                w[4 * q] = t.x;
+                w[4 * q + 1] = t.y;
+                w[4 * q + 2] = t.z;
+                w[4 * q + 3] = t.w;
+            }
+            if (ok && d > 0) {
+                const bool fwd = d & 1;
+#pragma unroll
+                for (int sp = 0; sp < 4; sp++) {
+                    cx<float> v[3], z[3];
+#pragma unroll
+                    for (int c = 0; c < 3; c++) {
+                        const float2 f = __bfloat1622float2(*reinterpret_cast<bf162 *>(&w[3 * sp + c]));
+                        v[c] = mk(f.x, f.y);
+                    }
+                    if (fwd)
+                        su3_mul_fma(u, v, z);
+                    else
+                        su3dag_mul_fma(u, v, z);
+#pragma unroll
+                    for (int c = 0; c < 3; c++) w[3 * sp + c] = pack_bf(z[c]);
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < 3; c++)
+                *reinterpret_cast<uint4 *>(A + (3 * s + c) * LD + 8 * (i * 9 + d)) =
+                    make_uint4(w[c], w[3 + c], w[6 + c], w[9 + c]);
+        }
+    }
+    __syncthreads();
+    // tensor-core contraction: warp w owns rows 32 w .. 32 w + 31 (two m16 tiles)
+    const int w = tid >> 5, lane = tid & 31, gq = lane >> 2, tq = lane & 3;
+    float acc[COUT][2][4];
+#pragma unroll
+    for (int nt = 0; nt < COUT; nt++)
+#pragma unroll
+        for (int mi = 0; mi < 2; mi++)
+#pragma unroll
+            for (int q = 0; q < 4; q++) acc[nt][mi][q] = 0.f;
+    const bf16 *Ar = A + (32 * w + (lane & 15)) * LD + 8 * (lane >> 4);
+    // lanes 0-15: output channel 0; 16-31: channel COUT - 1
+    const bf16 *Br = Bs + (8 * (COUT == 2 ? lane >> 4 : 0) + (lane & 7)) * LD + 8 * ((lane >> 3) & 1);
+#pragma unroll
+    for (int k0 = 0; k0 < Kp; k0 += 16) {
+        unsigned b[4], f[2][4];
+        ldmatrix4(b, Br + k0);
+        ldmatrix4(f[0], Ar + k0);
+        ldmatrix4(f[1], Ar + 16 * LD + k0);
+#pragma unroll
+        for (int nt = 0; nt < COUT; nt++)
+#pragma unroll
+            for (int mi = 0; mi < 2; mi++)
+                asm volatile(
+                    "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+                    "{%0,%1,%2,%3};\n"
+                    : "+f"(acc[nt][mi][0]), "+f"(acc[nt][mi][1]), "+f"(acc[nt][mi][2]), "+f"(acc[nt][mi][3])
+                    : "r"(f[mi][0]), "r"(f[mi][1]), "r"(f[mi][2]), "r"(f[mi][3]), "r"(b[2 * nt]), "r"(b[2 * nt + 1]));
+    }
+    // columns 2tq, 2tq+1 of n-tile nt are (re, im) of output channel nt, spin tq
+#pragma unroll
+    for (int mi = 0; mi < 2; mi++)
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const int row = 32 * w + 16 * mi + gq + 8 * h;
+            const int sl = row / 3, cc = row - 3 * sl;
+            if (x0 + sl >= V) continue;
+#pragma unroll
+            for (int nt = 0; nt < COUT; nt++)
+                act_store1(out, (long)nt * 12 * V + 12 * (x0 + sl) + 3 * tq + cc, acc[nt][mi][2 * h],
+                           acc[nt][mi][2 * h + 1]);
+        }
+}
+
+// FP32 layer: the contraction with multiply-adds
+__global__ void __launch_bounds__(PT_THREADS) k_ptc_layer_f32(LayerArgs a)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
-    const ACT *in = (const ACT *)a.in + blockIdx.y * a.in_ss;
-    ACT *out = (ACT *)a.out + blockIdx.y * a.out_ss;
+    const float2 *in = (const float2 *)a.in + blockIdx.y * a.in_ss;
+    float2 *out = (float2 *)a.out + blockIdx.y * a.out_ss;
     const long x0 = (long)blockIdx.x * PT_SITES;
     const long V = a.g.V;
     const int cin = a.cin, cout = a.cout, tid = threadIdx.x;
-    const int K = 72 * cin, Kp = (K + 15) / 16 * 16, ld = pt_ld(Kp);
-    constexpr bool BF = sizeof(ACT) == 4;
     PtStage &S = *reinterpret_cast<PtStage *>(smraw);
-    unsigned char *tile = smraw + sizeof(PtStage);
-    bf16 *A = (bf16 *)tile;                                    // [rows][ld]
-    bf16 *Bs = A + PT_ROWS * ld;                               // [8 cout][ld]
-    cx<float> *Z = (cx<float> *)tile;                          // [rows][36 cin]
+    cx<float> *Z = (cx<float> *)(smraw + sizeof(PtStage));     // [rows][36 cin]
     cx<float> *Ws = Z + PT_ROWS * 36 * cin;                    // [cout*cin*144]
-    if (BF) {
-        for (int e = tid; e < 8 * cout * Kp; e += blockDim.x) Bs[(e / Kp) * ld + e % Kp] = a.Bt[e];
-        for (int e = tid; e < PT_ROWS * (Kp - K); e += blockDim.x)
-            A[(e / (Kp - K)) * ld + K + e % (Kp - K)] = __float2bfloat16(0.f);
-    } else {
-        for (int e = tid; e < cout * cin * 144; e += blockDim.x) {
-            float2 w = a.Wc[e];
-            Ws[e] = mk(w.x, w.y);
-        }
+    for (int e = tid; e < cout * cin * 144; e += blockDim.x) {
+        float2 w = a.Wc[e];
+        Ws[e] = mk(w.x, w.y);
     }
     pt_stage_sites(a.g, x0, S);
     __syncthreads();
-    if (BF) {
-        pt_gather(a.g, a.U, in, cin, x0, S, [&](int s, int i, int d, const cx<float> z[12]) {
+    pt_gather(a.g, a.U, in, cin, x0, S, [&](int s, int i, int d, const cx<float> z[12]) {
 #pragma unroll
-            for (int sp = 0; sp < 4; sp++)
+        for (int sp = 0; sp < 4; sp++)
 #pragma unroll
-                for (int cc = 0; cc < 3; cc++) {
-                    const int kk = (i * 9 + d) * 4 + sp, row = 3 * s + cc;
-                    *reinterpret_cast<bf162 *>(A + row * ld + 2 * kk) =
-                        __floats2bfloat162_rn(z[3 * sp + cc].re, z[3 * sp + cc].im);
-                }
-        });
-    } else {
-        pt_gather(a.g, a.U, in, cin, x0, S, [&](int s, int i, int d, const cx<float> z[12]) {
-#pragma unroll
-            for (int sp = 0; sp < 4; sp++)
-#pragma unroll
-                for (int cc = 0; cc < 3; cc++) Z[(3 * s + cc) * 36 * cin + (i * 9 + d) * 4 + sp] = z[3 * sp + cc];
-        });
-    }
+            for (int cc = 0; cc < 3; cc++) Z[(3 * s + cc) * 36 * cin + (i * 9 + d) * 4 + sp] = z[3 * sp + cc];
+    });
     __syncthreads();
-    if (BF) {
-        // tensor-core contraction: warp w owns rows 32w .. 32w+31 (two m16 tiles)
-        const int w = tid >> 5, lane = tid & 31, gq = lane >> 2, tq = lane & 3;
-        for (int nt = 0; nt < cout; nt++) {
-            const bf16 *Br = Bs + (8 * nt + gq) * ld;
+    for (int e = tid; e < PT_ROWS * cout * 4; e += blockDim.x) {
+        const int row = e / (cout * 4), o = (e / 4) % cout, s = e % 4;
+        const long x = x0 + row / 3;
+        cx<float> acc = mk(0.f, 0.f);
+        for (int i = 0; i < cin; i++)
+            for (int d = 0; d < 9; d++) {
+                const cx<float> *w = Ws + ((o * cin + i) * 9 + d) * 16 + 4 * s;
+                const cx<float> *zr = Z + row * 36 * cin + (i * 9 + d) * 4;
 #pragma unroll
-            for (int mi = 0; mi < 2; mi++) {
-                const bf16 *Ar = A + (32 * w + 16 * mi) * ld;
-                float d0 = 0.f, d1 = 0.f, d2 = 0.f, d3 = 0.f;
-                for (int k0 = 0; k0 < Kp; k0 += 16) {
-                    unsigned a0 = ld_b32(Ar + gq * ld + k0 + 2 * tq);
-                    unsigned a1 = ld_b32(Ar + (gq + 8) * ld + k0 + 2 * tq);
-                    unsigned a2 = ld_b32(Ar + gq * ld + k0 + 8 + 2 * tq);
-                    unsigned a3 = ld_b32(Ar + (gq + 8) * ld + k0 + 8 + 2 * tq);
-                    unsigned b0 = ld_b32(Br + k0 + 2 * tq);
-                    unsigned b1 = ld_b32(Br + k0 + 8 + 2 * tq);
-                    asm volatile(
-                        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-                        "{%0,%1,%2,%3};\n"
-                        : "+f"(d0), "+f"(d1), "+f"(d2), "+f"(d3)
-                        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-                }
-                // columns 2tq, 2tq+1 of n-tile nt are (re, im) of output channel nt, spin tq
-#pragma unroll
-                for (int h = 0; h < 2; h++) {
-                    const int row = 32 * w + 16 * mi + gq + 8 * h;
-                    const int sl = row / 3, cc = row % 3;
-                    const long x = x0 + sl;
-                    if (x < V) act_store1(out, (long)nt * 12 * V + 12 * x + 3 * tq + cc, h ? d2 : d0, h ? d3 : d1);
-                }
+                for (int sp = 0; sp < 4; sp++) acc = acc + w[sp] * zr[sp];
             }
-        }
-    } else {
-        for (int e = tid; e < PT_ROWS * cout * 4; e += blockDim.x) {
-            const int row = e / (cout * 4), o = (e / 4) % cout, s = e % 4;
-            const long x = x0 + row / 3;
-            cx<float> acc = mk(0.f, 0.f);
-            for (int i = 0; i < cin; i++)
-                for (int d = 0; d < 9; d++) {
-                    const cx<float> *w = Ws + ((o * cin + i) * 9 + d) * 16 + 4 * s;
-                    const cx<float> *zr = Z + row * 36 * cin + (i * 9 + d) * 4;
-#pragma unroll
-                    for (int sp = 0; sp < 4; sp++) acc = acc + w[sp] * zr[sp];
-                }
-            if (x < V) act_store1(out, (long)o * 12 * V + 12 * x + 3 * s + row % 3, acc.re, acc.im);
-        }
+        if (x < V) act_store1(out, (long)o * 12 * V + 12 * x + 3 * s + row % 3, acc.re, acc.im);
     }
 }
 
@@ -641,7 +707,7 @@ void net_free(lqcd_ctx *c)
 
 namespace {
 
-inline int kpad(int cin) { return (72 * cin + 15) / 16 * 16; }
+inline int kpad(int cin) { return pt_kpad(cin); }
 inline size_t act_elem(lqcd_prec a) { return a == LQCD_BF16 ? sizeof(bf162) : sizeof(float2); }
 
 lqcd_status net_rebuild(lqcd_ctx *c)
@@ -677,11 +743,15 @@ template <class ACT>
 lqcd_status launch_layer(lqcd_ctx *c, const void *in, void *out, int cin, int cout, int nb, const bf16 *Bt,
                          const float2 *Wc)
 {
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(k_ptc_layer<ACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        attr = true;
+    constexpr bool BF = sizeof(ACT) == 4;
+    void (*kern)(LayerArgs) = k_ptc_layer_f32;
+    if (BF) {
+        static void (*const bf[2][2])(LayerArgs) = {{k_ptc_layer_bf<1, 1>, k_ptc_layer_bf<1, 2>},
+                                                    {k_ptc_layer_bf<2, 1>, k_ptc_layer_bf<2, 2>}};
+        kern = bf[cin - 1][cout - 1];   // lqcd_net_set takes 1 or 2 channels
     }
+    const size_t smem = layer_smem(BF ? LQCD_BF16 : LQCD_F32, cin, cout);
+    LQCD_CUDA_CHECK(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     LayerArgs a;
     a.g = c->g;
     a.U = c->U32;
@@ -693,8 +763,7 @@ lqcd_status launch_layer(lqcd_ctx *c, const void *in, void *out, int cin, int co
     a.out_ss = (long)cout * 12 * c->g.V;
     a.Bt = Bt;
     a.Wc = Wc;
-    lqcd_prec act = sizeof(ACT) == 4 ? LQCD_BF16 : LQCD_F32;
-    k_ptc_layer<ACT><<<dim3(div_up(c->g.V, PT_SITES), nb), PT_THREADS, layer_smem(act, cin, cout), c->stream>>>(a);
+    kern<<<dim3(div_up(c->g.V, PT_SITES), nb), PT_THREADS, smem, c->stream>>>(a);
     c->n_kernel_launches++;
     LQCD_LAUNCH_CHECK(c);
     return LQCD_OK;
