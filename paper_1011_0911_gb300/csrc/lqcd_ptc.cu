@@ -264,14 +264,15 @@ __device__ __forceinline__ unsigned pack_bf(cx<float> v)
 // transported spin.  A path's four spins of a row are one 16-byte store (kk runs
 // over the spin fastest), the contraction reads its fragments with ldmatrix,
 // each A fragment once for all output channels, and the sizes are compile-time.
-// 32 x 16^3, 4 samples: 671 -> 453 us for the three layers of 1-2-2-1 channels
+// A CTA keeps its sites for spc samples: their coordinates, neighbours and the
+// weights are staged once, and the loads of the next path (and sample) are issued
+// before the arithmetic of the current one.
+// 32 x 16^3, 4 samples: 671 -> 372 us for the three layers of 1-2-2-1 channels (453 with one sample per CTA and no prefetch)
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(PT_THREADS) k_ptc_layer_bf(LayerArgs a)
+__global__ void __launch_bounds__(PT_THREADS, CIN == 1 ? 4 : 3) k_ptc_layer_bf(LayerArgs a, int nb, int spc)
 {
     constexpr int K = 72 * CIN, Kp = pt_kpad(CIN), LD = pt_ld(Kp);
     extern __shared__ __align__(16) unsigned char smraw[];
-    const bf162 *in = (const bf162 *)a.in + blockIdx.y * a.in_ss;
-    bf162 *out = (bf162 *)a.out + blockIdx.y * a.out_ss;
     const long x0 = (long)blockIdx.x * PT_SITES;
     const long V = a.g.V;
     const int tid = threadIdx.x;
@@ -285,90 +286,139 @@ __global__ void __launch_bounds__(PT_THREADS) k_ptc_layer_bf(LayerArgs a)
     if (K < Kp) *reinterpret_cast<uint4 *>(A + tid * LD + K) = make_uint4(0, 0, 0, 0);   // Kp - K = 8, 192 rows
     pt_stage_sites(a.g, x0, S);
     __syncthreads();
-    for (int it = tid; it < 9 * PT_SITES; it += PT_THREADS) {
-        const int s = it % PT_SITES, d = it / PT_SITES;
-        const bool ok = x0 + s < V;
-        cx<float> u[3][3];
-        if (ok && d > 0) pt_link(a.g, a.U, S, s, d, u);
-        const int y = ok ? S.nbr[d][s] : 0;
+    // this thread's items: site s, paths d0, d0 + 3, d0 + 6; the loads of the next
+    // path are issued before the arithmetic of the current one
+    static_assert(PT_THREADS == 3 * PT_SITES, "three paths per thread");
+    const int s = tid % PT_SITES, d0 = tid / PT_SITES;
+    const bool ok = x0 + s < V;
+    float4 lk[3];
+    uint4 av[CIN][3];
+    const int b0 = blockIdx.y * spc, b1 = min(nb, b0 + spc);
+    const bf162 *in = (const bf162 *)a.in + b0 * a.in_ss;
+    auto fetch = [&](int d) {
+        if (!ok) return;
+        if (d > 0) {
+            const float4 *p = a.U + S.lnk[d][s];
 #pragma unroll
-        for (int i = 0; i < CIN; i++) {
-            unsigned w[12];   // component 3 spin + colour
-            const uint4 *src = reinterpret_cast<const uint4 *>(in + (long)i * 12 * V + 12L * y);
+            for (int q = 0; q < 3; q++) lk[q] = __ldg(p + q * (long)a.g.Vh);
+        }
+        const int y = S.nbr[d][s];
+#pragma unroll
+        for (int i = 0; i < CIN; i++)
+#pragma unroll
+            for (int q = 0; q < 3; q++)
+                av[i][q] = __ldg(reinterpret_cast<const uint4 *>(in + (long)i * 12 * V + 12L * y) + q);
+    };
+#pragma unroll
+    for (int i = 0; i < CIN; i++)
+#pragma unroll
+        for (int q = 0; q < 3; q++) av[i][q] = make_uint4(0, 0, 0, 0);
+    fetch(d0);
+#pragma unroll 1
+    for (int smp = b0; smp < b1; smp++) {
+        bf162 *out = (bf162 *)a.out + smp * a.out_ss;
+        if (smp > b0) __syncthreads();   // the tile of the sample before has been read
+#pragma unroll 1
+        for (int j = 0; j < 3; j++) {
+            const int d = d0 + 3 * j;
+            cx<float> u[3][3];
+            unsigned w[CIN][12];   // component 3 spin + colour
 #pragma unroll
             for (int q = 0; q < 3; q++) {
-                const uint4 t = ok ? __ldg(src + q) : make_uint4(0, 0, 0, 0);
-                w[4 * q] = t.x;
-                w[4 * q + 1] = t.y;
-                w[4 * q + 2] = t.z;
-                w[4 * q + 3] = t.w;
+                u[(2 * q) / 3][(2 * q) % 3] = mk(lk[q].x, lk[q].y);
+                u[(2 * q + 1) / 3][(2 * q + 1) % 3] = mk(lk[q].z, lk[q].w);
+            }
+#pragma unroll
+            for (int i = 0; i < CIN; i++)
+#pragma unroll
+                for (int q = 0; q < 3; q++) {
+                    w[i][4 * q] = av[i][q].x;
+                    w[i][4 * q + 1] = av[i][q].y;
+                    w[i][4 * q + 2] = av[i][q].z;
+                    w[i][4 * q + 3] = av[i][q].w;
+                }
+            if (j < 2) {
+                fetch(d + 3);
+            } else if (smp + 1 < b1) {
+                in += a.in_ss;
+                fetch(d0);
             }
             if (ok && d > 0) {
+                su3_third_row(u);
+                if (S.sg[d][s] < 0.f)
+#pragma unroll
+                    for (int p = 0; p < 3; p++)
+#pragma unroll
+                        for (int k = 0; k < 3; k++) u[p][k] = -u[p][k];
                 const bool fwd = d & 1;
 #pragma unroll
-                for (int sp = 0; sp < 4; sp++) {
-                    cx<float> v[3], z[3];
+                for (int i = 0; i < CIN; i++)
 #pragma unroll
-                    for (int c = 0; c < 3; c++) {
-                        const float2 f = __bfloat1622float2(*reinterpret_cast<bf162 *>(&w[3 * sp + c]));
-                        v[c] = mk(f.x, f.y);
+                    for (int sp = 0; sp < 4; sp++) {
+                        cx<float> v[3], z[3];
+#pragma unroll
+                        for (int c = 0; c < 3; c++) {
+                            const float2 f = __bfloat1622float2(*reinterpret_cast<bf162 *>(&w[i][3 * sp + c]));
+                            v[c] = mk(f.x, f.y);
+                        }
+                        if (fwd)
+                            su3_mul_fma(u, v, z);
+                        else
+                            su3dag_mul_fma(u, v, z);
+#pragma unroll
+                        for (int c = 0; c < 3; c++) w[i][3 * sp + c] = pack_bf(z[c]);
                     }
-                    if (fwd)
-                        su3_mul_fma(u, v, z);
-                    else
-                        su3dag_mul_fma(u, v, z);
-#pragma unroll
-                    for (int c = 0; c < 3; c++) w[3 * sp + c] = pack_bf(z[c]);
-                }
             }
 #pragma unroll
-            for (int c = 0; c < 3; c++)
-                *reinterpret_cast<uint4 *>(A + (3 * s + c) * LD + 8 * (i * 9 + d)) =
-                    make_uint4(w[c], w[3 + c], w[6 + c], w[9 + c]);
+            for (int i = 0; i < CIN; i++)
+#pragma unroll
+                for (int c = 0; c < 3; c++)
+                    *reinterpret_cast<uint4 *>(A + (3 * s + c) * LD + 8 * (i * 9 + d)) =
+                        make_uint4(w[i][c], w[i][3 + c], w[i][6 + c], w[i][9 + c]);
         }
-    }
-    __syncthreads();
-    // tensor-core contraction: warp w owns rows 32 w .. 32 w + 31 (two m16 tiles)
-    const int w = tid >> 5, lane = tid & 31, gq = lane >> 2, tq = lane & 3;
-    float acc[COUT][2][4];
-#pragma unroll
-    for (int nt = 0; nt < COUT; nt++)
-#pragma unroll
-        for (int mi = 0; mi < 2; mi++)
-#pragma unroll
-            for (int q = 0; q < 4; q++) acc[nt][mi][q] = 0.f;
-    const bf16 *Ar = A + (32 * w + (lane & 15)) * LD + 8 * (lane >> 4);
-    // lanes 0-15: output channel 0; 16-31: channel COUT - 1
-    const bf16 *Br = Bs + (8 * (COUT == 2 ? lane >> 4 : 0) + (lane & 7)) * LD + 8 * ((lane >> 3) & 1);
-#pragma unroll
-    for (int k0 = 0; k0 < Kp; k0 += 16) {
-        unsigned b[4], f[2][4];
-        ldmatrix4(b, Br + k0);
-        ldmatrix4(f[0], Ar + k0);
-        ldmatrix4(f[1], Ar + 16 * LD + k0);
+        __syncthreads();
+        // tensor-core contraction: warp wp owns rows 32 wp .. 32 wp + 31 (two m16 tiles)
+        const int wp = tid >> 5, lane = tid & 31, gq = lane >> 2, tq = lane & 3;
+        float acc[COUT][2][4];
 #pragma unroll
         for (int nt = 0; nt < COUT; nt++)
 #pragma unroll
             for (int mi = 0; mi < 2; mi++)
-                asm volatile(
-                    "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-                    "{%0,%1,%2,%3};\n"
-                    : "+f"(acc[nt][mi][0]), "+f"(acc[nt][mi][1]), "+f"(acc[nt][mi][2]), "+f"(acc[nt][mi][3])
-                    : "r"(f[mi][0]), "r"(f[mi][1]), "r"(f[mi][2]), "r"(f[mi][3]), "r"(b[2 * nt]), "r"(b[2 * nt + 1]));
-    }
-    // columns 2tq, 2tq+1 of n-tile nt are (re, im) of output channel nt, spin tq
 #pragma unroll
-    for (int mi = 0; mi < 2; mi++)
+                for (int q = 0; q < 4; q++) acc[nt][mi][q] = 0.f;
+        const bf16 *Ar = A + (32 * wp + (lane & 15)) * LD + 8 * (lane >> 4);
+        // lanes 0-15: output channel 0; 16-31: channel COUT - 1
+        const bf16 *Br = Bs + (8 * (COUT == 2 ? lane >> 4 : 0) + (lane & 7)) * LD + 8 * ((lane >> 3) & 1);
 #pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const int row = 32 * w + 16 * mi + gq + 8 * h;
-            const int sl = row / 3, cc = row - 3 * sl;
-            if (x0 + sl >= V) continue;
+        for (int k0 = 0; k0 < Kp; k0 += 16) {
+            unsigned b[4], f[2][4];
+            ldmatrix4(b, Br + k0);
+            ldmatrix4(f[0], Ar + k0);
+            ldmatrix4(f[1], Ar + 16 * LD + k0);
 #pragma unroll
             for (int nt = 0; nt < COUT; nt++)
-                act_store1(out, (long)nt * 12 * V + 12 * (x0 + sl) + 3 * tq + cc, acc[nt][mi][2 * h],
-                           acc[nt][mi][2 * h + 1]);
+#pragma unroll
+                for (int mi = 0; mi < 2; mi++)
+                    asm volatile(
+                        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+                        "{%0,%1,%2,%3};\n"
+                        : "+f"(acc[nt][mi][0]), "+f"(acc[nt][mi][1]), "+f"(acc[nt][mi][2]), "+f"(acc[nt][mi][3])
+                        : "r"(f[mi][0]), "r"(f[mi][1]), "r"(f[mi][2]), "r"(f[mi][3]), "r"(b[2 * nt]), "r"(b[2 * nt + 1]));
         }
+        // columns 2tq, 2tq+1 of n-tile nt are (re, im) of output channel nt, spin tq
+#pragma unroll
+        for (int mi = 0; mi < 2; mi++)
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const int row = 32 * wp + 16 * mi + gq + 8 * h;
+                const int sl = row / 3, cc = row - 3 * sl;
+                if (x0 + sl >= V) continue;
+#pragma unroll
+                for (int nt = 0; nt < COUT; nt++)
+                    act_store1(out, (long)nt * 12 * V + 12 * (x0 + sl) + 3 * tq + cc, acc[nt][mi][2 * h],
+                               acc[nt][mi][2 * h + 1]);
+            }
+    }
 }
 
 // FP32 layer: the contraction with multiply-adds
@@ -744,14 +794,15 @@ lqcd_status launch_layer(lqcd_ctx *c, const void *in, void *out, int cin, int co
                          const float2 *Wc)
 {
     constexpr bool BF = sizeof(ACT) == 4;
-    void (*kern)(LayerArgs) = k_ptc_layer_f32;
+    void (*kbf)(LayerArgs, int, int) = nullptr;
     if (BF) {
-        static void (*const bf[2][2])(LayerArgs) = {{k_ptc_layer_bf<1, 1>, k_ptc_layer_bf<1, 2>},
+        static void (*const bf[2][2])(LayerArgs, int, int) = {{k_ptc_layer_bf<1, 1>, k_ptc_layer_bf<1, 2>},
                                                     {k_ptc_layer_bf<2, 1>, k_ptc_layer_bf<2, 2>}};
-        kern = bf[cin - 1][cout - 1];   // lqcd_net_set takes 1 or 2 channels
+        kbf = bf[cin - 1][cout - 1];   // lqcd_net_set takes 1 or 2 channels
     }
     const size_t smem = layer_smem(BF ? LQCD_BF16 : LQCD_F32, cin, cout);
-    LQCD_CUDA_CHECK(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    LQCD_CUDA_CHECK(c, cudaFuncSetAttribute(BF ? (const void *)kbf : (const void *)k_ptc_layer_f32,
+                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     LayerArgs a;
     a.g = c->g;
     a.U = c->U32;
@@ -763,7 +814,14 @@ lqcd_status launch_layer(lqcd_ctx *c, const void *in, void *out, int cin, int co
     a.out_ss = (long)cout * 12 * c->g.V;
     a.Bt = Bt;
     a.Wc = Wc;
-    kern<<<dim3(div_up(c->g.V, PT_SITES), nb), PT_THREADS, smem, c->stream>>>(a);
+    const int tiles = div_up(c->g.V, PT_SITES);
+    if (BF) {
+        // samples per CTA while about four waves of three CTAs per SM remain
+        const int spc = std::max(1, std::min(nb, (int)((long)tiles * nb / (12 * 152))));
+        kbf<<<dim3(tiles, div_up(nb, spc)), PT_THREADS, smem, c->stream>>>(a, nb, spc);
+    } else {
+        k_ptc_layer_f32<<<dim3(tiles, nb), PT_THREADS, smem, c->stream>>>(a);
+    }
     c->n_kernel_launches++;
     LQCD_LAUNCH_CHECK(c);
     return LQCD_OK;
