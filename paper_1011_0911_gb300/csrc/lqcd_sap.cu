@@ -387,6 +387,8 @@ __device__ __forceinline__ void gstore(float4 *f, long Vh, long r, const cx<floa
 }
 __device__ __forceinline__ void gstore(h16s *f, long Vh, long r, const cx<float> v[12]) { f16s_store(f, Vh, r, v); }
 
+constexpr int SAPS_NH = 128;   // sites of one parity per block (4^4 blocks)
+
 template <int P>
 __global__ void __launch_bounds__(128) k_sap_block(SapArgs<P> a)
 {
@@ -521,6 +523,380 @@ __global__ void __launch_bounds__(128) k_sap_block(SapArgs<P> a)
 }
 
 // ------------------------------------------------------------------------
+// FP64 block solve, four threads a site.
+//
+// The FP64 pipe bounds it (2 multiply-adds a clock and SM; operands from shared
+// memory and L2 have ten times the time they need), so the split is the one with
+// the fewest FP64 instructions issued:
+//  - thread group mu takes both hops of direction mu, its sites ordered with x_mu
+//    slowest: for 4^4 blocks a warp is a plane of constant x_mu, so the hops that
+//    leave the block, a quarter of all, are skipped by whole warps;
+//  - the backward product is accumulated on top of the forward one, which gives
+//    the upper spins w+ + w- without an addition and the lower ones as
+//    (w+ + w-) - 2 w+;
+//  - signs and factors i are integer operations on the sign bit;
+//  - each thread then adds the four directions' shares of one spin (group k owns
+//    spin k, through shared memory), applies three rows of the clover block and
+//    does the MinRes updates of its three components; the factor -1/2 of the
+//    hops between the two parities is applied once, at the end (-1/4).
+// All phases are one loop, so that the four directions' code is there once.
+// 32 x 16^3, 256 blocks of 4^4 a launch, 5 steps: 862 us (one thread a site: 1268 us), the FP64
+// pipe 85 % busy on an SM that has a block; 256 blocks on 152 SMs leave a third of
+// the SMs idle in the second half.
+struct SapD {
+    double2 *X, *rho, *to;   // shares [4][12][nh]; block vectors [12][nh]
+    double *red;             // [3][16], then alpha (2) and <p,p>
+};
+constexpr size_t sap_d_smem(int nh) { return (size_t)72 * nh * sizeof(double2) + 51 * sizeof(double); }
+
+__device__ __forceinline__ double flip_if(bool neg, double v)
+{
+    return __hiloint2double(__double2hiint(v) ^ (neg ? 0x80000000 : 0), __double2loint(v));
+}
+__device__ __forceinline__ double minus(double v) { return flip_if(true, v); }
+
+// w += U h (DAG: U^dag h), or w = ... (INIT), for both spins; u points at the
+// link's nine entries, Vh apart
+template <bool DAG, bool INIT>
+__device__ __forceinline__ void d_su3(const double2 *__restrict__ u, long Vh, const cx<double> h[2][3],
+                                      cx<double> w[2][3])
+{
+    double2 m[9];
+#pragma unroll
+    for (int e = 0; e < 9; e++) m[e] = __ldg(u + e * Vh);
+#pragma unroll
+    for (int j = 0; j < 3; j++)
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            const double2 q = DAG ? m[3 * j + i] : m[3 * i + j];
+#pragma unroll
+            for (int s = 0; s < 2; s++) {
+                const cx<double> x = h[s][j];
+                cx<double> &y = w[s][i];
+                y.re = INIT && j == 0 ? q.x * x.re : fmx(q.x, x.re, y.re);
+                y.re = fmx(DAG ? q.y : -q.y, x.im, y.re);
+                y.im = INIT && j == 0 ? q.x * x.im : fmx(q.x, x.im, y.im);
+                y.im = fmx(DAG ? -q.y : q.y, x.re, y.im);
+            }
+        }
+}
+
+// projected neighbour spinor, times the time-boundary sign
+template <int MU, int SGN>
+__device__ __forceinline__ void d_project(const double2 *src, int nh, bool neg, cx<double> h[2][3])
+{
+    stencil::Spinor<double> v;
+#pragma unroll
+    for (int c = 0; c < 12; c++) {
+        const double2 t = src[c * nh];
+        v.s[c / 3][c % 3] = mk(t.x, t.y);
+    }
+    stencil::project<double, MU, SGN>(v, h);
+    if (MU == 0)
+#pragma unroll
+        for (int i = 0; i < 6; i++)
+            h[i / 3][i % 3] = mk(flip_if(neg, h[i / 3][i % 3].re), flip_if(neg, h[i / 3][i % 3].im));
+}
+
+// Share of direction MU in the hop sum (before the -1/2) of one site, into
+// X[MU][.][t].  nf, nb: slots of the neighbours in src, or -1; uf, ub: the links.
+template <int MU>
+__device__ __forceinline__ void d_hops(const double2 *uf, const double2 *ub, long Vh, const double2 *src, int nh,
+                                       int nf, int nb, bool negf, bool negb, double2 *X)
+{
+    cx<double> h[2][3], w[2][3], d[2][3];
+    if (nf >= 0) {
+        d_project<MU, -1>(src + nf, nh, negf, h);
+        d_su3<false, true>(uf, Vh, h, w);
+        if (nb >= 0) {
+            cx<double> f[2][3];
+#pragma unroll
+            for (int i = 0; i < 6; i++) f[i / 3][i % 3] = w[i / 3][i % 3];
+            d_project<MU, 1>(src + nb, nh, negb, h);
+            d_su3<true, false>(ub, Vh, h, w);
+#pragma unroll
+            for (int i = 0; i < 6; i++) {
+                const cx<double> a = f[i / 3][i % 3], b = w[i / 3][i % 3];
+                d[i / 3][i % 3] = mk(fmx(-2.0, a.re, b.re), fmx(-2.0, a.im, b.im));
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 6; i++) {
+                const cx<double> a = w[i / 3][i % 3];
+                d[i / 3][i % 3] = mk(minus(a.re), minus(a.im));
+            }
+        }
+    } else if (nb >= 0) {
+        d_project<MU, 1>(src + nb, nh, negb, h);
+        d_su3<true, true>(ub, Vh, h, w);
+#pragma unroll
+        for (int i = 0; i < 6; i++) d[i / 3][i % 3] = w[i / 3][i % 3];
+    } else {
+#pragma unroll
+        for (int i = 0; i < 6; i++) w[i / 3][i % 3] = d[i / 3][i % 3] = mk(0.0, 0.0);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        const cx<double> a = d[0][c], b = d[1][c];
+        double2 l0, l1;   // e_mu^dag d
+        switch (MU) {
+            case 0:
+                l0 = make_double2(minus(a.re), minus(a.im));
+                l1 = make_double2(minus(b.re), minus(b.im));
+                break;
+            case 1:
+                l0 = make_double2(minus(b.im), b.re);
+                l1 = make_double2(minus(a.im), a.re);
+                break;
+            case 2:
+                l0 = make_double2(b.re, b.im);
+                l1 = make_double2(minus(a.re), minus(a.im));
+                break;
+            default:
+                l0 = make_double2(minus(a.im), a.re);
+                l1 = make_double2(b.im, minus(b.re));
+                break;
+        }
+        X[c * nh] = make_double2(w[0][c].re, w[0][c].im);
+        X[(3 + c) * nh] = make_double2(w[1][c].re, w[1][c].im);
+        X[(6 + c) * nh] = l0;
+        X[(9 + c) * nh] = l1;
+    }
+}
+
+// rows 3 HALF .. 3 HALF + 2 of a packed Hermitian 6x6 block (entries Vh apart)
+// times in[0..5] (nh apart)
+template <int HALF>
+__device__ __forceinline__ void d_rows(const double2 *__restrict__ A, long Vh, const double2 *in, int nh,
+                                       cx<double> out[3])
+{
+    const double2 d0 = __ldg(A + (HALF ? 1 : 0) * Vh), d1 = __ldg(A + (HALF ? 2 : 1) * Vh);
+    const double dg[3] = {HALF ? d0.y : d0.x, HALF ? d1.x : d0.y, HALF ? d1.y : d1.x};
+    cx<double> v[6];
+#pragma unroll
+    for (int i = 0; i < 6; i++) v[i] = mk(in[i * nh].x, in[i * nh].y);
+#pragma unroll
+    for (int i = 0; i < 3; i++) out[i] = mk(dg[i] * v[3 * HALF + i].re, dg[i] * v[3 * HALF + i].im);
+    int k = 3;
+#pragma unroll
+    for (int i = 0; i < 6; i++)
+#pragma unroll
+        for (int j = i + 1; j < 6; j++, k++) {
+            const bool ri = i / 3 == HALF, rj = j / 3 == HALF;
+            if (!ri && !rj) continue;
+            const double2 o = __ldg(A + k * Vh);
+            if (ri) {   // out_i += o v_j
+                cx<double> &y = out[i - 3 * HALF];
+                y.re = fmx(o.x, v[j].re, y.re);
+                y.re = fmx(-o.y, v[j].im, y.re);
+                y.im = fmx(o.x, v[j].im, y.im);
+                y.im = fmx(o.y, v[j].re, y.im);
+            }
+            if (rj) {   // out_j += conj(o) v_i
+                cx<double> &y = out[j - 3 * HALF];
+                y.re = fmx(o.x, v[i].re, y.re);
+                y.re = fmx(o.y, v[i].im, y.re);
+                y.im = fmx(o.x, v[i].im, y.im);
+                y.im = fmx(-o.y, v[i].re, y.im);
+            }
+        }
+}
+
+// Site i (0 .. nh-1) of parity par with x_mu slowest, and its neighbours along mu
+struct SapDSite {
+    int t, rank, nf, nb, rb;   // slot, global rank, neighbours' slots or -1, rank of the backward one
+    bool negf, negb;           // time-boundary sign of the two hops
+};
+__device__ __forceinline__ SapDSite d_site(const Geom &g, const BlkGeom &B, const int org[4], int mu, int par, int i)
+{
+    const int last = mu == 3 ? 2 : 3, hl = B.bs[last] >> 1;   // the direction halved by parity
+    int l[4], r = i / hl, sum = par;
+    const int lh = i - r * hl;
+#pragma unroll
+    for (int m = 3; m >= 0; m--) {
+        if (m == last || m == mu) continue;
+        l[m] = r % B.bs[m];
+        r /= B.bs[m];
+        sum += l[m];
+    }
+    l[mu] = r;
+    l[last] = 2 * lh + ((sum + r) & 1);
+    int x[4];
+#pragma unroll
+    for (int m = 0; m < 4; m++) x[m] = org[m] + l[m];
+    SapDSite s;
+    s.t = (l[3] + B.bs[3] * (l[2] + B.bs[2] * (l[1] + B.bs[1] * l[0]))) >> 1;
+    s.rank = (int)coords_rank(g, x);
+    s.nf = blk_nbr(B, l, mu, 1);
+    s.nb = blk_nbr(B, l, mu, -1);
+    s.negf = mu == 0 && x[0] == g.L[0] - 1 && g.bc_t < 0;
+    s.negb = mu == 0 && x[0] == 0 && g.bc_t < 0;
+    x[mu] = x[mu] == 0 ? g.L[mu] - 1 : x[mu] - 1;
+    s.rb = (int)coords_rank(g, x);
+    return s;
+}
+
+__global__ void __launch_bounds__(4 * SAPS_NH, 1) k_sap_block_d(SapArgs<LQCD_F64> a)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const BlkGeom &B = a.B;
+    const int nh = B.nh, gs = blockDim.x >> 2;
+    SapD S;
+    S.X = (double2 *)smem_raw;
+    S.rho = S.X + 48 * nh;
+    S.to = S.rho + 12 * nh;
+    S.red = (double *)(S.to + 12 * nh);
+    const long Vh = a.g.Vh;
+    const long half = 12 * Vh, foff = blockIdx.y * a.fstride;
+    const int k = threadIdx.x / gs, i = threadIdx.x - k * gs;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool act = i < nh;
+    int org[4];
+    {
+        int q = a.blocks[blockIdx.x];
+#pragma unroll
+        for (int m = 3; m >= 0; m--) {
+            org[m] = q % B.nb[m] * B.bs[m];
+            q /= B.nb[m];
+        }
+    }
+    const SapDSite so = d_site(a.g, B, org, k, 1, act ? i : 0), se = d_site(a.g, B, org, k, 0, act ? i : 0);
+    // three components of spin k of the two parities
+    const long co = 3 * k * Vh + so.rank, ce = 3 * k * Vh + se.rank;
+    cx<double> chi[3], s[3], w[3];
+#pragma unroll
+    for (int j = 0; j < 3; j++) chi[j] = s[j] = w[j] = mk(0.0, 0.0);
+    const int last = 2 * a.nmr + 1;
+    //   ph = -1            to = A_oo^-1 r_o
+    //   ph = 0             rho = r_e - H_eo to = r_e + 1/2 S(to)
+    //   odd ph < last      to = A_oo^-1 S(rho) = -2 A_oo^-1 H_oe rho
+    //   even ph            p = A_ee rho - 1/4 S(to); the MinRes step
+    //   ph = last          chi_o = A_oo^-1 (r_o + 1/2 S(chi_e)), chi_e read from to
+#pragma unroll 1
+    for (int ph = -1; ph <= last; ph++) {
+        const bool odd = ph & 1;
+        const int t = odd ? so.t : se.t;
+        if (ph >= 0) {
+            if (act) {
+                const double2 *src = odd && ph < last ? S.rho : S.to;
+                const int nf = odd ? so.nf : se.nf, nb = odd ? so.nb : se.nb;
+                const bool negf = odd ? so.negf : se.negf, negb = odd ? so.negb : se.negb;
+                const double2 *uf = a.U + (long)((odd * 4 + k) * 9) * Vh + (odd ? so.rank : se.rank);
+                const double2 *ub = a.U + (long)((!odd * 4 + k) * 9) * Vh + (odd ? so.rb : se.rb);
+                double2 *X = S.X + 12 * k * nh + t;
+                switch (k) {
+                    case 0: d_hops<0>(uf, ub, Vh, src, nh, nf, nb, negf, negb, X); break;
+                    case 1: d_hops<1>(uf, ub, Vh, src, nh, nf, nb, negf, negb, X); break;
+                    case 2: d_hops<2>(uf, ub, Vh, src, nh, nf, nb, negf, negb, X); break;
+                    default: d_hops<3>(uf, ub, Vh, src, nh, nf, nb, negf, negb, X); break;
+                }
+            }
+            __syncthreads();
+            if (act)
+#pragma unroll
+                for (int j = 0; j < 3; j++) {
+                    const double2 *x = S.X + (3 * k + j) * nh + t;
+                    const double2 x0 = x[0], x1 = x[12 * nh], x2 = x[24 * nh], x3 = x[36 * nh];
+                    s[j] = mk(((x0.x + x1.x) + x2.x) + x3.x, ((x0.y + x1.y) + x2.y) + x3.y);
+                }
+        }
+        bool fin = ph == last - 1;   // the next phase is the last
+        if (ph == 0) {
+            if (act)
+#pragma unroll
+                for (int j = 0; j < 3; j++) {
+                    const double2 r = a.r[foff + ce + j * Vh];
+                    S.rho[(3 * k + j) * nh + t] = make_double2(fmx(0.5, s[j].re, r.x), fmx(0.5, s[j].im, r.y));
+                }
+        } else {
+            // input of the clover rows: rho itself, or the odd phases' sum by way of
+            // X, whose entries of this site and spin no other thread reads
+            if (odd) {
+                if (act)
+#pragma unroll
+                    for (int j = 0; j < 3; j++) {
+                        if (ph < 0 || ph == last) {
+                            const double2 r = a.r[foff + half + co + j * Vh];
+                            s[j] = mk(fmx(0.5, s[j].re, r.x), fmx(0.5, s[j].im, r.y));
+                        }
+                        S.X[(3 * k + j) * nh + t] = make_double2(s[j].re, s[j].im);
+                    }
+                __syncthreads();
+            }
+            if (act) {
+                const double2 *in = (odd ? S.X : S.rho) + 6 * (k >> 1) * nh + t;
+                const double2 *A = (odd ? a.Aio : a.Ae) + (long)(18 * (k >> 1)) * Vh + (odd ? so.rank : se.rank);
+                if (k & 1)
+                    d_rows<1>(A, Vh, in, nh, w);
+                else
+                    d_rows<0>(A, Vh, in, nh, w);
+            }
+            if (odd) {
+                if (act && ph < last)
+#pragma unroll
+                    for (int j = 0; j < 3; j++) S.to[(3 * k + j) * nh + t] = make_double2(w[j].re, w[j].im);
+            } else {
+                double dot[4] = {0, 0, 0, 0};   // <p,p>, <p,rho>
+                cx<double> rv[3];
+                if (act)
+#pragma unroll
+                    for (int j = 0; j < 3; j++) {
+                        const double2 r = S.rho[(3 * k + j) * nh + t];
+                        rv[j] = mk(r.x, r.y);
+                        w[j] = mk(fmx(-0.25, s[j].re, w[j].re), fmx(-0.25, s[j].im, w[j].im));
+                        dot[0] = fmx(w[j].im, w[j].im, fmx(w[j].re, w[j].re, dot[0]));
+                        dot[1] = fmx(w[j].im, r.y, fmx(w[j].re, r.x, dot[1]));
+                        dot[2] = fmx(-w[j].im, r.x, fmx(w[j].re, r.y, dot[2]));
+                    }
+                warp_multi_sum<4>(dot);
+                if ((lane & 7) == 0 && lane < 24) S.red[16 * (lane >> 3) + warp] = dot[0];
+                __syncthreads();
+                if (warp == 0) {
+                    const bool has = lane < (int)(blockDim.x >> 5);
+                    double f[4] = {has ? S.red[lane] : 0, has ? S.red[16 + lane] : 0, has ? S.red[32 + lane] : 0, 0};
+                    warp_multi_sum<4>(f);
+                    const double pp = __shfl_sync(0xffffffffu, f[0], 0);
+                    if (lane == 0) S.red[50] = pp;
+                    if ((lane == 8 || lane == 16) && pp != 0) S.red[47 + lane / 8] = f[0] / pp;
+                }
+                __syncthreads();
+                if (S.red[50] == 0) {   // rho = 0: the block is solved
+                    fin = true;
+                    ph = last - 1;
+                } else if (act) {
+                    const double ar = S.red[48], ai = S.red[49];
+#pragma unroll
+                    for (int j = 0; j < 3; j++) {
+                        // chi += alpha rho, rho -= alpha p
+                        chi[j].re = fmx(-ai, rv[j].im, fmx(ar, rv[j].re, chi[j].re));
+                        chi[j].im = fmx(ai, rv[j].re, fmx(ar, rv[j].im, chi[j].im));
+                        S.rho[(3 * k + j) * nh + t] = make_double2(fmx(ai, w[j].im, fmx(-ar, w[j].re, rv[j].re)),
+                                                                   fmx(-ai, w[j].re, fmx(-ar, w[j].im, rv[j].im)));
+                    }
+                }
+            }
+        }
+        if (fin && act)
+#pragma unroll
+            for (int j = 0; j < 3; j++) S.to[(3 * k + j) * nh + se.t] = make_double2(chi[j].re, chi[j].im);
+        __syncthreads();
+    }
+    // psi += chi; delta = chi; r <- (rho, 0), as in k_sap_block
+    if (act)
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            const long e = foff + ce + j * Vh, o = foff + half + co + j * Vh;
+            const double2 pe = a.psi[e], po = a.psi[o];
+            a.psi[e] = make_double2(pe.x + chi[j].re, pe.y + chi[j].im);
+            a.psi[o] = make_double2(po.x + w[j].re, po.y + w[j].im);
+            a.delta[e] = make_double2(chi[j].re, chi[j].im);
+            a.delta[o] = make_double2(w[j].re, w[j].im);
+            a.r[e] = S.rho[(3 * k + j) * nh + se.t];
+            a.r[o] = make_double2(0.0, 0.0);
+        }
+}
+
+// ------------------------------------------------------------------------
 // FP32 block solve with the whole block resident in shared memory.
 //
 // At the start of a block visit the CTA stages the block's forward links (two
@@ -531,7 +907,6 @@ __global__ void __launch_bounds__(128) k_sap_block(SapArgs<P> a)
 // exchanges its partial sums by a lane shuffle, and each thread then applies
 // one chirality block (spins 2h, 2h+1) of the clover term.  Same arithmetic
 // as k_sap_block, different summation order.
-constexpr int SAPS_NH = 128;   // sites of one parity per block (4^4 blocks)
 
 // Shared memory of the resident block kernel.  SA: the clover term of the
 // block is staged too (172 KB, one CTA per SM); without it every clover
@@ -1342,6 +1717,16 @@ lqcd_status sap_run(lqcd_ctx *c, SapPlan &P_, int ncy, int nmr, const void *eta,
     // FP32 / F16S with blocks of <= 128 sites per parity (whole warps of site
     // pairs): the shared-memory resident kernel
     bool resident = false;
+    // FP64 with blocks of <= 128 sites per parity: four threads a site (512 of 128
+    // registers at most); larger ones one thread a site in turns
+    const bool four = P == LQCD_F64 && Pl.B.nh <= SAPS_NH && !sap_force_generic();
+    if constexpr (P == LQCD_F64) {
+        static bool attr_d = false;
+        if (!attr_d) {
+            cudaFuncSetAttribute(k_sap_block_d, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sap_d_smem(SAPS_NH));
+            attr_d = true;
+        }
+    }
     if constexpr (P != LQCD_F64) {
         static bool attr_s = false;
         if (!attr_s) {
@@ -1404,6 +1789,8 @@ lqcd_status sap_run(lqcd_ctx *c, SapPlan &P_, int ncy, int nmr, const void *eta,
                         <<<dim3(Pl.count[col], nrhs), 2 * Pl.B.nh, sizeof(SapSmem<P, false>), c->stream>>>(a);
                 else
                     k_sap_block<P><<<dim3(Pl.count[col], nrhs), threads, smem, c->stream>>>(a);
+            } else if (four) {
+                k_sap_block_d<<<dim3(Pl.count[col], nrhs), 4 * ((Pl.B.nh + 31) & ~31), sap_d_smem(Pl.B.nh), c->stream>>>(a);
             } else {
                 k_sap_block<P><<<dim3(Pl.count[col], nrhs), threads, smem, c->stream>>>(a);
             }
