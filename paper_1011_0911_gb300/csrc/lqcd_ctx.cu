@@ -288,10 +288,17 @@ __global__ void k_conv64to32(long Vh, long nhalf, long ih, long oh, const double
     if (r >= Vh || h >= nhalf) return;
     const double2 *i = in + h * ih * 12 * Vh + r;
     float4 *o = out + h * oh * 6 * Vh + r;
-    for (int q = 0; q < 6; q++) {
-        double2 a = i[(2 * q) * Vh], b = i[(2 * q + 1) * Vh];
-        o[q * Vh] = make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
+    double x[24];
+    float f[24];
+#pragma unroll
+    for (int k = 0; k < 12; k++) {
+        const double2 a = i[k * Vh];
+        x[2 * k] = a.x;
+        x[2 * k + 1] = a.y;
     }
+    narrow(x, f);
+#pragma unroll
+    for (int q = 0; q < 6; q++) o[q * Vh] = make_float4(f[4 * q], f[4 * q + 1], f[4 * q + 2], f[4 * q + 3]);
 }
 __global__ void k_conv32to64(long Vh, long nhalf, long ih, long oh, const float4 *__restrict__ in, double2 *out)
 {
@@ -300,20 +307,35 @@ __global__ void k_conv32to64(long Vh, long nhalf, long ih, long oh, const float4
     if (r >= Vh || h >= nhalf) return;
     const float4 *i = in + h * ih * 6 * Vh + r;
     double2 *o = out + h * oh * 12 * Vh + r;
+    double x[24];
+    float f[24];
+#pragma unroll
     for (int q = 0; q < 6; q++) {
-        float4 a = i[q * Vh];
-        o[(2 * q) * Vh] = make_double2(a.x, a.y);
-        o[(2 * q + 1) * Vh] = make_double2(a.z, a.w);
+        const float4 a = i[q * Vh];
+        f[4 * q] = a.x;
+        f[4 * q + 1] = a.y;
+        f[4 * q + 2] = a.z;
+        f[4 * q + 3] = a.w;
     }
+    widen(f, x);
+#pragma unroll
+    for (int k = 0; k < 12; k++) o[k * Vh] = make_double2(x[2 * k], x[2 * k + 1]);
 }
 
 // native F64 / F32 <-> native F16S, nhalf half fields
 __device__ __forceinline__ void nat_load(const double2 *f, long Vh, long r, cx<float> v[12])
 {
+    double x[24];
+    float t[24];
+#pragma unroll
     for (int c = 0; c < 12; c++) {
-        double2 a = f[c * Vh + r];
-        v[c] = mk((float)a.x, (float)a.y);
+        const double2 a = f[c * Vh + r];
+        x[2 * c] = a.x;
+        x[2 * c + 1] = a.y;
     }
+    narrow(x, t);
+#pragma unroll
+    for (int c = 0; c < 12; c++) v[c] = mk(t[2 * c], t[2 * c + 1]);
 }
 __device__ __forceinline__ void nat_load(const float4 *f, long Vh, long r, cx<float> v[12])
 {
@@ -325,7 +347,16 @@ __device__ __forceinline__ void nat_load(const float4 *f, long Vh, long r, cx<fl
 }
 __device__ __forceinline__ void nat_store(double2 *f, long Vh, long r, const cx<float> v[12])
 {
-    for (int c = 0; c < 12; c++) f[c * Vh + r] = make_double2(v[c].re, v[c].im);
+    double x[24];
+    float t[24];
+#pragma unroll
+    for (int c = 0; c < 12; c++) {
+        t[2 * c] = v[c].re;
+        t[2 * c + 1] = v[c].im;
+    }
+    widen(t, x);
+#pragma unroll
+    for (int c = 0; c < 12; c++) f[c * Vh + r] = make_double2(x[2 * c], x[2 * c + 1]);
 }
 __device__ __forceinline__ void nat_store(float4 *f, long Vh, long r, const cx<float> v[12])
 {

@@ -64,12 +64,15 @@ __device__ __forceinline__ float f16s_maxabs(const cx<float> *v, int n)
     for (int i = 0; i < n; i++) m = fmaxf(m, fmaxf(fabsf(v[i].re), fabsf(v[i].im)));
     return m;
 }
+// 1 / scale of a site whose largest |real part| is m; 0 (the site is stored as zero)
+// below float's normal range, where 1 / m overflows and would leave NaN
+__device__ __forceinline__ float f16s_inv(float m) { return m >= 1.17549435e-38f ? 1.f / m : 0.f; }
 __device__ __forceinline__ void f16s_store(h16s *f, long Vh, long r, const cx<float> v[12])
 {
     float m = 0.f;
 #pragma unroll
     for (int i = 0; i < 12; i++) m = fmaxf(m, fmaxf(fabsf(v[i].re), fabsf(v[i].im)));
-    const float inv = m > 0.f ? 1.f / m : 0.f;
+    const float inv = f16s_inv(m);
     uint4 *q = reinterpret_cast<uint4 *>(f);
 #pragma unroll
     for (int k = 0; k < 3; k++)

@@ -93,6 +93,48 @@ __device__ __forceinline__ void warp_multi_sum(double (&v)[V])
     for (; off > 0; off /= 2) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
 }
 
+// double <-> float of N numbers in integer arithmetic, the same values as the casts.
+// A cast takes a slot of the FP64 pipe (2 a clock and SM), eight integer
+// instructions a sixteenth of the chip's rate: with 24 casts per site each way a
+// conversion pass is bound by the pipe and not by memory.  Numbers outside float's
+// normal range (zero, too) send all N through the casts.
+template <int N>
+__device__ __forceinline__ void narrow(const double (&x)[N], float (&f)[N])
+{
+    bool odd = false;
+#pragma unroll
+    for (int i = 0; i < N; i++) {
+        const unsigned hi = __double2hiint(x[i]), lo = __double2loint(x[i]), t = hi & 0x7fffffffu;
+        odd |= t - 0x38100000u >= 0x0fe00000u;   // |x| < 2^-126 or >= 2^128
+        // mantissa cut to 23 bits, then rounded to nearest, ties to even (a carry
+        // runs on into the exponent)
+        unsigned u = __funnelshift_l(lo, t - 0x38000000u, 3);
+        u += ((lo & 0x1fffffffu) + (u & 1u) + 0x0fffffffu) >> 29;
+        f[i] = __uint_as_float(u | (hi & 0x80000000u));
+    }
+    if (odd) {
+        asm volatile("");   // a branch: the compiler would rather run the casts always
+#pragma unroll
+        for (int i = 0; i < N; i++) f[i] = (float)x[i];
+    }
+}
+template <int N>
+__device__ __forceinline__ void widen(const float (&f)[N], double (&x)[N])
+{
+    bool odd = false;
+#pragma unroll
+    for (int i = 0; i < N; i++) {
+        const unsigned u = __float_as_uint(f[i]), t = u & 0x7fffffffu;
+        odd |= t - 0x00800000u >= 0x7f000000u;   // zero, subnormal, infinite, NaN
+        x[i] = __hiloint2double((int)((u & 0x80000000u) | ((t >> 3) + 0x38000000u)), (int)(u << 29));
+    }
+    if (odd) {
+        asm volatile("");
+#pragma unroll
+        for (int i = 0; i < N; i++) x[i] = f[i];
+    }
+}
+
 // third row of an SU(3) matrix from the first two, u2 = (u0 x u1)^*, each real
 // part one product and three fused multiply-adds
 template <class R>
@@ -440,3 +482,5 @@ void dfl_free(lqcd_ctx *c);
 // smoother: SAP (net = false) or the network (net = true) after the deflation step
 lqcd_status dfl_precond_native(lqcd_ctx *c, const lqcd_sap_params *sp, const double2 *rho,
                                double2 *phi, int nrhs, bool net = false);
+lqcd_status dfl_precond_native32(lqcd_ctx *c, const lqcd_sap_params *sp, const double2 *rho, float4 *phi,
+                                 int halves, int nrhs, bool *done);

@@ -1166,7 +1166,7 @@ __device__ __forceinline__ void half_store(h16s *f, long Vh, long r, int h, cons
 #pragma unroll
     for (int i = 0; i < 6; i++) m = fmaxf(m, fmaxf(fabsf(v[i].re), fabsf(v[i].im)));
     m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
-    const float inv = m > 0.f ? 1.f / m : 0.f;
+    const float inv = f16s_inv(m);
     uint4 *q = reinterpret_cast<uint4 *>(f);
     const cx<float> e0 = h ? v[2] : v[0], e1 = h ? v[3] : v[1], e2 = h ? v[4] : v[2], e3 = h ? v[5] : v[3];
     const cx<float> m0 = h ? v[0] : v[4], m1 = h ? v[1] : v[5];
