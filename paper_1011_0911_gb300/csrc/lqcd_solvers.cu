@@ -200,8 +200,8 @@ struct Krylov32 {
           frho(24 * (long)ctx->g.Vh)
     {
     }
-    // the preconditioner's output in F32: SAP in F32 writes it directly, other
-    // forms are converted from their own output precision (the halves in use)
+    // the preconditioner's output in F32: SAP in F32 and the deflated SAP write it
+    // directly, other forms are converted from their own output precision (the halves in use)
     lqcd_status precond_with(const lqcd_solver_params *p, const double2 *rho, T *ph)
     {
         const lqcd_sap_params &sap = p->sap;
@@ -216,6 +216,11 @@ struct Krylov32 {
             LQCD_TRY(ws_get(c, WS_SAP_PSI, fb, &b));
             LQCD_TRY(sap_apply(c, &sap, a, b, nrhs));
             return convert_native(c, sap.prec, LQCD_F32, b, ph, nh * nrhs, hs, hs);
+        }
+        if (p->solver == LQCD_SOLVER_DFL_SAP_GCR) {
+            bool done;
+            LQCD_TRY(dfl_precond_native32(c, &sap, rho, ph, nh, nrhs, &done));
+            if (done) return LQCD_OK;
         }
         void *t;
         LQCD_TRY(ws_get(c, WS_PHI64, (size_t)frho * nrhs * sizeof(double2), &t));
