@@ -445,97 +445,6 @@ __device__ __forceinline__ void hop1f(int mu, int sgn, const stencil::Spinor<flo
     }
 }
 
-// The little Dirac build of an FP32 subspace in FP32 arithmetic: the FP32
-// operator (2-row links, FP32 clover), FP32 products and per-thread sums,
-// warp sums in float and the sum over warps in double.  The subspace itself is
-// FP32, so its entries carry FP32 accuracy either way; GB300's FP64 pipe made
-// the FP64 form of this kernel the largest single cost of the subspace build.
-__global__ void k_little_build32(Geom g, DBlk B, const float4 *phi, int Ns, long fstride, const float4 *U32,
-                                 const float4 *A0, const float4 *A1, double2 *Aint)
-{
-    extern __shared__ double sh[];
-    double *res = sh + 2 * RCHUNK * 32;
-    const int b = blockIdx.x, l = blockIdx.y, t = threadIdx.x;
-    BSite s;
-    bsite(g, B, b, t, s);
-    const long hs = fstride / 2;
-    const float4 *pl = phi + l * fstride;
-    for (int j = 0; j < 9; j++) {
-        stencil::Spinor<float> w;
-#pragma unroll
-        for (int sp = 0; sp < 4; sp++)
-#pragma unroll
-            for (int c = 0; c < 3; c++) w.s[sp][c] = mk(0.f, 0.f);
-        if (j == 0) {
-            stencil::Spinor<float> v;
-            stencil::load_spinor(pl + s.p * hs, g.Vh, (int)s.r, v);
-            stencil::clover_apply<float, float4>(s.p ? A1 : A0, g.Vh, (int)s.r, v, w);
-        }
-        stencil::Spinor<float> acc;
-#pragma unroll
-        for (int sp = 0; sp < 4; sp++)
-#pragma unroll
-            for (int c = 0; c < 3; c++) acc.s[sp][c] = mk(0.f, 0.f);
-        // W_j (j >= 1) vanishes on the sites that its hop does not reach: they
-        // skip the subspace loads below (their products would all be zero)
-        bool nz = j == 0;
-        for (int mu = 0; mu < 4; mu++)
-            for (int d = -1; d <= 1; d += 2) {
-                const int jj = d > 0 ? 1 + 2 * mu : 2 + 2 * mu;
-                const int lm = s.l[mu] + d;
-                const bool inside = (lm >= 0 && lm < B.bs[mu]) || B.wrap[mu];
-                if ((j == 0) != inside) continue;
-                if (j != 0 && j != jj) continue;
-                nz = true;
-                int y[4] = {s.x[0], s.x[1], s.x[2], s.x[3]};
-                y[mu] = (y[mu] + d + g.L[mu]) % g.L[mu];
-                const int ry = coords_rank(g, y);
-                stencil::Spinor<float> v;
-                cx<float> u[3][3];
-                stencil::load_spinor(pl + (1 - s.p) * hs, g.Vh, ry, v);
-                if (d > 0) {
-                    const float sign = (mu == 0 && s.x[0] == g.L[0] - 1) ? (float)g.bc_t : 1.f;
-                    stencil::load_link(U32, g.Vh, s.p, mu, (int)s.r, u);
-                    hop1f(mu, -1, v, u, false, sign, acc);
-                } else {
-                    const float sign = (mu == 0 && s.x[0] == 0) ? (float)g.bc_t : 1.f;
-                    stencil::load_link(U32, g.Vh, 1 - s.p, mu, ry, u);
-                    hop1f(mu, +1, v, u, true, sign, acc);
-                }
-            }
-#pragma unroll
-        for (int sp = 0; sp < 4; sp++)
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-                w.s[sp][c].re = fmx(-0.5f, acc.s[sp][c].re, w.s[sp][c].re);
-                w.s[sp][c].im = fmx(-0.5f, acc.s[sp][c].im, w.s[sp][c].im);
-            }
-        for (int k0 = 0; k0 < Ns; k0 += RCHUNK) {
-            float dd[2 * RCHUNK];
-            const int kn = min(RCHUNK, Ns - k0);
-#pragma unroll
-            for (int i = 0; i < RCHUNK; i++) {
-                dd[2 * i] = dd[2 * i + 1] = 0.f;
-                if (i < kn && nz) {
-                    stencil::Spinor<float> q;
-                    stencil::load_spinor(phi + (k0 + i) * fstride + s.p * hs, g.Vh, (int)s.r, q);
-#pragma unroll
-                    for (int sp = 0; sp < 4; sp++)
-#pragma unroll
-                        for (int c = 0; c < 3; c++) {
-                            const cx<float> a = q.s[sp][c], z = w.s[sp][c];
-                            dd[2 * i] = fmx(a.re, z.re, fmx(a.im, z.im, dd[2 * i]));
-                            dd[2 * i + 1] = fmx(a.re, z.im, fmx(-a.im, z.re, dd[2 * i + 1]));
-                        }
-                }
-            }
-            block_sum_f<2 * RCHUNK>(dd, 2 * kn, sh, res);
-            if (t < kn) Aint[(((long)b * 9 + j) * Ns + k0 + t) * Ns + l] = make_double2(res[2 * t], res[2 * t + 1]);
-            __syncthreads();
-        }
-    }
-}
-
 // c_r[b*Ns + k] = <phi_k|_b, in_r>  (in_r: native F64 full fields, stride in_rs;
 // c_r stride c_rs).  The nrhs CTAs of one block are consecutive, so the block's
 // subspace vectors are read from DRAM once and from L2 by the other fields.
@@ -686,6 +595,151 @@ __global__ void __launch_bounds__(512, 1) k_project_h(Geom g, DBlk B, const floa
         for (int w = 0; w < nw; w++) sum += red[i >> 5][w][i & 31];
         const int k = i / (2 * PJ_R), r = (i >> 1) % PJ_R, comp = i & 1;
         if (r < nr) reinterpret_cast<double *>(c + (long)(r0 + r) * c_rs + (long)b * Ns + k)[comp] = sum;
+    }
+}
+
+// The little Dirac build of an FP32 subspace in FP32 arithmetic: the FP32
+// operator (2-row links, FP32 clover), FP32 products and per-thread sums,
+// warp sums in float and the sum over warps in double.  The subspace itself is
+// FP32, so its entries carry FP32 accuracy either way; GB300's FP64 pipe made
+// the FP64 form of this kernel the largest single cost of the subspace build.
+//
+// The reads of the subspace vectors through L2 bound it, and the products themselves
+// next.  A CTA takes LB_L columns l of one block in one of three parts: the sites of
+// the block with the hops inside it (j = 0), or the sites of its four forward or
+// backward faces with the one hop that leaves there, so that every thread has a hop
+// to do (a quarter of a block's sites lie on a face).  A thread keeps W phi_l of its
+// site for the LB_L columns and reads each phi_k once for all of them; LB_K x LB_L
+// complex sums share one halving exchange, the warps' sums meet at the end.
+// 48 x 24^3 in 4^4 blocks, 20 vectors: 7.0 ms (one column a CTA, every face over all
+// sites of the block: 41 ms).
+constexpr int LB_L = 4, LB_K = 4;
+static_assert(LB_L * LB_K * 2 == 32, "one value per lane in the warp reduction");
+constexpr int LB_THREADS = 256;
+// warps of the faces' sites: each face in whole warps; wrapped directions have none
+__host__ __device__ __forceinline__ int lb_face_warps(const DBlk &B, int mu)
+{
+    return B.wrap[mu] ? 0 : (B.vol / B.bs[mu] + 31) / 32;
+}
+inline size_t lb_smem(const DBlk &B, int Ns)
+{
+    int nf = 0;
+    for (int mu = 0; mu < 4; mu++) nf += lb_face_warps(B, mu);
+    return (size_t)std::max(nf, B.vol / 32) * ((Ns + LB_K - 1) / LB_K) * 32 * sizeof(float);
+}
+__global__ void __launch_bounds__(LB_THREADS, 1)
+    k_little_build32(Geom g, DBlk B, const float4 *__restrict__ phi, int Ns, long fstride, const float4 *__restrict__ U32,
+                     const float4 *__restrict__ A0, const float4 *__restrict__ A1, double2 *Aint, int ngl)
+{
+    extern __shared__ float lb_red[];   // [warp][step of LB_K vectors][32]
+    const int part = blockIdx.x % 3, bl = blockIdx.x / 3, l0 = bl % ngl * LB_L, b = bl / ngl;
+    const int lane = threadIdx.x & 31, nk = (Ns + LB_K - 1) / LB_K, d = part == 1 ? 1 : -1;
+    const long hs = fstride / 2;
+    int nw = 0;
+    if (part == 0)
+        nw = B.vol / 32;
+    else
+        for (int mu = 0; mu < 4; mu++) nw += lb_face_warps(B, mu);
+    for (int w = threadIdx.x >> 5; w < nw; w += LB_THREADS / 32) {
+        // this warp's sites: place t in the block
+        int t = w * 32 + lane, fmu = -1;
+        bool on = true;
+        if (part) {
+            int ww = w;
+            for (fmu = 0; ww >= lb_face_warps(B, fmu); fmu++) ww -= lb_face_warps(B, fmu);
+            int f = ww * 32 + lane, below = 1;   // site of the face; volume of the directions after fmu
+            on = f < B.vol / B.bs[fmu];
+            if (!on) f = 0;
+            for (int m = fmu + 1; m < 4; m++) below *= B.bs[m];
+            const int up = f / below;
+            t = (up * B.bs[fmu] + (d > 0 ? B.bs[fmu] - 1 : 0)) * below + f - up * below;
+        }
+        BSite s;
+        bsite(g, B, b, t, s);
+        stencil::Spinor<float> acc[LB_L];
+#pragma unroll
+        for (int i = 0; i < LB_L; i++)
+#pragma unroll
+            for (int c = 0; c < 12; c++) acc[i].s[c / 3][c % 3] = mk(0.f, 0.f);
+        if (on) {
+#pragma unroll 1
+            for (int h = part ? 2 * fmu + (d > 0) : 0; h < 8; h += part ? 8 : 1) {
+                const int mu = h >> 1, dd = h & 1 ? 1 : -1, lm = s.l[mu] + dd;
+                if (part == 0 && !((lm >= 0 && lm < B.bs[mu]) || B.wrap[mu])) continue;
+                int y[4] = {s.x[0], s.x[1], s.x[2], s.x[3]};
+                y[mu] = (y[mu] + dd + g.L[mu]) % g.L[mu];
+                const int ry = coords_rank(g, y);
+                const float sign = (mu == 0 && s.x[0] == (dd > 0 ? g.L[0] - 1 : 0)) ? (float)g.bc_t : 1.f;
+                cx<float> u[3][3];
+                if (dd > 0)
+                    stencil::load_link(U32, g.Vh, s.p, mu, (int)s.r, u);
+                else
+                    stencil::load_link(U32, g.Vh, 1 - s.p, mu, ry, u);
+#pragma unroll
+                for (int i = 0; i < LB_L; i++) {
+                    stencil::Spinor<float> v;
+                    stencil::load_spinor(phi + min(l0 + i, Ns - 1) * fstride + (1 - s.p) * hs, g.Vh, ry, v);
+                    hop1f(mu, dd > 0 ? -1 : 1, v, u, dd < 0, sign, acc[i]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < LB_L; i++) {
+                stencil::Spinor<float> cl;
+                if (part == 0) {
+                    stencil::Spinor<float> v;
+                    stencil::load_spinor(phi + min(l0 + i, Ns - 1) * fstride + s.p * hs, g.Vh, (int)s.r, v);
+                    stencil::clover_apply<float, float4>(s.p ? A1 : A0, g.Vh, (int)s.r, v, cl);
+                }
+#pragma unroll
+                for (int c = 0; c < 12; c++) {
+                    cx<float> &z = acc[i].s[c / 3][c % 3];
+                    const cx<float> q = part == 0 ? cl.s[c / 3][c % 3] : mk(0.f, 0.f);
+                    z = mk(fmx(-0.5f, z.re, q.re), fmx(-0.5f, z.im, q.im));
+                }
+            }
+        }
+        // <phi_k, W phi_l>; W phi_l is zero on the lanes without a site
+        const float4 *f = phi + s.p * hs + s.r;
+#pragma unroll 1
+        for (int k = 0; k < nk; k++) {
+            float v[32];
+#pragma unroll
+            for (int kk = 0; kk < LB_K; kk++) {
+                const float4 *fk = f + min(k * LB_K + kk, Ns - 1) * fstride;
+                float4 q[6];
+#pragma unroll
+                for (int i = 0; i < 6; i++) q[i] = fk[i * g.Vh];
+#pragma unroll
+                for (int i = 0; i < LB_L; i++) {
+                    float re = 0.f, im = 0.f;
+#pragma unroll
+                    for (int c = 0; c < 6; c++) {
+                        const cx<float> z0 = acc[i].s[(2 * c) / 3][(2 * c) % 3], z1 = acc[i].s[(2 * c + 1) / 3][(2 * c + 1) % 3];
+                        re = fmx(q[c].x, z0.re, fmx(q[c].y, z0.im, fmx(q[c].z, z1.re, fmx(q[c].w, z1.im, re))));
+                        im = fmx(q[c].x, z0.im, fmx(-q[c].y, z0.re, fmx(q[c].z, z1.im, fmx(-q[c].w, z1.re, im))));
+                    }
+                    v[(kk * LB_L + i) * 2] = re;
+                    v[(kk * LB_L + i) * 2 + 1] = im;
+                }
+            }
+            warp_reduce_scatter32(v);
+            lb_red[(w * nk + k) * 32 + lane] = v[0];
+        }
+    }
+    __syncthreads();
+    // entries [j][k][l] of this part: the sums over the warps of the block or the face
+    const int per = Ns * LB_L * 2;
+    for (int e = threadIdx.x; e < (part ? 4 : 1) * per; e += LB_THREADS) {
+        const int mu = e / per, i = e - mu * per, k = i / (2 * LB_L), l = l0 + (i >> 1) % LB_L, comp = i & 1;
+        int w0 = 0, n = nw;
+        if (part) {
+            for (int m = 0; m < mu; m++) w0 += lb_face_warps(B, m);
+            n = lb_face_warps(B, mu);
+        }
+        double sum = 0;
+        for (int w = w0; w < w0 + n; w++) sum += lb_red[(w * nk + k / LB_K) * 32 + i % 32];
+        const int j = part ? (d > 0 ? 1 : 2) + 2 * mu : 0;
+        if (l < Ns) reinterpret_cast<double *>(Aint + (((long)b * 9 + j) * Ns + k) * Ns + l)[comp] = sum;
     }
 }
 
@@ -2296,8 +2350,13 @@ lqcd_status lqcd_dfl_build(lqcd_ctx *c, const lqcd_dfl_params *p, const double *
         k_little_build<double2><<<grid, B.vol, sm2, c->stream>>>(c->g, B, (const double2 *)d->phi, p->Ns, fe,
                                                                 c->U64, c->A64[0], c->A64[1], d->Aint);
     else
-        k_little_build32<<<grid, B.vol, sm2, c->stream>>>(c->g, B, (const float4 *)d->phi, p->Ns, fe, c->U32,
-                                                          c->A32[0], c->A32[1], d->Aint);
+    {
+        const int ngl = div_up(p->Ns, LB_L);
+        const size_t sm3 = lb_smem(B, p->Ns);
+        LQCD_CUDA_CHECK(c, cudaFuncSetAttribute(k_little_build32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3));
+        k_little_build32<<<3 * ngl * B.nblk, LB_THREADS, sm3, c->stream>>>(
+            c->g, B, (const float4 *)d->phi, p->Ns, fe, c->U32, c->A32[0], c->A32[1], d->Aint, ngl);
+    }
     c->n_kernel_launches++;
     LQCD_LAUNCH_CHECK(c);
     // block-Jacobi preconditioner of the coarse solve: inverses of the diagonal blocks
