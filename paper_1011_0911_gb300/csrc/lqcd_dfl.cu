@@ -1055,6 +1055,7 @@ __global__ void __launch_bounds__(256) k_fdot_partial(long n, const float2 *__re
                                                       const float2 *__restrict__ B, long fb, int k0, int kn,
                                                       double2 *partial)
 {
+    after_previous();
     const int r = blockIdx.y;
     const float2 *Br = B + r * fb, *Ar = A + r * fa;
     float re[FDOT_K], im[FDOT_K];
@@ -1159,10 +1160,15 @@ __global__ void k_fsub(long n, const float2 *a, const float2 *b, float2 *out)
 // AT [b][j-1][l][k] and DT [b][l][k]; the input segment of neighbour j sits in
 // shared memory as [l][r] (one broadcast read per pair of right-hand sides).
 // The eight partial sums are added in the order j = 1 .. 8, then Dinv is
-// applied by thread (k, r).  Short dependent chains per warp (Ns loads of one
-// matrix) and 8 warps per row block keep enough loads in flight.
+// applied by thread (k, r).  What a CTA reads comes from L2 and a row block is a few
+// microseconds of work, so latencies bound it: Dinv, the rows of xadd and the first
+// entries of the matrix are under way before the neighbours' segments are known, and
+// each group of entries is loaded while the one before it is used.  1296 rows,
+// Ns = 20, 12 right-hand sides: 30 us (33 with
+// each of these loaded where it is used); launched dependently (launch_pdl), the six
+// kernels of a coarse step together 30 us less.
 constexpr int CW_R = 12;   // right-hand sides per pass
-__global__ void __launch_bounds__(256) k_coarse_hop_eo_j(int Ns, long Nin, long Nout, int nrhs,
+__global__ void __launch_bounds__(256, 3) k_coarse_hop_eo_j(int Ns, long Nin, long Nout, int nrhs,
                                                          const int *__restrict__ rows, const int *__restrict__ npos,
                                                          const float2 *__restrict__ AT,
                                                          const float2 *__restrict__ DT, int use_dinv,
@@ -1176,10 +1182,31 @@ __global__ void __launch_bounds__(256) k_coarse_hop_eo_j(int Ns, long Nin, long 
     const int tile = Ns * CW_R;
     float2 *xj = sm + j * tile;     // input segment of neighbour j, then its partial sum
     float2 *hs = sm + 8 * tile;     // hop sum [k][r] for the Dinv stage
+    float2 *Ds = hs + tile;         // Dinv of the row, as DT
     in += r0 * Nin;
     out += r0 * Nout;
     if (xadd) xadd += r0 * Nout;
+    constexpr int G = 8;            // matrix entries in a group
+    const float2 *Aj = AT + ((long)b * 8 + j) * Ns * Ns + lane;
+    float2 av[G];
+    if (lane < Ns)
+#pragma unroll
+        for (int u = 0; u < G; u++) av[u] = u < Ns ? __ldg(Aj + u * Ns) : make_float2(0.f, 0.f);
     const long seg = (long)npos[i * 8 + j] * Ns;
+    // Ns <= 32: at most two outputs and four entries of Dinv a thread
+    float2 base[2], dv[4];
+    if (use_dinv)
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const int o = threadIdx.x + 256 * u;
+            if (o < Ns * Ns) dv[u] = __ldg(DT + (long)b * Ns * Ns + o);
+        }
+    after_previous();   // the operator above is constant, in and xadd are not
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+        const int o = threadIdx.x + 256 * u, k = o / CW_R, r = o - k * CW_R;
+        base[u] = xadd && o < tile && r < nr ? xadd[r * Nout + (long)i * Ns + k] : make_float2(0.f, 0.f);
+    }
     if (lane < Ns)
 #pragma unroll
         for (int r = 0; r < CW_R; r++)
@@ -1189,14 +1216,13 @@ __global__ void __launch_bounds__(256) k_coarse_hop_eo_j(int Ns, long Nin, long 
 #pragma unroll
     for (int r = 0; r < CW_R; r++) re[r] = im[r] = 0.f;
     if (lane < Ns) {
-        const float2 *Aj = AT + ((long)b * 8 + j) * Ns * Ns + lane;
-        // the matrix column in groups of 8 entries, each group's loads issued together
-        for (int l0 = 0; l0 < Ns; l0 += 8) {
-            float2 av[8];
+        for (int l0 = 0; l0 < Ns; l0 += G) {
+            float2 an[G];
 #pragma unroll
-            for (int u = 0; u < 8; u++) av[u] = l0 + u < Ns ? __ldg(Aj + (l0 + u) * Ns) : make_float2(0.f, 0.f);
+            for (int u = 0; u < G; u++)
+                an[u] = l0 + G + u < Ns ? __ldg(Aj + (l0 + G + u) * Ns) : make_float2(0.f, 0.f);
 #pragma unroll
-            for (int u = 0; u < 8; u++) {
+            for (int u = 0; u < G; u++) {
                 if (l0 + u >= Ns) break;
                 const float2 a = av[u];
                 const float4 *y4 = reinterpret_cast<const float4 *>(xj + (l0 + u) * CW_R);
@@ -1209,46 +1235,52 @@ __global__ void __launch_bounds__(256) k_coarse_hop_eo_j(int Ns, long Nin, long 
                     im[2 * q + 1] = fmx(a.x, y.w, fmx(a.y, y.z, im[2 * q + 1]));
                 }
             }
+#pragma unroll
+            for (int u = 0; u < G; u++) av[u] = an[u];
         }
     }
     __syncwarp();
     if (lane < Ns)
 #pragma unroll
         for (int r = 0; r < CW_R; r++) xj[lane * CW_R + r] = make_float2(re[r], im[r]);
+    if (use_dinv)
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const int o = threadIdx.x + 256 * u;
+            if (o < Ns * Ns) Ds[o] = dv[u];
+        }
     __syncthreads();
-    for (int o = threadIdx.x; o < tile; o += blockDim.x) {
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+        const int o = threadIdx.x + 256 * u;
+        if (o >= tile) break;
         float2 t = sm[o];
 #pragma unroll
         for (int jj = 1; jj < 8; jj++) {
-            const float2 u = sm[jj * tile + o];
-            t.x += u.x;
-            t.y += u.y;
+            const float2 p = sm[jj * tile + o];
+            t.x += p.x;
+            t.y += p.y;
         }
         const int k = o / CW_R, r = o - k * CW_R;
-        if (use_dinv) {
+        if (use_dinv)
             hs[o] = t;
-        } else if (r < nr) {
-            const long oi = r * Nout + (long)i * Ns + k;
-            const float2 base = xadd ? xadd[oi] : make_float2(0.f, 0.f);
-            out[oi] = make_float2(base.x + sign * t.x, base.y + sign * t.y);
-        }
+        else if (r < nr)
+            out[r * Nout + (long)i * Ns + k] = make_float2(base[u].x + sign * t.x, base[u].y + sign * t.y);
     }
     if (!use_dinv) return;
     __syncthreads();
-    for (int o = threadIdx.x; o < tile; o += blockDim.x) {
-        const int k = o / CW_R, r = o - k * CW_R;
-        if (r >= nr) continue;
-        const float2 *D = DT + (long)b * Ns * Ns + k;
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+        const int o = threadIdx.x + 256 * u, k = o / CW_R, r = o - k * CW_R;
+        if (o >= tile || r >= nr) continue;
         float dre = 0.f, dim = 0.f;
 #pragma unroll 4
         for (int l = 0; l < Ns; l++) {
-            const float2 a = __ldg(D + l * Ns), y = hs[l * CW_R + r];
+            const float2 a = Ds[l * Ns + k], y = hs[l * CW_R + r];
             dre = fmx(a.x, y.x, fmx(-a.y, y.y, dre));
             dim = fmx(a.x, y.y, fmx(a.y, y.x, dim));
         }
-        const long oi = r * Nout + (long)i * Ns + k;
-        const float2 base = xadd ? xadd[oi] : make_float2(0.f, 0.f);
-        out[oi] = make_float2(base.x + sign * dre, base.y + sign * dim);
+        out[r * Nout + (long)i * Ns + k] = make_float2(base[u].x + sign * dre, base[u].y + sign * dim);
     }
 }
 // column-major FP32 copies of the eight hopping matrices and of the diagonal
@@ -1515,6 +1547,7 @@ __global__ void k_c_norm(int nrhs, int k, CoarseScal *s)
 // other took 20 us for 50 of them)
 __global__ void __launch_bounds__(32) k_c_norm_p(int k, int nbp, const double2 *partial, CoarseScal *s)
 {
+    after_previous();
     const int r = blockIdx.x, lane = threadIdx.x;
     double v[4] = {0, 0, 0, 0};
     for (int b = lane; b < nbp; b += 32) {
@@ -1565,6 +1598,7 @@ __global__ void __launch_bounds__(256) k_fgs_norm(long n, int k, int nbp, const 
                                                   CoarseScal *S, const float2 *__restrict__ Q, long sa, float2 *qk,
                                                   const float2 *__restrict__ rho, double2 *partial2)
 {
+    after_previous();
     const int r = blockIdx.y;
     __shared__ float2 cs[CG_K];
     __shared__ double sh[8][3];
@@ -1636,6 +1670,7 @@ __global__ void __launch_bounds__(256) k_fgs_norm(long n, int k, int nbp, const 
 // vector p_{k+1} = rho (pnext may be null)
 __global__ void k_fc_update(long n, const CoarseScal *S, float2 *qk, float2 *rho, float2 *pnext)
 {
+    after_previous();
     const int r = blockIdx.y;
     const float cr = (float)S->cfR[r].x, ci = (float)S->cfR[r].y, cs = (float)S->cfS[r].x;
     float2 *qr = qk + r * n, *pr = rho + r * n, *nr = pnext ? pnext + r * n : nullptr;
@@ -1876,10 +1911,12 @@ lqcd_status coarse_gcr32_eo(lqcd_ctx *c, const double2 *b, double2 *x, int nrhs,
     const int nb = std::max(1, std::min<int>(std::max(8, 4 * 152 / nrhs), (int)((Ne + 255) / 256)));
     const int ga = std::max(1, std::min<int>(4 * 152 / std::max(1, nrhs), (int)((Ne + 255) / 256)));
     if (!d->AT32) return set_err(c, LQCD_ERR_STATE, "even-odd coarse solve without its FP32 matrix copies");
-    const size_t wsm = (size_t)9 * Ns * CW_R * sizeof(float2);
+    const size_t wsm = ((size_t)9 * Ns * CW_R + Ns * Ns) * sizeof(float2);
+    const bool pdl = !c->capturing;   // a step is six kernels of a few microseconds each
     auto hop = [&](const int *rows, int nrows, long Nin, long Nout, const float2 *in, int dinv, const float2 *xadd,
                    float sign, float2 *out) -> lqcd_status {
-        k_coarse_hop_eo_j<<<dim3(nrows, div_up(nrhs, CW_R)), 256, wsm, c->stream>>>(
+        launch_pdl_smem(
+            pdl, k_coarse_hop_eo_j, dim3(nrows, div_up(nrhs, CW_R)), 256, wsm, c->stream,
             Ns, Nin, Nout, nrhs, rows, d->npos + 8 * (rows - d->blist), d->AT32, d->DT32, dinv, in, xadd, sign, out);
         c->n_kernel_launches++;
         LQCD_LAUNCH_CHECK(c);
@@ -1939,12 +1976,13 @@ lqcd_status coarse_gcr32_eo(lqcd_ctx *c, const double2 *b, double2 *x, int nrhs,
             if (k > 0)
                 for (int k0 = 0; k0 < k; k0 += FDOT_K) {
                     const int kn = std::min(FDOT_K, k - k0);
-                    k_fdot_partial<<<dim3(nb, nrhs), 256, 0, c->stream>>>(Ne, Q, bE, Ne, qk, Ne, k0, kn, partial);
+                    launch_pdl(pdl, k_fdot_partial, dim3(nb, nrhs), 256, c->stream, Ne, Q, bE, Ne, qk, Ne, k0, kn, partial);
                     c->n_kernel_launches++;
                 }
-            k_fgs_norm<<<dim3(nb, nrhs), 256, 0, c->stream>>>(Ne, k, nb, partial, S, Q, bE, qk, rho, partial2);
-            k_c_norm_p<<<nrhs, 32, 0, c->stream>>>(k, nb, partial2, S);
-            k_fc_update<<<dim3(ga, nrhs), 256, 0, c->stream>>>(Ne, S, qk, rho, k + 1 < nkv ? pk + bE : nullptr);
+            launch_pdl(pdl, k_fgs_norm, dim3(nb, nrhs), 256, c->stream, Ne, k, nb, partial, S, Q, bE, qk, rho, partial2);
+            launch_pdl(pdl, k_c_norm_p, nrhs, 32, c->stream, k, nb, partial2, S);
+            launch_pdl(pdl, k_fc_update, dim3(ga, nrhs), 256, c->stream, Ne, S, qk, rho,
+                       k + 1 < nkv ? pk + bE : (float2 *)nullptr);
             c->n_kernel_launches += 3;
             LQCD_LAUNCH_CHECK(c);
             it++;

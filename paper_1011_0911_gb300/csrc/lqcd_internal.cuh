@@ -362,15 +362,17 @@ inline long native_half_units(const lqcd_ctx *c, lqcd_prec p)   // in 16-byte un
 // signalled before it, the launches of a chain pile up on the SMs (43.6 us).  In
 // captured graphs plain launches are faster (CGNR on 8^4: 6.97 against 7.97 ms).
 template <class... KP, class... A>
-inline cudaError_t launch_pdl(bool pdl, void (*kernel)(KP...), dim3 grid, dim3 block, cudaStream_t st, A... args)
+inline cudaError_t launch_pdl_smem(bool pdl, void (*kernel)(KP...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                   A... args)
 {
     if (!pdl) {
-        kernel<<<grid, block, 0, st>>>(args...);
+        kernel<<<grid, block, smem, st>>>(args...);
         return cudaGetLastError();
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -378,6 +380,11 @@ inline cudaError_t launch_pdl(bool pdl, void (*kernel)(KP...), dim3 grid, dim3 b
     cfg.attrs = at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KP>(args)...);
+}
+template <class... KP, class... A>
+inline cudaError_t launch_pdl(bool pdl, void (*kernel)(KP...), dim3 grid, dim3 block, cudaStream_t st, A... args)
+{
+    return launch_pdl_smem(pdl, kernel, grid, block, 0, st, args...);
 }
 __device__ __forceinline__ void after_previous()
 {
