@@ -1781,6 +1781,12 @@ lqcd_status sap_run(lqcd_ctx *c, SapPlan &P_, int ncy, int nmr, const void *eta,
     // the residual is not needed after the last sweep
     int last_col = Pl.count[1] > 0 ? 1 : 0;
     int sweep = 0;
+    // Dependent launches where the blocks of a sweep are at most one wave (three CTAs
+    // an SM): there launch and staging are a part of a sweep's time (500 sweeps of 256
+    // blocks at 32 x 16^3: 49.9 -> 48.4 ms).  Over many waves the CTAs that are set up
+    // early only get in the way of the kernel before (48 x 24^3 with 12 right-hand
+    // sides, 15552 blocks a sweep: 3.1 ms a sweep plain, 3.5 ms dependent).
+    const bool dependent = !c->capturing && (long)std::max(Pl.count[0], Pl.count[1]) * nrhs <= 3 * 152;
     for (int cyc = 0; cyc < ncy; cyc++)
         for (int col = 0; col < 2; col++) {
             if (Pl.count[col] == 0) continue;
@@ -1791,10 +1797,9 @@ lqcd_status sap_run(lqcd_ctx *c, SapPlan &P_, int ncy, int nmr, const void *eta,
                 cudaEventRecord(ev[0], c->stream);
             }
             if constexpr (P != LQCD_F64) {
-                // dependent launches (the links are staged while the kernel before still
-                // runs: a solve of 500 sweeps at 32 x 16^3 49.9 -> 48.4 ms) but for the
-                // first, which may follow the kernels that make the operator's copy
-                const bool pdl = !c->capturing && sweep > 0;
+                // (the first may follow the kernels that make the operator's copy, whose
+                // writes it would stage too early)
+                const bool pdl = dependent && sweep > 0;
                 if (resident && stage)
                     launch_pdl_smem(pdl, k_sap_block_s<P, true>, dim3(Pl.count[col], nrhs), 2 * Pl.B.nh,
                                     sizeof(SapSmem<P, true>), c->stream, a);
@@ -1822,7 +1827,7 @@ lqcd_status sap_run(lqcd_ctx *c, SapPlan &P_, int ncy, int nmr, const void *eta,
             sweep++;
             if (cyc == ncy - 1 && col == last_col) continue;
             if (Pl.nface[col] > 0)
-                launch_pdl(!c->capturing, k_sap_face_l<P>, dim3(div_up(Pl.nface[col], 128), nrhs), 128, c->stream, a,
+                launch_pdl(dependent, k_sap_face_l<P>, dim3(div_up(Pl.nface[col], 128), nrhs), 128, c->stream, a,
                            (const int2 *)Pl.face_dev[col], Pl.nface[col]);
             c->n_kernel_launches++;
             LQCD_LAUNCH_CHECK(c);
@@ -1841,41 +1846,6 @@ lqcd_status sap_run(lqcd_ctx *c, SapPlan &P_, int ncy, int nmr, const void *eta,
 }
 
 }  // namespace
-
-// r = eta - r on native full fields
-namespace {
-template <class T>
-__global__ void k_eta_minus(long n, const T *__restrict__ eta, T *r);
-template <>
-__global__ void k_eta_minus<double2>(long n, const double2 *__restrict__ eta, double2 *r)
-{
-    for (long j = blockIdx.x * (long)blockDim.x + threadIdx.x; j < n; j += (long)gridDim.x * blockDim.x) {
-        double2 a = eta[j], b = r[j];
-        r[j] = make_double2(a.x - b.x, a.y - b.y);
-    }
-}
-template <>
-__global__ void k_eta_minus<float4>(long n, const float4 *__restrict__ eta, float4 *r)
-{
-    for (long j = blockIdx.x * (long)blockDim.x + threadIdx.x; j < n; j += (long)gridDim.x * blockDim.x) {
-        float4 a = eta[j], b = r[j];
-        r[j] = make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
-    }
-}
-}  // namespace
-
-lqcd_status sap_axpby_native(lqcd_ctx *c, lqcd_prec p, const void *eta, void *r)
-{
-    long n = 2 * (long)c->g.Vh * (p == LQCD_F64 ? 12 : 6);
-    int grid = (int)std::min<long>(4 * 152, (n + 255) / 256);
-    if (p == LQCD_F64)
-        k_eta_minus<double2><<<grid, 256, 0, c->stream>>>(n, (const double2 *)eta, (double2 *)r);
-    else
-        k_eta_minus<float4><<<grid, 256, 0, c->stream>>>(n, (const float4 *)eta, (float4 *)r);
-    c->n_kernel_launches++;
-    LQCD_LAUNCH_CHECK(c);
-    return LQCD_OK;
-}
 
 lqcd_status sap_apply(lqcd_ctx *c, const lqcd_sap_params *sp, const void *eta, void *psi, int nrhs)
 {
