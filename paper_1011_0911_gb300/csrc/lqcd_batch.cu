@@ -790,11 +790,21 @@ lqcd_status lqcd_batch_solve_dhat(lqcd_batch *b, const double *const *eta_dev, d
     LQCD_CUDA_CHECK(hc, cudaMemsetAsync(b->bar, 0, sizeof(GridBar), b->st));
     LQCD_CUDA_CHECK(hc, cudaStreamSynchronize(b->st));
     std::vector<BScal> S(n);
-    std::vector<cudaStream_t> saved(n);
-    for (int l = 0; l < n; l++) {
-        saved[l] = b->ctx[l]->stream;
-        b->ctx[l]->stream = b->st;
-    }
+    struct OnBatchStream {   // the contexts work on the batch's stream until the return
+        lqcd_batch *b;
+        std::vector<cudaStream_t> saved;
+        explicit OnBatchStream(lqcd_batch *batch) : b(batch)
+        {
+            for (lqcd_ctx *c : b->ctx) {
+                saved.push_back(c->stream);
+                c->stream = b->st;
+            }
+        }
+        ~OnBatchStream()
+        {
+            for (size_t l = 0; l < saved.size(); l++) b->ctx[l]->stream = saved[l];
+        }
+    } on_batch_stream(b);
     LQCD_TRY(sap_batch_refresh(b->sap, b->ctx.data(), n, b->p.sap.bs));
     for (int l = 0; l < n; l++) {
         lqcd_ctx *c = b->ctx[l];
@@ -885,7 +895,6 @@ lqcd_status lqcd_batch_solve_dhat(lqcd_batch *b, const double *const *eta_dev, d
             info[l].net_fallbacks = 0;
         }
         if (worst == LQCD_OK && S[l].status != LQCD_OK) worst = (lqcd_status)S[l].status;
-        c->stream = saved[l];
     }
     cudaEventRecord(ev, b->st);
     cudaStreamWaitEvent(b->user, ev, 0);

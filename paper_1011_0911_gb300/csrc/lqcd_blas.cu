@@ -16,13 +16,6 @@ __global__ void k_axpy(long n, double ar, double ai, const double2 *__restrict__
         y[j] = caxpy(make_double2(ar, ai), x[j], y[j]);
     }
 }
-__global__ void k_xpay(long n, const double2 *__restrict__ x, double ar, double2 *y)
-{
-    for (long j = blockIdx.x * (long)blockDim.x + threadIdx.x; j < n; j += (long)gridDim.x * blockDim.x) {
-        double2 a = x[j], b = y[j];
-        y[j] = make_double2(a.x + ar * b.x, a.y + ar * b.y);
-    }
-}
 __global__ void k_scal(long n, double ar, double ai, double2 *y)
 {
     for (long j = blockIdx.x * (long)blockDim.x + threadIdx.x; j < n; j += (long)gridDim.x * blockDim.x) {
@@ -595,14 +588,6 @@ lqcd_status blas_axpy(lqcd_ctx *c, long n2, double ar, double ai, const double *
 {
     long n = n2 / 2;
     k_axpy<<<grid_for(n), 256, 0, c->stream>>>(n, ar, ai, (const double2 *)x, (double2 *)y);
-    c->n_kernel_launches++;
-    LQCD_LAUNCH_CHECK(c);
-    return LQCD_OK;
-}
-lqcd_status blas_xpay(lqcd_ctx *c, long n2, const double *x, double ar, double *y)
-{
-    long n = n2 / 2;
-    k_xpay<<<grid_for(n), 256, 0, c->stream>>>(n, (const double2 *)x, ar, (double2 *)y);
     c->n_kernel_launches++;
     LQCD_LAUNCH_CHECK(c);
     return LQCD_OK;

@@ -419,7 +419,6 @@ lqcd_status blas_dot(lqcd_ctx *c, long n2, const double *a, const double *b, int
                      double *host_out);  // k dots <a_i, b>, host_out: 2k doubles
 lqcd_status blas_norm2(lqcd_ctx *c, long n2, const double *a, double *host_out);
 lqcd_status blas_axpy(lqcd_ctx *c, long n2, double ar, double ai, const double *x, double *y);
-lqcd_status blas_xpay(lqcd_ctx *c, long n2, const double *x, double ar, double *y);  // y = x + a y
 lqcd_status blas_scal(lqcd_ctx *c, long n2, double ar, double ai, double *y);
 lqcd_status blas_copy(lqcd_ctx *c, long n2, const double *x, double *y);
 lqcd_status blas_sub(lqcd_ctx *c, long n2, const double *x, const double *y, double *z);  // z = x - y
@@ -462,7 +461,6 @@ lqcd_status blas_zero(lqcd_ctx *c, size_t bytes, void *p);
 lqcd_status cgnr_native(lqcd_ctx *c, const double2 *eta, double2 *x, double tol, int nmx, lqcd_solve_info *info);
 
 // sap
-lqcd_status sap_axpby_native(lqcd_ctx *c, lqcd_prec p, const void *eta, void *r);
 void sap_free_plans(lqcd_ctx *c);
 lqcd_status sap_apply(lqcd_ctx *c, const lqcd_sap_params *sp, const void *eta_native,
                       void *psi_native, int nrhs = 1);
