@@ -266,7 +266,9 @@ lqcd_status cgnr_native(lqcd_ctx *c, const double2 *eta, double2 *x, double tol,
                     own.graph = nullptr;   // plain launches serve
                 }
             }
-            if (own.graph) {
+            // (a graph is kept for later starts; one with fewer iterations left than a graph
+            // holds runs plainly: nothing would be sent, and H still has the start before)
+            if (own.graph && limit >= CG_RING) {
                 const long graphs = limit / CG_RING;
                 long done = 0, sent = 0;
                 while (last.code == CG_RUN && done < graphs) {
@@ -298,11 +300,12 @@ lqcd_status cgnr_native(lqcd_ctx *c, const double2 *eta, double2 *x, double tol,
                 seen++;
             }
             LQCD_CUDA_CHECK(c, cudaStreamSynchronize(c->stream));   // iterations past the end are no-ops
+            const bool moved = last.iters > it;
             it = last.iters;
             rr = last.rr;
             if (last.code == CG_NAN) st = LQCD_ERR_NAN;
             if (last.code == CG_BREAKDOWN) st = LQCD_ERR_BREAKDOWN;
-            if (last.code != CG_BELOW) break;
+            if (last.code != CG_BELOW || !moved) break;   // no start without an iteration is repeated
             // recompute the residual before accepting; too large: another start from it
             LQCD_TRY(dhat(x, w));
             LQCD_TRY(blas_sub(c, n2, (const double *)eta, (const double *)w, (double *)r));
