@@ -217,13 +217,13 @@ lqcd_status cgnr_native(lqcd_ctx *c, const double2 *eta, double2 *x, double tol,
         CgState *cur = S + i % CG_RING, *nxt = S + (i + 1) % CG_RING;
         const bool pdl = !c->capturing;
         LQCD_TRY(dhat(p, w));
-        LQCD_CUDA_CHECK(c, launch_pdl(pdl, k_cg_norm, nb, CG_THREADS, c->stream, n, w, pw));
-        LQCD_CUDA_CHECK(c, launch_pdl(pdl, k_cg_xr, nb, CG_THREADS, c->stream, n, nb, cur, pw, p, w, x, r, t, prr));
+        launch_pdl(pdl, k_cg_norm, nb, CG_THREADS, c->stream, n, w, pw);
+        launch_pdl(pdl, k_cg_xr, nb, CG_THREADS, c->stream, n, nb, cur, pw, p, w, x, r, t, prr);
         LQCD_TRY(dhat(t, z));
-        LQCD_CUDA_CHECK(c, launch_pdl(pdl, k_cg_norm, nb, CG_THREADS, c->stream, n, z, pzz));
-        LQCD_CUDA_CHECK(c, launch_pdl(pdl, k_cg_p, nb, CG_THREADS, c->stream, n, nb, cur, nxt, H + i % CG_RING, tol2, pw,
-                                      prr, pzz, z, p));
+        launch_pdl(pdl, k_cg_norm, nb, CG_THREADS, c->stream, n, z, pzz);
+        launch_pdl(pdl, k_cg_p, nb, CG_THREADS, c->stream, n, nb, cur, nxt, H + i % CG_RING, tol2, pw, prr, pzz, z, p);
         c->n_kernel_launches += 4;
+        LQCD_LAUNCH_CHECK(c);
         return LQCD_OK;
     };
     int it = 0;

@@ -132,15 +132,14 @@ lqcd_status launch_var(lqcd_ctx *c, int var, dim3 b, const HopArgs<SP, LK, CL> &
     if (nb > 0x7fffffffL) return set_err(c, LQCD_ERR_ARG, "stencil: grid of %ld CTAs", nb);
     const dim3 grid((unsigned)nb, hop_grid_y<MODE>());
     const bool pdl = !c->capturing;
-    cudaError_t e;
     switch (var) {
-        case 0: e = launch_pdl(pdl, k_hop<R, SP, LK, CL, MODE, 0>, grid, b, c->stream, a, ngy); break;
-        case 1: e = launch_pdl(pdl, k_hop<R, SP, LK, CL, MODE, 1>, grid, b, c->stream, a, ngy); break;
-        case 2: e = launch_pdl(pdl, k_hop<R, SP, LK, CL, MODE, 2>, grid, b, c->stream, a, ngy); break;
-        default: e = launch_pdl(pdl, k_hop<R, SP, LK, CL, MODE, 3>, grid, b, c->stream, a, ngy); break;
+        case 0: launch_pdl(pdl, k_hop<R, SP, LK, CL, MODE, 0>, grid, b, c->stream, a, ngy); break;
+        case 1: launch_pdl(pdl, k_hop<R, SP, LK, CL, MODE, 1>, grid, b, c->stream, a, ngy); break;
+        case 2: launch_pdl(pdl, k_hop<R, SP, LK, CL, MODE, 2>, grid, b, c->stream, a, ngy); break;
+        default: launch_pdl(pdl, k_hop<R, SP, LK, CL, MODE, 3>, grid, b, c->stream, a, ngy); break;
     }
     c->n_kernel_launches++;
-    LQCD_CUDA_CHECK(c, e);
+    LQCD_LAUNCH_CHECK(c);
     return LQCD_OK;
 }
 

@@ -330,15 +330,14 @@ lqcd_status launch_d(lqcd_ctx *c, int G, const HopArgs<double2, double2, double2
     if (nb > 0x7fffffffL) return set_err(c, LQCD_ERR_ARG, "FP64 stencil: grid of %ld CTAs", nb);
     const dim3 grid((unsigned)nb, hop_grid_y<MODE>());
     const bool pdl = !c->capturing;
-    cudaError_t e = cudaSuccess;
     switch (G) {
-        case 1: e = launch_pdl(pdl, k_hop_d<MODE, 1, BLK>, grid, HOP_D_THREADS, c->stream, a, bx); break;
-        case 2: e = launch_pdl(pdl, k_hop_d<MODE, 2, BLK>, grid, HOP_D_THREADS, c->stream, a, bx); break;
-        case 4: e = launch_pdl(pdl, k_hop_d<MODE, 4, BLK>, grid, HOP_D_THREADS, c->stream, a, bx); break;
+        case 1: launch_pdl(pdl, k_hop_d<MODE, 1, BLK>, grid, HOP_D_THREADS, c->stream, a, bx); break;
+        case 2: launch_pdl(pdl, k_hop_d<MODE, 2, BLK>, grid, HOP_D_THREADS, c->stream, a, bx); break;
+        case 4: launch_pdl(pdl, k_hop_d<MODE, 4, BLK>, grid, HOP_D_THREADS, c->stream, a, bx); break;
         default: return set_err(c, LQCD_ERR_ARG, "FP64 stencil: split %d", G);
     }
     c->n_kernel_launches++;
-    LQCD_CUDA_CHECK(c, e);
+    LQCD_LAUNCH_CHECK(c);
     return LQCD_OK;
 }
 }  // namespace

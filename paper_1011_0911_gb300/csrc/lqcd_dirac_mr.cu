@@ -183,12 +183,12 @@ __global__ void __launch_bounds__(VarMR<VAR>::T, VarMR<VAR>::B) k_hop_mr(const H
 }
 
 template <class R, class SP, class LK, class CL, int MODE, int NR>
-cudaError_t launch_nr(bool pdl, int var, dim3 grid, dim3 b, int ngy, cudaStream_t st, const HopArgs<SP, LK, CL> &a)
+void launch_nr(bool pdl, int var, dim3 grid, dim3 b, int ngy, cudaStream_t st, const HopArgs<SP, LK, CL> &a)
 {
     switch (var) {
-        case 0: return launch_pdl(pdl, k_hop_mr<R, SP, LK, CL, MODE, NR, 0>, grid, b, st, a, ngy);
-        case 1: return launch_pdl(pdl, k_hop_mr<R, SP, LK, CL, MODE, NR, 1>, grid, b, st, a, ngy);
-        default: return launch_pdl(pdl, k_hop_mr<R, SP, LK, CL, MODE, NR, 2>, grid, b, st, a, ngy);
+        case 0: launch_pdl(pdl, k_hop_mr<R, SP, LK, CL, MODE, NR, 0>, grid, b, st, a, ngy); break;
+        case 1: launch_pdl(pdl, k_hop_mr<R, SP, LK, CL, MODE, NR, 1>, grid, b, st, a, ngy); break;
+        default: launch_pdl(pdl, k_hop_mr<R, SP, LK, CL, MODE, NR, 2>, grid, b, st, a, ngy); break;
     }
 }
 
@@ -202,15 +202,14 @@ lqcd_status launch_hop_mr(lqcd_ctx *c, int nr, int var, dim3 b, const HopArgs<SP
     const long grid = (long)div_up(c->g.Vh, b.x) * ngy;
     if (grid > 0x7fffffffL) return set_err(c, LQCD_ERR_ARG, "blocked stencil: grid of %ld CTAs", grid);
     const dim3 g((unsigned)grid, hop_grid_y<MODE>());
-    cudaError_t e;
     if (nr == 2)
-        e = launch_nr<R, SP, LK, CL, MODE, 2>(!c->capturing, var, g, b, ngy, c->stream, a);
+        launch_nr<R, SP, LK, CL, MODE, 2>(!c->capturing, var, g, b, ngy, c->stream, a);
     else if (nr == 3)
-        e = launch_nr<R, SP, LK, CL, MODE, 3>(!c->capturing, var, g, b, ngy, c->stream, a);
+        launch_nr<R, SP, LK, CL, MODE, 3>(!c->capturing, var, g, b, ngy, c->stream, a);
     else
         return set_err(c, LQCD_ERR_ARG, "no blocked stencil for %d fields per thread", nr);
     c->n_kernel_launches++;
-    LQCD_CUDA_CHECK(c, e);
+    LQCD_LAUNCH_CHECK(c);
     return LQCD_OK;
 }
 

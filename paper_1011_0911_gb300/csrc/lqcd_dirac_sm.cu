@@ -192,12 +192,12 @@ __global__ void __launch_bounds__(VarSM<VAR>::T, VarSM<VAR>::B) k_hop_sm(const H
 }
 
 template <class SP, class LK, class CL, int MODE, int TS>
-cudaError_t launch_ts(bool pdl, int var, dim3 grid, dim3 b, int ngy, cudaStream_t st, const HopArgs<SP, LK, CL> &a)
+void launch_ts(bool pdl, int var, dim3 grid, dim3 b, int ngy, cudaStream_t st, const HopArgs<SP, LK, CL> &a)
 {
     switch (var) {
-        case 0: return launch_pdl(pdl, k_hop_sm<SP, LK, CL, MODE, TS, 0>, grid, b, st, a, ngy);
-        case 1: return launch_pdl(pdl, k_hop_sm<SP, LK, CL, MODE, TS, 1>, grid, b, st, a, ngy);
-        default: return launch_pdl(pdl, k_hop_sm<SP, LK, CL, MODE, TS, 2>, grid, b, st, a, ngy);
+        case 0: launch_pdl(pdl, k_hop_sm<SP, LK, CL, MODE, TS, 0>, grid, b, st, a, ngy); break;
+        case 1: launch_pdl(pdl, k_hop_sm<SP, LK, CL, MODE, TS, 1>, grid, b, st, a, ngy); break;
+        default: launch_pdl(pdl, k_hop_sm<SP, LK, CL, MODE, TS, 2>, grid, b, st, a, ngy); break;
     }
 }
 
@@ -210,15 +210,14 @@ lqcd_status launch_hop_sm(lqcd_ctx *c, int var, dim3 b, const HopArgs<SP, LK, CL
     const long nb = (long)div_up(c->g.Vh, b.x) * ngy;
     if (nb > 0x7fffffffL) return set_err(c, LQCD_ERR_ARG, "staged stencil: grid of %ld CTAs", nb);
     const dim3 g((unsigned)nb, hop_grid_y<MODE>());
-    cudaError_t e;
     if (b.x == 16)
-        e = launch_ts<SP, LK, CL, MODE, 16>(!c->capturing, var, g, b, ngy, c->stream, a);
+        launch_ts<SP, LK, CL, MODE, 16>(!c->capturing, var, g, b, ngy, c->stream, a);
     else if (b.x == 32)
-        e = launch_ts<SP, LK, CL, MODE, 32>(!c->capturing, var, g, b, ngy, c->stream, a);
+        launch_ts<SP, LK, CL, MODE, 32>(!c->capturing, var, g, b, ngy, c->stream, a);
     else
         return set_err(c, LQCD_ERR_ARG, "staged stencil: tile of %d sites", (int)b.x);
     c->n_kernel_launches++;
-    LQCD_CUDA_CHECK(c, e);
+    LQCD_LAUNCH_CHECK(c);
     return LQCD_OK;
 }
 

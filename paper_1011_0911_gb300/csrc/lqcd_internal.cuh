@@ -361,13 +361,14 @@ inline long native_half_units(const lqcd_ctx *c, lqcd_prec p)   // in 16-byte un
 // -> 19.3 us.  Kernels must let the next one be set up only after their own wait:
 // signalled before it, the launches of a chain pile up on the SMs (43.6 us).  In
 // captured graphs plain launches are faster (CGNR on 8^4: 6.97 against 7.97 ms).
+// A launch that fails leaves its error for LQCD_LAUNCH_CHECK, as <<< >>> does.
 template <class... KP, class... A>
-inline cudaError_t launch_pdl_smem(bool pdl, void (*kernel)(KP...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+inline void launch_pdl_smem(bool pdl, void (*kernel)(KP...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                    A... args)
 {
     if (!pdl) {
         kernel<<<grid, block, smem, st>>>(args...);
-        return cudaGetLastError();
+        return;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -379,12 +380,12 @@ inline cudaError_t launch_pdl_smem(bool pdl, void (*kernel)(KP...), dim3 grid, d
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KP>(args)...);
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<KP>(args)...);
 }
 template <class... KP, class... A>
-inline cudaError_t launch_pdl(bool pdl, void (*kernel)(KP...), dim3 grid, dim3 block, cudaStream_t st, A... args)
+inline void launch_pdl(bool pdl, void (*kernel)(KP...), dim3 grid, dim3 block, cudaStream_t st, A... args)
 {
-    return launch_pdl_smem(pdl, kernel, grid, block, 0, st, args...);
+    launch_pdl_smem(pdl, kernel, grid, block, 0, st, args...);
 }
 __device__ __forceinline__ void after_previous()
 {
