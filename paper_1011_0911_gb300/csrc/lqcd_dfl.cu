@@ -621,6 +621,8 @@ __host__ __device__ __forceinline__ int lb_face_warps(const DBlk &B, int mu)
 {
     return B.wrap[mu] ? 0 : (B.vol / B.bs[mu] + 31) / 32;
 }
+// at most 4 x 16 warps of faces or 32 of sites (1024 sites in a block), NS_MAX vectors
+constexpr int LB_SMEM_MAX = 64 * (NS_MAX / LB_K) * 32 * sizeof(float);
 inline size_t lb_smem(const DBlk &B, int Ns)
 {
     int nf = 0;
@@ -2391,7 +2393,10 @@ lqcd_status lqcd_dfl_build(lqcd_ctx *c, const lqcd_dfl_params *p, const double *
     {
         const int ngl = div_up(p->Ns, LB_L);
         const size_t sm3 = lb_smem(B, p->Ns);
-        LQCD_CUDA_CHECK(c, cudaFuncSetAttribute(k_little_build32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3));
+        // set once, for all contexts and threads
+        static const cudaError_t attr =
+            cudaFuncSetAttribute(k_little_build32, cudaFuncAttributeMaxDynamicSharedMemorySize, LB_SMEM_MAX);
+        LQCD_CUDA_CHECK(c, attr);
         k_little_build32<<<3 * ngl * B.nblk, LB_THREADS, sm3, c->stream>>>(
             c->g, B, (const float4 *)d->phi, p->Ns, fe, c->U32, c->A32[0], c->A32[1], d->Aint, ngl);
     }

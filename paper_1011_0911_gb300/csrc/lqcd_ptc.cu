@@ -789,20 +789,37 @@ size_t wgrad_smem(int cin, int cout)
            (size_t)PT_ROWS * 4 * cout * sizeof(cx<float>);
 }
 
+using LayerBf = void (*)(LayerArgs, int, int);
+LayerBf layer_bf(int cin, int cout)   // lqcd_net_set takes 1 or 2 channels
+{
+    static const LayerBf k[2][2] = {{k_ptc_layer_bf<1, 1>, k_ptc_layer_bf<1, 2>},
+                                    {k_ptc_layer_bf<2, 1>, k_ptc_layer_bf<2, 2>}};
+    return k[cin - 1][cout - 1];
+}
+// The most shared memory that each layer kernel takes, set once: the limit belongs to the
+// kernel, so to all contexts and threads of the process, and one that was set for a call
+// could be lowered by another thread before that call's launch.
+cudaError_t layer_limits()
+{
+    static const cudaError_t err = [] {
+        const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        cudaError_t e = cudaFuncSetAttribute(k_ptc_layer_f32, attr, (int)layer_smem(LQCD_F32, 2, 2));
+        for (int ci = 1; ci <= 2; ci++)
+            for (int co = 1; co <= 2; co++)
+                if (e == cudaSuccess)
+                    e = cudaFuncSetAttribute(layer_bf(ci, co), attr, (int)layer_smem(LQCD_BF16, ci, co));
+        return e;
+    }();
+    return err;
+}
+
 template <class ACT>
 lqcd_status launch_layer(lqcd_ctx *c, const void *in, void *out, int cin, int cout, int nb, const bf16 *Bt,
                          const float2 *Wc)
 {
     constexpr bool BF = sizeof(ACT) == 4;
-    void (*kbf)(LayerArgs, int, int) = nullptr;
-    if (BF) {
-        static void (*const bf[2][2])(LayerArgs, int, int) = {{k_ptc_layer_bf<1, 1>, k_ptc_layer_bf<1, 2>},
-                                                    {k_ptc_layer_bf<2, 1>, k_ptc_layer_bf<2, 2>}};
-        kbf = bf[cin - 1][cout - 1];   // lqcd_net_set takes 1 or 2 channels
-    }
+    LQCD_CUDA_CHECK(c, layer_limits());
     const size_t smem = layer_smem(BF ? LQCD_BF16 : LQCD_F32, cin, cout);
-    LQCD_CUDA_CHECK(c, cudaFuncSetAttribute(BF ? (const void *)kbf : (const void *)k_ptc_layer_f32,
-                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     LayerArgs a;
     a.g = c->g;
     a.U = c->U32;
@@ -818,7 +835,7 @@ lqcd_status launch_layer(lqcd_ctx *c, const void *in, void *out, int cin, int co
     if (BF) {
         // samples per CTA while about four waves of three CTAs per SM remain
         const int spc = std::max(1, std::min(nb, (int)((long)tiles * nb / (12 * 152))));
-        kbf<<<dim3(tiles, div_up(nb, spc)), PT_THREADS, smem, c->stream>>>(a, nb, spc);
+        layer_bf(cin, cout)<<<dim3(tiles, div_up(nb, spc)), PT_THREADS, smem, c->stream>>>(a, nb, spc);
     } else {
         k_ptc_layer_f32<<<dim3(tiles, nb), PT_THREADS, smem, c->stream>>>(a);
     }
