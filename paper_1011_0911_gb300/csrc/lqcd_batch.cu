@@ -373,13 +373,13 @@ __global__ void k_b_restart(const BLat *lat, const double2 *part, int *act, BSca
     S.rn2 = s.x;
     S.nk = 0;
     if (S.iters > 0) S.restarts++;
-    if (!(s.x > S.tol2)) {
-        S.done = 1;
-        S.status = LQCD_OK;
-        act[l] = 0;
-    } else if (!isfinite(s.x)) {
+    if (!isfinite(s.x)) {   // also where the source, and so tol2, is not finite
         S.done = 1;
         S.status = LQCD_ERR_NAN;
+        act[l] = 0;
+    } else if (s.x <= S.tol2) {
+        S.done = 1;
+        S.status = LQCD_OK;
         act[l] = 0;
     } else {
         S.cyc_tol2 = fmax(S.tol2, s.x * gain2);
