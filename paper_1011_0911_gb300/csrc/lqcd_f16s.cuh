@@ -65,8 +65,12 @@ __device__ __forceinline__ float f16s_maxabs(const cx<float> *v, int n)
     return m;
 }
 // 1 / scale of a site whose largest |real part| is m; 0 (the site is stored as zero)
-// below float's normal range, where 1 / m overflows and would leave NaN
-__device__ __forceinline__ float f16s_inv(float m) { return m >= 1.17549435e-38f ? 1.f / m : 0.f; }
+// where 1 / m overflows, at m of 2^-128 or less, and would leave NaN
+__device__ __forceinline__ float f16s_inv(float m)
+{
+    const float inv = 1.f / m;
+    return inv <= 3.40282347e38f ? inv : 0.f;
+}
 __device__ __forceinline__ void f16s_store(h16s *f, long Vh, long r, const cx<float> v[12])
 {
     float m = 0.f;
