@@ -1657,6 +1657,15 @@ lqcd_status sap_operator(lqcd_ctx *c, SapPlan &pl, SapArgs<P> &a)
     a.Ub = a.U;
     a.Aeb = a.Ae;
     a.Aiob = a.Aio;
+    // A caller's graph reads the lattice-ordered arrays (the same bits): replayed after
+    // the links have changed it would find the copy of the operator it was captured
+    // with, and a copy recorded here would not be made before the next eager call.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) {
+        cudaGetLastError();   // the legacy stream, while another one is captured
+        cap = cudaStreamCaptureStatusNone;
+    }
+    if (cap != cudaStreamCaptureStatusNone) return LQCD_OK;
     if (!pm.p && !pm.failed) {
         if (cudaMalloc(&pm.p, (24 + 2 * 18) * Vh * sizeof(LK)) != cudaSuccess) {
             cudaGetLastError();
