@@ -181,7 +181,7 @@ LQCD_API lqcd_status lqcd_apply_Dhat_native_static(lqcd_ctx *ctx, lqcd_prec prec
 /* Autotuner of launch shapes and kernel forms (the paper has no counterpart;
  * the kernels' results do not depend on the choice).  The first call with a
  * new key -- kernel, mode, precision, number of right-hand sides, lattice
- * extents, GPU name -- times every candidate (stencil: occupancy variant,
+ * extents, GPU name, generation of the kernels -- times every candidate (stencil: occupancy variant,
  * CTA shape, fields per thread, kernel form; SAP: clover staged in shared
  * memory or read through L1, timed over the sweeps of the first
  * application; batched solver: tile size) with CUDA events on the context's

@@ -83,6 +83,10 @@ void save_locked()
 
 }  // namespace
 
+// Part of every key: raised when the kernels behind the keys change, so that timings of
+// older ones in a cache file decide nothing.
+constexpr int KERNELS = 2;
+
 std::string tune_key(const lqcd_ctx *c, const char *kernel, int mode, int prec, int nrhs)
 {
     if (g_gpu.empty()) {
@@ -95,7 +99,7 @@ std::string tune_key(const lqcd_ctx *c, const char *kernel, int mode, int prec, 
     }
     std::ostringstream s;
     s << kernel << "/m" << mode << "/p" << prec << "/n" << nrhs << "/" << c->g.L[0] << "x" << c->g.L[1] << "x"
-      << c->g.L[2] << "x" << c->g.L[3] << "/" << g_gpu;
+      << c->g.L[2] << "x" << c->g.L[3] << "/" << g_gpu << "/k" << KERNELS;
     return s.str();
 }
 
