@@ -8,12 +8,19 @@
 // the stopping test runs on the device, and the host stays ahead: an iteration
 // past the end finds the state closed and changes nothing.  gamma5 is applied in
 // the updates, so that Dhat^dag = gamma5 Dhat gamma5 costs no pass of its own.
-// On lattices whose iterations take less than the eight launches do
-// (CG_GRAPH_SITES), four iterations are captured as a graph for the solve and
-// replayed, on a stream of the context's own (a legacy default stream cannot be
-// captured); elsewhere the host runs two iterations ahead with plain launches.
-// Measured on 8^4 (131 iterations): 16.0 -> 7.0 ms (plain launches 7.8 ms; with
-// the state copied to the host instead of written there 8.7 ms).
+//
+// An iteration past the end still costs its two Dhat, so the host sends one unit
+// (an iteration, or a graph) beyond the one it waits for, and only while the mean
+// decay of the residual so far puts the end behind it: solves of one to four
+// iterations took up to twice the time with two units always ahead (16384 even
+// sites, one iteration: 1820 us; 549 us now; 861 us with the scalars on the host).
+// On lattices of up to CG_GRAPH_SITES even sites, where launching takes as long as
+// the kernels, four iterations are captured as a graph once CG_GRAPH_FROM are
+// expected, on a stream of the context's own (a legacy default stream cannot be
+// captured).  Making the graph takes about 250 us; an iteration costs, with plain
+// launches / in graphs, at 2048 even sites 61 / 50 us, 4096 98 / 74, 8192 173 / 120,
+// 16384 220 / 205.  131 iterations on 8^4: 16.0 -> 6.9 ms (with the state copied to the
+// host instead of written there 8.7 ms).
 #include <cmath>
 
 #include "lqcd_internal.cuh"
@@ -21,9 +28,9 @@
 namespace {
 
 constexpr int CG_THREADS = 256;
-constexpr int CG_AHEAD = 2;     // iterations launched beyond the last one seen (plain launches)
 constexpr int CG_RING = 4;      // states in flight; iterations of a graph
 constexpr int CG_GRAPH_SITES = 16384;   // even sites
+constexpr int CG_GRAPH_FROM = 16;       // iterations still to come
 
 enum { CG_RUN = 0, CG_BELOW, CG_BREAKDOWN, CG_NAN };
 
@@ -144,7 +151,7 @@ __global__ void __launch_bounds__(CG_THREADS) k_cg_p(long n, int nb, const CgSta
 namespace {
 
 struct CgEvents {
-    cudaEvent_t e[CG_RING] = {};
+    cudaEvent_t e[2] = {};
     ~CgEvents()
     {
         for (cudaEvent_t v : e)
@@ -157,7 +164,7 @@ struct CgStream {
     cudaStream_t user;
     cudaEvent_t ev = nullptr;
     cudaGraphExec_t graph = nullptr;
-    bool on = false;
+    bool on = false, failed = false;
     explicit CgStream(lqcd_ctx *ctx) : c(ctx), user(ctx->stream) {}
     lqcd_status enter()
     {
@@ -226,6 +233,28 @@ lqcd_status cgnr_native(lqcd_ctx *c, const double2 *eta, double2 *x, double tol,
         LQCD_LAUNCH_CHECK(c);
         return LQCD_OK;
     };
+    // CG_RING iterations as a graph; without it plain launches serve
+    auto make_graph = [&]() -> lqcd_status {
+        cudaGraph_t g = nullptr;
+        const long before = c->n_kernel_launches;
+        c->capturing = true;
+        lqcd_status cs = LQCD_OK;
+        bool ok = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+        if (ok) {
+            for (int i = 0; i < CG_RING && cs == LQCD_OK; i++) cs = iteration(i);
+            ok = cudaStreamEndCapture(c->stream, &g) == cudaSuccess && cs == LQCD_OK && g &&
+                 cudaGraphInstantiate(&own.graph, g, 0) == cudaSuccess;
+        }
+        c->capturing = false;
+        c->n_kernel_launches = before;   // recorded, not run
+        if (g) cudaGraphDestroy(g);
+        if (!ok) {
+            cudaGetLastError();
+            own.graph = nullptr;
+            own.failed = true;
+        }
+        return LQCD_OK;
+    };
     int it = 0;
     lqcd_status st = LQCD_ERR_NOT_CONVERGED;
     double rr = eta2;
@@ -244,62 +273,52 @@ lqcd_status cgnr_native(lqcd_ctx *c, const double2 *eta, double2 *x, double tol,
             H[CG_RING] = s0;
             LQCD_CUDA_CHECK(c, cudaMemcpyAsync(S, H + CG_RING, sizeof(CgState), cudaMemcpyHostToDevice, c->stream));
             const long limit = (long)nmx - it;
-            long seen = 0;
+            const double rr0 = rr;
             CgState last = s0;
-            // whole graphs of CG_RING iterations within the limit, one beyond the last one seen
-            if (own.on && limit >= CG_RING && !own.graph) {
-                cudaGraph_t g = nullptr;
-                const long before = c->n_kernel_launches;
-                c->capturing = true;
-                lqcd_status cs = LQCD_OK;
-                bool ok = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-                if (ok) {
-                    for (int i = 0; i < CG_RING && cs == LQCD_OK; i++) cs = iteration(i);
-                    ok = cudaStreamEndCapture(c->stream, &g) == cudaSuccess && cs == LQCD_OK && g &&
-                         cudaGraphInstantiate(&own.graph, g, 0) == cudaSuccess;
+            last.rr = rr0;
+            long sent = 0, seen = 0;   // iterations of this start launched / whose state is known
+            long end[2] = {0, 0};      // of the units in flight: a graph, or one iteration
+            int first = 0, flying = 0;
+            // Iterations still to come by the mean decay so far (CGNR's residual never
+            // grows; its decay slows down, so the estimate is rather too small).
+            auto left = [&]() -> double {
+                const int k = last.iters - s0.iters;
+                const double d = k > 0 ? std::log(rr0 / last.rr) : 0;
+                return d > 0 ? k * std::log(last.rr / tol2) / d : 0;
+            };
+            auto send = [&]() -> lqcd_status {
+                const double more = std::min(left(), (double)(limit - seen)) - (sent - seen);
+                if (own.on && !own.graph && !own.failed && more >= CG_GRAPH_FROM) LQCD_TRY(make_graph());
+                if (own.graph && sent % CG_RING == 0 && more >= CG_RING) {
+                    LQCD_CUDA_CHECK(c, cudaGraphLaunch(own.graph, c->stream));
+                    c->n_kernel_launches += 8 * CG_RING;
+                    sent += CG_RING;
+                } else {
+                    LQCD_TRY(iteration(sent));
+                    sent++;
                 }
-                c->capturing = false;
-                c->n_kernel_launches = before;   // recorded, not run
-                if (g) cudaGraphDestroy(g);
-                if (!ok) {
-                    cudaGetLastError();
-                    own.graph = nullptr;   // plain launches serve
-                }
-            }
-            // (a graph is kept for later starts; one with fewer iterations left than a graph
-            // holds runs plainly: nothing would be sent, and H still has the start before)
-            if (own.graph && limit >= CG_RING) {
-                const long graphs = limit / CG_RING;
-                long done = 0, sent = 0;
-                while (last.code == CG_RUN && done < graphs) {
-                    // one graph beyond the one waited for.  It may already have
-                    // overwritten the host copy that is read: a later state of the
-                    // same solve, and a closed one stays as it is.
-                    for (; sent < std::min(graphs, done + 2); sent++) {
-                        LQCD_CUDA_CHECK(c, cudaGraphLaunch(own.graph, c->stream));
-                        LQCD_CUDA_CHECK(c, cudaEventRecord(ev.e[sent % CG_RING], c->stream));
-                        c->n_kernel_launches += 8 * CG_RING;
-                    }
-                    LQCD_CUDA_CHECK(c, cudaEventSynchronize(ev.e[done % CG_RING]));
-                    done++;
-                    last.code = ((volatile CgState *)H)[CG_RING - 1].code;
-                }
-                LQCD_CUDA_CHECK(c, cudaStreamSynchronize(c->stream));
-                last = H[CG_RING - 1];
-                seen = sent * CG_RING;
-            }
-            long launched = seen;
+                const int u = (first + flying++) % 2;
+                end[u] = sent;
+                LQCD_CUDA_CHECK(c, cudaEventRecord(ev.e[u], c->stream));
+                return LQCD_OK;
+            };
             while (last.code == CG_RUN && seen < limit) {
-                while (launched < seen + 1 + CG_AHEAD && launched < limit) {
-                    LQCD_TRY(iteration(launched));
-                    LQCD_CUDA_CHECK(c, cudaEventRecord(ev.e[launched % CG_RING], c->stream));
-                    launched++;
-                }
-                LQCD_CUDA_CHECK(c, cudaEventSynchronize(ev.e[seen % CG_RING]));
-                last = H[seen % CG_RING];
-                seen++;
+                if (flying == 0) LQCD_TRY(send());
+                // a second unit while the end is expected behind the first
+                if (flying == 1 && sent < limit && left() >= (double)(sent - seen + 1)) LQCD_TRY(send());
+                LQCD_CUDA_CHECK(c, cudaEventSynchronize(ev.e[first]));
+                seen = end[first];
+                first = (first + 1) % 2;
+                flying--;
+                // a graph in flight may have overwritten it: with a later state of this
+                // start, and a closed one stays as it is
+                volatile CgState *h = H + (seen - 1) % CG_RING;
+                last.code = h->code;
+                last.rr = h->rr;
+                last.iters = h->iters;
             }
             LQCD_CUDA_CHECK(c, cudaStreamSynchronize(c->stream));   // iterations past the end are no-ops
+            last = H[(sent - 1) % CG_RING];
             const bool moved = last.iters > it;
             it = last.iters;
             rr = last.rr;
