@@ -181,10 +181,11 @@ LQCD_API lqcd_status lqcd_apply_Dhat_native_static(lqcd_ctx *ctx, lqcd_prec prec
 /* Autotuner of launch shapes and kernel forms (the paper has no counterpart;
  * the kernels' results do not depend on the choice).  The first call with a
  * new key -- kernel, mode, precision, number of right-hand sides, lattice
- * extents, GPU name, generation of the kernels -- times every candidate (stencil: occupancy variant,
- * CTA shape, fields per thread, kernel form; SAP: clover staged in shared
- * memory or read through L1, timed over the sweeps of the first
- * application; batched solver: tile size) with CUDA events on the context's
+ * extents, GPU name, generation of the kernels -- times every candidate
+ * (stencil: occupancy variant, CTA shape, fields per thread, kernel form, and
+ * for D and Dhat whether their kernels are launched dependently; SAP: clover
+ * staged in shared memory or read through L1, timed over the sweeps of the
+ * first application; batched solver: tile size) with CUDA events on the context's
  * stream, keeps the fastest and appends it to the cache file
  * $LQCD_TUNE_CACHE (default $HOME/.cache/lqcd_tune.json; one line per key:
  * "key": [variant, tx, ty, microseconds, fields per thread, kind]), so later

@@ -131,7 +131,7 @@ lqcd_status launch_var(lqcd_ctx *c, int var, dim3 b, const HopArgs<SP, LK, CL> &
     const long nb = (long)div_up(c->g.Vh, b.x) * ngy;
     if (nb > 0x7fffffffL) return set_err(c, LQCD_ERR_ARG, "stencil: grid of %ld CTAs", nb);
     const dim3 grid((unsigned)nb, hop_grid_y<MODE>());
-    const bool pdl = !c->capturing;
+    const bool pdl = c->hop_dep && !c->capturing;
     switch (var) {
         case 0: launch_pdl(pdl, k_hop<R, SP, LK, CL, MODE, 0>, grid, b, c->stream, a, ngy); break;
         case 1: launch_pdl(pdl, k_hop<R, SP, LK, CL, MODE, 1>, grid, b, c->stream, a, ngy); break;
@@ -292,7 +292,7 @@ lqcd_status launch_hop(lqcd_ctx *c, int p_out, const SP *in_other, long in_rs, c
                                       {"k_hop_dx2", "k_hop_d1x2", "k_hop_d2x2", "", "k_hop_d4x2"}};
     constexpr int both = MODE == MODE_D;
     const int split = dbl ? hop_force_split() : 0;
-    TuneMemo &memo = c->tune[MODE][prec][p_out];
+    TuneMemo &memo = c->tune[MODE][prec][p_out][nrhs % TUNE_SLOTS];
     const int forced = dbl ? 16 + split : force;
     TuneChoice tc;
     if (memo.gen == tune_generation() && memo.nrhs == nrhs && memo.force == forced) {
@@ -359,43 +359,88 @@ lqcd_status launch_hop(lqcd_ctx *c, int p_out, const SP *in_other, long in_rs, c
 
 }  // namespace
 
+// Dependent launches (launch_pdl) are a choice for each operator, precision, number of
+// fields and lattice.  They hide the set-up of a kernel's CTAs behind the kernel
+// before; but the CTAs set up early go to the SMs that are through first, so a kernel
+// of about one wave may have several CTAs on some SMs and none on others.  Plain /
+// dependent, us an application in a run: FP64 Dhat, one field, 2048 even sites 20.5 / 15.3,
+// 8192 45 / 60, 16384 82 / 78; F16S, three fields, 23520 even sites 20.5 / 25.2 or 15.4 by
+// the kernels' forms.  So a run of applications is timed both ways once the forms are
+// settled (0.3 ms to 15 ms on the first call); above DEP_LONG_US an application the
+// difference is below 1 % and the launches are dependent.  Over 126 operators and sizes
+// the choice is 1.2 % faster than dependent launches throughout, at most 17 % where
+// those lost.
+constexpr float DEP_LONG_US = 300.f;
+enum { OP_DHAT = 0, OP_D = 1 };
+namespace {
+template <class Run>
+lqcd_status run_operator(lqcd_ctx *c, int op, lqcd_prec p, int nrhs, Run run)
+{
+    DepMemo &m = c->dep[op][p][nrhs % TUNE_SLOTS];
+    c->hop_dep = true;
+    if (m.gen == tune_generation() && m.nrhs == nrhs) {
+        c->hop_dep = m.dep;
+        return run();
+    }
+    const std::string key = tune_key(c, "k_hop_dep", op, (int)p, nrhs);
+    TuneChoice t;
+    if (!tune_lookup(key, &t)) {
+        if (!tune_enabled()) return run();
+        LQCD_TRY(run());   // settles the forms
+        float us, best[2] = {1e30f, 1e30f};
+        LQCD_TRY(tune_time(c, run, 1, &us));
+        constexpr int N = 6;   // applications in a run
+        for (int rep = 0; rep < 4 && us < DEP_LONG_US; rep++) {
+            c->hop_dep = rep & 1;
+            LQCD_TRY(tune_time(
+                c,
+                [&]() -> lqcd_status {
+                    for (int i = 0; i < N; i++) LQCD_TRY(run());
+                    return LQCD_OK;
+                },
+                1, &us));
+            us /= N;
+            if (tune_verbose()) fprintf(stderr, "tune %s: dependent=%d %.1f us\n", key.c_str(), rep & 1, us);
+            best[rep & 1] = std::min(best[rep & 1], us);
+        }
+        t.variant = best[1] <= 1.01f * best[0];
+        t.us = std::min(us, best[t.variant]);
+        tune_store(key, t);
+    }
+    m = DepMemo{tune_generation(), nrhs, t.variant != 0};
+    c->hop_dep = m.dep;
+    return run();
+}
+template <class R, class SP, class LK, class CL>
+lqcd_status launch_dhat(lqcd_ctx *c, lqcd_prec p, const void *in, long in_rs, void *out, long out_rs, void *tmp_o,
+                        const LK *U, const CL *Aio, const CL *Ae, int nrhs)
+{
+    auto *i = (const SP *)in;
+    auto *o = (SP *)out;
+    auto *t = (SP *)tmp_o;
+    const long rs = native_half_units(c, p);
+    return run_operator(c, OP_DHAT, p, nrhs, [&]() -> lqcd_status {
+        LQCD_TRY((launch_hop<R, SP, LK, CL, MODE_DHAT1>(c, 1, i, in_rs, nullptr, 0, t, rs, U, Aio, nrhs)));
+        return launch_hop<R, SP, LK, CL, MODE_DHAT2>(c, 0, t, rs, i, in_rs, o, out_rs, U, Ae, nrhs);
+    });
+}
+}  // namespace
+
 // Dhat on native half fields: in / out even, in_rs / out_rs units apart per rhs
 // (native units: double2, float4, h16s); tmp_o: nrhs odd half fields one after the other.
 lqcd_status dirac_dhat_s(lqcd_ctx *c, lqcd_prec p, const void *in, long in_rs, void *out, long out_rs, void *tmp_o,
                          int nrhs)
 {
     if (!c->have_clover) return set_err(c, LQCD_ERR_STATE, "clover term not built");
-    const long rs = native_half_units(c, p);
-    if (p == LQCD_F64) {
-        auto *i = (const double2 *)in;
-        auto *o = (double2 *)out;
-        auto *t = (double2 *)tmp_o;
-        LQCD_TRY((launch_hop<double, double2, double2, double2, MODE_DHAT1>(
-            c, 1, i, in_rs, nullptr, 0, t, rs, c->U64, c->Ai64[1], nrhs)));
-        LQCD_TRY((launch_hop<double, double2, double2, double2, MODE_DHAT2>(
-            c, 0, t, rs, i, in_rs, o, out_rs, c->U64, c->A64[0], nrhs)));
-        return LQCD_OK;
-    }
-    if (p == LQCD_F32) {
-        auto *i = (const float4 *)in;
-        auto *o = (float4 *)out;
-        auto *t = (float4 *)tmp_o;
-        LQCD_TRY((launch_hop<float, float4, float4, float4, MODE_DHAT1>(
-            c, 1, i, in_rs, nullptr, 0, t, rs, c->U32, c->Ai32[1], nrhs)));
-        LQCD_TRY((launch_hop<float, float4, float4, float4, MODE_DHAT2>(
-            c, 0, t, rs, i, in_rs, o, out_rs, c->U32, c->A32[0], nrhs)));
-        return LQCD_OK;
-    }
-    if (p == LQCD_F16S) {
-        auto *i = (const h16s *)in;
-        auto *o = (h16s *)out;
-        auto *t = (h16s *)tmp_o;
-        LQCD_TRY((launch_hop<float, h16s, uint2, uint2, MODE_DHAT1>(c, 1, i, in_rs, nullptr, 0, t, rs, c->U16,
-                                                                    c->Ai16[1], nrhs)));
-        LQCD_TRY((launch_hop<float, h16s, uint2, uint2, MODE_DHAT2>(c, 0, t, rs, i, in_rs, o, out_rs, c->U16,
-                                                                    c->A16[0], nrhs)));
-        return LQCD_OK;
-    }
+    if (p == LQCD_F64)
+        return launch_dhat<double, double2, double2, double2>(c, p, in, in_rs, out, out_rs, tmp_o, c->U64, c->Ai64[1],
+                                                              c->A64[0], nrhs);
+    if (p == LQCD_F32)
+        return launch_dhat<float, float4, float4, float4>(c, p, in, in_rs, out, out_rs, tmp_o, c->U32, c->Ai32[1],
+                                                          c->A32[0], nrhs);
+    if (p == LQCD_F16S)
+        return launch_dhat<float, h16s, uint2, uint2>(c, p, in, in_rs, out, out_rs, tmp_o, c->U16, c->Ai16[1],
+                                                      c->A16[0], nrhs);
     return set_err(c, LQCD_ERR_ARG, "precision %d not supported for Dhat", (int)p);
 }
 lqcd_status dirac_dhat(lqcd_ctx *c, lqcd_prec p, const void *in, void *out, void *tmp_o, int nrhs)
@@ -409,22 +454,24 @@ lqcd_status dirac_dhat(lqcd_ctx *c, lqcd_prec p, const void *in, void *out, void
 // filled wave (FP32, 28 x 12 x 10 x 14, 5 fields: two launches of 16.3 us -> 27.6 us).
 namespace {
 template <class R, class SP, class LK, class CL>
-lqcd_status launch_D(lqcd_ctx *c, const void *in, void *out, long h, const LK *U, CL *const A[2], int nrhs)
+lqcd_status launch_D(lqcd_ctx *c, lqcd_prec p, const void *in, void *out, const LK *U, CL *const A[2], int nrhs)
 {
     auto *i = (const SP *)in;
     auto *o = (SP *)out;
-    return launch_hop<R, SP, LK, CL, MODE_D>(c, 0, i + h, 2 * h, i, 2 * h, o, 2 * h, U, A[0], nrhs, i, i + h, o + h,
-                                             A[1]);
+    const long h = native_half_units(c, p);
+    return run_operator(c, OP_D, p, nrhs, [&]() {
+        return launch_hop<R, SP, LK, CL, MODE_D>(c, 0, i + h, 2 * h, i, 2 * h, o, 2 * h, U, A[0], nrhs, i, i + h,
+                                                 o + h, A[1]);
+    });
 }
 }  // namespace
 
 lqcd_status dirac_D(lqcd_ctx *c, lqcd_prec p, const void *in, void *out, int nrhs)
 {
     if (!c->have_clover) return set_err(c, LQCD_ERR_STATE, "clover term not built");
-    const long h = native_half_units(c, p);
-    if (p == LQCD_F64) return launch_D<double, double2, double2, double2>(c, in, out, h, c->U64, c->A64, nrhs);
-    if (p == LQCD_F32) return launch_D<float, float4, float4, float4>(c, in, out, h, c->U32, c->A32, nrhs);
-    if (p == LQCD_F16S) return launch_D<float, h16s, uint2, uint2>(c, in, out, h, c->U16, c->A16, nrhs);
+    if (p == LQCD_F64) return launch_D<double, double2, double2, double2>(c, p, in, out, c->U64, c->A64, nrhs);
+    if (p == LQCD_F32) return launch_D<float, float4, float4, float4>(c, p, in, out, c->U32, c->A32, nrhs);
+    if (p == LQCD_F16S) return launch_D<float, h16s, uint2, uint2>(c, p, in, out, c->U16, c->A16, nrhs);
     return set_err(c, LQCD_ERR_ARG, "precision %d not supported for D", (int)p);
 }
 
@@ -432,6 +479,7 @@ lqcd_status dirac_D(lqcd_ctx *c, lqcd_prec p, const void *in, void *out, int nrh
 lqcd_status dirac_hop_parity(lqcd_ctx *c, lqcd_prec p, int p_out, const void *in_other, void *out,
                              long in_rstride, long out_rstride, int nrhs)
 {
+    c->hop_dep = true;
     if (p == LQCD_F64)
         return launch_hop<double, double2, double2, double2, MODE_HOP>(
             c, p_out, (const double2 *)in_other, in_rstride, nullptr, 0, (double2 *)out, out_rstride,

@@ -329,7 +329,7 @@ lqcd_status launch_d(lqcd_ctx *c, int G, const HopArgs<double2, double2, double2
     const long nb = (long)div_up(c->g.Vh, sites) * a.nrhs;
     if (nb > 0x7fffffffL) return set_err(c, LQCD_ERR_ARG, "FP64 stencil: grid of %ld CTAs", nb);
     const dim3 grid((unsigned)nb, hop_grid_y<MODE>());
-    const bool pdl = !c->capturing;
+    const bool pdl = c->hop_dep && !c->capturing;
     switch (G) {
         case 1: launch_pdl(pdl, k_hop_d<MODE, 1, BLK>, grid, HOP_D_THREADS, c->stream, a, bx); break;
         case 2: launch_pdl(pdl, k_hop_d<MODE, 2, BLK>, grid, HOP_D_THREADS, c->stream, a, bx); break;
@@ -356,6 +356,7 @@ lqcd_status launch_dhat_block_d(lqcd_ctx *c, const int bs[4], const double2 *in,
     a.in_rs = a.same_rs = a.out_rs = 0;
     a.U = c->U64;
     const BlkExt bx = {{bs[0], bs[1], bs[2], bs[3]}};
+    c->hop_dep = true;
     // as the untuned rule of the lattice-wide operator
     const int G = c->g.Vh >= 16 * 1216 ? 1 : (c->g.Vh >= 16 * 608 ? 2 : 4);
     a.p_out = 1;

@@ -203,9 +203,9 @@ lqcd_status launch_hop_mr(lqcd_ctx *c, int nr, int var, dim3 b, const HopArgs<SP
     if (grid > 0x7fffffffL) return set_err(c, LQCD_ERR_ARG, "blocked stencil: grid of %ld CTAs", grid);
     const dim3 g((unsigned)grid, hop_grid_y<MODE>());
     if (nr == 2)
-        launch_nr<R, SP, LK, CL, MODE, 2>(!c->capturing, var, g, b, ngy, c->stream, a);
+        launch_nr<R, SP, LK, CL, MODE, 2>(c->hop_dep && !c->capturing, var, g, b, ngy, c->stream, a);
     else if (nr == 3)
-        launch_nr<R, SP, LK, CL, MODE, 3>(!c->capturing, var, g, b, ngy, c->stream, a);
+        launch_nr<R, SP, LK, CL, MODE, 3>(c->hop_dep && !c->capturing, var, g, b, ngy, c->stream, a);
     else
         return set_err(c, LQCD_ERR_ARG, "no blocked stencil for %d fields per thread", nr);
     c->n_kernel_launches++;

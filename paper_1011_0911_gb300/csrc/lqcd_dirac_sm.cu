@@ -211,9 +211,9 @@ lqcd_status launch_hop_sm(lqcd_ctx *c, int var, dim3 b, const HopArgs<SP, LK, CL
     if (nb > 0x7fffffffL) return set_err(c, LQCD_ERR_ARG, "staged stencil: grid of %ld CTAs", nb);
     const dim3 g((unsigned)nb, hop_grid_y<MODE>());
     if (b.x == 16)
-        launch_ts<SP, LK, CL, MODE, 16>(!c->capturing, var, g, b, ngy, c->stream, a);
+        launch_ts<SP, LK, CL, MODE, 16>(c->hop_dep && !c->capturing, var, g, b, ngy, c->stream, a);
     else if (b.x == 32)
-        launch_ts<SP, LK, CL, MODE, 32>(!c->capturing, var, g, b, ngy, c->stream, a);
+        launch_ts<SP, LK, CL, MODE, 32>(c->hop_dep && !c->capturing, var, g, b, ngy, c->stream, a);
     else
         return set_err(c, LQCD_ERR_ARG, "staged stencil: tile of %d sites", (int)b.x);
     c->n_kernel_launches++;

@@ -224,10 +224,18 @@ struct Workspace {
 // the autotuner's choice for a stencil launch, kept with the context while nothing
 // it depends on changes (building and looking up its key took longer than the
 // launch)
+constexpr int TUNE_SLOTS = 4;   // calls with one and with several right-hand sides take turns
 struct TuneMemo {
     long gen = -1;      // generation of the tuner's table
     int nrhs = 0, force = 0;
     int variant = 0, tx = 0, ty = 0, nr = 0, kind = 0;
+};
+
+// the same for an operator: are its kernels launched dependently?
+struct DepMemo {
+    long gen = -1;
+    int nrhs = 0;
+    bool dep = true;
 };
 
 struct DflState;   // deflation subspace (lqcd_dfl.cu)
@@ -262,7 +270,9 @@ struct lqcd_ctx {
     NetState *net = nullptr;
     ChronoState *chrono = nullptr;
     long n_kernel_launches = 0;
-    TuneMemo tune[4][3][2];   // [mode][precision][output parity]
+    TuneMemo tune[4][3][2][TUNE_SLOTS];   // [mode][precision][output parity][nrhs % TUNE_SLOTS]
+    DepMemo dep[2][3][TUNE_SLOTS];        // [Dhat, D][precision][nrhs % TUNE_SLOTS]
+    bool hop_dep = true;      // the choice for the stencil launches of the operator under way
     bool capturing = false;               // launches go into a graph being captured
     cudaStream_t cg_stream = nullptr;     // CGNR on small lattices (lqcd_cgnr.cu)
     // LQCD_PROFILE=1: synchronised wall time of solver phases, reported on
