@@ -1790,12 +1790,14 @@ lqcd_status sap_run(lqcd_ctx *c, SapPlan &P_, int ncy, int nmr, const void *eta,
     // the residual is not needed after the last sweep
     int last_col = Pl.count[1] > 0 ? 1 : 0;
     int sweep = 0;
-    // Dependent launches where the blocks of a sweep are at most one wave (three CTAs
-    // an SM): there launch and staging are a part of a sweep's time (500 sweeps of 256
-    // blocks at 32 x 16^3: 49.9 -> 48.4 ms).  Over many waves the CTAs that are set up
-    // early only get in the way of the kernel before (48 x 24^3 with 12 right-hand
-    // sides, 15552 blocks a sweep: 3.1 ms a sweep plain, 3.5 ms dependent).
-    const bool dependent = !c->capturing && (long)std::max(Pl.count[0], Pl.count[1]) * nrhs <= 3 * 152;
+    // Dependent launches hide launch and staging, a part of a short sweep's time, but the
+    // CTAs set up early go to the SMs that the kernel before leaves first.  Eight steps of
+    // a GCR, 4 x 5 sweeps each, dependent / plain, by CTAs a sweep: FP32 8 to 128 0.90 to
+    // 0.93, 192 to 400 0.96 to 1.03 (0.98 at 32 x 16^3, one field), 576 to 6000 0.99 to 1.03;
+    // F16S (three CTAs an SM, so the packing is the tightest) 8 to 128 0.91 to 0.93, 192 0.97
+    // to 1.00, 243 1.22, 256 1.20, 384 to 6000 1.02 to 1.10.  FP64 (faces only): 0.996.
+    const long sweep_ctas = (long)std::max(Pl.count[0], Pl.count[1]) * nrhs;
+    const bool dependent = !c->capturing && sweep_ctas <= (P == LQCD_F16S ? 152 : 3 * 152);
     for (int cyc = 0; cyc < ncy; cyc++)
         for (int col = 0; col < 2; col++) {
             if (Pl.count[col] == 0) continue;
