@@ -91,10 +91,10 @@ __device__ __forceinline__ void hop_site(const HopArgs<SP, LK, CL> &a, int r, in
 // so the CTAs of all fields of a site tile run next to each other and share
 // its links and clover term through L1/L2
 template <class R, class SP, class LK, class CL, int MODE, int VAR>
-__global__ void __launch_bounds__(Var<VAR>::T, Var<VAR>::B) k_hop(const HopArgs<SP, LK, CL> args, int ngy)
+__global__ void __launch_bounds__(Var<VAR>::T, Var<VAR>::B) k_hop(const HopParam<MODE, SP, LK, CL> args, int ngy)
 {
     after_previous();
-    const HopArgs<SP, LK, CL> a = hop_args<MODE>(args);
+    const HopArgs<SP, LK, CL> &a = hop_args(args);
     const int gy = blockIdx.x % ngy, tile = blockIdx.x / ngy;
     const int r = tile * blockDim.x + threadIdx.x;
     const int k = gy * blockDim.y + threadIdx.y;
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(256) k_hop_batch(const HopArgs<SP, LK, CL> *ar
 }
 
 template <class R, class SP, class LK, class CL, int MODE>
-lqcd_status launch_var(lqcd_ctx *c, int var, dim3 b, const HopArgs<SP, LK, CL> &a)
+lqcd_status launch_var(lqcd_ctx *c, int var, dim3 b, const HopArgs2<SP, LK, CL> &a)
 {
     const int ngy = div_up(a.nrhs, b.y);
     const long nb = (long)div_up(c->g.Vh, b.x) * ngy;
@@ -247,7 +247,7 @@ std::vector<TuneChoice> hop_d_candidates(int only)
 }
 
 template <class R, class SP, class LK, class CL, int MODE>
-lqcd_status launch_choice(lqcd_ctx *c, const TuneChoice &t, const HopArgs<SP, LK, CL> &a)
+lqcd_status launch_choice(lqcd_ctx *c, const TuneChoice &t, const HopArgs2<SP, LK, CL> &a)
 {
     if constexpr (std::is_same<R, float>::value && MODE != MODE_HOP) {
         if (t.kind == KIND_MR) return launch_hop_mr<R, SP, LK, CL, MODE>(c, t.nr, t.variant, dim3(t.tx, t.ty), a);
@@ -265,7 +265,7 @@ lqcd_status launch_hop(lqcd_ctx *c, int p_out, const SP *in_other, long in_rs, c
                        const SP *in_other1 = nullptr, const SP *in_same1 = nullptr, SP *out1 = nullptr,
                        const CL *clov1 = nullptr)
 {
-    HopArgs<SP, LK, CL> a;
+    HopArgs2<SP, LK, CL> a;
     a.in_other1 = in_other1;
     a.in_same1 = in_same1;
     a.out1 = out1;

@@ -185,12 +185,12 @@ struct BlkExt {
     int bs[4];
 };
 template <int MODE, int G, bool BLK = false>
-__global__ void __launch_bounds__(HOP_D_THREADS, 3) k_hop_d(const HopArgs<double2, double2, double2> args,
+__global__ void __launch_bounds__(HOP_D_THREADS, 3) k_hop_d(const HopParam<MODE, double2, double2, double2> args,
                                                             BlkExt bx)
 {
     constexpr int P = 2 * G, SW = 32 / P;
     after_previous();
-    const HopArgs<double2, double2, double2> a = hop_args<MODE>(args);
+    const HopArgs<double2, double2, double2> &a = hop_args(args);
     const long Vh = a.g.Vh;
     const int kf = blockIdx.x % a.nrhs;
     const int lane = threadIdx.x & 31, part = lane / SW, s = part & 1;
@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(HOP_D_THREADS, 3) k_hop_d(const HopArgs<double
 
 namespace {
 template <int MODE, bool BLK>
-lqcd_status launch_d(lqcd_ctx *c, int G, const HopArgs<double2, double2, double2> &a, BlkExt bx)
+lqcd_status launch_d(lqcd_ctx *c, int G, const HopArgs2<double2, double2, double2> &a, BlkExt bx)
 {
     const int sites = HOP_D_THREADS / (2 * G);   // per CTA
     const long nb = (long)div_up(c->g.Vh, sites) * a.nrhs;
@@ -343,14 +343,14 @@ lqcd_status launch_d(lqcd_ctx *c, int G, const HopArgs<double2, double2, double2
 }  // namespace
 
 template <int MODE>
-lqcd_status launch_hop_d(lqcd_ctx *c, int G, const HopArgs<double2, double2, double2> &a)
+lqcd_status launch_hop_d(lqcd_ctx *c, int G, const HopArgs2<double2, double2, double2> &a)
 {
     return launch_d<MODE, false>(c, G, a, BlkExt{});
 }
 
 lqcd_status launch_dhat_block_d(lqcd_ctx *c, const int bs[4], const double2 *in, double2 *tmp, double2 *out)
 {
-    HopArgs<double2, double2, double2> a = {};
+    HopArgs2<double2, double2, double2> a = {};
     a.g = c->g;
     a.nrhs = 1;
     a.in_rs = a.same_rs = a.out_rs = 0;
@@ -373,9 +373,9 @@ lqcd_status launch_dhat_block_d(lqcd_ctx *c, const int bs[4], const double2 *in,
     return launch_d<MODE_DHAT2, true>(c, G, a, bx);
 }
 
-template lqcd_status launch_hop_d<MODE_HOP>(lqcd_ctx *, int, const HopArgs<double2, double2, double2> &);
-template lqcd_status launch_hop_d<MODE_DHAT1>(lqcd_ctx *, int, const HopArgs<double2, double2, double2> &);
-template lqcd_status launch_hop_d<MODE_DHAT2>(lqcd_ctx *, int, const HopArgs<double2, double2, double2> &);
-template lqcd_status launch_hop_d<MODE_D>(lqcd_ctx *, int, const HopArgs<double2, double2, double2> &);
+template lqcd_status launch_hop_d<MODE_HOP>(lqcd_ctx *, int, const HopArgs2<double2, double2, double2> &);
+template lqcd_status launch_hop_d<MODE_DHAT1>(lqcd_ctx *, int, const HopArgs2<double2, double2, double2> &);
+template lqcd_status launch_hop_d<MODE_DHAT2>(lqcd_ctx *, int, const HopArgs2<double2, double2, double2> &);
+template lqcd_status launch_hop_d<MODE_D>(lqcd_ctx *, int, const HopArgs2<double2, double2, double2> &);
 
 }  // namespace stencil

@@ -99,10 +99,10 @@ struct VarMR<2> {
 // all field groups of a site tile run next to each other and share its links
 // and clover term through L1/L2.
 template <class R, class SP, class LK, class CL, int MODE, int NR, int VAR>
-__global__ void __launch_bounds__(VarMR<VAR>::T, VarMR<VAR>::B) k_hop_mr(const HopArgs<SP, LK, CL> args, int ngy)
+__global__ void __launch_bounds__(VarMR<VAR>::T, VarMR<VAR>::B) k_hop_mr(const HopParam<MODE, SP, LK, CL> args, int ngy)
 {
     after_previous();
-    const HopArgs<SP, LK, CL> a = hop_args<MODE>(args);
+    const HopArgs<SP, LK, CL> &a = hop_args(args);
     const int gy = blockIdx.x % ngy, tile = blockIdx.x / ngy;
     const int r = tile * blockDim.x + threadIdx.x;
     const int k0 = (gy * blockDim.y + threadIdx.y) * NR;
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(VarMR<VAR>::T, VarMR<VAR>::B) k_hop_mr(const H
 }
 
 template <class R, class SP, class LK, class CL, int MODE, int NR>
-void launch_nr(bool pdl, int var, dim3 grid, dim3 b, int ngy, cudaStream_t st, const HopArgs<SP, LK, CL> &a)
+void launch_nr(bool pdl, int var, dim3 grid, dim3 b, int ngy, cudaStream_t st, const HopArgs2<SP, LK, CL> &a)
 {
     switch (var) {
         case 0: launch_pdl(pdl, k_hop_mr<R, SP, LK, CL, MODE, NR, 0>, grid, b, st, a, ngy); break;
@@ -195,7 +195,7 @@ void launch_nr(bool pdl, int var, dim3 grid, dim3 b, int ngy, cudaStream_t st, c
 }  // namespace
 
 template <class R, class SP, class LK, class CL, int MODE>
-lqcd_status launch_hop_mr(lqcd_ctx *c, int nr, int var, dim3 b, const HopArgs<SP, LK, CL> &a)
+lqcd_status launch_hop_mr(lqcd_ctx *c, int nr, int var, dim3 b, const HopArgs2<SP, LK, CL> &a)
 {
     const int groups = (a.nrhs + nr - 1) / nr;
     const int ngy = div_up(groups, b.y);
@@ -214,7 +214,7 @@ lqcd_status launch_hop_mr(lqcd_ctx *c, int nr, int var, dim3 b, const HopArgs<SP
 }
 
 #define LQCD_MR_INST(R, SP, LK, CL, MODE) \
-    template lqcd_status launch_hop_mr<R, SP, LK, CL, MODE>(lqcd_ctx *, int, int, dim3, const HopArgs<SP, LK, CL> &);
+    template lqcd_status launch_hop_mr<R, SP, LK, CL, MODE>(lqcd_ctx *, int, int, dim3, const HopArgs2<SP, LK, CL> &);
 LQCD_MR_INST(float, float4, float4, float4, MODE_DHAT1)
 LQCD_MR_INST(float, float4, float4, float4, MODE_DHAT2)
 LQCD_MR_INST(float, float4, float4, float4, MODE_D)

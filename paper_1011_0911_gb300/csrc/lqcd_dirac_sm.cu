@@ -119,10 +119,10 @@ struct VarSM<2> {
 };
 
 template <class SP, class LK, class CL, int MODE, int TS, int VAR>
-__global__ void __launch_bounds__(VarSM<VAR>::T, VarSM<VAR>::B) k_hop_sm(const HopArgs<SP, LK, CL> args, int ngy)
+__global__ void __launch_bounds__(VarSM<VAR>::T, VarSM<VAR>::B) k_hop_sm(const HopParam<MODE, SP, LK, CL> args, int ngy)
 {
     after_previous();
-    const HopArgs<SP, LK, CL> a = hop_args<MODE>(args);
+    const HopArgs<SP, LK, CL> &a = hop_args(args);
     __shared__ SmStage<TS> S;
     const long Vh = a.g.Vh;
     // one-dimensional grid, the field blocks of a site tile next to each other
@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(VarSM<VAR>::T, VarSM<VAR>::B) k_hop_sm(const H
 }
 
 template <class SP, class LK, class CL, int MODE, int TS>
-void launch_ts(bool pdl, int var, dim3 grid, dim3 b, int ngy, cudaStream_t st, const HopArgs<SP, LK, CL> &a)
+void launch_ts(bool pdl, int var, dim3 grid, dim3 b, int ngy, cudaStream_t st, const HopArgs2<SP, LK, CL> &a)
 {
     switch (var) {
         case 0: launch_pdl(pdl, k_hop_sm<SP, LK, CL, MODE, TS, 0>, grid, b, st, a, ngy); break;
@@ -204,7 +204,7 @@ void launch_ts(bool pdl, int var, dim3 grid, dim3 b, int ngy, cudaStream_t st, c
 }  // namespace
 
 template <class R, class SP, class LK, class CL, int MODE>
-lqcd_status launch_hop_sm(lqcd_ctx *c, int var, dim3 b, const HopArgs<SP, LK, CL> &a)
+lqcd_status launch_hop_sm(lqcd_ctx *c, int var, dim3 b, const HopArgs2<SP, LK, CL> &a)
 {
     const int ngy = div_up(a.nrhs, b.y);
     const long nb = (long)div_up(c->g.Vh, b.x) * ngy;
@@ -222,7 +222,7 @@ lqcd_status launch_hop_sm(lqcd_ctx *c, int var, dim3 b, const HopArgs<SP, LK, CL
 }
 
 #define LQCD_SM_INST(SP, LK, CL, MODE) \
-    template lqcd_status launch_hop_sm<float, SP, LK, CL, MODE>(lqcd_ctx *, int, dim3, const HopArgs<SP, LK, CL> &);
+    template lqcd_status launch_hop_sm<float, SP, LK, CL, MODE>(lqcd_ctx *, int, dim3, const HopArgs2<SP, LK, CL> &);
 LQCD_SM_INST(float4, float4, float4, MODE_DHAT1)
 LQCD_SM_INST(float4, float4, float4, MODE_DHAT2)
 LQCD_SM_INST(float4, float4, float4, MODE_D)
