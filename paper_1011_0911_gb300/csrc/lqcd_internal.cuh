@@ -356,8 +356,6 @@ enum {
 lqcd_status ws_get(lqcd_ctx *c, int slot, size_t bytes, void **out);
 
 // native element counts per site
-inline int native_chunks(lqcd_prec p) { return p == LQCD_F64 ? 12 : (p == LQCD_F32 ? 6 : 3); }
-inline size_t native_chunk_bytes(lqcd_prec p) { return p == LQCD_F64 ? 16 : (p == LQCD_F32 ? 16 : 16); }
 size_t native_half_bytes(const lqcd_ctx *c, lqcd_prec p);   // one rhs, one parity
 inline long native_half_units(const lqcd_ctx *c, lqcd_prec p)   // in 16-byte units
 {
@@ -368,9 +366,15 @@ inline long native_half_units(const lqcd_ctx *c, lqcd_prec p)   // in 16-byte un
 // still running (programmatic dependent launch); the kernel begins with
 // after_previous(), which waits until that kernel has finished and its writes are
 // visible.  It hides about 2 us per kernel: Dhat FP64 on 8^4 (four kernels) 28.7
-// -> 19.3 us.  Kernels must let the next one be set up only after their own wait:
-// signalled before it, the launches of a chain pile up on the SMs (43.6 us).  In
-// captured graphs plain launches are faster (CGNR on 8^4: 6.97 against 7.97 ms).
+// -> 19.3 us.  The CTAs set up early go to the SMs that come free first; where that
+// spreads a kernel of about one wave unevenly it costs up to a third, so stencils
+// (run_operator) and SAP sweeps choose.  The coarse solve's kernels are faster with it
+// at every size timed (a deflated step of one field 0.68 at 8^4 to 0.93 at 48 x 24^3 of
+// its time with plain launches), the canonical conversions at all but a few (calls of
+// 0.8 to 1.03, one of 1.2, of their time with plain launches).  Kernels must let the
+// next one be set up only after their own wait: signalled before it, the launches of
+// a chain pile up on the SMs (43.6 us).  In captured graphs plain launches are faster
+// (CGNR on 8^4: 6.97 against 7.97 ms).
 // A launch that fails leaves its error for LQCD_LAUNCH_CHECK, as <<< >>> does.
 template <class... KP, class... A>
 inline void launch_pdl_smem(bool pdl, void (*kernel)(KP...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,

@@ -8,9 +8,10 @@
 // is, the even half of its output is the search direction, and D phi_k needs
 // Dhat phi_e alone (as many hops as D).  Every Krylov vector, dot product and
 // update has half the length, and the residual is that of the Dhat system
-// itself (Eq. 5 only bounds it by the full one).  Measured with unchanged
-// iteration counts: 32 x 16^3, one source, FP32 SAP, FP64 Krylov vectors 70.9 ->
-// 58.4 ms; 48 x 24^3, 12 sources, deflated, build included 1218 -> 1101 ms.
+// itself (Eq. 5 only bounds it by the full one, so that the full-lattice form went
+// on with a tighter tolerance where needed).  Iteration counts are the same or
+// lower: 62 at 32 x 16^3, one source, FP32 SAP, FP64 Krylov vectors, 70.9 -> 58.4 ms; 27 ->
+// 26 at 48 x 24^3, 12 sources, deflated, build included 1218 -> 1101 ms.
 //
 // Precision: the residual, the solution update and the restart residual
 // eta - D psi are FP64.  The preconditioner and D phi_k may run in FP32
