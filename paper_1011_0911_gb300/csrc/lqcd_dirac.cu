@@ -94,7 +94,7 @@ template <class R, class SP, class LK, class CL, int MODE, int VAR>
 __global__ void __launch_bounds__(Var<VAR>::T, Var<VAR>::B) k_hop(const HopParam<MODE, SP, LK, CL> args, int ngy)
 {
     after_previous();
-    const HopArgs<SP, LK, CL> &a = hop_args(args);
+    const HopArgs<SP, LK, CL> &a = hop_args<MODE>(args);
     const int gy = blockIdx.x % ngy, tile = blockIdx.x / ngy;
     const int r = tile * blockDim.x + threadIdx.x;
     const int k = gy * blockDim.y + threadIdx.y;

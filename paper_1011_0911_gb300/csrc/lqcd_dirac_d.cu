@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(HOP_D_THREADS, 3) k_hop_d(const HopParam<MODE,
 {
     constexpr int P = 2 * G, SW = 32 / P;
     after_previous();
-    const HopArgs<double2, double2, double2> &a = hop_args(args);
+    const HopArgs<double2, double2, double2> &a = hop_args<MODE>(args);
     const long Vh = a.g.Vh;
     const int kf = blockIdx.x % a.nrhs;
     const int lane = threadIdx.x & 31, part = lane / SW, s = part & 1;

@@ -122,7 +122,7 @@ template <class SP, class LK, class CL, int MODE, int TS, int VAR>
 __global__ void __launch_bounds__(VarSM<VAR>::T, VarSM<VAR>::B) k_hop_sm(const HopParam<MODE, SP, LK, CL> args, int ngy)
 {
     after_previous();
-    const HopArgs<SP, LK, CL> &a = hop_args(args);
+    const HopArgs<SP, LK, CL> &a = hop_args<MODE>(args);
     __shared__ SmStage<TS> S;
     const long Vh = a.g.Vh;
     // one-dimensional grid, the field blocks of a site tile next to each other

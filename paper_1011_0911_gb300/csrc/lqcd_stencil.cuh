@@ -383,9 +383,11 @@ struct HopArgs {
     const CL *clov;   // parity p_out: A^-1 (DHAT1) or A (DHAT2, D)
 };
 // MODE_D writes both parities in one launch: the members of HopArgs are output
-// parity 0 (blockIdx.y = 0), these parity 1.  Kernels of the other modes take HopArgs:
-// with these members in their parameters the compiler made DHAT1 up to 9 % slower
-// (FP32, five fields at 48 x 24^3: 141 -> 153 us).
+// parity 0 (blockIdx.y = 0), these parity 1.  Kernels of the other modes take HopArgs
+// but for DHAT2 in FP32: the size of the parameters alone changes what the compiler
+// makes of a kernel.  48 x 24^3, with / without these members: DHAT1 FP32, five fields
+// 153 / 141 us, twelve 312 / 308; DHAT2 FP32 159 / 165, 344 / 351; F16S, three fields, DHAT1
+// 88 / 82, DHAT2 94 / 90.
 template <class SP, class LK, class CL>
 struct HopArgs2 : HopArgs<SP, LK, CL> {
     const SP *in_other1, *in_same1;
@@ -393,18 +395,19 @@ struct HopArgs2 : HopArgs<SP, LK, CL> {
     const CL *clov1;
 };
 template <int MODE, class SP, class LK, class CL>
-using HopParam = std::conditional_t<MODE == MODE_D, HopArgs2<SP, LK, CL>, HopArgs<SP, LK, CL>>;
+using HopParam = std::conditional_t<MODE == MODE_D || (MODE == MODE_DHAT2 && std::is_same<SP, float4>::value),
+                                    HopArgs2<SP, LK, CL>, HopArgs<SP, LK, CL>>;
 // the arguments of this CTA's output parity
-template <class SP, class LK, class CL>
+template <int MODE, class SP, class LK, class CL>
 __device__ __forceinline__ const HopArgs<SP, LK, CL> &hop_args(const HopArgs<SP, LK, CL> &a)
 {
     return a;
 }
-template <class SP, class LK, class CL>
+template <int MODE, class SP, class LK, class CL>
 __device__ __forceinline__ HopArgs<SP, LK, CL> hop_args(const HopArgs2<SP, LK, CL> &a)
 {
     HopArgs<SP, LK, CL> b = a;
-    if (blockIdx.y) {
+    if (MODE == MODE_D && blockIdx.y) {
         b.p_out = 1;
         b.in_other = a.in_other1;
         b.in_same = a.in_same1;
