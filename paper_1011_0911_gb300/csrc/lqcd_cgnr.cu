@@ -19,7 +19,7 @@
 // expected, on a stream of the context's own (a legacy default stream cannot be
 // captured).  Making the graph takes about 250 us; an iteration costs, with plain
 // launches / in graphs, at 2048 even sites 61 / 50 us, 4096 98 / 74, 8192 173 / 120,
-// 16384 220 / 205.  131 iterations on 8^4: 16.0 -> 6.9 ms (with the state copied to the
+// 16384 220 / 205.  131 iterations on 8^4: 16.0 -> 6.7 ms (with the state copied to the
 // host instead of written there 8.7 ms).
 #include <cmath>
 
