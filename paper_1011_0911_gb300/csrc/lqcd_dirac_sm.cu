@@ -119,7 +119,7 @@ struct VarSM<2> {
 };
 
 template <class SP, class LK, class CL, int MODE, int TS, int VAR>
-__global__ void __launch_bounds__(VarSM<VAR>::T, VarSM<VAR>::B) k_hop_sm(const HopParam<MODE, SP, LK, CL> args, int ngy)
+__global__ void __launch_bounds__(VarSM<VAR>::T, VarSM<VAR>::B) k_hop_sm(const HopArgs2<SP, LK, CL> args, int ngy)
 {
     after_previous();
     const HopArgs<SP, LK, CL> &a = hop_args<MODE>(args);

@@ -384,10 +384,10 @@ struct HopArgs {
 };
 // MODE_D writes both parities in one launch: the members of HopArgs are output
 // parity 0 (blockIdx.y = 0), these parity 1.  Kernels of the other modes take HopArgs
-// but for DHAT2 in FP32: the size of the parameters alone changes what the compiler
-// makes of a kernel.  48 x 24^3, with / without these members: DHAT1 FP32, five fields
-// 153 / 141 us, twelve 312 / 308; DHAT2 FP32 159 / 165, 344 / 351; F16S, three fields, DHAT1
-// 88 / 82, DHAT2 94 / 90.
+// but for DHAT2 in FP32 and the staged form: the size of the parameters alone changes
+// what the compiler makes of a kernel.  48 x 24^3, with / without these members: DHAT1
+// FP32, five fields 153 / 141 us, twelve 312 / 308; DHAT2 FP32 159 / 165, 344 / 351; F16S,
+// three fields, DHAT1 88 / 82, DHAT2 94 / 90; Dhat staged, F16S, twelve fields at 16^4 62 / 75.
 template <class SP, class LK, class CL>
 struct HopArgs2 : HopArgs<SP, LK, CL> {
     const SP *in_other1, *in_same1;
