@@ -371,6 +371,7 @@ lqcd_status launch_hop(lqcd_ctx *c, int p_out, const SP *in_other, long in_rs, c
 // the choice is 1.2 % faster than dependent launches throughout, at most 17 % where
 // those lost.
 constexpr float DEP_LONG_US = 300.f;
+constexpr float DEP_MARGIN = 1.05f;   // behind other kernels dependent launches still save their set-up
 enum { OP_DHAT = 0, OP_D = 1 };
 namespace {
 template <class Run>
@@ -403,7 +404,7 @@ lqcd_status run_operator(lqcd_ctx *c, int op, lqcd_prec p, int nrhs, Run run)
             if (tune_verbose()) fprintf(stderr, "tune %s: dependent=%d %.1f us\n", key.c_str(), rep & 1, us);
             best[rep & 1] = std::min(best[rep & 1], us);
         }
-        t.variant = best[1] <= 1.01f * best[0];
+        t.variant = best[1] <= DEP_MARGIN * best[0];
         t.us = std::min(us, best[t.variant]);
         tune_store(key, t);
     }

@@ -1,6 +1,6 @@
 """D and Dhat with their kernels launched dependently or plainly: the same bits; without a
 recorded choice both are timed, the faster one is kept (dependent launches where they
-are at most 1 % slower), persists in the cache file and is read back."""
+are at most 5 % slower), persists in the cache file and is read back."""
 import json
 import re
 
@@ -44,7 +44,7 @@ def test_choice(op, prec, tmp_path, monkeypatch, capfd):
     (key,) = [k for k in entries if k.startswith(head)]
     plain, dep = min(times["0"]), min(times["1"])
     # printed to 0.1 us
-    assert dep <= 1.01 * plain + 0.11 if entries[key][0] else dep >= 1.01 * plain - 0.11
+    assert dep <= 1.05 * plain + 0.11 if entries[key][0] else dep >= 1.05 * plain - 0.11
     for choice in (0, 1):
         entries[key][0] = choice
         cache.write_text("{\n" + ",\n".join(f'  "{k}": {json.dumps(v)}' for k, v in entries.items()) + "\n}\n")
