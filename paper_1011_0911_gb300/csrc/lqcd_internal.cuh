@@ -378,7 +378,7 @@ inline long native_half_units(const lqcd_ctx *c, lqcd_prec p)   // in 16-byte un
 // A launch that fails leaves its error for LQCD_LAUNCH_CHECK, as <<< >>> does.
 template <class... KP, class... A>
 inline void launch_pdl_smem(bool pdl, void (*kernel)(KP...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                                   A... args)
+                            const A &...args)
 {
     if (!pdl) {
         kernel<<<grid, block, smem, st>>>(args...);
@@ -397,7 +397,7 @@ inline void launch_pdl_smem(bool pdl, void (*kernel)(KP...), dim3 grid, dim3 blo
     cudaLaunchKernelEx(&cfg, kernel, static_cast<KP>(args)...);
 }
 template <class... KP, class... A>
-inline void launch_pdl(bool pdl, void (*kernel)(KP...), dim3 grid, dim3 block, cudaStream_t st, A... args)
+inline void launch_pdl(bool pdl, void (*kernel)(KP...), dim3 grid, dim3 block, cudaStream_t st, const A &...args)
 {
     launch_pdl_smem(pdl, kernel, grid, block, 0, st, args...);
 }
